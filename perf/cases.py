@@ -185,6 +185,114 @@ def run(state):
     return xhat, q8.q8_ste_backward(state["grad"]), S
 
 
+# ------------------------------------------------------------------ the same results in 64 bits, in plain torch
+def _plain_scale(x):
+    m = x.abs().max().float()
+    return torch.full_like(m, 127.0) / m  # (127.0 / m would be computed as 127 times the rounded reciprocal)
+
+
+def _plain_quantize(x, S):
+    """Integers of Eq. 1 as float64.  The paper's product x * S is formed in the precision of x."""
+    return torch.clamp(torch.round(x * S.to(x.dtype)), -127, 127).double()
+
+
+def _plain_linear(Xq, S_x, Wq, S_w, bias, act):
+    """Integer operands held as float64: the matrix product is exact."""
+    S = S_x * S_w
+    y = (Xq @ Wq.T + torch.round(bias * S).double()) / S.double()
+    return torch.nn.functional.gelu(y) if act else y
+
+
+def _plain_layer(g, M, K, N, act, static):
+    """The draws of _layer(), in its order."""
+    X, W = _activation(g, M, K), _weight(g, N, K)
+    S_w = _plain_scale(W)
+    lay = dict(X=X, Wq=_plain_quantize(W, S_w), S_w=S_w, bias=_weight(g, N), act=act)
+    lay["S_x"] = _plain_scale(_activation(g, M, K) if static else X)
+    return lay
+
+
+def _plain_encoder(case, seed):
+    """The whole forward in float64.  A value next to a rounding boundary of a quantiser may fall on its other side here,
+    as it may in any other implementation: the results agree to the size of that noise (see tolerance())."""
+    dims, B, S = DIMS[case["model"]], case["B"], case["S"]
+    H, heads = dims["hidden"], dims["heads"]
+
+    def draw_weight(n, k, index):
+        w = torch.from_numpy(synth.weight(n, k, synth.seed_for(seed, index))).cuda()
+        S_w = _plain_scale(w)
+        return _plain_quantize(w, S_w), S_w
+
+    tables = [draw_weight(n, H, 100 + i) for i, n in enumerate((dims["vocab"], dims["max_pos"], 2))]
+    layers = [[draw_weight(N, K, 200 + 20 * l + 2 * i)
+               + (torch.from_numpy(synth.bias(N, synth.seed_for(seed, 200 + 20 * l + 2 * i + 1))).cuda(), act)
+               for i, (_, K, N, act) in enumerate(synth.fc_set(H, dims["ffn"]))] for l in range(case["layers"])]
+
+    def norm(x):
+        x = x - x.mean(1, keepdim=True)
+        return x / torch.sqrt((x * x).mean(1, keepdim=True) + 1e-12)
+
+    def forward(ids, scales):
+        seen = iter(scales) if scales is not None else None
+        taken = []
+
+        def fc(x, layer):
+            S_x = next(seen) if seen is not None else _plain_scale(x)
+            taken.append(S_x)
+            return _plain_linear(_plain_quantize(x, S_x), S_x, *layer)
+
+        places = torch.arange(S, device="cuda").repeat(B)
+        rows = (ids.long(), places, torch.zeros_like(places))
+        h = norm(sum(E[r] / S_e.double() for (E, S_e), r in zip(tables, rows)))
+        for qkv, attn_out, ffn1, ffn2 in layers:
+            q, k, v = fc(h, qkv).view(B, S, 3, heads, H // heads).permute(2, 0, 3, 1, 4)
+            ctx = torch.softmax(q @ k.transpose(2, 3) / math.sqrt(H // heads), dim=3) @ v
+            h = norm(fc(ctx.transpose(1, 2).reshape(B * S, H), attn_out) + h)
+            h = norm(fc(fc(h, ffn1), ffn2) + h)
+        return h, taken
+
+    ids = random_ids(B * S, dims["vocab"], seed)
+    if case["mode"] == "dynamic":
+        return forward(ids, None)[0]
+    # the first calibration batch sets the running maximum
+    return forward(ids, forward(random_ids(B * S, dims["vocab"], seed + 1), None)[1])[0]
+
+
+def exact(case, seed):
+    g = _generator(seed)
+    kind = case["kind"]
+    if kind == "linear":
+        a = _plain_layer(g, case["M"], case["K"], case["N"], case["act"], case["scale"] == "static")
+        return _plain_linear(_plain_quantize(a["X"], a["S_x"]), a["S_x"], a["Wq"], a["S_w"], a["bias"], a["act"])
+    if kind == "ffn":
+        M, H, F = case["M"], case["H"], case["F"]
+        a, b = _plain_layer(g, M, H, F, 1, True), _plain_layer(g, M, F, H, 0, True)
+        mid = _plain_linear(_plain_quantize(a["X"], a["S_x"]), a["S_x"], a["Wq"], a["S_w"], a["bias"], a["act"])
+        mid = _plain_quantize(mid.float(), b["S_x"])
+        return _plain_linear(mid, b["S_x"], b["Wq"], b["S_w"], b["bias"], b["act"]), mid.to(torch.int8)
+    if kind == "fc_set":
+        dims, M = DIMS[case["model"]], case["M"]
+        outs = []
+        for _, K, N, act in synth.fc_set(dims["hidden"], dims["ffn"]):
+            a = _plain_layer(g, M, K, N, act, True)
+            outs.append(_plain_linear(_plain_quantize(a["X"], a["S_x"]), a["S_x"], a["Wq"], a["S_w"], a["bias"], a["act"]))
+        E = _weight(g, dims["vocab"], dims["hidden"])
+        ids = torch.randint(dims["vocab"], (M,), generator=g, device="cuda", dtype=torch.int32)
+        S_e = _plain_scale(E)
+        return [_plain_quantize(E[ids.long()], S_e) / S_e.double()] + outs
+    if kind == "encoder":
+        return _plain_encoder(case, seed)
+    if kind == "weights":
+        W = _weight(g, case["N"], case["K"])
+        S_w = _plain_scale(W)
+        return _plain_quantize(W, S_w).to(torch.int8), S_w.double().reshape(1)
+    X = _activation(g, case["M"], case["K"])
+    ema = _activation(g, case["M"], case["K"]).abs().max().double()
+    grad = torch.randn(X.shape, generator=g, device="cuda")
+    S = _plain_scale(ema + (1.0 - DECAY) * (X.abs().max().double() - ema))
+    return _plain_quantize(X, S) / S.double(), grad.double(), S.double().reshape(1)
+
+
 # ------------------------------------------------------------------ what a pass cannot do without
 def _linear_work(M, K, N, in_bytes=4, out_bytes=4):
     return M * K * in_bytes + N * K + 4 * N + M * N * out_bytes, 2 * M * N * K
