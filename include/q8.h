@@ -248,13 +248,12 @@ const char *q8_status_string(q8_status s);
  * any pointer may be NULL. */
 void q8_last_launch_info(int *gemm_kernel, int *launches, int *block_n, int *grid, int *ctas);
 
-/* q8_attention / q8_attention_quant run on the tensor cores when the padded sequence fits the accumulator
- * memory (S rounded up to a multiple of 64, plus 64, at most 512 columns: S <= 448) and the pointers are
- * 16-byte aligned: both products as tcgen05.mma kind::tf32 on operands split into a TF32-exact high part and a
- * low remainder, three partial products accumulated in fp32, which keeps fp32-grade accuracy.  Otherwise a
- * CUDA-core fp32 kernel computes the same thing.  The tensor-core kernel bounds
- * its waits; a time-out sets the Q8_ERR_TIMEOUT bit in a per-device status word whose device address
- * q8_attention_status_word returns (poll it with q8_poll_status). */
+/* q8_attention / q8_attention_quant run on the tensor cores when the pointers are 16-byte aligned: both products as
+ * tcgen05.mma on operands split into two 16-bit (kind::f16, scaled by powers of two) or TF32 parts each, three
+ * partial products accumulated in fp32, which keeps fp32-grade accuracy (an infinite input gives NaN where the
+ * exact result would be infinite).  Otherwise a CUDA-core fp32 kernel computes the same thing.  The tensor-core
+ * kernels bound their waits; a time-out sets the Q8_ERR_TIMEOUT bit in a per-device status word whose device
+ * address q8_attention_status_word returns (poll it with q8_poll_status). */
 q8_status q8_attention_status_word(void **dev_status);
 
 #ifdef __cplusplus

@@ -536,7 +536,7 @@ def q8_selftest_wait_timeout(limit_ns: int, dev_status: torch.Tensor, dev_report
 
 
 def q8_tune_attention(use_tensor_cores: bool = True) -> None:
-    """Chooses between the tensor-core (3 x TF32) and the CUDA-core fp32 attention kernel for later calls."""
+    """Chooses between the tensor-core (split operands) and the CUDA-core fp32 attention kernel for later calls."""
     load().q8_tune_attention(1 if use_tensor_cores else 0)
 
 

@@ -1,28 +1,36 @@
-// Multi-head self-attention (head dimension 64, no mask) on the Blackwell tensor cores with fp32-grade
-// accuracy: both products, Q K^T and P V, run as tcgen05.mma kind::tf32 with every fp32 operand split into
-// a TF32-exact high part (x rounded to nearest TF32) and the low remainder (x = hi + lo exactly), and
-// the three significant partial products hi*hi + hi*lo + lo*hi are accumulated in fp32 in TMEM.  The dropped
-// lo*lo term is below 2^-22 relative per product, i.e. at the rounding level of a plain fp32 dot product.
+// Multi-head self-attention (head dimension 64, no mask, any sequence length) on the Blackwell tensor cores with
+// fp32-grade accuracy.  Both products, Q K^T and P V, run as tcgen05.mma kind::f16 with every fp32 operand x scaled by
+// a power of two (exactly) and split into two fp16 numbers, hi = fp16(x) and lo = fp16(x - hi): 22 to 23 significant
+// bits, accumulated in fp32 in TMEM as lo*hi + hi*lo + hi*hi; the dropped lo*lo term is below 2^-22 relative per product,
+// i.e. at the rounding level of a plain fp32 dot product.  The scale comes from the data (largest finite |x| of a Q row, of
+// each K chunk and of each V chunk brought into [2^13, 2^14)), so fp16's narrow exponent costs nothing: relative to
+// that largest value a smaller one keeps an absolute error of 2^-39.  The scales are undone in fp32, inside the FFMA that
+// the softmax needs anyway.  (Split TF32 operands, which need no scales, have half the MMA rate and twice the
+// shared-memory bytes; grids that do not fill the device still use them, see launch_attention_tc().)
 // (The paper keeps attention in fp32 and quantises only the FC layers; this kernel is the fp32 attention an
 // encoder forward needs around them.)
 //
-// One CTA = 128 queries of one (sequence, head): 16 worker warps plus one warp that only issues MMAs.
-// All operands are staged by the workers themselves (global -> registers -> split -> shared memory in the
-// K-major 128-byte-swizzled layout the MMA reads); no TMA, no multicast.  Chunks of keys go through two (phase 1)
-// or three (phase 2) buffer sets, so the MMAs of chunk c run while the workers prepare the chunks after it:
-//   phase 1  Q tile (scaled by log2(e)/8) -> Q_hi, Q_lo; per 128 keys: K rows -> K_hi, K_lo; 24 MMAs with N = 128
-//            (2 swizzle spans x 4 K steps x 3 partial products) -> scores in TMEM columns [128 c, 128 c + 128); the
-//            row maxima are read from TMEM chunk by chunk behind the MMAs (a row is shared by four threads)
-//   phase 2  per chunk: p = 2^(s - max) -> P_hi (back into tensor memory over the chunk's scores: the A operand is
-//            read from there), P_lo (shared memory; keys along K); V chunk transposed ->
-//            [V_hi ; V_lo] stacked as one 128-row B operand, so that one N = 128 MMA yields P_hi V_hi (columns
-//            0..63 of the O accumulator) and P_hi V_lo (columns 64..127), and one N = 64 MMA adds P_lo V_hi to the
-//            latter: 16 MMAs per chunk.  Keeping the small products in columns of their own also leaves a single
-//            rounding per K step on the long accumulation chain.
-//   phase 3  (O_main + O_corr) / row sum -> ctx (and optionally Int8 at the next layer's scale)
-// The whole score row block lives in TMEM (S_pad + 128 <= 512 columns), so the softmax needs no running
-// rescale.  Workers and the MMA warp meet only through mbarriers, and every wait on one is bounded: on a
-// time-out the CTA raises Q8_ERR_TIMEOUT in the status word, every role leaves its loops and TMEM is freed.
+// One CTA = 128 queries of one (sequence, head), two CTAs per SM (97 KB of shared memory and 256 TMEM columns each), so that
+// one CTA's waits run under the other's work.  Keys come in chunks of 64 through two buffers each for K, V and the scores,
+// so the scores of chunk c + 1 are computed while the softmax works on chunk c.  Roles:
+//   warps 0..3  softmax: one thread per query row (no exchange between threads at all): scores out of TMEM, running
+//               maximum, p = 2^(s - max), both fp16 parts of p back into TMEM over the scores, from where the second
+//               product takes them as its A operand.  P V of one chunk is a fresh accumulation (small partial products
+//               first); the running output lives in 64 registers of the row's thread and is added to in fp32, because the
+//               tensor core truncates when it accumulates: one chain over 512 keys had an error of 6.6e-7 of |ctx|, growing
+//               with the length (now 1.7e-7 at any length, inputs ~ N(0, 0.55); plain fp32 FMAs: 4.2e-7).  The output is
+//               rescaled only when a row's maximum has risen by more than 2^8 (p has room for that).
+//   warps 4..7  staging: K and V global -> registers -> scale, split -> shared memory, 128-byte-swizzled rows of 64 fp16.  K
+//               is a K-major operand; V keeps its [key][feature] order and is read as an MN-major operand.
+//   warp 8      issues the MMAs (converged, one elected lane); the rest of its warpgroup is there for setmaxnreg, which gives
+//               the softmax 120 registers a thread and the staging 96 (with 96 for all, O was spilled).
+// Measured (64 x 384 x 16 heads / 16 x 512 x 12 / 32 x 128 x 12, Int8 output): 236 / 77 / 19.5 us; split TF32 with whole score
+// rows in TMEM, one CTA per SM, 512 threads staging: 304 / - / 23.8 us (it takes S <= 384; plain fp32 FMAs needed 413 us at
+// 512).  What bounds it now is latency: loads of K and V (without them 25 % less) and the chain softmax -> P V -> scores
+// between the roles, with the issue slots 40 % busy and the tensor pipe 20 %.  Tried and dropped: a persistent grid (the
+// item loop's state does not fit the registers, 250 us), 16-column softmax loops (242 us), Q in shared memory (259 us).
+// The roles meet only through mbarriers, and every wait on one is bounded: on a time-out the CTA raises Q8_ERR_TIMEOUT
+// in the status word, every role leaves its loop and TMEM is freed.
 
 #include "q8_internal.cuh"
 #include "q8_sm100_ptx.cuh"
@@ -34,33 +42,28 @@ namespace {
 using namespace ptx;
 
 constexpr int kHeadDim = 64;
-constexpr int kQTile = 128;    // queries per CTA = TMEM lanes
-constexpr int kChunk = 64;     // keys per chunk = N of the score MMA = K extent of one P / V chunk
-constexpr int kWorkers = 512;  // 16 warps: four per TMEM lane quarter, each taking 16 of a chunk's 64 columns
-constexpr int kThreads = kWorkers + 32;        // + the MMA warp
-constexpr int kSpanBytesA = kQTile * 128;      // one swizzle span (32 fp32 of K) of a 128-row operand: 16 KB
-constexpr int kSpanBytesB = 2 * kChunk * 128;  // ... of the 64-row operand, hi rows then lo rows: 16 KB
-constexpr int kLoRowsB = kChunk * 128;         // offset of the lo rows inside a B span
-constexpr int kBufQP = 4 * kSpanBytesA;        // {hi, lo} x 2 spans: Q, then P
-constexpr int kBufKV = 2 * kSpanBytesB;        // 2 spans x [hi ; lo]: K, then V^T
-constexpr int kAttnTcSmemBytes = 1024 + 2 * kBufQP + 2 * kBufKV;  // 193 KB
-// Phase 2 needs V^T (hi and lo: kBufKV) and P_lo (half of kBufQP) per chunk: three such sets fill the same 192 KB
-// (against two sets: 325.7 -> 322.5 us for 64 x 384 x 16 heads).
-constexpr int kSets2 = 3;
-constexpr int kSet2Bytes = kBufKV + kBufQP / 2;
-static_assert(kSets2 * kSet2Bytes == 2 * kBufQP + 2 * kBufKV, "three phase-2 buffer sets use the whole allocation");
-// Phase 1 takes keys 128 at a time (N = 128 score MMAs: half as many instructions, each reading Q once for twice
-// the columns).  Its two K buffers of 64 KB ([hi 128 rows | lo 128 rows] per span) lie behind Q; phase 2 reuses the
-// whole allocation for its three buffer sets.
-constexpr int kBigChunk = 2 * kChunk;
-constexpr int kSpanBytesK = 2 * kBigChunk * 128;  // one span of a 128-key K buffer, hi rows then lo rows: 32 KB
-constexpr int kLoRowsK = kBigChunk * 128;
-static_assert(kBufQP + 2 * (2 * kSpanBytesK) == 2 * kBufQP + 2 * kBufKV, "Q and the two K buffers of phase 1 fill the allocation");
+constexpr int kQTile = 128;  // queries per CTA = TMEM lanes
+constexpr int kChunk = 64;   // keys per chunk
+constexpr int kSoftmaxWarps = 4, kStagingWarps = 4;
+constexpr int kThreads = 384;  // three warpgroups: softmax, staging, and one whose first warp issues the MMAs
+// Registers per thread after the redistribution between the warpgroups; their sum must not exceed what the CTA is launched
+// with (checked on the host: an increase that cannot be served would wait for ever).
+constexpr int kLaunchRegs = 80, kSoftmaxRegs = 120, kStagingRegs = 96, kIssuerRegs = 24;
+static_assert(kSoftmaxRegs + kStagingRegs + kIssuerRegs <= 3 * kLaunchRegs, "register split");
+constexpr int kRowBytes = kHeadDim * 4;      // an fp32 row of Q or of the output
+constexpr int kQBytes = kQTile * kRowBytes;  // fp32 Q on its way in, the output on its way out: 32 KB
+constexpr int kKvHalfBytes = kChunk * 128;   // rows of 64 fp16: the hi (or the lo) half of a K or V chunk, 8 KB
+constexpr int kKvBytes = 2 * kKvHalfBytes;
+constexpr int kAttnTcSmemBytes = 1024 + 4 * kKvBytes + kQBytes;  // two K, two V buffers, Q: 97 KB
+constexpr uint32_t kTmemCols = 256;  // scores / P of two chunks, P V of one, Q (32 columns of hi parts, 32 of lo parts)
+constexpr uint32_t kColPV = 128, kColQ = 192;
+constexpr float kLog2eOver8 = 1.4426950408889634f / 8.0f;  // log2(e) / sqrt(64): the softmax uses 2^x
+constexpr int kPShift = 7;           // p is split as 2^7 p: at most 2^15 with the stale-maximum slack below, and small p keep
+constexpr float kStaleSlack = 8.0f;  // their precision (fp16 rounds absolutely below 2^-14)
 
-// tcgen05.mma kind::tf32 instruction descriptor: D = F32, A = B = TF32, both K-major, M = 128.
-constexpr uint32_t kIdescBase = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kQTile >> 4) << 24);
-constexpr uint32_t kIdescN64 = kIdescBase | ((uint32_t)(kChunk >> 3) << 17);         // N = 64
-constexpr uint32_t kIdescN128 = kIdescBase | ((uint32_t)((2 * kChunk) >> 3) << 17);  // N = 128
+// tcgen05.mma kind::f16 instruction descriptor: D = F32, A = B = F16, M = 128; bit 16: B is MN-major.
+constexpr uint32_t kIdescBase = (1u << 4) | ((uint32_t)(kQTile >> 4) << 24);
+constexpr uint32_t kIdescPV = kIdescBase | (1u << 16) | ((uint32_t)(kHeadDim >> 3) << 17);
 
 // Byte offset of the 16-byte piece `piece` (0..7) of row `row` inside one swizzle span (rows of 128 bytes,
 // groups of 8 rows 1024 bytes apart, piece index XORed with the row's position in its group).
@@ -69,46 +72,157 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int piece)
     return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((piece ^ (row & 7)) << 4));
 }
 
-// x = hi + lo with hi = x rounded to nearest TF32 (10 explicit mantissa bits, ties away from zero), so
-// |lo| <= 2^-12 |x|; lo has up to 12 significant bits, of which the tensor core's truncation of its operands
-// keeps 11: an error below 2^-23 |x|.  (Clearing the low bits of x instead would double |lo| and with it that
-// error.)  The rounding is done on the integer pipe - add half a TF32 ulp to the bit pattern, clear the 13 low
-// bits - which gives what cvt.rna.tf32.f32 gives without loading the conversion unit (22 results per clock and SM).
-__device__ __forceinline__ float round_tf32(float x)
+// Descriptor of the [key][feature] tile of V as an MN-major B operand: 64 features (one 128-byte swizzle span) per atom of 8
+// keys, atoms 1024 bytes apart along the keys (stride byte offset); the leading byte offset would be the step to further
+// features.
+__device__ __forceinline__ uint64_t smem_desc_v(uint32_t saddr)
 {
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(kKvHalfBytes >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           (1ull << 46) | (2ull << 61);
 }
 
-__device__ __forceinline__ void store_split4(uint8_t *hi_at, uint8_t *lo_at, float4 v)
+// D[tmem] (+)= A B^T, fp32 accumulation.  A from tensor memory: lane = row, two fp16 of K per 32-bit column (8 columns per
+// instruction); read from shared memory, a 128 x 16 operand costs more than the 64 x 16 one of K or V (48 against 32 cycles).
+__device__ __forceinline__ void umma_f16_ts_elected(uint32_t elected, uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b,
+                                                    uint32_t idesc, uint32_t accumulate)
 {
-    float4 h;
-    h.x = round_tf32(v.x);
-    h.y = round_tf32(v.y);
-    h.z = round_tf32(v.z);
-    h.w = round_tf32(v.w);
-    *reinterpret_cast<float4 *>(hi_at) = h;
-    *reinterpret_cast<float4 *>(lo_at) = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);  // exact
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(elected)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x8(uint32_t taddr, const uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
 }
 
-__device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+// {hi, lo} = fp16 pairs of two values (the first in the low half): hi = fp16(x), lo = fp16(x - hi), the difference exact in
+// fp32.  The subtraction is the mixed-precision FMA hi * -1 + x, which takes hi as it is.
+__device__ __forceinline__ uint32_t pack_f16x2(float a, float b)
+{
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    return r;
+}
+__device__ __forceinline__ void split2(uint64_t x2, uint32_t &hi, uint32_t &lo)
+{
+    float a, b, la, lb;
+    unpack_f32x2(x2, a, b);
+    hi = pack_f16x2(a, b);
+    asm("{\n\t.reg .b16 h0, h1, m;\n\t"
+        "mov.b32 {h0, h1}, %2;\n\t"
+        "mov.b16 m, 0xBC00;\n\t"
+        "fma.rn.f32.f16 %0, h0, m, %3;\n\t"
+        "fma.rn.f32.f16 %1, h1, m, %4;\n\t}"
+        : "=f"(la), "=f"(lb) : "r"(hi), "f"(a), "f"(b));
+    lo = pack_f16x2(la, lb);
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float exp2_fast(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t at)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
+    return v;
+}
 
-__global__ void __launch_bounds__(kThreads, 1)
-attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float scale, float *__restrict__ ctx,
+// Largest finite magnitude among N float4, as fp32 bits (NaN and infinities do not take part).
+template <int N>
+__device__ __forceinline__ uint32_t absmax_bits(const float4 (&v)[N])
+{
+    float m = 0.0f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        m = fmaxf(fmaxf(m, fabsf(v[i].x)), fabsf(v[i].y));
+        m = fmaxf(fmaxf(m, fabsf(v[i].z)), fabsf(v[i].w));
+    }
+    if (m == INFINITY) {  // rare: leave the infinities out (fmaxf has left the NaN out)
+        auto finite = [](float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.0f; };
+        m = 0.0f;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            m = fmaxf(fmaxf(fmaxf(m, finite(v[i].x)), fmaxf(finite(v[i].y), finite(v[i].z))), finite(v[i].w));
+    }
+    return __float_as_uint(m);
+}
+// Exponent g with max * 2^-g in [2^13, 2^14) for a maximum given as fp32 bits (at least -126, so that 2^-g is a normal number)
+__device__ __forceinline__ int scale_exponent(uint32_t max_bits) { return max((int)(max_bits >> 23), 14) - 140; }
+__device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }  // -126 <= e <= 127
+
+// Tile staging by 128 threads: thread t holds float4 piece t % 16 (of 16 per row) of rows t / 16 + 8 i.
+template <int ROWS>
+struct Tile {
+    float4 v[ROWS / 8];
+    // Rows past the last one repeat it: a K row there gives scores that are masked, a V row is multiplied by p = 0.
+    __device__ __forceinline__ void fetch(const float *base, uint32_t pitch_bytes, int t, int rows)
+    {
+#pragma unroll
+        for (int i = 0; i < ROWS / 8; ++i)
+            v[i] = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(base) +
+                                                          ((uint32_t)min((t >> 4) + 8 * i, rows - 1) * pitch_bytes + 16u * (t & 15))));
+    }
+    __device__ __forceinline__ void store(uint32_t tile, int t, float mult) const
+    {
+        // (rows t / 16 + 8 i: the same place in every group of 8 rows)
+        const uint32_t at = tile + sw128_offset(t >> 4, (t & 15) >> 1) + 8 * (t & 1);
+        const uint64_t m2 = pack_f32x2(mult, mult);
+#pragma unroll
+        for (int i = 0; i < ROWS / 8; ++i) {
+            uint2 hi, lo;
+            split2(mul_f32x2(pack_f32x2(v[i].x, v[i].y), m2), hi.x, lo.x);
+            split2(mul_f32x2(pack_f32x2(v[i].z, v[i].w), m2), hi.y, lo.y);
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + 1024 * i), "r"(hi.x), "r"(hi.y) : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + 1024 * i + ROWS * 128), "r"(lo.x), "r"(lo.y) : "memory");
+        }
+    }
+};
+
+template <int N>
+__device__ __forceinline__ void grow_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void shrink_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
+__device__ __forceinline__ void staging_barrier() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+
+__global__ void __launch_bounds__(kThreads, 2)
+attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__restrict__ ctx,
                     const float *__restrict__ S_q, int8_t *__restrict__ ctx_q, uint32_t *__restrict__ amax,
-                    uint32_t tmem_cols, int32_t *status)
+                    int32_t *status)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    // [ Q, then P buffer 0 | K / V buffer 0 | K / V buffer 1 | P buffer 1 ]
-    uint8_t *const q_buf = smem;
-    auto k_buf = [&](int b) { return smem + kBufQP + b * (2 * kSpanBytesK); };  // phase 1: two buffers behind Q
-    auto v_buf = [&](int b) { return smem + b * kSet2Bytes; };                  // phase 2: three sets of [V^T | P_lo]
-    auto plo_buf = [&](int b) { return smem + b * kSet2Bytes + kBufKV; };
-    __shared__ __align__(8) uint64_t ready_bar[kSets2];  // workers -> MMA warp: the operands of a chunk are in place
-    __shared__ __align__(8) uint64_t done_bar[kSets2];   // MMA warp -> workers: the MMAs of a chunk have completed
+    const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    auto k_tile = [&](int buf) { return smem + (uint32_t)(buf * kKvBytes); };
+    auto v_tile = [&](int buf) { return smem + (uint32_t)((2 + buf) * kKvBytes); };
+    const uint32_t q_rows = smem + 4 * kKvBytes;
+    __shared__ __align__(8) uint64_t bars[11];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ float row_part[4][kQTile];  // per-row partial maxima, then partial sums, of the four column quarters
+    __shared__ __align__(16) uint32_t warp_max[2][2][kStagingWarps];  // [chunk parity][K, V][warp]
+    // K = K' 2^exponent, V = V' 2^exponent, by chunk number modulo 4 (K of chunk c + 2 may be staged while the softmax of
+    // chunk c still reads its exponent; K of chunk c + 4 is staged after P of chunk c + 1 was handed over)
+    __shared__ int k_exponent[4], v_exponent[4];
+    // barrier of each kind for buffer `buf` = chunk parity
+    const uint32_t bar0 = smem_u32(bars), q_ready = bar0 + 80;
+    auto k_ready = [&](int buf) { return bar0 + 8 * buf; };        // staging -> MMA: K is in place
+    auto v_ready = [&](int buf) { return bar0 + 16 + 8 * buf; };   // staging -> MMA, softmax: V (and its exponent)
+    auto s_done = [&](int buf) { return bar0 + 32 + 8 * buf; };    // MMA -> softmax, staging: scores complete, K read
+    auto p_ready = [&](int buf) { return bar0 + 48 + 8 * buf; };   // softmax -> MMA: P is in tensor memory
+    auto pv_done = [&](int buf) { return bar0 + 64 + 8 * buf; };   // MMA -> staging, softmax: P V complete, P and V read
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q0 = blockIdx.x * kQTile;
@@ -116,275 +230,344 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float scale
     const int64_t row_pitch = 3 * H;
     const float *base = qkv + seq * (int64_t)S * row_pitch + head * kHeadDim;
     const int chunks = (S + kChunk - 1) / kChunk;
-    const int s_pad = chunks * kChunk;
-    const int big_chunks = (S + kBigChunk - 1) / kBigChunk;
+    // columns of chunk c: whole chunks are 64 wide, the last one is rounded up to 32
+    auto chunk_cols = [&](int c) { return c + 1 < chunks ? kChunk : ((S - c * kChunk + 31) & ~31); };
 
     if (tid == 0) {
-        for (int b = 0; b < kSets2; ++b) {
-            mbar_init(smem_u32(&ready_bar[b]), kWorkers / 32);  // one arrival per worker warp
-            mbar_init(smem_u32(&done_bar[b]), 1);
+        mbar_init(q_ready, kSoftmaxWarps);
+        for (int buf = 0; buf < 2; ++buf) {
+            mbar_init(k_ready(buf), kStagingWarps);
+            mbar_init(v_ready(buf), kStagingWarps);
+            mbar_init(s_done(buf), 1);
+            mbar_init(p_ready(buf), kSoftmaxWarps);
+            mbar_init(pv_done(buf), 1);
         }
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == kWorkers / 32) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
+    if (warp == kSoftmaxWarps + kStagingWarps) tmem_alloc(smem_u32(&tmem_slot), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
-    const uint32_t tmem_o = tmem_base + (uint32_t)s_pad;  // O_main: 64 columns behind the scores; O_corr: the next 64
-    grid_dependency_release_next(gridDim.x * gridDim.y * gridDim.z <= 600u);  // up to ~4 waves of CTAs count as small
+    grid_dependency_release_next(gridDim.x * gridDim.y * gridDim.z <= 600u);  // up to ~2 waves of CTAs count as small
     grid_dependency_wait();  // the set-up above may overlap the tail of the kernel that produced qkv
 
-    if (warp == kWorkers / 32) {
-        // ================= MMA warp: stays converged (all lanes wait and compute the same descriptors, which the
-        // compiler can then keep in uniform registers); one elected lane issues, chunk after chunk, as the workers
-        // report operands ready
-        {
+    bool ok = true;
+    // Whole warp, same outcome in every lane; bounded.  (One short polling loop instead of mbar_wait(), whose copies were a
+    // fifth of the kernel's code.  A try may sleep in hardware for up to 0.2 ms: waits of several hundred cycles are the rule
+    // here, and a polling warp takes issue slots from the other CTA: 64 x 384 x 16 heads 241 -> 233 us.)
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        uint64_t t0 = 0;
+#pragma unroll 1
+        while (!__all_sync(0xffffffffu, mbar_try_wait_for(bar, parity, 200000u))) {
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kWaitLimitNs) {
+                *(volatile int *)&abort_flag = 1;
+                if (status) atomicOr(status, 1 << Q8_ERR_TIMEOUT);
+            }
+            if (__any_sync(0xffffffffu, *(volatile int *)&abort_flag)) {
+                ok = false;
+                break;
+            }
+        }
+        tc_fence_after();
+        return ok;
+    };
+    // one arrival per warp, after every lane's writes (tensor memory, and shared memory with the fence) are visible to the
+    // tensor core
+    auto arrive = [&](uint32_t bar, bool wrote_smem) {
+        if (wrote_smem) fence_proxy_async_smem();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+    };
+
+    if (warp >= kSoftmaxWarps + kStagingWarps) {
+        // ================= MMA issuer (the other warps of its group have nothing to do)
+        shrink_registers<kIssuerRegs>();
+        if (warp == kSoftmaxWarps + kStagingWarps) {
             const uint32_t elected = elect_one();
-            uint32_t ready_phase = 0u;  // bit b: parity of the next phase of ready_bar[b]
-            bool ok = true;
-            const uint32_t q_hi = smem_u32(q_buf), q_lo = q_hi + 2 * kSpanBytesA;
-            for (int kc = 0; kc < big_chunks && ok; ++kc) {  // scores of the 128 keys of big chunk kc
-                const int b = kc & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ready_bar[b]), (ready_phase >> b) & 1u, &abort_flag, status));
-                ready_phase ^= 1u << b;
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t d = tmem_base + (uint32_t)(kc * kBigChunk), kb = smem_u32(k_buf(b));
-                uint32_t acc = 0u;
+            auto issue_scores = [&](int c) {  // S(c) = Q K(c)^T into the columns of buffer c % 2
+                const int buf = c & 1;
+                const uint32_t par = (uint32_t)((c >> 1) & 1), d = tmem_base + (uint32_t)(buf * kChunk);
+                if (!wait(k_ready(buf), par)) return;
+                if (c >= 2 && !wait(pv_done(buf), par ^ 1u)) return;  // P of chunk c - 2 lies there
+                const uint64_t k_hi = smem_desc_sw128(k_tile(buf)), k_lo = k_hi + (uint64_t)(kKvHalfBytes >> 4);
+                const uint32_t idesc = kIdescBase | ((uint32_t)(chunk_cols(c) >> 3) << 17);
+                const uint32_t q_hi = tmem_base + kColQ, q_lo = q_hi + 32;
 #pragma unroll
-                for (int span = 0; span < 2; ++span) {
-                    const uint64_t ah = smem_desc_sw128(q_hi + span * kSpanBytesA), al = smem_desc_sw128(q_lo + span * kSpanBytesA);
-                    const uint64_t bh = smem_desc_sw128(kb + span * kSpanBytesK), bl = smem_desc_sw128(kb + span * kSpanBytesK + kLoRowsK);
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {  // 8 fp32 = 32 bytes of K per instruction: +2 in the (address >> 4) field
-                        const uint64_t adv = (uint64_t)(2 * ks);
-                        umma_tf32_elected(elected, d, al + adv, bh + adv, kIdescN128, acc);  // small terms first
-                        umma_tf32_elected(elected, d, ah + adv, bl + adv, kIdescN128, 1u);
-                        umma_tf32_elected(elected, d, ah + adv, bh + adv, kIdescN128, 1u);
-                        acc = 1u;
-                    }
+                for (int ks = 0; ks < 4; ++ks) {  // 16 fp16 = 32 bytes of K per instruction: +2 in the (address >> 4) field
+                    umma_f16_ts_elected(elected, d, q_lo + 8 * ks, k_hi + 2 * ks, idesc, ks > 0 ? 1u : 0u);  // small terms first
+                    umma_f16_ts_elected(elected, d, q_hi + 8 * ks, k_lo + 2 * ks, idesc, 1u);
                 }
-                umma_commit_elected(elected, smem_u32(&done_bar[b]));
-            }
-            for (int kc = 0, b = 0; kc < chunks && ok; ++kc, b = (b + 1 == kSets2 ? 0 : b + 1)) {  // O += P V of chunk kc
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ready_bar[b]), (ready_phase >> b) & 1u, &abort_flag, status));
-                ready_phase ^= 1u << b;
-                if (!ok) break;
-                tc_fence_after();
-                // P_hi is read from tensor memory, where it has replaced the chunk's scores (row = lane, key = column)
-                const uint32_t p_hi = tmem_base + (uint32_t)(kc * kChunk);
-                const uint32_t p_lo = smem_u32(plo_buf(b)), vb = smem_u32(v_buf(b));
-                uint32_t acc = kc > 0 ? 1u : 0u;
 #pragma unroll
-                for (int span = 0; span < 2; ++span) {
-                    const uint64_t al = smem_desc_sw128(p_lo + span * kSpanBytesA);
-                    const uint64_t bhl = smem_desc_sw128(vb + span * kSpanBytesB);  // 128 rows: V_hi then V_lo
+                for (int ks = 0; ks < 4; ++ks) umma_f16_ts_elected(elected, d, q_hi + 8 * ks, k_hi + 2 * ks, idesc, 1u);
+                umma_commit_elected(elected, s_done(buf));
+            };
+            auto issue_pv = [&](int c) {  // P(c) V(c) into the product columns (the softmax has read P(c - 1) V(c - 1) before)
+                const int buf = c & 1, steps = chunk_cols(c) / 16;
+                const uint32_t par = (uint32_t)((c >> 1) & 1), d = tmem_base + kColPV;
+                if (!wait(v_ready(buf), par) || !wait(p_ready(buf), par)) return;
+                const uint64_t v_hi = smem_desc_v(v_tile(buf)), v_lo = v_hi + (uint64_t)(kKvHalfBytes >> 4);
+                // P: per 16 keys 8 columns of hi parts, then 8 of lo parts; 16 keys are two atoms (2048 bytes) of V
+                auto p_at = [&](int ks) { return tmem_base + (uint32_t)(buf * kChunk + 16 * ks); };
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {  // 8 keys per instruction: 8 TMEM columns of P_hi, +2 in the (address >> 4) field
-                        const uint64_t adv = (uint64_t)(2 * ks);
-                        umma_tf32_ts_elected(elected, tmem_o, p_hi + (uint32_t)(32 * span + 8 * ks), bhl + adv, kIdescN128, acc);  // [P_hi V_hi | P_hi V_lo]
-                        umma_tf32_elected(elected, tmem_o + kHeadDim, al + adv, bhl + adv, kIdescN64, 1u);  // += P_lo V_hi
-                        acc = 1u;
-                    }
+                for (int ks = 0; ks < 4; ++ks) {
+                    if (ks >= steps) break;
+                    umma_f16_ts_elected(elected, d, p_at(ks) + 8, v_hi + ks * (2048 >> 4), kIdescPV, ks > 0 ? 1u : 0u);
+                    umma_f16_ts_elected(elected, d, p_at(ks), v_lo + ks * (2048 >> 4), kIdescPV, 1u);
                 }
-                umma_commit_elected(elected, smem_u32(&done_bar[b]));
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    if (ks >= steps) break;
+                    umma_f16_ts_elected(elected, d, p_at(ks), v_hi + ks * (2048 >> 4), kIdescPV, 1u);
+                }
+                umma_commit_elected(elected, pv_done(buf));
+            };
+            // P(c - 1) becomes ready about when the softmax turns to S(c); the products of chunk c - 1 and, when they have
+            // read P(c - 1), the scores of chunk c + 1 in its place then run under the softmax of chunk c
+            if (wait(q_ready, 0)) issue_scores(0);
+#pragma unroll 1
+            for (int c = 0; c < chunks && ok; ++c) {
+                if (c + 1 < chunks) issue_scores(c + 1);
+                if (ok) issue_pv(c);
             }
+            if (!ok) {  // aborting: let the MMAs issued so far finish before the tensor memory is freed
+                const uint64_t t0 = global_timer_ns();
+                while (global_timer_ns() - t0 < 1000000ull) {}
+            }
+        }
+    } else if (warp >= kSoftmaxWarps) {
+        // ================= staging warps
+        grow_registers<kStagingRegs>();
+        const int t = tid - 32 * kSoftmaxWarps, w = warp - kSoftmaxWarps;
+        const float *kbase = base + H, *vbase = base + 2 * H;
+        const uint32_t pitch_bytes = (uint32_t)row_pitch * 4u;
+        Tile<kChunk> kt, vt;
+        auto chunk_exponent = [&](const Tile<kChunk> &tile, int which, int c) {
+            const uint32_t m = __reduce_max_sync(0xffffffffu, absmax_bits(tile.v));
+            if (lane == 0) warp_max[c & 1][which][w] = m;
+            staging_barrier();
+            const uint4 x = *reinterpret_cast<const uint4 *>(warp_max[c & 1][which]);
+            return scale_exponent(max(max(x.x, x.y), max(x.z, x.w)));
+        };
+        int gv_largest = -126;
+        // (chunk -1: nothing to stage yet, its fetches bring in chunk 0; after a time-out the loop still runs, for the
+        // barriers of its group alone)
+#pragma unroll 1
+        for (int c = -1; c < chunks; ++c) {
+            const int buf = c & 1, left = S - (c + 1) * kChunk;  // keys behind this chunk
+            const uint32_t freed = (uint32_t)(((c >> 1) & 1) ^ 1);
+            if (c >= 0) {
+                const int gk = chunk_exponent(kt, 0, c);
+                if (c >= 2 && ok) wait(s_done(buf), freed);  // K of chunk c - 2 has been read
+                if (ok) {
+                    kt.store(k_tile(buf), t, pow2(-gk));
+                    if (t == 0) k_exponent[c & 3] = gk;
+                    arrive(k_ready(buf), true);
+                }
+            }
+            if (left > 0) kt.fetch(kbase + (int64_t)(c + 1) * kChunk * row_pitch, pitch_bytes, t, left);
+            if (c >= 0) {
+                // (a chunk of far smaller values shares the scale of the largest so far to within 2^60: P carries the exponent
+                // too, and fp32 has to hold it for the row sum)
+                const int gv = max(chunk_exponent(vt, 1, c), gv_largest - 60);
+                gv_largest = max(gv_largest, gv);
+                if (c >= 2 && ok) wait(pv_done(buf), freed);  // V of chunk c - 2 has been read
+                if (ok) {
+                    vt.store(v_tile(buf), t, pow2(-gv));
+                    if (t == 0) v_exponent[c & 3] = gv;
+                    arrive(v_ready(buf), true);
+                }
+            }
+            if (left > 0) vt.fetch(vbase + (int64_t)(c + 1) * kChunk * row_pitch, pitch_bytes, t, left);
         }
     } else {
-        // ================= workers
-        const int quarter = warp & 3, cq = warp >> 2;  // TMEM lane quarter this warp may read; its 16 columns of a chunk
-        const int row = quarter * 32 + lane;           // query row (TMEM lane) of this thread in the softmax
-        const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        uint32_t done_phase = 0u;  // bit b: parity of the next phase of done_bar[b]
-        bool ok = true;
-        // waits (whole warp, same outcome in every lane) until the MMAs of the chunk that used buffer set b are done
-        auto wait_done = [&](int b) {
-            const bool mine = mbar_wait(smem_u32(&done_bar[b]), (done_phase >> b) & 1u, &abort_flag, status);
-            done_phase ^= 1u << b;
-            ok = __all_sync(0xffffffffu, mine);
-            tc_fence_after();
-        };
-        // every thread makes its shared-memory writes visible to the tensor core; then one lane reports for the warp
-        // (16 arrivals on the barrier instead of 512)
-        auto report_ready = [&](int b) {
-            fence_proxy_async_smem();
-            tc_fence_before();  // (a tcgen05.st of P_hi has completed by now: tmem_st_wait() before this call)
+        // ================= softmax warps: thread = query row = TMEM lane
+        grow_registers<kSoftmaxRegs>();
+        const float Sq = ctx_q != nullptr ? __ldg(S_q) : 1.0f;
+        const uint32_t t_row = tmem_base + ((uint32_t)(warp * 32) << 16);
+        const bool warp_live = q0 + 32 * warp < S;  // a warp whose rows all lie past the end only keeps the barriers going
+        const uint32_t my_rows = q_rows + (uint32_t)(warp * (32 * kRowBytes));  // 16-byte pieces XORed with the row
+        auto piece = [&](int r, int i) { return my_rows + (uint32_t)(r * kRowBytes + ((i ^ (r & 15)) << 4)); };
+        // Q: this warp's 32 rows to shared memory (whole lines), every thread takes its row, scales it by a power of two of its
+        // own and puts both fp16 parts into tensor memory: the A operand of the scores.
+        int gq = 0;
+        {
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i) {
+                const int r = 2 * i + (lane >> 4), pc = lane & 15;
+                const bool in = q0 + 32 * warp + r < S;  // rows past the end are filled with zeros
+                const float *src = base + (int64_t)(in ? q0 + 32 * warp + r : 0) * row_pitch + 4 * pc;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(piece(r, pc)), "l"(src), "r"(in ? 16 : 0) : "memory");
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ready_bar[b]));
-        };
-
-        // ---------------- phase 1: scores = (Q * log2(e)/8) K^T
-        constexpr int kPiecesK = (kBigChunk * 16) / kWorkers;  // 16-byte pieces of a 128-key K chunk per thread
-        float4 kreg[kPiecesK];
-        auto fetch_k = [&](int j0) {  // 128 keys x 64 fp32
+            float4 v[4];
+            uint32_t mq = 0;
+#pragma unroll 1
+            for (int h = 0; h < 4; ++h) {
 #pragma unroll
-            for (int i = 0; i < kPiecesK; ++i) {
-                const int c = tid + i * kWorkers, r = c >> 4, pc = c & 15;
-                kreg[i] = (j0 + r < S) ? __ldg(reinterpret_cast<const float4 *>(base + (int64_t)(j0 + r) * row_pitch + H) + pc)
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = 0; i < 4; ++i) v[i] = ld_shared_f4(piece(lane, 4 * h + i));
+                mq = max(mq, absmax_bits(v));
             }
-        };
-        fetch_k(0);  // the first K chunk travels while Q is split and staged
-        // a 16-byte piece c of a [rows x 64] fp32 tile: row c / 16, span (c % 16) / 8, piece (c % 16) % 8
+            gq = scale_exponent(mq);
+            const uint64_t m2 = pack_f32x2(pow2(-gq), pow2(-gq));
+#pragma unroll 1
+            for (int h = 0; h < 4; ++h) {
+                uint32_t hi[8], lo[8];
 #pragma unroll
-        for (int i = 0; i < (kQTile * 16) / kWorkers; ++i) {
-            const int c = tid + i * kWorkers, r = c >> 4, pc = c & 15;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (q0 + r < S) v = __ldg(reinterpret_cast<const float4 *>(base + (int64_t)(q0 + r) * row_pitch) + pc);
-            v.x *= scale;
-            v.y *= scale;
-            v.z *= scale;
-            v.w *= scale;
-            uint8_t *at = q_buf + (pc >> 3) * kSpanBytesA + sw128_offset(r, pc & 7);
-            store_split4(at, at + 2 * kSpanBytesA, v);
-        }
-        float m = -INFINITY;
-        uint32_t sv[32];  // this thread's 32 score columns of a big chunk, on their way out of TMEM
-        auto load_scores = [&](int c) { tmem_ld_32x32(t_row + (uint32_t)(c * kBigChunk + cq * 32), sv); };
-        auto take_max = [&](int c) {  // after load_scores(c): waits for the load, folds the 32 columns into m
-            uint32_t(&v)[32] = sv;
-            const int col0 = c * kBigChunk + cq * 32;
-            tmem_ld_wait();
-            if (col0 + 32 <= S) {
+                for (int i = 0; i < 4; ++i) v[i] = ld_shared_f4(piece(lane, 4 * h + i));
 #pragma unroll
-                for (int j = 0; j < 32; ++j) m = fmaxf(m, __uint_as_float(v[j]));
-            } else {
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (col0 + j < S) m = fmaxf(m, __uint_as_float(v[j]));
-            }
-        };
-        for (int kc = 0; kc < big_chunks && ok; ++kc) {
-            const int b = kc & 1;
-            if (kc >= 2) {  // buffer b was read by the MMAs of big chunk kc - 2, whose scores are final after this wait
-                wait_done(b);
-                if (!ok) break;
-                load_scores(kc - 2);  // in flight while the next K chunk is staged below
-            }
-#pragma unroll
-            for (int i = 0; i < kPiecesK; ++i) {
-                const int c = tid + i * kWorkers, r = c >> 4, pc = c & 15;
-                uint8_t *at = k_buf(b) + (pc >> 3) * kSpanBytesK + sw128_offset(r, pc & 7);
-                store_split4(at, at + kLoRowsK, kreg[i]);
-            }
-            if (kc + 1 < big_chunks) fetch_k((kc + 1) * kBigChunk);  // next K chunk, in flight during the MMAs
-            report_ready(b);
-            if (kc >= 2) take_max(kc - 2);
-        }
-        for (int c = (big_chunks > 2 ? big_chunks - 2 : 0); c < big_chunks && ok; ++c) {  // the last two big chunks
-            wait_done(c & 1);
-            if (ok) {
-                load_scores(c);
-                take_max(c);
-            }
-        }
-        row_part[cq][row] = m;
-        worker_barrier();
-        m = fmaxf(fmaxf(row_part[0][row], row_part[1][row]), fmaxf(row_part[2][row], row_part[3][row]));
-        worker_barrier();  // row_part is reused for the sums; every score MMA has completed: Q may be overwritten
-
-        // ---------------- phase 2: P = 2^(scores - max), O = P V, chunk by chunk
-        float l = 0.0f;
-        // V chunk as a 64 x 64 tile of blocks of 4 keys x 2 features: thread = (key block vkb, feature pair vfp); the
-        // block is transposed in registers so that each feature row of V^T gets 4 consecutive keys (one 16-byte piece)
-        const int vkb = tid >> 5, vfp = tid & 31;
-        float2 vreg[4];
-        auto fetch_v = [&](int j0) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = j0 + 4 * vkb + i;
-                vreg[i] = (j < S) ? __ldg(reinterpret_cast<const float2 *>(base + (int64_t)j * row_pitch + 2 * H) + vfp)
-                                  : make_float2(0.f, 0.f);
-            }
-        };
-        if (ok) fetch_v(0);
-        // All scores are final, so a chunk's 16 score columns are fetched from TMEM one chunk ahead, and its
-        // exponentials are taken before the wait for the buffer set they will be stored into.
-        uint32_t pv[16];
-        if (ok) tmem_ld_32x16(t_row + (uint32_t)(cq * 16), pv);
-        for (int kc = 0, b = 0; kc < chunks && ok; ++kc, b = (b + 1 == kSets2 ? 0 : b + 1)) {
-            // p = hi + lo (hi = p rounded to TF32).  The hi parts go back into tensor memory over the chunk's scores, from
-            // where the MMA takes them as its A operand (no trip through shared memory: 64 x 384 x 16 heads 338 -> 325 us;
-            // the same for Q in phase 1 measured slower, 360 us, and is not done); the lo parts go to shared memory.
-            float p_lo[16];
-            {
-                const int col0 = kc * kChunk + cq * 16;
-                tmem_ld_wait();
-                const bool whole = col0 + 16 <= S;
-                uint32_t ph[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    float e;
-                    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__uint_as_float(pv[j]) - m));
-                    const float pj = (whole || col0 + j < S) ? e : 0.0f;
-                    l += pj;
-                    const float h = round_tf32(pj);
-                    ph[j] = __float_as_uint(h);
-                    p_lo[j] = pj - h;  // exact
+                for (int i = 0; i < 4; ++i) {
+                    split2(mul_f32x2(pack_f32x2(v[i].x, v[i].y), m2), hi[2 * i], lo[2 * i]);
+                    split2(mul_f32x2(pack_f32x2(v[i].z, v[i].w), m2), hi[2 * i + 1], lo[2 * i + 1]);
                 }
-                if (kc + 1 < chunks) tmem_ld_32x16(t_row + (uint32_t)(col0 + kChunk), pv);
-                tmem_st_32x16(t_row + (uint32_t)col0, ph);
-            }
-            if (kc >= kSets2) {  // buffer set b was last read by the MMAs of chunk kc - 3
-                wait_done(b);
-                if (!ok) break;
-            }
-            // V^T[d][key]: rows = features (64, hi block then lo block), K = keys of this chunk (2 spans of 32)
-            {
-                uint8_t *sb = v_buf(b) + (vkb >> 3) * kSpanBytesB;  // keys 4 vkb .. 4 vkb + 3: span vkb / 8, piece vkb % 8
-                uint8_t *a0 = sb + sw128_offset(2 * vfp + 0, vkb & 7), *a1 = sb + sw128_offset(2 * vfp + 1, vkb & 7);
-                store_split4(a0, a0 + kLoRowsB, make_float4(vreg[0].x, vreg[1].x, vreg[2].x, vreg[3].x));
-                store_split4(a1, a1 + kLoRowsB, make_float4(vreg[0].y, vreg[1].y, vreg[2].y, vreg[3].y));
-            }
-            if (kc + 1 < chunks) fetch_v((kc + 1) * kChunk);
-            // P_lo[row][key]: this thread's 16 keys are pieces 4 (cq & 1) .. + 3 of span cq / 2 of the chunk
-            {
-                uint8_t *sb = plo_buf(b) + (cq >> 1) * kSpanBytesA;
-#pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    *reinterpret_cast<float4 *>(sb + sw128_offset(row, 4 * (cq & 1) + g)) =
-                        make_float4(p_lo[4 * g], p_lo[4 * g + 1], p_lo[4 * g + 2], p_lo[4 * g + 3]);
+                tmem_st_32x8(t_row + kColQ + 8 * h, hi);
+                tmem_st_32x8(t_row + kColQ + 32 + 8 * h, lo);
             }
             tmem_st_wait();
-            report_ready(b);
+            arrive(q_ready, false);
         }
-        tmem_ld_wait();  // (a load is still in flight only when the loop above was left early)
-        row_part[cq][row] = l;  // the row sums are exchanged while the last MMAs run
-        worker_barrier();
-        for (int c = (chunks > kSets2 ? chunks - kSets2 : 0); c < chunks && ok; ++c) wait_done(c % kSets2);  // the last three chunks
-
-        // ---------------- phase 3: ctx = (O_main + O_corr) / row sum
-        if (ok) {  // (warp-uniform: the TMEM loads below are warp-wide instructions, only the stores depend on the row)
-            const float inv = 1.0f / ((row_part[0][row] + row_part[1][row]) + (row_part[2][row] + row_part[3][row]));
-            uint32_t v[16], w[16];
-            tmem_ld_32x16(t_row + (uint32_t)(s_pad + cq * 16), v);
-            tmem_ld_32x16(t_row + (uint32_t)(s_pad + kHeadDim + cq * 16), w);
-            tmem_ld_wait();
-            const bool row_ok = q0 + row < S;
-            const int64_t at = (seq * (int64_t)S + q0 + row) * H + head * kHeadDim + cq * 16;
-            float y[16];
+        // Reference maxima, whole numbers so that every power of two between them is exact: M of s + v_exponent
+        // (P is 2^(s + v_exponent - M)), ml of s (for the row sum l)
+        float M = 0.0f, ml = 0.0f;
+        float l = 0.0f;
+        uint64_t O[kHeadDim / 2];  // running output of the row, in units of 2^M
 #pragma unroll
-            for (int j = 0; j < 16; ++j) y[j] = (__uint_as_float(v[j]) + __uint_as_float(w[j])) * inv;
-            if (amax != nullptr) {  // max|ctx| for a dynamically quantised consumer (Sec. 4.1); rows past S do not count
-                float am = 0.0f;
-                if (row_ok) {
+        for (int j = 0; j < kHeadDim / 2; ++j) O[j] = 0;  // (+0, +0)
+        auto add_product = [&](int c) {  // O += P(c) V(c)
+            if (!wait(pv_done(c & 1), (uint32_t)((c >> 1) & 1))) return;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) am = fmaxf(am, fabsf(y[j]));
+            for (int h = 0; h < 2; ++h) {
+                uint32_t x[32];
+                tmem_ld_32x32(t_row + kColPV + (uint32_t)(32 * h), x);
+                tmem_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    O[16 * h + j] = add_f32x2(O[16 * h + j], pack_f32x2(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1])));
+            }
+        };
+        for (int c = 0; c < chunks && ok; ++c) {
+            const int buf = c & 1, left = S - c * kChunk;
+            const uint32_t par = (uint32_t)((c >> 1) & 1), t_s = t_row + (uint32_t)(buf * kChunk);
+            if (!wait(s_done(buf), par) || !wait(v_ready(buf), par)) break;
+            if (warp_live) {
+                const float f = pow2(max(-126, min(120, gq + k_exponent[c & 3]))) * kLog2eOver8, gv = (float)v_exponent[c & 3];
+                // half 1 of the scores is read twice (for the maximum, then for the exponentials), half 0 stays in registers
+                uint32_t sv[32];
+                float mc = -INFINITY;
+                auto load_half = [&](int h) {
+                    tmem_ld_32x32(t_s + (uint32_t)(32 * h), sv);
+                    tmem_ld_wait();
+                    if (left < 32 * h + 32) {  // the last columns of a ragged sequence: keys past its end get p = 2^-inf
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            if (32 * h + j >= left) sv[j] = 0xFF800000u;
+                    }
+                };
+                auto take_max = [&](int h) {
+                    load_half(h);
+                    float m1 = -INFINITY;
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        mc = fmaxf(fmaxf(mc, __uint_as_float(sv[j])), __uint_as_float(sv[j + 1]));
+                        m1 = fmaxf(fmaxf(m1, __uint_as_float(sv[j + 2])), __uint_as_float(sv[j + 3]));
+                    }
+                    mc = fmaxf(mc, m1);
+                };
+                const bool two = left > 32;
+                if (two) take_max(1);
+                take_max(0);
+                mc = ceilf(mc * f);
+                const float a = mc + gv;
+                float rescale = 1.0f;
+                if (c == 0) {
+                    M = a;
+                    ml = mc;
+                } else {
+                    if (a > M + kStaleSlack) {
+                        rescale = exp2_fast(M - a);
+                        M = a;
+                    }
+                    if (mc > ml + 20.0f) {
+                        l *= exp2_fast(ml - mc);
+                        ml = mc;
+                    }
                 }
-                warp_fold_absmax(am, amax);
-            }
-            if (ctx != nullptr && row_ok) {
+                const float b = gv - M;
+                const uint64_t f2 = pack_f32x2(f, f), b2 = pack_f32x2(b, b);
+                const uint64_t shift2 = pack_f32x2((float)(1 << kPShift), (float)(1 << kPShift));
+                uint64_t sum_a = 0, sum_b = 0;  // (+0, +0)
+                auto exponentials = [&](int h) {  // 16 keys: 8 columns of hi parts, then 8 of lo parts, over their scores
 #pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    *reinterpret_cast<float4 *>(ctx + at + 4 * g) = make_float4(y[4 * g], y[4 * g + 1], y[4 * g + 2], y[4 * g + 3]);
+                    for (int q = 0; q < 2; ++q) {
+                        uint32_t hi[8], lo[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            float x0, x1;
+                            const int k = 16 * q + 2 * j;
+                            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[k]), __uint_as_float(sv[k + 1])), f2, b2), x0, x1);
+                            const uint64_t e2 = pack_f32x2(exp2_fast(x0), exp2_fast(x1));
+                            if (j & 1) sum_a = add_f32x2(sum_a, e2);
+                            else sum_b = add_f32x2(sum_b, e2);
+                            split2(mul_f32x2(e2, shift2), hi[j], lo[j]);
+                        }
+                        tmem_st_32x8(t_s + (uint32_t)(32 * h + 16 * q), hi);
+                        tmem_st_32x8(t_s + (uint32_t)(32 * h + 16 * q + 8), lo);
+                    }
+                };
+                exponentials(0);
+                if (two) {
+                    load_half(1);
+                    exponentials(1);
+                }
+                float sum0, sum1, sum2, sum3;
+                unpack_f32x2(sum_a, sum0, sum1);
+                unpack_f32x2(sum_b, sum2, sum3);
+                l = fmaf((sum0 + sum1) + (sum2 + sum3), exp2_fast(-b - ml), l);
+                if (c > 0) {
+                    add_product(c - 1);
+                    if (__any_sync(0xffffffffu, rescale != 1.0f)) {
+                        const uint64_t r2 = pack_f32x2(rescale, rescale);
+#pragma unroll
+                        for (int j = 0; j < kHeadDim / 2; ++j) O[j] = mul_f32x2(O[j], r2);
+                    }
+                }
+                tmem_st_wait();
             }
-            if (ctx_q != nullptr && row_ok) {  // the same fp32 values, quantised for the next quantised layer (Eq. 1)
-                const float Sq = __ldg(S_q);
-                *reinterpret_cast<uint4 *>(ctx_q + at) =
-                    make_uint4(quantize_pack4(y[0], y[1], y[2], y[3], Sq), quantize_pack4(y[4], y[5], y[6], y[7], Sq),
-                               quantize_pack4(y[8], y[9], y[10], y[11], Sq), quantize_pack4(y[12], y[13], y[14], y[15], Sq));
+            arrive(p_ready(buf), false);
+        }
+        // ---------------- ctx = O / row sum
+        if (ok && warp_live) add_product(chunks - 1);
+        if (ok && warp_live) {
+            // Normalised rows to shared memory (where Q came in), then a half-warp takes a row at a time, so that whole lines
+            // are stored.  In a short loop: written out for a thread's 64 values this was a third of the kernel's code.
+            const float inv = exp2_fast(M - (float)kPShift - ml) / l;
+            const uint64_t inv2 = pack_f32x2(inv, inv);
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                asm volatile("st.shared.v2.b64 [%0], {%1, %2};"
+                             ::"r"(piece(lane, i)), "l"(mul_f32x2(O[2 * i], inv2)), "l"(mul_f32x2(O[2 * i + 1], inv2))
+                             : "memory");
+            __syncwarp();
+            const int live_rows = min(32, S - q0 - 32 * warp), pc = lane & 15;
+            const int64_t out0 = (seq * (int64_t)S + q0 + 32 * warp) * H + head * kHeadDim + 4 * pc;
+            float am = 0.0f;
+#pragma unroll 2
+            for (int r = lane >> 4; r < live_rows; r += 2) {
+                const float4 y = ld_shared_f4(piece(r, pc));
+                const int64_t at = out0 + (int64_t)r * H;
+                am = fmaxf(fmaxf(am, fmaxf(fabsf(y.x), fabsf(y.y))), fmaxf(fabsf(y.z), fabsf(y.w)));
+                if (ctx != nullptr) *reinterpret_cast<float4 *>(ctx + at) = y;
+                // the same fp32 values, quantised for the next quantised layer (Eq. 1)
+                if (ctx_q != nullptr) *reinterpret_cast<uint32_t *>(ctx_q + at) = quantize_pack4(y.x, y.y, y.z, y.w, Sq);
+            }
+            if (amax != nullptr) {  // max|ctx| for a dynamically quantised consumer (Sec. 4.1); rows past S do not count
+                __syncwarp();
+                warp_fold_absmax(am, amax);
             }
         }
     }
@@ -392,19 +575,29 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float scale
     // ---------------- teardown (reached by every thread, also after a time-out)
     tc_fence_before();
     __syncthreads();
-    if (warp == kWorkers / 32) {
+    if (warp == kSoftmaxWarps + kStagingWarps) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, tmem_cols);
+        tmem_dealloc(tmem_base, kTmemCols);
     }
 }
 
 bool g_attention_tc_enabled = true;
 
+int device_sms(int dev)
+{
+    static int cached[64] = {};
+    if (cached[dev] == 0) {
+        int v = 0;
+        cached[dev] = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 148;
+    }
+    return cached[dev];
+}
+
 }  // namespace
 
 void set_attention_tensor_cores(bool enable) { g_attention_tc_enabled = enable; }
 
-// Device status word of the tensor-core attention kernel (one per device, in a file-scope array).
+// Device status word of the tensor-core attention kernels (one per device, in a file-scope array).
 static __device__ int32_t g_attention_status[1];
 
 int32_t *attention_status_word()
@@ -422,10 +615,10 @@ int32_t *attention_status_word()
 
 bool attention_tc_supported(const float *qkv, int64_t S, int64_t heads, const float *ctx, const int8_t *ctx_q)
 {
-    const int64_t s_pad = (S + kChunk - 1) / kChunk * kChunk;
     auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-    (void)heads;  // H = 64 * heads keeps every row 16-byte aligned
-    return g_attention_tc_enabled && s_pad + 2 * kHeadDim <= 512 && al16(qkv) && al16(ctx) && al16(ctx_q);
+    // 16-byte loads and stores (H = 64 * heads keeps every row aligned); byte offsets within a chunk and key positions fit
+    // 32 bits (65535 heads: 64 rows of 50 MB)
+    return g_attention_tc_enabled && S <= (int64_t(1) << 30) && heads <= 65535 && al16(qkv) && al16(ctx) && al16(ctx_q);
 }
 
 cudaError_t launch_attention_tc(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,
@@ -436,18 +629,25 @@ cudaError_t launch_attention_tc(const float *qkv, int64_t B, int64_t S, int64_t 
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    // With at most one CTA per SM the time is that of a single CTA, which the kernel with 512 threads per CTA has the shorter
+    // (12 heads of 128: 12 CTAs 8.4 against 9.2 us, 144 CTAs 8.8 / 10.1; 144 CTAs of 384: 14.9 / 17.8); beyond, two of this
+    // kernel's CTAs share an SM where the other needs a second round (192 CTAs of 128: 16.4 / 11.7 us, 288: 16.9 / 12.1).
+    if ((S + kQTile - 1) / kQTile * heads * B <= device_sms(dev) && attention_small_supported(S))
+        return launch_attention_small(qkv, B, S, heads, ctx, S_q, ctx_q, amax, s);
     if (!attr_set[dev]) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, attention_tc_kernel);
+        if (e != cudaSuccess) return e;
+        if (fa.numRegs * 3 < kSoftmaxRegs + kStagingRegs + kIssuerRegs) return cudaErrorLaunchOutOfResources;
         e = cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnTcSmemBytes);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    const int64_t s_pad = (S + kChunk - 1) / kChunk * kChunk;
-    uint32_t cols = 32;
-    while (cols < (uint32_t)(s_pad + 2 * kHeadDim)) cols <<= 1;  // scores, O_main, O_corr
     dim3 grid((unsigned)((S + kQTile - 1) / kQTile), (unsigned)heads, (unsigned)B);
-    const float scale = 1.4426950408889634f / 8.0f;  // log2(e) / sqrt(64): the softmax then uses 2^x
     return launch_overlapping_tail(attention_tc_kernel, grid, dim3(kThreads), kAttnTcSmemBytes, s, qkv, (int)S,
-                                   heads * kHeadDim, scale, ctx, S_q, ctx_q, amax, cols, attention_status_word());
+                                   heads * kHeadDim, ctx, S_q, ctx_q, amax, attention_status_word());
 }
 
 }  // namespace q8

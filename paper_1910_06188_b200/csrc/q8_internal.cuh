@@ -91,10 +91,14 @@ cudaError_t launch_add_layernorm(const float *x, const float *r1, const float *r
 cudaError_t launch_attention(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,
                              int8_t *ctx_q, uint32_t *amax, cudaStream_t s);
 
-// Tensor-core attention (q8_attention_sm100.cu): 3 x TF32 split products with fp32 accumulation in TMEM.
+// Tensor-core attention (q8_attention_sm100.cu): split fp16 products with fp32 accumulation.
 bool attention_tc_supported(const float *qkv, int64_t S, int64_t heads, const float *ctx, const int8_t *ctx_q);
 cudaError_t launch_attention_tc(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,
                                 int8_t *ctx_q, uint32_t *amax, cudaStream_t s);
+// Grids of at most one CTA per SM, S <= 384 (q8_attention_small_sm100.cu): split TF32 products, shorter latency of a CTA.
+bool attention_small_supported(int64_t S);
+cudaError_t launch_attention_small(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,
+                                   int8_t *ctx_q, uint32_t *amax, cudaStream_t s);
 void set_attention_tensor_cores(bool enable);
 int32_t *attention_status_word();  // device word that receives Q8_ERR_TIMEOUT from the tensor-core attention kernel
 

@@ -41,6 +41,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// The same with a time limit (ns) for which the hardware may suspend the thread.
+__device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t limit_ns)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(limit_ns)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ uint64_t global_timer_ns()
 {
     uint64_t t;
@@ -102,18 +115,7 @@ __device__ __forceinline__ void umma_i8(uint32_t tmem_d, uint64_t desc_a, uint64
         : "memory");
 }
 // D[tmem] (+)= A[smem] * B[smem]^T with TF32 operands (the upper 19 bits of each fp32 word) and fp32 accumulation.
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
-                                          uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// The same instruction for a converged warp: every lane executes the call with identical operands and one elected
-// lane issues.  Keeping the issuing warp converged lets the compiler hold descriptors and addresses in uniform
+// For a converged warp: every lane executes the call with identical operands and one elected lane issues.  Keeping the issuing warp converged lets the compiler hold descriptors and addresses in uniform
 // registers instead of moving them there for every instruction.  `elected` comes from elect_one().
 __device__ __forceinline__ uint32_t elect_one()
 {

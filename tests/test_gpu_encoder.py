@@ -333,3 +333,56 @@ def test_dynamic_forward_without_absmax_passes_equals_the_unfused_dynamic_forwar
     assert torch.equal(got, want)
     assert enc.poll() == ((q8.Q8_OK, 0), (q8.Q8_OK, 0))
     assert enc.launches_per_forward("dynamic", fused=True) < enc.launches_per_forward("dynamic")
+
+
+# ------------------------------------------------------------------ tensor-core attention at the edges of its chunks
+# Operands carry 22 bits (relative error 2^-23 each), so a score q.k / 8 of 64 products of N(0, 1) values (|s| up to ~6) is
+# off by less than 64 * 2^-22 * E|q k| / 8 ~ 1.2e-6 and its weight by as much; v adds 2^-22: 2e-6 of the largest output.
+EDGE_TOL = 2e-6
+FULL = 150  # sequences of one head that make more CTAs than there are SMs: the kernel for grids that fill the device
+
+
+def _attention_errors(qkv, S):
+    """FULL copies of one sequence of one head: (error of the first, error of the last) against the oracle."""
+    got = q8.q8_attention(dev(np.tile(qkv, (FULL, 1))), FULL, S, 1).cpu().numpy()
+    assert q8.q8_attention_status() == (q8.Q8_OK, 0)
+    ref = o.attention(qkv, 1, S, 1)
+    return [np.abs(x - ref).max() / np.abs(ref).max() for x in (got[:S], got[-S:])]
+
+
+@pytest.mark.parametrize("S", [1, 31, 33, 63, 65, 95, 97, 127, 129, 193, 385, 512, 513])
+def test_attention_at_chunk_and_tile_edges(S):
+    assert max(_attention_errors(synth.normal((S, 3 * 64), 1.0, 3300 + S), S)) <= EDGE_TOL
+
+
+@pytest.mark.parametrize("S", [100, 200])
+def test_attention_scales_of_its_operands(S):
+    """Powers of two moved between Q and K, and between the chunks of V, leave the accuracy as it is: every operand tile is
+    brought into fp16's range by a scale of its own.  A maximum that rises from chunk to chunk rescales what is summed."""
+    qkv = synth.normal((S, 3 * 64), 1.0, 3400 + S)
+    moved = qkv.copy()
+    moved[:, :64] *= 2.0 ** 40
+    moved[:, 64:128] *= 2.0 ** -40
+    assert max(_attention_errors(moved, S)) <= EDGE_TOL
+    for first, later in ((2.0 ** 20, 2.0 ** -20), (2.0 ** -20, 2.0 ** 20), (1.0, 0.0), (0.0, 1.0)):
+        v = qkv.copy()
+        v[:64, 128:] *= np.float32(first)
+        v[64:, 128:] *= np.float32(later)
+        assert max(_attention_errors(v, S)) <= EDGE_TOL
+    rising = qkv.copy()
+    rising[:, 64:128] *= np.linspace(0.1, 8.0, S, dtype=np.float32)[:, None]  # scores up to ~50: EDGE_TOL * 8 by the same sum
+    assert max(_attention_errors(rising, S)) <= 8 * EDGE_TOL
+
+
+def test_attention_non_finite_rows_stay_in_their_rows():
+    S = 130
+    qkv = synth.normal((S, 3 * 64), 1.0, 3500)
+    bad = qkv.copy()
+    bad[70, 0] = np.nan                # a query: its own row
+    bad[71, 3] = np.inf
+    bad[100, 128 + 5] = np.inf         # a value: its feature of every row
+    got = q8.q8_attention(dev(np.tile(bad, (FULL, 1))), FULL, S, 1).cpu().numpy()[-S:]
+    ref = o.attention(qkv, 1, S, 1)
+    rows, features = np.delete(np.arange(S), [70, 71]), np.delete(np.arange(64), 5)
+    assert np.isnan(got[70]).all() and np.isnan(got[71]).all() and not np.isfinite(got[:, 5]).any()
+    assert np.abs(got[np.ix_(rows, features)] - ref[np.ix_(rows, features)]).max() <= EDGE_TOL * np.abs(ref).max()
