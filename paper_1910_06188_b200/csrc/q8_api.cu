@@ -31,6 +31,16 @@ q8_status quantize_tensor(const float *X, int64_t numel, const float *S_given, i
 {
     LaunchInfo &li = last_launch_info();
     const float *S = S_given;
+    if (S_given == nullptr && quantize_dynamic_small_supported(X, numel, Xq, Xq_copy)) {
+        Q8_CUDA_TRY(launch_quantize_dynamic_small(X, numel, S_dyn, status, false, Xq, Xq_copy, s));
+        li.launches += 1;
+        return Q8_OK;
+    }
+    if (S_given == nullptr && quantize_dynamic_grid_supported(X, numel, Xq, Xq_copy)) {
+        Q8_CUDA_TRY(launch_quantize_dynamic_grid(X, numel, S_dyn, status, Xq, Xq_copy, s));
+        li.launches += 1;
+        return Q8_OK;
+    }
     if (S_given == nullptr) {
         // The scale word first holds the float bits of the running maximum, then the scale itself.
         if (!S_dyn_is_zero) Q8_CUDA_TRY(cudaMemsetAsync(S_dyn, 0, sizeof(float), s));
@@ -90,8 +100,8 @@ q8_status linear_impl(const float *X, const int8_t *Wq, const float *S_w, const 
     WorkspaceHeader *hdr = static_cast<WorkspaceHeader *>(workspace);
     int8_t *Xq = static_cast<int8_t *>(workspace) + kWorkspaceHeaderBytes;
     // Eq. 1.  With a given scale the quantise kernel itself starts the call's status word at zero (no separate
-    // clearing operation in the stream); with the Sec. 4.1 dynamic scale (S_x NULL) the header is zeroed first, then
-    // come the abs-max pass and one kernel that turns the maximum into the scale and quantises with it.
+    // clearing operation in the stream); with the Sec. 4.1 dynamic scale (S_x NULL) come an abs-max pass and one
+    // kernel that turns its partial maxima into the scale and quantises with it.
     if ((x_absmax && !aligned_to(x_absmax, 4)) || (y_absmax && !aligned_to(y_absmax, 4))) return Q8_ERR_ALIGN;
     if (S_x != nullptr) {
         Q8_CUDA_TRY(launch_quantize(X, M * K, S_x, Xq, dbg_Xq, s, &hdr->status));
@@ -103,12 +113,13 @@ q8_status linear_impl(const float *X, const int8_t *Wq, const float *S_w, const 
         last_launch_info().launches += 1;
     } else if (quantize_dynamic_small_supported(X, M * K, Xq, dbg_Xq)) {
         // a small activation (up to 256 x 768): abs-max, scale and Eq. 1 in one launch of one cluster, no memset
-        Q8_CUDA_TRY(launch_quantize_dynamic_small(X, M * K, &hdr->S_x_dyn, &hdr->status, Xq, dbg_Xq, s));
+        Q8_CUDA_TRY(launch_quantize_dynamic_small(X, M * K, &hdr->S_x_dyn, &hdr->status, true, Xq, dbg_Xq, s));
         last_launch_info().launches += 1;
     } else {
-        Q8_CUDA_TRY(cudaMemsetAsync(hdr, 0, sizeof(WorkspaceHeader), s));
-        Q8_CUDA_TRY(launch_absmax(X, M * K, &hdr->absmax_bits, s));
-        Q8_CUDA_TRY(launch_quantize_dynamic(X, M * K, &hdr->absmax_bits, &hdr->S_x_dyn, &hdr->status, Xq, dbg_Xq, s));
+        int words = 0;
+        Q8_CUDA_TRY(launch_absmax_partial(X, M * K, hdr->absmax_partial,
+                                          (int)(sizeof(hdr->absmax_partial) / sizeof(hdr->absmax_partial[0])), &words, s));
+        Q8_CUDA_TRY(launch_quantize_dynamic(X, M * K, hdr->absmax_partial, &hdr->S_x_dyn, &hdr->status, Xq, dbg_Xq, s, true, words));
         last_launch_info().launches += 2;
     }
 
@@ -212,9 +223,8 @@ q8_status q8_calibrate(const float *X, int64_t numel, float decay, void *state, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     CalibState *st = static_cast<CalibState *>(state);
     if (numel == 0) return Q8_OK;  // an empty batch is no observation of max|x|: the running state stays as it is
-    Q8_CUDA_TRY(launch_absmax(X, numel, &st->scratch_bits, s));
-    Q8_CUDA_TRY(launch_ema_update(st, decay, s));
-    last_launch_info().launches = 2;
+    Q8_CUDA_TRY(launch_absmax(X, numel, &st->scratch_bits, s, st, decay));
+    last_launch_info().launches = 1;
     return Q8_OK;
 }
 

@@ -4,6 +4,8 @@
 // All of them stream their input once with 16-byte loads and stores; the grid is a multiple of
 // the SM count with a grid-stride loop so every SM keeps several independent loads in flight.
 
+#include <cooperative_groups.h>
+
 #include "q8_internal.cuh"
 
 namespace q8 {
@@ -40,10 +42,15 @@ __device__ __forceinline__ float absmax4(float m, float4 v)
     return fmaxf(m, fabsf(v.w));
 }
 
+__device__ __forceinline__ void ema_update(CalibState *st, float m, float decay);
+
+// With st the last CTA to finish (counted in the state's own counter, which it leaves at zero) also makes the Eq. 4 update.
 template <bool VEC>
-__global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restrict__ x, int64_t n,
-                                                          uint32_t *__restrict__ bits)
+__global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restrict__ x, int64_t n, uint32_t *bits,
+                                                          CalibState *st, float decay)
 {
+    grid_dependency_release_next(n <= kSmallProblemElems);
+    grid_dependency_wait();
     float m = 0.0f;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
@@ -51,11 +58,13 @@ __global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restric
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
         const int64_t n4 = n >> 2;
         int64_t i = tid;
-        // four independent 16-byte loads per iteration
-        for (; i + 3 * nthreads < n4; i += 4 * nthreads) {
-            float4 a = __ldg(x4 + i), b = __ldg(x4 + i + nthreads), c = __ldg(x4 + i + 2 * nthreads),
-                   d = __ldg(x4 + i + 3 * nthreads);
-            m = absmax4(absmax4(absmax4(absmax4(m, a), b), c), d);
+        // eight independent 16-byte loads per iteration
+        for (; i + 7 * nthreads < n4; i += 8 * nthreads) {
+            float4 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = __ldg(x4 + i + k * nthreads);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m = absmax4(m, v[k]);
         }
         for (; i < n4; i += nthreads) m = absmax4(m, __ldg(x4 + i));
         for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
@@ -71,14 +80,74 @@ __global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restric
         m = threadIdx.x < kThreads / 32 ? warp_max[threadIdx.x] : 0.0f;
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        // non-negative floats (and +Inf) order like their bit patterns
-        if (threadIdx.x == 0 && m > 0.0f) atomicMax(bits, __float_as_uint(m));
+        if (threadIdx.x == 0) {
+            // non-negative floats (and +Inf) order like their bit patterns
+            if (m > 0.0f) atomicMax(bits, __float_as_uint(m));
+            if (st != nullptr) {
+                __threadfence();
+                if (atomicInc(&st->finished_ctas, gridDim.x - 1) == gridDim.x - 1)
+                    ema_update(st, __uint_as_float(atomicExch(bits, 0u)), decay);
+            }
+        }
     }
+}
+
+// max|x| as one partial maximum per cluster of CTAs (exchanged through distributed shared memory): every word of `partial`
+// is written, so nothing has to be cleared first (a dynamic q8_linear on 1421 x 768 -> 768: 12.7 -> 10.8 us).
+constexpr int kAmCluster = 8;
+
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads) absmax_partial_kernel(const float *__restrict__ x, int64_t n,
+                                                                  uint32_t *__restrict__ partial)
+{
+    grid_dependency_release_next(n <= kSmallProblemElems);
+    grid_dependency_wait();
+    float m = 0.0f;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        const float4 *x4 = reinterpret_cast<const float4 *>(x);
+        const int64_t n4 = n >> 2;
+        int64_t i = tid;
+        for (; i + 7 * nthreads < n4; i += 8 * nthreads) {
+            float4 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = __ldg(x4 + i + k * nthreads);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m = absmax4(m, v[k]);
+        }
+        for (; i < n4; i += nthreads) m = absmax4(m, __ldg(x4 + i));
+        for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
+    } else {
+        for (int64_t j = tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
+    }
+    __shared__ uint32_t cta_max;
+    if (threadIdx.x == 0) cta_max = 0u;
+    __syncthreads();
+    const uint32_t bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) atomicMax(&cta_max, bits);
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (blockIdx.x % kAmCluster == 0 && threadIdx.x < 32) {
+        uint32_t p = 0;
+        if (threadIdx.x < kAmCluster) {
+            uint32_t remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                         : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(&cta_max)), "r"((uint32_t)threadIdx.x));
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(p) : "r"(remote) : "memory");
+        }
+        p = __reduce_max_sync(0xffffffffu, p);
+        if (threadIdx.x == 0) partial[blockIdx.x / kAmCluster] = p;
+    }
+    // no CTA may exit (and give up its shared memory) while a peer can still read it
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // S = 127 / max|.| (Eq. 3), in place over the scratch word when bits and S alias.
 __global__ void scale_from_absmax_kernel(const uint32_t *bits, float *S, int32_t *status)
 {
+    grid_dependency_release_next(true);
+    grid_dependency_wait();
     float a = __uint_as_float(*bits);
     float s;
     if (!(a > 0.0f) || isinf(a)) {
@@ -105,7 +174,7 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
                                                             const float *__restrict__ S_ptr,
                                                             int8_t *__restrict__ xq, int8_t *__restrict__ xq_copy,
                                                             const uint32_t *__restrict__ absmax_bits = nullptr,
-                                                            float *__restrict__ S_out = nullptr,
+                                                            int absmax_count = 1, float *__restrict__ S_out = nullptr,
                                                             int32_t *__restrict__ status = nullptr,
                                                             int32_t *__restrict__ clear_word = nullptr)
 {
@@ -115,7 +184,14 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
     if (clear_word != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *clear_word = 0;
     float S;
     if (absmax_bits != nullptr) {
-        const float a = __uint_as_float(__ldg(absmax_bits));
+        uint32_t am = 0u;  // the maximum, or the largest of absmax_count partial maxima
+        if (absmax_count == 1) {
+            am = __ldg(absmax_bits);
+        } else {
+            for (int k = threadIdx.x & 31; k < absmax_count; k += 32) am = max(am, __ldg(absmax_bits + k));
+            am = __reduce_max_sync(0xffffffffu, am);
+        }
+        const float a = __uint_as_float(am);
         const bool bad = !(a > 0.0f) || isinf(a);
         S = bad ? 1.0f : __fdiv_rn(127.0f, a);
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -184,7 +260,7 @@ constexpr int64_t kDqMaxElems = (int64_t)kDqCluster * kDqThreads * kDqVecPerThre
 
 __global__ void __launch_bounds__(kDqThreads) quantize_dynamic_cluster_kernel(const float *__restrict__ x, int64_t n,
                                                                               float *__restrict__ S_out,
-                                                                              int32_t *__restrict__ status,
+                                                                              int32_t *__restrict__ status, int set_status,
                                                                               int8_t *__restrict__ xq,
                                                                               int8_t *__restrict__ xq_copy)
 {
@@ -239,7 +315,10 @@ __global__ void __launch_bounds__(kDqThreads) quantize_dynamic_cluster_kernel(co
     const float S = bad ? 1.0f : __fdiv_rn(127.0f, a);
     if (rank == 0 && threadIdx.x == 0) {
         *S_out = S;
-        if (status) *status = bad ? (1 << Q8_ERR_SCALE) : 0;  // first kernel of the call: starts the status word
+        if (status != nullptr) {
+            if (set_status) *status = bad ? (1 << Q8_ERR_SCALE) : 0;  // first kernel of a call: starts its status word
+            else if (bad) atomicOr(status, 1 << Q8_ERR_SCALE);
+        }
     }
     uint32_t *q4 = reinterpret_cast<uint32_t *>(xq);
     uint32_t *c4 = reinterpret_cast<uint32_t *>(xq_copy);
@@ -255,11 +334,88 @@ __global__ void __launch_bounds__(kDqThreads) quantize_dynamic_cluster_kernel(co
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// ------------------------------------------------------------------ Eq. 4
-__global__ void ema_update_kernel(CalibState *st, float decay)
+// The same in ONE launch for tensors that no longer fit one cluster's registers: a cooperative grid finds max|x|, meets,
+// derives S and quantises.  Up to kCoopMaxElems: the barriers cost about as much device time as the launches they replace
+// (a 2048 x 768 weight 8.55 against 8.59 us for memset, abs-max, scale, quantise), but one call to the driver takes the place
+// of four; a 125 MB matrix would take 54 us instead of 51, the second pass being bound by the conversions and latency
+// even where it hits L2.
+// *word holds the running maximum (float bits) during the first pass and S at the end, so a single device word is enough;
+// a bad maximum is OR-ed into *status (may be NULL).
+constexpr int kCoopThreads = 256, kCoopCtasPerSm = 4;
+constexpr int64_t kCoopMaxElems = int64_t(4) << 20;
+
+__global__ void __launch_bounds__(kCoopThreads, kCoopCtasPerSm)
+quantize_dynamic_grid_kernel(const float *__restrict__ x, int64_t n, uint32_t *word, int32_t *status,
+                             int8_t *__restrict__ xq, int8_t *__restrict__ xq_copy)
 {
-    float m = __uint_as_float(st->scratch_bits);
-    st->scratch_bits = 0u;
+    namespace cg = cooperative_groups;
+    cg::grid_group grid = cg::this_grid();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *word = 0u;
+    auto word_cleared = grid.barrier_arrive();  // waited for after the first pass
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+    const float4 *x4 = reinterpret_cast<const float4 *>(x);
+    const int64_t n4 = n >> 2, rest = n4 << 2;  // the last n % 4 values go to the first threads
+    float m = 0.0f;
+    int64_t i = tid;
+    for (; i + 7 * nthreads < n4; i += 8 * nthreads) {
+        float4 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __ldg(x4 + i + k * nthreads);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m = absmax4(m, v[k]);
+    }
+    for (; i < n4; i += nthreads) m = absmax4(m, __ldg(x4 + i));
+    if (rest + tid < n) m = fmaxf(m, fabsf(x[rest + tid]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    __shared__ float warp_max[kCoopThreads / 32];
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+    grid.barrier_wait(static_cast<cg::grid_group::arrival_token &&>(word_cleared));
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 0; w < kCoopThreads / 32; ++w) m = fmaxf(m, warp_max[w]);
+        if (m > 0.0f) atomicMax(word, __float_as_uint(m));  // non-negative floats (and +Inf) order like their bit patterns
+    }
+    grid.sync();
+    const float a = __uint_as_float(*reinterpret_cast<volatile uint32_t *>(word));
+    auto word_read = grid.barrier_arrive();  // waited for before S takes the maximum's place
+    const bool bad = !(a > 0.0f) || isinf(a);
+    const float S = bad ? 1.0f : __fdiv_rn(127.0f, a);
+    uint32_t *q4 = reinterpret_cast<uint32_t *>(xq);
+    uint32_t *c4 = reinterpret_cast<uint32_t *>(xq_copy);
+    if (rest + tid < n) {
+        const int8_t q = (int8_t)quantize_one(x[rest + tid], S);
+        xq[rest + tid] = q;
+        if (xq_copy) xq_copy[rest + tid] = q;
+    }
+    i = n4 - 1 - tid;
+    for (; i - 3 * nthreads >= 0; i -= 4 * nthreads) {
+        float4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldg(x4 + i - k * nthreads);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t q = quantize_pack4(v[k], S);
+            __stcs(q4 + i - k * nthreads, q);
+            if (xq_copy) __stcs(c4 + i - k * nthreads, q);
+        }
+    }
+    for (; i >= 0; i -= nthreads) {
+        const uint32_t q = quantize_pack4(__ldg(x4 + i), S);
+        q4[i] = q;
+        if (xq_copy) c4[i] = q;
+    }
+    grid.barrier_wait(static_cast<cg::grid_group::arrival_token &&>(word_read));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *reinterpret_cast<float *>(word) = S;
+        if (bad && status != nullptr) atomicOr(status, 1 << Q8_ERR_SCALE);
+    }
+}
+
+// ------------------------------------------------------------------ Eq. 4
+__device__ __forceinline__ void ema_update(CalibState *st, float m, float decay)
+{
     float ema;
     if (st->n_batches == 0 || decay == 0.0f) {
         ema = m;  // first batch, or no history kept: exactly this batch's maximum (the dynamic scale of Sec. 4.1)
@@ -347,28 +503,44 @@ __global__ void __launch_bounds__(kThreads) embedding_kernel(const int32_t *__re
 }
 
 // ------------------------------------------------------------------ training mode: fake quantisation (Sec. 2.2)
-// x_hat = Quantize(x | S) / S: the rounding of Eq. 1 simulated in floating point (one fp32 division per element).
-__device__ __forceinline__ float fake_one(float x, float S) { return __fdiv_rn((float)quantize_value(x, S), S); }
-
+// x_hat = Quantize(x | S) / S: the rounding of Eq. 1 simulated in floating point.  The quotient of an integer of -127..127
+// and S takes one of 255 values: each CTA makes the table of them with correctly rounded divisions and every element is
+// a shared-memory look-up instead of a division (4096 x 3072: 24.6 -> 16.2 us, 16384 x 3072: 99.5 -> 70.8 us =
+// 5.7 TB/s; four loads in flight instead of one are part of that).
 template <bool VEC>
-__global__ void __launch_bounds__(kThreads) fake_quantize_kernel(const float *__restrict__ x, int64_t n,
-                                                                 const float *__restrict__ S_ptr,
-                                                                 float *__restrict__ xhat)
+__global__ void __launch_bounds__(kThreads) fake_quantize_kernel(const float *x, int64_t n,
+                                                                 const float *__restrict__ S_ptr, float *xhat)
 {
+    static_assert(kThreads == 256, "one table entry per thread");
+    __shared__ float table[256];
+    grid_dependency_release_next(n <= kSmallProblemElems);
+    grid_dependency_wait();
     const float S = __ldg(S_ptr);
+    table[threadIdx.x] = __fdiv_rn((float)((int)threadIdx.x - 128), S);
+    __syncthreads();
+    auto fake = [&](float v) { return table[128 + quantize_value(v, S)]; };
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     if (VEC) {
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
         float4 *o4 = reinterpret_cast<float4 *>(xhat);
         const int64_t n4 = n >> 2;
-        for (int64_t i = tid; i < n4; i += nthreads) {
-            const float4 v = __ldg(x4 + i);
-            o4[i] = make_float4(fake_one(v.x, S), fake_one(v.y, S), fake_one(v.z, S), fake_one(v.w, S));
+        int64_t i = tid;
+        for (; i + 3 * nthreads < n4; i += 4 * nthreads) {  // four loads in flight
+            float4 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = x4[i + k * nthreads];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                o4[i + k * nthreads] = make_float4(fake(v[k].x), fake(v[k].y), fake(v[k].z), fake(v[k].w));
         }
-        for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) xhat[j] = fake_one(x[j], S);
+        for (; i < n4; i += nthreads) {
+            const float4 v = x4[i];
+            o4[i] = make_float4(fake(v.x), fake(v.y), fake(v.z), fake(v.w));
+        }
+        for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) xhat[j] = fake(x[j]);
     } else {
-        for (int64_t j = tid; j < n; j += nthreads) xhat[j] = fake_one(x[j], S);
+        for (int64_t j = tid; j < n; j += nthreads) xhat[j] = fake(x[j]);
     }
 }
 
@@ -376,21 +548,76 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 }  // namespace
 
-cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_t s)
+cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_t s, CalibState *st, float decay)
 {
     if (n <= 0) return cudaSuccess;
-    if (aligned16(x)) {
-        absmax_kernel<true><<<grid_for(n >> 2, kThreads * 4, 8), kThreads, 0, s>>>(x, n, bits);
-    } else {
-        absmax_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, bits);
+    if (aligned16(x))
+        return launch_overlapping_tail(absmax_kernel<true>, dim3(grid_for(n >> 2, kThreads * 4, 8)), dim3(kThreads), 0, s, x, n,
+                                       bits, st, decay);
+    return launch_overlapping_tail(absmax_kernel<false>, dim3(grid_for(n, kThreads * 4, 8)), dim3(kThreads), 0, s, x, n, bits,
+                                   st, decay);
+}
+
+cudaError_t launch_absmax_partial(const float *x, int64_t n, uint32_t *partial, int max_words, int *words, cudaStream_t s)
+{
+    const bool vec = aligned16(x);
+    int clusters = (grid_for(vec ? n >> 2 : n, kThreads * 4, 2) + kAmCluster - 1) / kAmCluster;
+    if (clusters > max_words) clusters = max_words;
+    *words = clusters;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * kAmCluster));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kAmCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, vec ? absmax_partial_kernel<true> : absmax_partial_kernel<false>, x, n, partial);
+}
+
+bool quantize_dynamic_grid_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy)
+{
+    return n > 0 && n <= kCoopMaxElems && aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy));
+}
+
+cudaError_t launch_quantize_dynamic_grid(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq, int8_t *xq_copy,
+                                         cudaStream_t s)
+{
+    static int resident[64] = {};  // CTAs of the kernel that fit on the device at a time
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (resident[dev] == 0) {
+        int per_sm = 0, sms = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quantize_dynamic_grid_kernel, kCoopThreads, 0);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1 || sms < 1) return cudaErrorCooperativeLaunchTooLarge;
+        resident[dev] = sms * (per_sm < kCoopCtasPerSm ? per_sm : kCoopCtasPerSm);
     }
-    return cudaGetLastError();
+    const int64_t want = ((n >> 2) + kCoopThreads * 4 - 1) / (kCoopThreads * 4);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(want < 1 ? 1 : want < resident[dev] ? want : resident[dev]));
+    cfg.blockDim = dim3(kCoopThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, quantize_dynamic_grid_kernel, x, n, reinterpret_cast<uint32_t *>(S_out), status,
+                              xq, xq_copy);
 }
 
 cudaError_t launch_scale_from_absmax(const uint32_t *bits, float *S, int32_t *status, cudaStream_t s)
 {
-    scale_from_absmax_kernel<<<1, 1, 0, s>>>(bits, S, status);
-    return cudaGetLastError();
+    return launch_overlapping_tail(scale_from_absmax_kernel, dim3(1), dim3(1), 0, s, bits, S, status);
 }
 
 // Grid of the vectorised quantise pass: CTAs per SM, grid-stride.  Measured on 24576 x 1024 / 24576 x 4096 fp32 inputs
@@ -405,25 +632,25 @@ cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *x
     if (n <= 0) return cudaSuccess;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
         return launch_overlapping_tail(quantize_kernel<true>, dim3(grid_for((n + 3) >> 2, kThreads * 4, kQuantCtasPerSm)),
-                                       dim3(kThreads), 0, s, x, n, S, xq, xq_copy, nullptr, nullptr, status, clear_word);
+                                       dim3(kThreads), 0, s, x, n, S, xq, xq_copy, nullptr, 1, nullptr, status, clear_word);
     } else {
-        quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, S, xq, xq_copy, nullptr, nullptr,
+        quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, S, xq, xq_copy, nullptr, 1, nullptr,
                                                                                  status, clear_word);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *absmax_bits, float *S_out, int32_t *status,
-                                    int8_t *xq, int8_t *xq_copy, cudaStream_t s, bool clear_status)
+                                    int8_t *xq, int8_t *xq_copy, cudaStream_t s, bool clear_status, int absmax_count)
 {
     if (n <= 0) return cudaSuccess;
     int32_t *clear_word = clear_status ? status : nullptr;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
         return launch_overlapping_tail(quantize_kernel<true>, dim3(grid_for((n + 3) >> 2, kThreads * 4, kQuantCtasPerSm)),
-                                       dim3(kThreads), 0, s, x, n, nullptr, xq, xq_copy, absmax_bits, S_out, status, clear_word);
+                                       dim3(kThreads), 0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
     } else {
         quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, nullptr, xq, xq_copy, absmax_bits,
-                                                                                 S_out, status, clear_word);
+                                                                                 absmax_count, S_out, status, clear_word);
     }
     return cudaGetLastError();
 }
@@ -434,7 +661,7 @@ bool quantize_dynamic_small_supported(const float *x, int64_t n, const int8_t *x
            (xq_copy == nullptr || aligned16(xq_copy));
 }
 
-cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq,
+cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_out, int32_t *status, bool set_status, int8_t *xq,
                                           int8_t *xq_copy, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -450,24 +677,17 @@ cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_ou
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, quantize_dynamic_cluster_kernel, x, n, S_out, status, xq, xq_copy);
+    return cudaLaunchKernelEx(&cfg, quantize_dynamic_cluster_kernel, x, n, S_out, status, set_status ? 1 : 0, xq, xq_copy);
 }
 
 cudaError_t launch_fake_quantize(const float *x, int64_t n, const float *S, float *xhat, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    if (aligned16(x) && aligned16(xhat)) {
-        fake_quantize_kernel<true><<<grid_for((n + 3) >> 2, kThreads * 4, 8), kThreads, 0, s>>>(x, n, S, xhat);
-    } else {
-        fake_quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, S, xhat);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ema_update(CalibState *st, float decay, cudaStream_t s)
-{
-    ema_update_kernel<<<1, 1, 0, s>>>(st, decay);
-    return cudaGetLastError();
+    if (aligned16(x) && aligned16(xhat))
+        return launch_overlapping_tail(fake_quantize_kernel<true>, dim3(grid_for((n + 3) >> 2, kThreads * 4, 4)), dim3(kThreads),
+                                       0, s, x, n, S, xhat);
+    return launch_overlapping_tail(fake_quantize_kernel<false>, dim3(grid_for(n, kThreads * 4, 8)), dim3(kThreads), 0, s, x, n,
+                                   S, xhat);
 }
 
 cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, const float *S_e, int64_t V,

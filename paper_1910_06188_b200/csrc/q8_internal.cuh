@@ -13,10 +13,11 @@ namespace q8 {
 struct WorkspaceHeader {
     int32_t status;        // OR of (1 << q8_status) bits raised by kernels
     float S_x_dyn;         // dynamic mode: 127 / max|X|, written by the quantise kernel
-    uint32_t absmax_bits;  // dynamic mode: float bits of max|X| (atomicMax scratch, zero at the start of a call)
-    int32_t pad;
+    int32_t pad[2];
+    uint32_t absmax_partial[60];  // dynamic mode: float bits of partial maxima of |X|
 };
 constexpr size_t kWorkspaceHeaderBytes = 256;
+static_assert(sizeof(WorkspaceHeader) == kWorkspaceHeaderBytes, "workspace header");
 
 // Device block behind q8_calibrate (Eq. 4 running state).
 struct CalibState {
@@ -25,7 +26,8 @@ struct CalibState {
     int32_t n_batches;
     uint32_t scratch_bits;
     int32_t status;
-    int32_t pad[3];
+    uint32_t finished_ctas;  // CTAs of the running q8_calibrate that are done; zero between calls
+    int32_t pad[2];
 };
 
 struct GemmArgs {
@@ -58,8 +60,12 @@ struct LaunchInfo {
 LaunchInfo &last_launch_info();
 
 // ---- elementwise / reduction launchers (q8_elementwise.cu) ----
-// max|x| folded into *bits (must hold 0 or an earlier maximum) with atomicMax on the float bits.
-cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_t s);
+// max|x| folded into *bits (must hold 0 or an earlier maximum) with atomicMax on the float bits.  With st the Eq. 4 update
+// of that state follows in the same launch and *bits is zero again afterwards.
+cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_t s, CalibState *st = nullptr,
+                          float decay = 0.0f);
+// max|x| as up to max_words partial maxima; *words receives how many were written (n > 0).
+cudaError_t launch_absmax_partial(const float *x, int64_t n, uint32_t *partial, int max_words, int *words, cudaStream_t s);
 // *S = 127 / float(*bits) in place (bits and S may alias); flags Q8_ERR_SCALE on 0 / non-finite.
 cudaError_t launch_scale_from_absmax(const uint32_t *bits, float *S, int32_t *status, cudaStream_t s);
 // clear_word (may be NULL): a device word the kernel sets to zero before anything else (a call's status word).
@@ -68,16 +74,20 @@ cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *x
                             cudaStream_t s, int32_t *clear_word = nullptr, int32_t *status = nullptr);
 // Eq. 1 with S = 127 / float(*absmax_bits) derived inside the kernel (dynamic scale); *S_out receives S and
 // *status the Q8_ERR_SCALE bit when the maximum is 0 or not finite (S = 1 then).  absmax_bits and S_out differ.
-// clear_status: start *status at zero first (the call's status word, when no memset precedes the kernel).
+// absmax_count: that many partial maxima from absmax_bits on.  clear_status: start *status at zero first (the call's status word, when no memset precedes the kernel).
 cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *absmax_bits, float *S_out,
                                     int32_t *status, int8_t *xq, int8_t *xq_copy, cudaStream_t s,
-                                    bool clear_status = false);
+                                    bool clear_status = false, int absmax_count = 1);
 // Small tensors (n <= 196608, n % 4 == 0, 16-byte aligned): abs-max, scale and Eq. 1 in one launch of one cluster.
-// *status (may be NULL) is SET (0 or the Q8_ERR_SCALE bit), not OR-ed into.
+// *status (may be NULL) is SET (0 or the Q8_ERR_SCALE bit) with set_status, else OR-ed into.
 bool quantize_dynamic_small_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
-cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq,
+cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_out, int32_t *status, bool set_status, int8_t *xq,
                                           int8_t *xq_copy, cudaStream_t s);
-cudaError_t launch_ema_update(CalibState *st, float decay, cudaStream_t s);
+// Larger ones, up to 4 Mi values (16-byte aligned): the same in one cooperative launch.  *S_out also serves as the reduction
+// word; *status (may be NULL) is OR-ed into.
+bool quantize_dynamic_grid_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
+cudaError_t launch_quantize_dynamic_grid(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq, int8_t *xq_copy,
+                                         cudaStream_t s);
 cudaError_t launch_fake_quantize(const float *x, int64_t n, const float *S, float *xhat, cudaStream_t s);
 cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, const float *S_e, int64_t V,
                              int64_t H, float *out, int8_t *rows_q, int32_t *status, cudaStream_t s);

@@ -338,3 +338,48 @@ def test_fused_projection_with_per_layer_scales_equals_separate_layers(M, H, seg
         assert_close_fp(Y[:, i * H:(i + 1) * H].cpu().numpy(), ref["y"], f"segment {i}")
     Xq, S_x = q8.q8_quantize_activation(dev(X))
     assert torch.equal(q8.q8_linear_q_wseg(Xq, S_x, Wq, S_w, seg, dev(b), act), Y)
+
+
+# ------------------------------------------------------------------ routes of the dynamic scale
+@pytest.mark.parametrize("n", [1, 3, 4, 4095, 196607, 196608, 196612, 300001, 1 << 20, (4 << 20) - 1, 4 << 20, (4 << 20) + 5])
+@pytest.mark.parametrize("peak_at", ["first", "last"])
+def test_dynamic_quantisation_in_one_or_several_launches(n, peak_at):
+    """One cluster, one cooperative grid or separate passes (by size): the same integers, the same scale, and the largest
+    value is found wherever it lies; a zero tensor flags the scale without clearing the caller's status word."""
+    x = synth.normal((n,), 1.0, 9000 + n % 1000)
+    x[0 if peak_at == "first" else -1] = -9.0
+    xq, s = q8.q8_quantize_activation(dev(x))
+    s_ref, _ = o.scale_from_absmax(o.absmax(x))
+    assert s.cpu().numpy()[0] == s_ref
+    assert np.array_equal(xq.cpu().numpy(), o.quantize(x, s_ref))
+    word = torch.full((1,), 1 << 20, dtype=torch.int32, device="cuda")
+    zq, zs = q8.q8_quantize_activation(torch.zeros(n, device="cuda"), dev_status=word)
+    assert zs.item() == 1.0 and not zq.any() and word.item() == (1 << 20) | (1 << q8.Q8_ERR_SCALE)
+
+
+@pytest.mark.parametrize("M,K", [(1, 13), (3, 65537), (257, 768), (1000, 300), (4096, 1040)])
+def test_dynamic_linear_finds_the_peak_of_every_share(M, K):
+    """The partial maxima of the abs-max pass: the scale is that of the largest value, in whichever CTA's share it lies."""
+    W = synth.weight(16, K, 9100)
+    for at in (0, M * K // 2, M * K - 1):
+        x = synth.normal((M, K), 1.0, 9101)
+        x.flat[at] = 11.0
+        Wq, S_w = q8.q8_quantize_weight(dev(W))
+        ws = q8.new_workspace(M, 16, K)
+        q8.q8_linear(dev(x), Wq, S_w, None, None, 0, workspace=ws)
+        assert ws[4:8].view(torch.float32).item() == np.float32(127.0) / np.float32(11.0)
+        assert q8.q8_poll_status(ws) == (q8.Q8_OK, 0)
+
+
+@pytest.mark.parametrize("n", [1, 5, 1023, 4096, 1 << 20, (1 << 20) + 3])
+def test_calibration_leaves_its_counter_at_zero_and_fake_quantisation_divides_exactly(n):
+    x = synth.activation(1, n, 9200)[0]
+    state = q8.new_calibrate_state()
+    for _ in range(3):
+        q8.q8_calibrate(dev(x), 0.9999, state)
+    words = state.cpu().numpy()
+    assert words[2] == 3 and words[3] == 0 and not words[4:].any()
+    S = np.float32(127.0) / np.abs(x).max()
+    assert q8.calibrate_S_x(state).item() == S
+    got = q8.q8_fake_quantize(dev(x), q8.calibrate_S_x(state)).cpu().numpy()
+    assert np.array_equal(got, o.quantize(x, S).astype(np.float32) / S)
