@@ -383,3 +383,35 @@ def test_calibration_leaves_its_counter_at_zero_and_fake_quantisation_divides_ex
     assert q8.calibrate_S_x(state).item() == S
     got = q8.q8_fake_quantize(dev(x), q8.calibrate_S_x(state)).cpu().numpy()
     assert np.array_equal(got, o.quantize(x, S).astype(np.float32) / S)
+
+
+# ------------------------------------------------------------------ operands that TMA cannot fetch
+@pytest.mark.parametrize("K", [8, 24, 56, 72, 4, 20, 132, 1, 3, 63, 65, 129, 1001])
+@pytest.mark.parametrize("M,N", [(1, 1), (63, 65), (65, 130), (1700, 1665)])
+def test_generic_gemm_pieces_and_tile_edges(M, N, K):
+    """Pieces of 8, 4 and single bytes of K, both tile sizes (1700 x 1665: more than 148 of 128 x 128), ragged everywhere."""
+    rng = np.random.default_rng(K * 7 + M)
+    Xq, Wq = (rng.integers(-127, 128, size=(n, K), dtype=np.int8) for n in (M, N))
+    acc = torch.empty((M, N), dtype=torch.int32, device="cuda")
+    q8.q8_linear_q(dev(Xq), torch.ones(1, device="cuda"), dev(Wq), torch.ones(1, device="cuda"), None, 0, dbg_acc=acc)
+    assert q8.q8_last_launch_info()["gemm_kernel"] == 2
+    assert np.array_equal(acc.cpu().numpy(), Xq.astype(np.int32) @ Wq.astype(np.int32).T)
+
+
+@pytest.mark.parametrize("offset_x,offset_w", [(8, 0), (4, 8), (1, 0), (0, 3), (2, 1)])
+def test_generic_gemm_pointers_at_any_byte(offset_x, offset_w):
+    M, N, K = 70, 66, 96
+    rng = np.random.default_rng(77)
+    Xq, Wq = (rng.integers(-127, 128, size=(n, K), dtype=np.int8) for n in (M, N))
+
+    def at(a, offset):
+        buf = torch.empty(a.size + offset, dtype=torch.int8, device="cuda")
+        buf[offset:] = dev(a).reshape(-1)
+        return buf[offset:].view(a.shape)
+
+    acc = torch.empty((M, N), dtype=torch.int32, device="cuda")
+    Y = torch.empty(M * N + 1, device="cuda")[1:].view(M, N)  # 4-byte aligned output: no 8-byte stores
+    one = torch.ones(1, device="cuda")
+    q8.q8_linear_q(at(Xq, offset_x), one, at(Wq, offset_w), one, None, 0, Y=Y, dbg_acc=acc)
+    ref = Xq.astype(np.int32) @ Wq.astype(np.int32).T
+    assert np.array_equal(acc.cpu().numpy(), ref) and np.array_equal(Y.cpu().numpy(), ref.astype(np.float32))
