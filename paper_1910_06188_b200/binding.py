@@ -4,6 +4,10 @@ Every function takes torch tensors that already live on the CUDA device (torch s
 memory and streams, nothing else), checks dtype / device / contiguity, passes raw pointers to
 the C ABI and raises :class:`Q8Error` on a non-zero status.  There is no CPU fallback: if the
 shared library is missing the first call raises.
+
+The calls of a forward or training pass do the same natively (``csrc/q8_python.cpp``) when their arguments are in the
+ordinary form; the Python form behind each of them takes what is left (a given stream, a tensor subclass, ...) and
+names what is wrong.
 """
 from __future__ import annotations
 
@@ -69,6 +73,11 @@ SIGNATURES = {
 }
 
 _lib: Optional[C.CDLL] = None
+_native_module = None
+_NATIVE_CALLS = ("q8_quantize_weight", "q8_fake_quantize", "q8_ste_backward", "q8_calibrate",
+                 "q8_linear", "q8_linear_workspace_bytes", "q8_linear_q", "q8_linear_requant", "q8_linear_q_requant",
+                 "q8_linear_dyn", "q8_embedding", "q8_add_layernorm", "q8_add_layernorm_quant", "q8_add_layernorm_absmax",
+                 "q8_attention", "q8_attention_quant", "q8_attention_absmax")
 
 
 class Q8Error(RuntimeError):
@@ -92,6 +101,21 @@ def load() -> C.CDLL:
             fn.argtypes = args
         _lib = lib
     return _lib
+
+
+def _native():
+    """The native marshalling module, bound to the loaded library."""
+    global _native_module
+    if _native_module is None:
+        lib = load()
+        try:
+            from . import _q8_native
+        except ImportError as ex:
+            raise RuntimeError("_q8_native.so not found or not loadable: build it first "
+                               "(python -m paper_1910_06188_b200.build)") from ex
+        _q8_native.bind({name: C.cast(getattr(lib, name), C.c_void_p).value for name in _NATIVE_CALLS}, _check)
+        _native_module = _q8_native
+    return _native_module
 
 
 def status_string(status: int) -> str:
@@ -136,6 +160,10 @@ def _check(status: int, where: str) -> None:
 def q8_quantize_weight(W: torch.Tensor, Wq: Optional[torch.Tensor] = None, S_w: Optional[torch.Tensor] = None,
                        dev_status: Optional[torch.Tensor] = None, stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """Eq. 3 + Eq. 1 on a weight (or embedding table) [N, K]; returns (W_q int8, S_w fp32[1])."""
+    if stream is None:
+        r = (_native_module or _native()).quantize_weight(W, Wq, S_w, dev_status)
+        if r is not NotImplemented:
+            return r
     N, K = W.shape
     if Wq is None:
         Wq = torch.empty((N, K), dtype=torch.int8, device=W.device)
@@ -165,6 +193,10 @@ def q8_quantize_activation(X: torch.Tensor, S_x: Optional[torch.Tensor] = None, 
 
 def q8_fake_quantize(X, S, Xhat=None, stream=None):
     """Training-mode fake quantisation: Xhat = Quantize(X | S) / S."""
+    if stream is None:
+        r = (_native_module or _native()).fake_quantize(X, S, Xhat)
+        if r is not NotImplemented:
+            return r
     if Xhat is None:
         Xhat = torch.empty_like(X)
     st = load().q8_fake_quantize(_ptr(X, torch.float32, "X"), X.numel(), _ptr(S, torch.float32, "S"),
@@ -175,6 +207,10 @@ def q8_fake_quantize(X, S, Xhat=None, stream=None):
 
 def q8_ste_backward(grad_out, grad_in=None, stream=None):
     """Straight-through estimator (Eq. 5): the gradient of fake quantisation is the incoming gradient."""
+    if stream is None:
+        r = (_native_module or _native()).ste_backward(grad_out, grad_in)
+        if r is not NotImplemented:
+            return r
     if grad_in is None:
         grad_in = torch.empty_like(grad_out)
     st = load().q8_ste_backward(_ptr(grad_out, torch.float32, "grad_out"), grad_out.numel(),
@@ -198,6 +234,10 @@ def calibrate_S_x(state: torch.Tensor) -> torch.Tensor:
 
 
 def q8_calibrate(X: torch.Tensor, decay: float, state: torch.Tensor, stream=None) -> None:
+    if stream is None:
+        r = (_native_module or _native()).calibrate(X, decay, state)
+        if r is not NotImplemented:
+            return r
     st = load().q8_calibrate(_ptr(X, torch.float32, "X"), X.numel(), float(decay), _any_ptr(state, "state"),
                              _stream(stream))
     _check(st, "q8_calibrate")
@@ -233,6 +273,10 @@ def _linear(fn_name: str, X, Wq, S_w, S_x, bias, act, Y, workspace, dbg_Xq, dbg_
 def q8_linear(X, Wq, S_w, S_x=None, bias=None, act: int = Q8_ACT_NONE, Y=None, workspace=None, dbg_Xq=None,
               dbg_acc=None, stream=None) -> torch.Tensor:
     """Inference-mode quantised FC (Sec. 3): quantise X, Int8 GEMM, Int32 bias, dequantise, act."""
+    if stream is None:
+        r = (_native_module or _native()).linear(X, Wq, S_w, S_x, bias, act, Y, workspace, dbg_Xq, dbg_acc)
+        if r is not NotImplemented:
+            return r
     return _linear("q8_linear", X, Wq, S_w, S_x, bias, act, Y, workspace, dbg_Xq, dbg_acc, stream)
 
 
@@ -243,6 +287,10 @@ def q8_linear_generic(X, Wq, S_w, S_x=None, bias=None, act: int = Q8_ACT_NONE, Y
 
 def q8_linear_q(Xq, S_x, Wq, S_w, bias=None, act: int = Q8_ACT_NONE, Y=None, dbg_acc=None, dev_status=None,
                 stream=None) -> torch.Tensor:
+    if stream is None:
+        r = (_native_module or _native()).linear_q(Xq, S_x, Wq, S_w, bias, act, Y, dbg_acc, dev_status)
+        if r is not NotImplemented:
+            return r
     M, K = Xq.shape
     N, K2 = Wq.shape
     if K != K2:
@@ -289,6 +337,10 @@ def q8_poll_status_at(address: int, stream=None) -> Tuple[int, int]:
 
 
 def q8_embedding(ids, Eq, S_e, out=None, rows_q=None, dev_status=None, stream=None) -> torch.Tensor:
+    if stream is None:
+        r = (_native_module or _native()).embedding(ids, Eq, S_e, out, rows_q, dev_status)
+        if r is not NotImplemented:
+            return r
     T = ids.numel()
     V, H = Eq.shape
     if out is None:
@@ -303,6 +355,10 @@ def q8_embedding(ids, Eq, S_e, out=None, rows_q=None, dev_status=None, stream=No
 
 def q8_add_layernorm(x, r1=None, r2=None, gamma=None, beta=None, eps: float = 1e-12, out=None, stream=None):
     """out = LayerNorm(x + r1 + r2) * gamma + beta over the last dimension (fp32, Sec. 3)."""
+    if stream is None:
+        r = (_native_module or _native()).add_layernorm(x, r1, r2, gamma, beta, eps, out, None, None, None)
+        if r is not NotImplemented:
+            return r
     rows, H = x.shape
     if out is None:
         out = torch.empty_like(x)
@@ -316,6 +372,10 @@ def q8_add_layernorm(x, r1=None, r2=None, gamma=None, beta=None, eps: float = 1e
 
 def q8_attention(qkv, B: int, S: int, heads: int, ctx=None, stream=None):
     """fp32 multi-head self-attention (head dimension 64, no mask) on the fused projection [B*S, 3*heads*64]."""
+    if stream is None:
+        r = (_native_module or _native()).attention(qkv, B, S, heads, ctx, None, None, None)
+        if r is not NotImplemented:
+            return r
     H = heads * 64
     if tuple(qkv.shape) != (B * S, 3 * H):
         raise ValueError(f"qkv must be [{B * S}, {3 * H}], got {tuple(qkv.shape)}")
@@ -330,6 +390,10 @@ def q8_attention(qkv, B: int, S: int, heads: int, ctx=None, stream=None):
 def q8_add_layernorm_absmax(x, absmax_bits, r1=None, r2=None, gamma=None, beta=None, eps: float = 1e-12, out=None,
                             stream=None):
     """q8_add_layernorm that also folds max|out| into the int32 device word `absmax_bits` (fp32 bits; Sec. 4.1)."""
+    if stream is None:
+        r = (_native_module or _native()).add_layernorm_absmax(x, r1, r2, gamma, beta, eps, out, None, None, absmax_bits)
+        if r is not NotImplemented:
+            return r
     rows, H = x.shape
     if out is None:
         out = torch.empty_like(x)
@@ -344,6 +408,10 @@ def q8_add_layernorm_absmax(x, absmax_bits, r1=None, r2=None, gamma=None, beta=N
 
 def q8_attention_absmax(qkv, B: int, S: int, heads: int, absmax_bits, ctx=None, stream=None):
     """q8_attention that also folds max|ctx| into the int32 device word `absmax_bits` (fp32 bits; Sec. 4.1)."""
+    if stream is None:
+        r = (_native_module or _native()).attention_absmax(qkv, B, S, heads, ctx, None, None, absmax_bits)
+        if r is not NotImplemented:
+            return r
     H = heads * 64
     if tuple(qkv.shape) != (B * S, 3 * H):
         raise ValueError(f"qkv must be [{B * S}, {3 * H}], got {tuple(qkv.shape)}")
@@ -359,6 +427,10 @@ def q8_linear_dyn(X, x_absmax, Wq, S_w, bias=None, act: int = Q8_ACT_NONE, Y=Non
                   dbg_Xq=None, dbg_acc=None, stream=None) -> torch.Tensor:
     """q8_linear with the dynamic scale 127 / max|X| taken from the device word `x_absmax` (written by the kernel
     that produced X); `y_absmax` optionally receives max|Y| for the next dynamically quantised layer."""
+    if stream is None:
+        r = (_native_module or _native()).linear_dyn(X, x_absmax, Wq, S_w, bias, act, Y, y_absmax, workspace, dbg_Xq, dbg_acc)
+        if r is not NotImplemented:
+            return r
     M, K = X.shape
     N, K2 = Wq.shape
     if K != K2:
@@ -424,6 +496,10 @@ def q8_linear_q_wseg(Xq, S_x, Wq, S_w, seg_rows: int, bias=None, act: int = Q8_A
 def q8_linear_requant(X, Wq, S_w, S_x, bias, act, S_y, Yq=None, Y=None, workspace=None, dbg_Xq=None, dbg_acc=None,
                       stream=None):
     """q8_linear whose output is (also) emitted as Int8 at the next layer's scale S_y.  Returns Yq."""
+    if stream is None:
+        r = (_native_module or _native()).linear_requant(X, Wq, S_w, S_x, bias, act, S_y, Yq, Y, workspace, dbg_Xq, dbg_acc)
+        if r is not NotImplemented:
+            return r
     M, K = X.shape
     N = Wq.shape[0]
     if Yq is None:
@@ -443,6 +519,10 @@ def q8_linear_requant(X, Wq, S_w, S_x, bias, act, S_y, Yq=None, Y=None, workspac
 
 def q8_linear_q_requant(Xq, S_x, Wq, S_w, bias, act, S_y, Yq=None, Y=None, dbg_acc=None, dev_status=None, stream=None):
     """q8_linear_q whose output is (also) emitted as Int8 at the next layer's scale S_y.  Returns Yq."""
+    if stream is None:
+        r = (_native_module or _native()).linear_q_requant(Xq, S_x, Wq, S_w, bias, act, S_y, Yq, Y, dbg_acc, dev_status)
+        if r is not NotImplemented:
+            return r
     M, K = Xq.shape
     N = Wq.shape[0]
     if Yq is None:
@@ -459,6 +539,10 @@ def q8_linear_q_requant(Xq, S_x, Wq, S_w, bias, act, S_y, Yq=None, Y=None, dbg_a
 
 def q8_add_layernorm_quant(x, r1, r2, S_q, out_q=None, out=None, gamma=None, beta=None, eps: float = 1e-12, stream=None):
     """LayerNorm(x + r1 + r2) written as fp32 (`out`, optional) and as Int8 at scale S_q (`out_q`)."""
+    if stream is None:
+        r = (_native_module or _native()).add_layernorm_quant(x, r1, r2, gamma, beta, eps, out, S_q, out_q, None)
+        if r is not NotImplemented:
+            return r
     rows, H = x.shape
     if out_q is None:
         out_q = torch.empty((rows, H), dtype=torch.int8, device=x.device)
@@ -473,6 +557,10 @@ def q8_add_layernorm_quant(x, r1, r2, S_q, out_q=None, out=None, gamma=None, bet
 
 def q8_attention_quant(qkv, B: int, S: int, heads: int, S_q, ctx_q=None, ctx=None, stream=None):
     """fp32 self-attention whose context is (also) emitted as Int8 at scale S_q."""
+    if stream is None:
+        r = (_native_module or _native()).attention_quant(qkv, B, S, heads, ctx, S_q, ctx_q, None)
+        if r is not NotImplemented:
+            return r
     H = heads * 64
     if ctx_q is None:
         ctx_q = torch.empty((B * S, H), dtype=torch.int8, device=qkv.device)

@@ -63,6 +63,13 @@ class Q8BertEncoder:
             self.layers.append(lay)
         self._bufs = None
 
+    def _static_scale(self, l: int, name: str) -> torch.Tensor:
+        """The S_x word of a layer's Eq. 4 state (the view is made once per state)."""
+        p = self.layers[l][name]
+        if p.get("S_x_state") is not p["state"]:
+            p["S_x_state"], p["S_x"] = p["state"], q8.calibrate_S_x(p["state"])
+        return p["S_x"]
+
     # ------------------------------------------------------------------ buffers
     def _buffers(self, T: int):
         if self._bufs is None or self._bufs["T"] != T:
@@ -100,7 +107,7 @@ class Q8BertEncoder:
             p = self.layers[l][name]
             if scales == "calibrate":
                 q8.q8_calibrate(X, decay, p["state"])
-            S_x = q8.calibrate_S_x(p["state"]) if scales == "static" else None
+            S_x = self._static_scale(l, name) if scales == "static" else None
             Xq = acc = None
             if debug:
                 if "dbg_xq" not in bf:
@@ -132,7 +139,7 @@ class Q8BertEncoder:
         if "hq" not in bf:
             i8 = lambda n: torch.empty((T, n), dtype=torch.int8, device=self.device)
             bf.update(hq=i8(self.H), ctxq=i8(self.H), h1q=i8(self.H), fq=i8(self.F))
-        sx = lambda l, name: q8.calibrate_S_x(self.layers[l][name]["state"])
+        sx = self._static_scale
         pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
         typ_ids = torch.zeros(T, dtype=torch.int32, device=self.device)
         q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])
@@ -168,9 +175,9 @@ class Q8BertEncoder:
         bf = self._buffers(T)
         if "amax" not in bf:
             bf["amax"] = torch.zeros(4 * self.L, dtype=torch.int32, device=self.device)
-        amax = bf["amax"]
-        amax.zero_()                      # the words only ever rise: start every forward at zero (one memset)
-        word = lambda l, i: amax[4 * l + i: 4 * l + i + 1]
+            bf["amax_words"] = bf["amax"].split(1)
+        bf["amax"].zero_()                # the words only ever rise: start every forward at zero (one memset)
+        word = lambda l, i: bf["amax_words"][4 * l + i]
         pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
         typ_ids = torch.zeros(T, dtype=torch.int32, device=self.device)
         q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])

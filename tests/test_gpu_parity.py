@@ -415,3 +415,59 @@ def test_generic_gemm_pointers_at_any_byte(offset_x, offset_w):
     q8.q8_linear_q(at(Xq, offset_x), one, at(Wq, offset_w), one, None, 0, Y=Y, dbg_acc=acc)
     ref = Xq.astype(np.int32) @ Wq.astype(np.int32).T
     assert np.array_equal(acc.cpu().numpy(), ref) and np.array_equal(Y.cpu().numpy(), ref.astype(np.float32))
+
+
+# ------------------------------------------------------------------ native marshalling and its Python form
+def _both_forms():
+    M, K, N, S, heads = 20, 64, 96, 10, 1
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    X, b, x64, qkv = r(M, K), r(N), r(M, 64), r(2 * S, 192)
+    Wq, S_w = q8.q8_quantize_weight(r(N, K))
+    Xq = torch.randint(-127, 128, (M, K), generator=g, device="cuda", dtype=torch.int8)
+    s, word = torch.full((1,), 20.0, device="cuda"), lambda: torch.zeros(1, dtype=torch.int32, device="cuda")
+    ids = torch.randint(0, N, (7,), generator=g, device="cuda", dtype=torch.int32)
+    state, peak = q8.new_calibrate_state(), X.abs().max().reshape(1).view(torch.int32)
+    return [
+        (q8.q8_linear, (X, Wq, S_w, s, b, 1)), (q8.q8_linear, (X, Wq, S_w)), (q8.q8_linear_q, (Xq, s, Wq, S_w, b)),
+        (q8.q8_linear_requant, (X, Wq, S_w, s, b, 1, s)), (q8.q8_linear_q_requant, (Xq, s, Wq, S_w, b, 1, s)),
+        (q8.q8_linear_dyn, (X, peak, Wq, S_w, b)), (q8.q8_embedding, (ids, Wq, S_w)), (q8.q8_add_layernorm, (x64, x64)),
+        (q8.q8_add_layernorm_quant, (x64, x64, None, s)), (q8.q8_add_layernorm_absmax, (x64, word())),
+        (q8.q8_attention, (qkv, 2, S, heads)), (q8.q8_attention_quant, (qkv, 2, S, heads, s)),
+        (q8.q8_attention_absmax, (qkv, 2, S, heads, word())), (q8.q8_quantize_weight, (X,)),
+        (q8.q8_fake_quantize, (X, s)), (q8.q8_ste_backward, (X,)), (q8.q8_calibrate, (X, 0.5, state)),
+    ]
+
+
+def test_native_and_python_forms_of_a_call_agree():
+    """A given stream selects the Python form; without one the same arguments take the native form."""
+    for fn, args in _both_forms():
+        native, python = fn(*args), fn(*args, stream=torch.cuda.current_stream())
+        for a, b in zip(*(v if isinstance(v, tuple) else (v,) for v in (native, python))):
+            assert a is None and b is None or torch.equal(a, b), fn.__name__
+        out = native[0] if isinstance(native, tuple) else native
+        if out is not None and fn not in (q8.q8_quantize_weight,):
+            name = {torch.int8: {"q8_linear_requant": "Yq", "q8_linear_q_requant": "Yq", "q8_add_layernorm_quant": "out_q",
+                                 "q8_attention_quant": "ctx_q"},
+                    torch.float32: {"q8_embedding": "out", "q8_fake_quantize": "Xhat", "q8_ste_backward": "grad_in"}}[out.dtype]
+            key = name.get(fn.__name__) or ("Y" if "linear" in fn.__name__ else "ctx" if "attention" in fn.__name__ else "out")
+            into = torch.empty_like(out)
+            assert fn(*args, **{key: into}) is into and torch.equal(into, out), fn.__name__
+
+
+def test_native_calls_refuse_what_the_python_form_refuses():
+    for fn, args in _both_forms():
+        for bad in (lambda t: t.cpu(), lambda t: t.double(), lambda t: torch.stack([t, t], -1)[..., 0]):
+            broken = (bad(args[0]),) + args[1:]
+            with pytest.raises(TypeError):
+                fn(*broken, stream=torch.cuda.current_stream())
+            with pytest.raises(TypeError):
+                fn(*broken)
+    X = torch.zeros((4, 32), device="cuda")
+    Wq, S_w = q8.q8_quantize_weight(torch.ones((8, 48), device="cuda"))
+    with pytest.raises(ValueError, match="X is"):
+        q8.q8_linear(X, Wq, S_w)
+    with pytest.raises(q8.Q8Error, match="q8_linear: q8_status 10"):
+        q8.q8_linear(X, Wq[:, :32].contiguous(), S_w, act=7)
+    with pytest.raises(q8.Q8Error, match="q8_status 7"):
+        q8.q8_linear(X, Wq[:, :32].contiguous(), S_w, workspace=torch.empty(256, dtype=torch.uint8, device="cuda"))
