@@ -248,6 +248,16 @@ const char *q8_status_string(q8_status s);
  * any pointer may be NULL. */
 void q8_last_launch_info(int *gemm_kernel, int *launches, int *block_n, int *grid, int *ctas);
 
+/* The input of an encoder: LayerNorm(word[ids[t]] + position[t mod S] + type[0]) for t < T, the three Int8 tables with
+ * their scales (word_q [V, H], pos_q [P, H], type_q [>= 1, H]), gamma 1, beta 0, in one pass.  Bit-identical to three
+ * q8_embedding calls and q8_add_layernorm.  out (fp32) and out_q (Int8 at scale S_q) are both optional, not both NULL;
+ * absmax_bits (may be NULL) receives max|out| as in q8_add_layernorm_absmax.  An id outside [0, V) or a position >= P
+ * counts as a zero row and flags Q8_ERR_INDEX.  H a multiple of 4, at most 1024; tables 4-byte, out 16-byte aligned. */
+q8_status q8_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, const int8_t *word_q, const float *S_word,
+                             int64_t V, const int8_t *pos_q, const float *S_pos, int64_t P, const int8_t *type_q,
+                             const float *S_type, float eps, int64_t H, float *out, const float *S_q, int8_t *out_q,
+                             uint32_t *absmax_bits, int32_t *dev_status, void *stream);
+
 /* q8_attention / q8_attention_quant run on the tensor cores when the pointers are 16-byte aligned: both products as
  * tcgen05.mma on operands split into two 16-bit (kind::f16, scaled by powers of two) or TF32 parts each, three
  * partial products accumulated in fp32, which keeps fp32-grade accuracy (an infinite input gives NaN where the

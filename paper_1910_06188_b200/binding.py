@@ -38,6 +38,8 @@ SIGNATURES = {
     "q8_linear_workspace_bytes": (_sz, [_i64, _i64, _i64]),
     "q8_linear_q": (_int, [_vp, _vp, _vp, _vp, _vp, _int, _vp, _i64, _i64, _i64, _vp, _vp, _vp]),
     "q8_linear_generic": (_int, [_vp, _vp, _vp, _vp, _vp, _int, _vp, _i64, _i64, _i64, _vp, _sz, _vp, _vp, _vp]),
+    "q8_embed_layernorm": (_int, [_vp, _i64, _i64, _vp, _vp, _i64, _vp, _vp, _i64, _vp, _vp, _f, _i64, _vp, _vp, _vp, _vp, _vp,
+                                  _vp]),
     "q8_linear_noalloc": (_int, [_vp, _vp, _vp, _vp, _vp, _int, _vp, _i64, _i64, _i64, _vp, _vp, C.POINTER(_vp), _vp]),
     "q8_embedding": (_int, [_vp, _i64, _vp, _vp, _i64, _i64, _vp, _vp, _vp, _vp]),
     "q8_add_layernorm": (_int, [_vp, _vp, _vp, _vp, _vp, _f, _i64, _i64, _vp, _vp]),
@@ -77,7 +79,7 @@ _native_module = None
 _NATIVE_CALLS = ("q8_quantize_weight", "q8_fake_quantize", "q8_ste_backward", "q8_calibrate",
                  "q8_linear", "q8_linear_workspace_bytes", "q8_linear_q", "q8_linear_requant", "q8_linear_q_requant",
                  "q8_linear_dyn", "q8_embedding", "q8_add_layernorm", "q8_add_layernorm_quant", "q8_add_layernorm_absmax",
-                 "q8_attention", "q8_attention_quant", "q8_attention_absmax")
+                 "q8_attention", "q8_attention_quant", "q8_attention_absmax", "q8_embed_layernorm")
 
 
 class Q8Error(RuntimeError):
@@ -351,6 +353,30 @@ def q8_embedding(ids, Eq, S_e, out=None, rows_q=None, dev_status=None, stream=No
                              _stream(stream))
     _check(st, "q8_embedding")
     return out
+
+
+def q8_embed_layernorm(ids, S: int, word, S_word, pos, S_pos, typ, S_typ, eps: float = 1e-12, out=None, S_q=None, out_q=None,
+                       absmax_bits=None, dev_status=None, stream=None):
+    """LayerNorm(word[ids[t]] + pos[t % S] + typ[0]) in one pass, as fp32 (`out`, allocated unless `out_q` is given) and
+    optionally as Int8 at scale S_q (`out_q`); optionally folds max|out| into the int32 device word `absmax_bits`."""
+    if stream is None:
+        r = (_native_module or _native()).embed_layernorm(ids, S, word, S_word, pos, S_pos, typ, S_typ, eps, out, S_q, out_q,
+                                                          absmax_bits, dev_status)
+        if r is not NotImplemented:
+            return r
+    T, (V, H), P = ids.numel(), word.shape, pos.shape[0]
+    if pos.shape[1] != H or typ.shape[1] != H or typ.shape[0] < 1:
+        raise ValueError(f"tables must have {H} columns, and typ at least one row")
+    if out is None and out_q is None:
+        out = torch.empty((T, H), dtype=torch.float32, device=word.device)
+    i8, f32 = torch.int8, torch.float32
+    st = load().q8_embed_layernorm(_ptr(ids, torch.int32, "ids"), T, S, _ptr(word, i8, "word"), _ptr(S_word, f32, "S_word"), V,
+                                   _ptr(pos, i8, "pos"), _ptr(S_pos, f32, "S_pos"), P, _ptr(typ, i8, "typ"),
+                                   _ptr(S_typ, f32, "S_typ"), float(eps), H, _ptr(out, f32, "out"), _ptr(S_q, f32, "S_q"),
+                                   _ptr(out_q, i8, "out_q"), _ptr(absmax_bits, torch.int32, "absmax_bits"),
+                                   _ptr(dev_status, torch.int32, "dev_status"), _stream(stream))
+    _check(st, "q8_embed_layernorm")
+    return out if out is not None else out_q
 
 
 def q8_add_layernorm(x, r1=None, r2=None, gamma=None, beta=None, eps: float = 1e-12, out=None, stream=None):

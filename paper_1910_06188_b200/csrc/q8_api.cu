@@ -439,6 +439,27 @@ q8_status q8_attention_absmax(const float *qkv, int64_t B, int64_t S, int64_t he
     return attention_impl(qkv, B, S, heads, ctx, nullptr, nullptr, stream, absmax_bits);
 }
 
+q8_status q8_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, const int8_t *word_q, const float *S_word, int64_t V,
+                             const int8_t *pos_q, const float *S_pos, int64_t P, const int8_t *type_q, const float *S_type,
+                             float eps, int64_t H, float *out, const float *S_q, int8_t *out_q, uint32_t *absmax_bits,
+                             int32_t *dev_status, void *stream)
+{
+    last_launch_info() = LaunchInfo();
+    if (T < 0 || S < 0 || V < 0 || P < 0 || H < 0 || (T > 0 && S == 0)) return Q8_ERR_SHAPE;
+    if (T == 0 || H == 0) return Q8_OK;
+    if (!ids || !word_q || !S_word || !pos_q || !S_pos || !type_q || !S_type || (!out && !out_q) || (out_q && !S_q)) return Q8_ERR_NULL;
+    if (H > 1024 || H % 4 != 0 || T > (int64_t)INT_MAX || V > (int64_t)INT_MAX || P > (int64_t)INT_MAX) return Q8_ERR_SHAPE;
+    if (!(eps >= 0.0f)) return Q8_ERR_ARG;
+    if (!aligned_to(ids, 4) || !aligned_to(S_word, 4) || !aligned_to(S_pos, 4) || !aligned_to(S_type, 4) || !aligned_to(S_q, 4) ||
+        !aligned_to(absmax_bits, 4) || !aligned_to(dev_status, 4) ||
+        !embed_layernorm_supported(word_q, pos_q, type_q, H, out, out_q))
+        return Q8_ERR_ALIGN;
+    Q8_CUDA_TRY(launch_embed_layernorm(ids, T, S, word_q, S_word, V, pos_q, S_pos, P, type_q, S_type, eps, H, out, S_q, out_q,
+                                       absmax_bits, dev_status, static_cast<cudaStream_t>(stream)));
+    last_launch_info().launches = 1;
+    return Q8_OK;
+}
+
 q8_status q8_linear_dyn(const float *X, const uint32_t *x_absmax, const int8_t *Wq, const float *S_w, const float *bias,
                         int act, float *Y, uint32_t *y_absmax, int64_t M, int64_t N, int64_t K, void *workspace,
                         size_t workspace_bytes, int8_t *dbg_Xq, int32_t *dbg_acc, void *stream)

@@ -98,6 +98,13 @@ cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, co
 cudaError_t launch_add_layernorm(const float *x, const float *r1, const float *r2, const float *gamma,
                                  const float *beta, float eps, int64_t rows, int64_t H, float *out, const float *S_q,
                                  int8_t *out_q, uint32_t *amax, cudaStream_t s);
+// The embedding sum and its LayerNorm in one pass (H % 4 == 0, H <= 1024).
+bool embed_layernorm_supported(const int8_t *word, const int8_t *pos, const int8_t *typ, int64_t H, const float *out,
+                               const int8_t *out_q);
+cudaError_t launch_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, const int8_t *word, const float *S_word, int64_t V,
+                                   const int8_t *pos, const float *S_pos, int64_t P, const int8_t *typ, const float *S_typ,
+                                   float eps, int64_t H, float *out, const float *S_q, int8_t *out_q, uint32_t *amax,
+                                   int32_t *status, cudaStream_t s);
 cudaError_t launch_attention(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,
                              int8_t *ctx_q, uint32_t *amax, cudaStream_t s);
 

@@ -24,7 +24,7 @@ namespace {
     X(q8_quantize_weight) X(q8_fake_quantize) X(q8_ste_backward) X(q8_calibrate) X(q8_linear)  \
     X(q8_linear_workspace_bytes) X(q8_linear_q) X(q8_linear_requant) X(q8_linear_q_requant) X(q8_linear_dyn)            \
     X(q8_embedding) X(q8_add_layernorm) X(q8_add_layernorm_quant) X(q8_add_layernorm_absmax) X(q8_attention)            \
-    X(q8_attention_quant) X(q8_attention_absmax)
+    X(q8_attention_quant) X(q8_attention_absmax) X(q8_embed_layernorm)
 #define Q8_DECLARE(name) decltype(&::name) p_##name = nullptr;
 Q8_CALLS(Q8_DECLARE)
 PyObject *g_check = nullptr;  // binding._check(status, where): raises
@@ -365,6 +365,33 @@ PyObject *attention(Args a)
     return out.result();
 }
 
+// (ids, S, word, S_word, pos, S_pos, typ, S_typ, eps, out, S_q, out_q, absmax_bits, dev_status)
+PyObject *embed_layernorm(Args a)
+{
+    Call c;
+    int64_t V, H, P, H2, rows, H3;
+    const at::Tensor *t = c.tensor(a[0]);
+    if (t == nullptr || !c.matrix(a[2], &V, &H) || !c.matrix(a[4], &P, &H2) || !c.matrix(a[6], &rows, &H3) || H2 != H || H3 != H ||
+        rows < 1 || (a[9] == Py_None && a[11] == Py_None))
+        return other_form();
+    const int64_t T = t->numel(), S = c.integer(a[1]);
+    auto ids = c.ptr<const int32_t>(a[0], kI32);
+    auto word = c.ptr<const int8_t>(a[2], kI8), pos = c.ptr<const int8_t>(a[4], kI8), typ = c.ptr<const int8_t>(a[6], kI8);
+    auto S_word = c.ptr<const float>(a[3], kF32), S_pos = c.ptr<const float>(a[5], kF32), S_typ = c.ptr<const float>(a[7], kF32);
+    const float eps = c.real(a[8]);
+    auto out = c.ptr<float>(a[9], kF32);
+    auto S_q = c.ptr<const float>(a[10], kF32);
+    auto out_q = c.ptr<int8_t>(a[11], kI8);
+    auto peak = c.ptr<uint32_t>(a[12], kI32);
+    auto status = c.ptr<int32_t>(a[13], kI32);
+    if (!c.plain) return other_form();
+    if (!run("q8_embed_layernorm", [&](void *s) {
+            return p_q8_embed_layernorm(ids, T, S, word, S_word, V, pos, S_pos, P, typ, S_typ, eps, H, out, S_q, out_q, peak, status, s);
+        }))
+        return nullptr;
+    return Py_NewRef(a[9] != Py_None ? a[9] : a[11]);
+}
+
 // (W, Wq, S_w, dev_status) -> (Wq, S_w)
 PyObject *quantize_weight(Args a)
 {
@@ -482,6 +509,7 @@ PyMethodDef kMethods[] = {
     Q8_ENTRY("attention", attention<0>, 8),
     Q8_ENTRY("attention_quant", attention<1>, 8),
     Q8_ENTRY("attention_absmax", attention<2>, 8),
+    Q8_ENTRY("embed_layernorm", embed_layernorm, 14),
     Q8_ENTRY("quantize_weight", quantize_weight, 4),
     Q8_ENTRY("calibrate", calibrate, 3),
     Q8_ENTRY("fake_quantize", fake_quantize, 3),

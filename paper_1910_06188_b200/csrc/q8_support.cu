@@ -130,43 +130,12 @@ __global__ void __launch_bounds__(kLnThreads) add_layernorm_vec_kernel(const flo
     if (amax) warp_fold_absmax(am, amax);
 }
 
-// One warp per row for H <= 1024 (BERT's hidden sizes): up to eight float4 per lane, both moments reduced with
-// shuffles only, eight rows per CTA, so there is no block-level barrier at all.
-__global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_kernel(const float *__restrict__ x,
-                                                                        const float *__restrict__ r1,
-                                                                        const float *__restrict__ r2,
-                                                                        const float *__restrict__ gamma,
-                                                                        const float *__restrict__ beta, float eps,
-                                                                        int64_t rows, int64_t H, float *__restrict__ out,
-                                                                        const float *__restrict__ S_q,
-                                                                        int8_t *__restrict__ out_q, uint32_t *__restrict__ amax)
+// The row of one warp, H <= 1024: v[i] holds the values 4 (lane + 32 i) .. + 3 of the summed row and s this lane's share of
+// their sum.  Both moments are reduced with shuffles only, so there is no block-level barrier at all.
+__device__ __forceinline__ void normalise_row(const float4 (&v)[8], float s, int lane, int n4, int64_t H, float eps,
+                                              const float *__restrict__ gamma, const float *__restrict__ beta, float4 *out4,
+                                              uint32_t *q4, float Sq, float &am)
 {
-    grid_dependency_release_next(rows * H <= kSmallProblemElems);
-    grid_dependency_wait();  // launched so that its start may overlap the tail of the kernel before it
-    const int lane = threadIdx.x & 31;
-    const int n4 = (int)(H >> 2);
-    const float Sq = out_q ? __ldg(S_q) : 1.0f;
-    float am = 0.0f;  // running max|y| of this lane over all rows of the warp
-    // the grid is sized to the device and every warp walks rows with a grid stride (no partial last wave)
-    for (int64_t row = (int64_t)blockIdx.x * (kLnThreads / 32) + (threadIdx.x >> 5); row < rows;
-         row += (int64_t)gridDim.x * (kLnThreads / 32)) {
-    const int64_t base4 = row * n4;
-    const float4 *x4 = reinterpret_cast<const float4 *>(x) + base4;
-    const float4 *a4 = r1 ? reinterpret_cast<const float4 *>(r1) + base4 : nullptr;
-    const float4 *b4 = r2 ? reinterpret_cast<const float4 *>(r2) + base4 : nullptr;
-    float4 v[8];
-    float s = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int c = lane + 32 * i;
-        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < n4) {
-            v[i] = __ldg(x4 + c);
-            if (a4) { const float4 t = __ldg(a4 + c); v[i].x += t.x; v[i].y += t.y; v[i].z += t.z; v[i].w += t.w; }
-            if (b4) { const float4 t = __ldg(b4 + c); v[i].x += t.x; v[i].y += t.y; v[i].z += t.z; v[i].w += t.w; }
-            s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
-        }
-    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const float mean = s / (float)H;
@@ -192,11 +161,102 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_k
         y.z = (v[i].z - mean) * rstd * g.z + b.z;
         y.w = (v[i].w - mean) * rstd * g.w + b.w;
         am = fmaxf(fmaxf(am, fmaxf(fabsf(y.x), fabsf(y.y))), fmaxf(fabsf(y.z), fabsf(y.w)));
-        if (out) reinterpret_cast<float4 *>(out)[base4 + c] = y;
-        if (out_q) reinterpret_cast<uint32_t *>(out_q)[base4 + c] = quantize_pack4(y.x, y.y, y.z, y.w, Sq);
+        if (out4) out4[c] = y;
+        if (q4) q4[c] = quantize_pack4(y.x, y.y, y.z, y.w, Sq);
     }
+}
+
+// One warp per row for H <= 1024 (BERT's hidden sizes): up to eight float4 per lane, eight rows per CTA.
+__global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_kernel(const float *__restrict__ x,
+                                                                        const float *__restrict__ r1,
+                                                                        const float *__restrict__ r2,
+                                                                        const float *__restrict__ gamma,
+                                                                        const float *__restrict__ beta, float eps,
+                                                                        int64_t rows, int64_t H, float *__restrict__ out,
+                                                                        const float *__restrict__ S_q,
+                                                                        int8_t *__restrict__ out_q, uint32_t *__restrict__ amax)
+{
+    grid_dependency_release_next(rows * H <= kSmallProblemElems);
+    grid_dependency_wait();  // launched so that its start may overlap the tail of the kernel before it
+    const int lane = threadIdx.x & 31;
+    const int n4 = (int)(H >> 2);
+    const float Sq = out_q ? __ldg(S_q) : 1.0f;
+    float am = 0.0f;  // running max|y| of this lane over all rows of the warp
+    // the grid is sized to the device and every warp walks rows with a grid stride (no partial last wave)
+    for (int64_t row = (int64_t)blockIdx.x * (kLnThreads / 32) + (threadIdx.x >> 5); row < rows;
+         row += (int64_t)gridDim.x * (kLnThreads / 32)) {
+        const int64_t base4 = row * n4;
+        const float4 *x4 = reinterpret_cast<const float4 *>(x) + base4;
+        const float4 *a4 = r1 ? reinterpret_cast<const float4 *>(r1) + base4 : nullptr;
+        const float4 *b4 = r2 ? reinterpret_cast<const float4 *>(r2) + base4 : nullptr;
+        float4 v[8];
+        float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int c = lane + 32 * i;
+            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c < n4) {
+                v[i] = __ldg(x4 + c);
+                if (a4) { const float4 t = __ldg(a4 + c); v[i].x += t.x; v[i].y += t.y; v[i].z += t.z; v[i].w += t.w; }
+                if (b4) { const float4 t = __ldg(b4 + c); v[i].x += t.x; v[i].y += t.y; v[i].z += t.z; v[i].w += t.w; }
+                s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+            }
+        }
+        normalise_row(v, s, lane, n4, H, eps, gamma, beta, out ? reinterpret_cast<float4 *>(out) + base4 : nullptr,
+                      out_q ? reinterpret_cast<uint32_t *>(out_q) + base4 : nullptr, Sq, am);
     }
     if (amax) warp_fold_absmax(am, amax);  // one atomic per warp: max|y| for a dynamically quantised consumer (Sec. 4.1)
+}
+
+// LayerNorm(word[ids[t]] + position[t % S] + type[0]) in one pass, one warp per token: the three Int8 rows are dequantised in
+// registers instead of travelling through three fp32 tensors (which is what the separate kernels are bound by: for
+// 24576 x 1024 they move 12 + 4 + 4 bytes per value where this one moves 4 and the table rows).  The same roundings as
+// q8_embedding and q8_add_layernorm: every product and sum is rounded by itself.
+__global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm)
+embed_layernorm_kernel(const int32_t *__restrict__ ids, int64_t T, int64_t S, const int8_t *__restrict__ word,
+                       const float *__restrict__ S_word, int64_t V, const int8_t *__restrict__ pos,
+                       const float *__restrict__ S_pos, int64_t P, const int8_t *__restrict__ typ,
+                       const float *__restrict__ S_typ, float eps, int64_t H, float *__restrict__ out,
+                       const float *__restrict__ S_q, int8_t *__restrict__ out_q, uint32_t *__restrict__ amax, int32_t *status)
+{
+    grid_dependency_release_next(T * H <= kSmallProblemElems);
+    grid_dependency_wait();
+    const int lane = threadIdx.x & 31;
+    const int n4 = (int)(H >> 2);
+    const float Sq = out_q ? __ldg(S_q) : 1.0f;
+    const float inv_w = __fdiv_rn(1.0f, __ldg(S_word)), inv_p = __fdiv_rn(1.0f, __ldg(S_pos)), inv_t = __fdiv_rn(1.0f, __ldg(S_typ));
+    float am = 0.0f;
+    for (int64_t t = (int64_t)blockIdx.x * (kLnThreads / 32) + (threadIdx.x >> 5); t < T;
+         t += (int64_t)gridDim.x * (kLnThreads / 32)) {
+        const int64_t id = __ldg(ids + t), place = t % S;
+        const bool id_ok = id >= 0 && id < V, place_ok = place < P;
+        if (!(id_ok && place_ok) && lane == 0 && status) atomicOr(status, 1 << Q8_ERR_INDEX);  // a zero row, as in q8_embedding
+        const uint32_t *w4 = reinterpret_cast<const uint32_t *>(word + (id_ok ? id : 0) * H);
+        const uint32_t *p4 = reinterpret_cast<const uint32_t *>(pos + (place_ok ? place : 0) * H);
+        const uint32_t *t4 = reinterpret_cast<const uint32_t *>(typ);
+        uint32_t qw[8], qp[8], qt[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int c = lane + 32 * i;
+            qw[i] = c < n4 && id_ok ? __ldg(w4 + c) : 0u;
+            qp[i] = c < n4 && place_ok ? __ldg(p4 + c) : 0u;
+            qt[i] = c < n4 ? __ldg(t4 + c) : 0u;
+        }
+        float4 v[8];
+        float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            auto sum = [&](int byte) {
+                auto value = [&](uint32_t w, float inv) { return __fmul_rn((float)(int8_t)((w >> (8 * byte)) & 0xffu), inv); };
+                return __fadd_rn(__fadd_rn(value(qw[i], inv_w), value(qp[i], inv_p)), value(qt[i], inv_t));
+            };
+            v[i] = make_float4(sum(0), sum(1), sum(2), sum(3));
+            if (lane + 32 * i < n4) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+        }
+        normalise_row(v, s, lane, n4, H, eps, nullptr, nullptr, out ? reinterpret_cast<float4 *>(out) + t * n4 : nullptr,
+                      out_q ? reinterpret_cast<uint32_t *>(out_q) + t * n4 : nullptr, Sq, am);
+    }
+    if (amax) warp_fold_absmax(am, amax);
 }
 
 // ------------------------------------------------------------------ self-attention, head dimension 64, no mask
@@ -381,6 +441,26 @@ cudaError_t launch_add_layernorm(const float *x, const float *r1, const float *r
                                                                                            H, out, S_q, out_q, amax);
     }
     return cudaGetLastError();
+}
+
+bool embed_layernorm_supported(const int8_t *word, const int8_t *pos, const int8_t *typ, int64_t H, const float *out,
+                               const int8_t *out_q)
+{
+    auto al = [](const void *p, uintptr_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; };
+    return H % 4 == 0 && H <= 1024 && al(word, 4) && al(pos, 4) && al(typ, 4) && al(out, 16) && al(out_q, 4);
+}
+
+cudaError_t launch_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, const int8_t *word, const float *S_word, int64_t V,
+                                   const int8_t *pos, const float *S_pos, int64_t P, const int8_t *typ, const float *S_typ,
+                                   float eps, int64_t H, float *out, const float *S_q, int8_t *out_q, uint32_t *amax,
+                                   int32_t *status, cudaStream_t s)
+{
+    if (T <= 0 || H <= 0) return cudaSuccess;
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t want = (T + kLnThreads / 32 - 1) / (kLnThreads / 32), cap = (int64_t)(sms > 0 ? sms : 148) * kLnCtasPerSm;
+    return launch_overlapping_tail(embed_layernorm_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kLnThreads), 0, s, ids, T,
+                                   S, word, S_word, V, pos, S_pos, P, typ, S_typ, eps, H, out, S_q, out_q, amax, status);
 }
 
 cudaError_t launch_attention(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,

@@ -88,6 +88,18 @@ class Q8BertEncoder:
         return n
 
     # ------------------------------------------------------------------ forward
+    def _one_pass_input(self) -> bool:
+        return self.H <= 1024  # what q8_embed_layernorm takes
+
+    def _embed(self, ids: torch.Tensor, B: int, S: int) -> None:
+        """The three table look-ups of B sequences of S tokens, each into its own fp32 buffer."""
+        bf = self._bufs
+        pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
+        typ_ids = torch.zeros(B * S, dtype=torch.int32, device=self.device)
+        q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])
+        q8.q8_embedding(pos_ids, self.pos, self.S_pos, out=bf["ep"], dev_status=bf["status"])
+        q8.q8_embedding(typ_ids, self.typ, self.S_typ, out=bf["et"], dev_status=bf["status"])
+
     def forward(self, ids: torch.Tensor, B: int, S: int, scales: str = "static", decay: float = 0.9999,
                 hook: Optional[Callable] = None, debug: bool = False) -> torch.Tensor:
         """ids: int32 [B*S] on the device.  scales: "static" (Eq. 4 scales from earlier calibrate passes),
@@ -96,11 +108,7 @@ class Q8BertEncoder:
         quantised FC; with debug=True, Xq / acc are that call's Int8 activation and Int32 accumulator copies."""
         T = B * S
         bf = self._buffers(T)
-        pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
-        typ_ids = torch.zeros(T, dtype=torch.int32, device=self.device)
-        q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])
-        q8.q8_embedding(pos_ids, self.pos, self.S_pos, out=bf["ep"], dev_status=bf["status"])
-        q8.q8_embedding(typ_ids, self.typ, self.S_typ, out=bf["et"], dev_status=bf["status"])
+        self._embed(ids, B, S)
         q8.q8_add_layernorm(bf["ew"], bf["ep"], bf["et"], eps=LN_EPS, out=bf["h"])
 
         def fc(l, name, X, Y):
@@ -140,12 +148,12 @@ class Q8BertEncoder:
             i8 = lambda n: torch.empty((T, n), dtype=torch.int8, device=self.device)
             bf.update(hq=i8(self.H), ctxq=i8(self.H), h1q=i8(self.H), fq=i8(self.F))
         sx = self._static_scale
-        pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
-        typ_ids = torch.zeros(T, dtype=torch.int32, device=self.device)
-        q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])
-        q8.q8_embedding(pos_ids, self.pos, self.S_pos, out=bf["ep"], dev_status=bf["status"])
-        q8.q8_embedding(typ_ids, self.typ, self.S_typ, out=bf["et"], dev_status=bf["status"])
-        q8.q8_add_layernorm_quant(bf["ew"], bf["ep"], bf["et"], sx(0, "qkv"), out_q=bf["hq"], out=bf["h"], eps=LN_EPS)
+        if self._one_pass_input():
+            q8.q8_embed_layernorm(ids, S, self.word, self.S_word, self.pos, self.S_pos, self.typ, self.S_typ, LN_EPS,
+                                  out=bf["h"], S_q=sx(0, "qkv"), out_q=bf["hq"], dev_status=bf["status"])
+        else:
+            self._embed(ids, B, S)
+            q8.q8_add_layernorm_quant(bf["ew"], bf["ep"], bf["et"], sx(0, "qkv"), out_q=bf["hq"], out=bf["h"], eps=LN_EPS)
         st = bf["status"]
         for l in range(self.L):
             p = self.layers[l]
@@ -178,12 +186,12 @@ class Q8BertEncoder:
             bf["amax_words"] = bf["amax"].split(1)
         bf["amax"].zero_()                # the words only ever rise: start every forward at zero (one memset)
         word = lambda l, i: bf["amax_words"][4 * l + i]
-        pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
-        typ_ids = torch.zeros(T, dtype=torch.int32, device=self.device)
-        q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])
-        q8.q8_embedding(pos_ids, self.pos, self.S_pos, out=bf["ep"], dev_status=bf["status"])
-        q8.q8_embedding(typ_ids, self.typ, self.S_typ, out=bf["et"], dev_status=bf["status"])
-        q8.q8_add_layernorm_absmax(bf["ew"], word(0, 0), bf["ep"], bf["et"], eps=LN_EPS, out=bf["h"])
+        if self._one_pass_input():
+            q8.q8_embed_layernorm(ids, S, self.word, self.S_word, self.pos, self.S_pos, self.typ, self.S_typ, LN_EPS,
+                                  out=bf["h"], absmax_bits=word(0, 0), dev_status=bf["status"])
+        else:
+            self._embed(ids, B, S)
+            q8.q8_add_layernorm_absmax(bf["ew"], word(0, 0), bf["ep"], bf["et"], eps=LN_EPS, out=bf["h"])
         for l in range(self.L):
             p = self.layers[l]
             lin = lambda name, X, xw, Y, yw=None: q8.q8_linear_dyn(X, xw, p[name]["Wq"], p[name]["S_w"], p[name]["b"],
@@ -213,12 +221,13 @@ class Q8BertEncoder:
         return graph, out
 
     def launches_per_forward(self, scales: str = "static", fused: bool = False) -> int:
+        first = 1 if fused and self._one_pass_input() else 4  # embeddings and their LayerNorm
         if fused and scales == "dynamic":
-            return 4 + self.L * 11          # per layer: 4 x (quantise + GEMM), attention, two LayerNorms
+            return first + self.L * 11      # per layer: 4 x (quantise + GEMM), attention, two LayerNorms
         if fused:
-            return 4 + self.L * 7
-        per_fc = 2 if scales == "static" else (3 if scales == "dynamic" else 5)
-        return 4 + self.L * (4 * per_fc + 3)
+            return first + self.L * 7
+        per_fc = 2 if scales == "static" else (3 if scales == "dynamic" else 4)
+        return first + self.L * (4 * per_fc + 3)
 
     def poll(self):
         """(code, bits) of the embedding status word and of the FC workspace, after synchronising."""

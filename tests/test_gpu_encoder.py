@@ -386,3 +386,42 @@ def test_attention_non_finite_rows_stay_in_their_rows():
     rows, features = np.delete(np.arange(S), [70, 71]), np.delete(np.arange(64), 5)
     assert np.isnan(got[70]).all() and np.isnan(got[71]).all() and not np.isfinite(got[:, 5]).any()
     assert np.abs(got[np.ix_(rows, features)] - ref[np.ix_(rows, features)]).max() <= EDGE_TOL * np.abs(ref).max()
+
+
+# ------------------------------------------------------------------ the input of an encoder in one pass
+@pytest.mark.parametrize("B,S,H", [(1, 1, 4), (3, 7, 100), (2, 33, 768), (5, 512, 1024), (700, 9, 132)])
+def test_embed_layernorm_equals_the_separate_calls(B, S, H):
+    T, V, P = B * S, 50, 512
+    g = torch.Generator(device="cuda").manual_seed(T + H)
+    (word, S_w), (pos, S_p), (typ, S_t) = (q8.q8_quantize_weight(torch.randn((n, H), generator=g, device="cuda") * 0.02) for n in (V, P, 2))
+    ids = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    places = torch.arange(S, dtype=torch.int32, device="cuda").repeat(B)
+    parts = [q8.q8_embedding(i, t, s) for i, t, s in ((ids, word, S_w), (places, pos, S_p), (torch.zeros_like(ids), typ, S_t))]
+    ref = q8.q8_add_layernorm(*parts)
+    scale, peak = torch.full((1,), 40.0, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref_q = q8.q8_add_layernorm_quant(*parts, scale)
+    out_q, status = torch.empty((T, H), dtype=torch.int8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    for stream in (None, torch.cuda.current_stream()):
+        peak.zero_()
+        out = q8.q8_embed_layernorm(ids, S, word, S_w, pos, S_p, typ, S_t, absmax_bits=peak, dev_status=status,
+                                    out=torch.empty((T, H), device="cuda"), S_q=scale, out_q=out_q, stream=stream)
+        assert torch.equal(out, ref) and torch.equal(out_q, ref_q) and peak.view(torch.float32).item() == ref.abs().max().item()
+        assert q8.q8_poll_status(status) == (q8.Q8_OK, 0)
+    assert torch.equal(q8.q8_embed_layernorm(ids, S, word, S_w, pos, S_p, typ, S_t), ref)
+
+
+def test_embed_layernorm_flags_what_is_out_of_range():
+    H, V = 64, 10
+    tables = [q8.q8_quantize_weight(torch.randn((n, H), device="cuda")) for n in (V, 4, 2)]
+    args = [x for t in tables for x in t]
+    for ids, S in (([1, V, 2, 3], 4), ([1, -1, 2, 3], 4), ([1, 2, 3, 4, 5], 5)):  # an id, an id, the fifth position
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        idt = torch.tensor(ids, dtype=torch.int32, device="cuda")
+        out = q8.q8_embed_layernorm(idt, S, *args, dev_status=status)
+        assert q8.q8_poll_status(status)[0] == q8.Q8_ERR_INDEX
+        places = torch.arange(S, dtype=torch.int32, device="cuda")
+        parts = [q8.q8_embedding(i, t, s) for i, (t, s) in zip((idt, places, torch.zeros_like(idt)), tables)]
+        assert torch.equal(out, q8.q8_add_layernorm(*parts))
+    with pytest.raises(q8.Q8Error, match="q8_status 2"):
+        wide = [x for n in (4, 4, 2) for x in q8.q8_quantize_weight(torch.ones((n, 1028), device="cuda"))]
+        q8.q8_embed_layernorm(torch.zeros(2, dtype=torch.int32, device="cuda"), 2, *wide)
