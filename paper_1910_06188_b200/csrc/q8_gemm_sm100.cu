@@ -594,6 +594,13 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
             best_cost = cost;
         }
     }
+    // Long K on few tiles: K split over a cluster of CTAs, where all CTAs still run at once (see q8_gemm_splitk_sm100.cu for
+    // both sides).  From K = 2048 on; with 1024 the exchange costs what it saves.
+    const int64_t narrow_tiles = tm * ((a.N + 31) / 32);
+    if (a.K >= 2048) {
+        if (4 * narrow_tiles <= sms) return launch_gemm_splitk(a, true, s);
+        if (best == 32 && 2 * tm * ((a.N + 63) / 64) <= sms) return launch_gemm_splitk(a, false, s);
+    }
     return launch_by_shape(best, 1, a, s);
 }
 

@@ -126,6 +126,8 @@ void set_gemm_tail_split(bool enable);
 void set_gemm_direct_store(int mode);
 void set_gemm_epilogue_warps(int warps);  // 0 automatic, 8 or 16
 cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s);  // q8_gemm_sm100.cu
+// K split over a cluster (q8_gemm_splitk_sm100.cu): four CTAs per 128 x 32 tile (rows) or two per 128 x 64 tile; K > 512.
+cudaError_t launch_gemm_splitk(const GemmArgs &a, bool rows, cudaStream_t s);
 cudaError_t launch_gemm_generic(const GemmArgs &a, cudaStream_t s);  // q8_gemm_generic.cu
 
 

@@ -471,3 +471,28 @@ def test_native_calls_refuse_what_the_python_form_refuses():
         q8.q8_linear(X, Wq[:, :32].contiguous(), S_w, act=7)
     with pytest.raises(q8.Q8Error, match="q8_status 7"):
         q8.q8_linear(X, Wq[:, :32].contiguous(), S_w, workspace=torch.empty(256, dtype=torch.uint8, device="cuda"))
+
+
+# ------------------------------------------------------------------ K split over a cluster
+@pytest.mark.parametrize("M,N,K", [(1, 32, 2048), (37, 90, 2064), (128, 768, 3072), (129, 500, 4096), (128, 1184, 2048),
+                                   (300, 1000, 2176), (512, 1152, 2048), (16, 33, 16400)])
+@pytest.mark.parametrize("act", [0, 1])
+def test_split_k_layers_bit_exact(M, N, K, act):
+    """Four CTAs per 128 x 32 tile (up to 37 tiles) and two per 128 x 64 tile: integers, fp32, and every output form."""
+    X, W, b = synth.activation(M, K, 9300 + M), synth.weight(N, K, 9301), synth.bias(N, 9302)
+    info = check_linear(X, W, b, act)
+    assert info["gemm_kernel"] == 1 and (info["block_n"], info["grid"]) in (
+        (32, 4 * ((M + 127) // 128) * ((N + 31) // 32)), (64, 2 * ((M + 127) // 128) * ((N + 63) // 64)))
+    Wq, S_w = q8.q8_quantize_weight(dev(W))
+    Xq, S_x = q8.q8_quantize_activation(dev(X))
+    S_y = torch.full((1,), 25.0, device="cuda")
+    peak = torch.zeros(1, dtype=torch.int32, device="cuda")
+    top = torch.tensor([float(np.abs(X).max())], device="cuda").view(torch.int32)
+    Y = q8.q8_linear_q(Xq, S_x, Wq, S_w, dev(b), act)
+    Y2 = torch.empty_like(Y)
+    both = q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), act, S_y, Y=Y2)
+    only = q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), act, S_y)
+    dyn = q8.q8_linear_dyn(dev(X), top, Wq, S_w, dev(b), act, y_absmax=peak)
+    assert torch.equal(Y2, Y) and torch.equal(both, only) and torch.equal(dyn, Y)
+    assert np.array_equal(only.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(25.0)))
+    assert peak.view(torch.float32).item() == Y.abs().max().item()
