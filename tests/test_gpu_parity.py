@@ -1,6 +1,8 @@
 """GPU parity: the CUDA path, called through the C ABI, against the CPU oracle on the same seeded
 inputs.  Integers (X_q, W_q, Int32 accumulators, scales' bits) must match exactly; fp32 outputs
 within 1e-5 of the output magnitude."""
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -11,6 +13,13 @@ from paper_1910_06188_b200 import synth
 from tests.gpu_util import REL_TOL, assert_close_fp, check_linear, dev
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _no_garbage_left_behind():
+    """Tensors that earlier tests left in reference cycles are freed here, not while another test counts allocations."""
+    yield
+    gc.collect()
 
 
 # ------------------------------------------------------------------ quantiser (Eq. 1, Eq. 3, Sec. 4.1)
@@ -496,3 +505,16 @@ def test_split_k_layers_bit_exact(M, N, K, act):
     assert torch.equal(Y2, Y) and torch.equal(both, only) and torch.equal(dyn, Y)
     assert np.array_equal(only.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(25.0)))
     assert peak.view(torch.float32).item() == Y.abs().max().item()
+
+
+@pytest.mark.parametrize("M,N,K", [(4096, 768, 256), (4000, 700, 144), (2900, 1024, 272)])
+def test_192_wide_tiles_bit_exact(M, N, K):
+    X, W, b = synth.activation(M, K, 9400 + N), synth.weight(N, K, 9401), synth.bias(N, 9402)
+    info = check_linear(X, W, b, 1)
+    assert (info["gemm_kernel"], info["block_n"], info["ctas"]) == (1, 192, 1)
+    Wq, S_w = q8.q8_quantize_weight(dev(W))
+    Xq, S_x = q8.q8_quantize_activation(dev(X))
+    S_y = torch.full((1,), 25.0, device="cuda")
+    Y = q8.q8_linear_q(Xq, S_x, Wq, S_w, dev(b), 1)
+    only = q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), 1, S_y)
+    assert np.array_equal(only.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(25.0)))
