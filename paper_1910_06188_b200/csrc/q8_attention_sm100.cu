@@ -23,8 +23,9 @@
 //   warps 4..7  staging: K and V global -> registers -> scale, split -> shared memory, 128-byte-swizzled rows of 64 fp16.  K
 //               is a K-major operand; V keeps its [key][feature] order and is read as an MN-major operand.
 //   warp 8      issues the MMAs (converged, one elected lane); the rest of its warpgroup is there for setmaxnreg, which gives
-//               the softmax 120 registers a thread and the staging 96 (with 96 for all, O was spilled).
-// Measured (64 x 384 x 16 heads / 16 x 512 x 12 / 32 x 128 x 12, Int8 output): 236 / 77 / 19.5 us; split TF32 with whole score
+//               the softmax 128 registers a thread and the staging 88, the one split without spills (120 / 96: 3 % slower, 112 / 104:
+//               8 %; with 96 for all, O was spilled).
+// Measured (64 x 384 x 16 heads / 16 x 512 x 12 / 32 x 128 x 12, Int8 output): 227 / 72 / 19.9 us; split TF32 with whole score
 // rows in TMEM, one CTA per SM, 512 threads staging: 304 / - / 23.8 us (it takes S <= 384; plain fp32 FMAs needed 413 us at
 // 512).  What bounds it now is latency: loads of K and V (without them 25 % less) and the chain softmax -> P V -> scores
 // between the roles, with the issue slots 40 % busy and the tensor pipe 20 %.  Tried and dropped: a persistent grid (the
@@ -48,7 +49,7 @@ constexpr int kSoftmaxWarps = 4, kStagingWarps = 4;
 constexpr int kThreads = 384;  // three warpgroups: softmax, staging, and one whose first warp issues the MMAs
 // Registers per thread after the redistribution between the warpgroups; their sum must not exceed what the CTA is launched
 // with (checked on the host: an increase that cannot be served would wait for ever).
-constexpr int kLaunchRegs = 80, kSoftmaxRegs = 120, kStagingRegs = 96, kIssuerRegs = 24;
+constexpr int kLaunchRegs = 80, kSoftmaxRegs = 128, kStagingRegs = 88, kIssuerRegs = 24;
 static_assert(kSoftmaxRegs + kStagingRegs + kIssuerRegs <= 3 * kLaunchRegs, "register split");
 constexpr int kRowBytes = kHeadDim * 4;      // an fp32 row of Q or of the output
 constexpr int kQBytes = kQTile * kRowBytes;  // fp32 Q on its way in, the output on its way out: 32 KB
