@@ -15,7 +15,12 @@ namespace {
 // One CTA per row.  The summed row is kept in shared memory, so the inputs are read once; mean and
 // variance are the two-pass forms (sum, then sum of squared deviations), reduced through warp shuffles.
 constexpr int kLnThreads = 256;
-constexpr int kLnCtasPerSm = 4;  // CTAs per SM of the warp-per-row kernel (64 registers x 256 threads each)
+// CTAs per SM of the warp-per-row kernel.  Two, with registers for all loads of a row and of its residual at once (with four CTAs
+// of 64 registers the loads of the two come one after the other: 128 x 768 3.85 -> 3.10 us, 1421 x 768 5.05 -> 4.10, 24576 x 1024
+// with Int8 copy 61.9 -> 54.0 us = 6.05 TB/s; three CTAs spill: 57.4).  Also where four would take all rows in one round and two
+// need a second one: 4096 x 768 10.2 -> 9.3.
+constexpr int kLnCtasPerSm = 2;
+constexpr int kEmbedLnCtasPerSm = 4;  // the one-pass input kernel: Int8 rows, fewer registers
 
 __device__ __forceinline__ float block_sum(float v, float *scratch)
 {
@@ -189,15 +194,19 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_k
         const float4 *x4 = reinterpret_cast<const float4 *>(x) + base4;
         const float4 *a4 = r1 ? reinterpret_cast<const float4 *>(r1) + base4 : nullptr;
         const float4 *b4 = r2 ? reinterpret_cast<const float4 *>(r2) + base4 : nullptr;
-        float4 v[8];
+        float4 v[8], r[8];
         float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = lane + 32 * i < n4 ? __ldg(x4 + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (a4) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) r[i] = lane + 32 * i < n4 ? __ldg(a4 + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int c = lane + 32 * i;
-            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (c < n4) {
-                v[i] = __ldg(x4 + c);
-                if (a4) { const float4 t = __ldg(a4 + c); v[i].x += t.x; v[i].y += t.y; v[i].z += t.z; v[i].w += t.w; }
+                if (a4) { v[i].x += r[i].x; v[i].y += r[i].y; v[i].z += r[i].z; v[i].w += r[i].w; }
                 if (b4) { const float4 t = __ldg(b4 + c); v[i].x += t.x; v[i].y += t.y; v[i].z += t.z; v[i].w += t.w; }
                 s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
             }
@@ -212,7 +221,7 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_k
 // registers instead of travelling through three fp32 tensors (which is what the separate kernels are bound by: for
 // 24576 x 1024 they move 12 + 4 + 4 bytes per value where this one moves 4 and the table rows).  The same roundings as
 // q8_embedding and q8_add_layernorm: every product and sum is rounded by itself.
-__global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm)
+__global__ void __launch_bounds__(kLnThreads, kEmbedLnCtasPerSm)
 embed_layernorm_kernel(const int32_t *__restrict__ ids, int64_t T, int64_t S, const int8_t *__restrict__ word,
                        const float *__restrict__ S_word, int64_t V, const int8_t *__restrict__ pos,
                        const float *__restrict__ S_pos, int64_t P, const int8_t *__restrict__ typ,
@@ -458,7 +467,7 @@ cudaError_t launch_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, con
     if (T <= 0 || H <= 0) return cudaSuccess;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (T + kLnThreads / 32 - 1) / (kLnThreads / 32), cap = (int64_t)(sms > 0 ? sms : 148) * kLnCtasPerSm;
+    const int64_t want = (T + kLnThreads / 32 - 1) / (kLnThreads / 32), cap = (int64_t)(sms > 0 ? sms : 148) * kEmbedLnCtasPerSm;
     return launch_overlapping_tail(embed_layernorm_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kLnThreads), 0, s, ids, T,
                                    S, word, S_word, V, pos, S_pos, P, typ, S_typ, eps, H, out, S_q, out_q, amax, status);
 }

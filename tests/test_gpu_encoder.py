@@ -425,3 +425,16 @@ def test_embed_layernorm_flags_what_is_out_of_range():
     with pytest.raises(q8.Q8Error, match="q8_status 2"):
         wide = [x for n in (4, 4, 2) for x in q8.q8_quantize_weight(torch.ones((n, 1028), device="cuda"))]
         q8.q8_embed_layernorm(torch.zeros(2, dtype=torch.int32, device="cuda"), 2, *wide)
+
+
+@pytest.mark.parametrize("rows", [2367, 2369, 4096, 4736, 4737])
+def test_add_layernorm_at_the_bounds_of_its_grids(rows):
+    """One, two and more rounds of rows (148 SMs x 16 rows): row by row the same results."""
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    x, r = (torch.randn((rows, 96), generator=g, device="cuda") for _ in range(2))
+    whole = q8.q8_add_layernorm(x, r)
+    parts = torch.cat([q8.q8_add_layernorm(x[i:i + 100], r[i:i + 100]) for i in range(0, rows, 100)])
+    assert torch.equal(whole, parts)
+    y = (x.double() + r.double())
+    y = (y - y.mean(1, keepdim=True)) / torch.sqrt(y.var(1, unbiased=False, keepdim=True) + 1e-12)
+    assert (whole.double() - y).abs().max().item() <= REL_TOL * y.abs().max().item()
