@@ -2,10 +2,13 @@
 // fp32-grade accuracy.  Both products, Q K^T and P V, run as tcgen05.mma kind::f16 with every fp32 operand x scaled by
 // a power of two (exactly) and split into two fp16 numbers, hi = fp16(x) and lo = fp16(x - hi): 22 to 23 significant
 // bits, accumulated in fp32 in TMEM as lo*hi + hi*lo + hi*hi; the dropped lo*lo term is below 2^-22 relative per product,
-// i.e. at the rounding level of a plain fp32 dot product.  The scale comes from the data (largest finite |x| of a Q row, of
-// each K chunk and of each V chunk brought into [2^13, 2^14)), so fp16's narrow exponent costs nothing: relative to
-// that largest value a smaller one keeps an absolute error of 2^-39.  The scales are undone in fp32, inside the FFMA that
-// the softmax needs anyway.  (Split TF32 operands, which need no scales, have half the MMA rate and twice the
+// i.e. at the rounding level of a plain fp32 dot product.  The scale comes from the data.  The largest finite |x| of a Q row and of
+// each K chunk is brought into [2^13, 2^14), that of each feature of V, over the keys so far, into [2^12, 2^15); a value below 2^-14
+// of that largest one keeps an absolute error of 2^-37 of it.  P, at most 1 beside its row's reference maximum, is split as
+// 2^13 P: an absolute error of 2^-38 where p < 2^-15.  So no feature of V is less accurate for the size of another.  (One
+// exponent for the 64 features of a V chunk, folded into P, lost 2^-10 for every 2^10 that one feature stood above the
+// others.)  Q's and K's scales are undone inside the FFMA that the softmax needs anyway, V's at the end: the running output is in
+// the units of V's features.  (Split TF32 operands, which need no scales, have half the MMA rate and twice the
 // shared-memory bytes; grids that do not fill the device still use them, see launch_attention_tc().)
 // (The paper keeps attention in fp32 and quantises only the FC layers; this kernel is the fp32 attention an
 // encoder forward needs around them.)
@@ -19,7 +22,7 @@
 //               first); the running output lives in 64 registers of the row's thread and is added to in fp32, because the
 //               tensor core truncates when it accumulates: one chain over 512 keys had an error of 6.6e-7 of |ctx|, growing
 //               with the length (now 1.7e-7 at any length, inputs ~ N(0, 0.55); plain fp32 FMAs: 4.2e-7).  The output is
-//               rescaled only when a row's maximum has risen by more than 2^8 (p has room for that).
+//               rescaled only when a row's maximum has risen by more than 2^2 (p has room for that), or V's unit in some feature.
 //   warps 4..7  staging: K and V global -> registers -> scale, split -> shared memory, 128-byte-swizzled rows of 64 fp16.  K
 //               is a K-major operand; V keeps its [key][feature] order and is read as an MN-major operand.
 //   warp 8      issues the MMAs (converged, one elected lane); the rest of its warpgroup is there for setmaxnreg, which gives
@@ -59,8 +62,8 @@ constexpr int kAttnTcSmemBytes = 1024 + 4 * kKvBytes + kQBytes;  // two K, two V
 constexpr uint32_t kTmemCols = 256;  // scores / P of two chunks, P V of one, Q (32 columns of hi parts, 32 of lo parts)
 constexpr uint32_t kColPV = 128, kColQ = 192;
 constexpr float kLog2eOver8 = 1.4426950408889634f / 8.0f;  // log2(e) / sqrt(64): the softmax uses 2^x
-constexpr int kPShift = 7;           // p is split as 2^7 p: at most 2^15 with the stale-maximum slack below, and small p keep
-constexpr float kStaleSlack = 8.0f;  // their precision (fp16 rounds absolutely below 2^-14)
+constexpr int kPShift = 13;          // p is split as 2^13 p: at most 2^15 with the stale-maximum slack below, and small p keep
+constexpr float kStaleSlack = 2.0f;  // their precision (fp16 rounds absolutely below 2^-14)
 
 // tcgen05.mma kind::f16 instruction descriptor: D = F32, A = B = F16, M = 128; bit 16: B is MN-major.
 constexpr uint32_t kIdescBase = (1u << 4) | ((uint32_t)(kQTile >> 4) << 24);
@@ -142,7 +145,18 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at)
     return v;
 }
 
-// Largest finite magnitude among N float4, as fp32 bits (NaN and infinities do not take part).
+// Largest finite magnitude among N float4 (NaN and infinities do not take part) of each component ...
+__device__ __forceinline__ float finite_abs(float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.0f; }
+template <int N>
+__device__ __forceinline__ float4 absmax_columns(const float4 (&v)[N])
+{
+    float4 m = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        m = make_float4(fmaxf(m.x, finite_abs(v[i].x)), fmaxf(m.y, finite_abs(v[i].y)), fmaxf(m.z, finite_abs(v[i].z)), fmaxf(m.w, finite_abs(v[i].w)));
+    return m;
+}
+// ... and of all of them, as fp32 bits.
 template <int N>
 __device__ __forceinline__ uint32_t absmax_bits(const float4 (&v)[N])
 {
@@ -153,11 +167,8 @@ __device__ __forceinline__ uint32_t absmax_bits(const float4 (&v)[N])
         m = fmaxf(fmaxf(m, fabsf(v[i].z)), fabsf(v[i].w));
     }
     if (m == INFINITY) {  // rare: leave the infinities out (fmaxf has left the NaN out)
-        auto finite = [](float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.0f; };
-        m = 0.0f;
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-            m = fmaxf(fmaxf(fmaxf(m, finite(v[i].x)), fmaxf(finite(v[i].y), finite(v[i].z))), finite(v[i].w));
+        const float4 c = absmax_columns(v);
+        m = fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w));
     }
     return __float_as_uint(m);
 }
@@ -177,16 +188,25 @@ struct Tile {
             v[i] = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(base) +
                                                           ((uint32_t)min((t >> 4) + 8 * i, rows - 1) * pitch_bytes + 16u * (t & 15))));
     }
-    __device__ __forceinline__ void store(uint32_t tile, int t, float mult) const
+    // mult: a power of two for each of this thread's four features
+    __device__ __forceinline__ void scale(float4 mult)
+    {
+        const uint64_t mult_xy = pack_f32x2(mult.x, mult.y), mult_zw = pack_f32x2(mult.z, mult.w);
+#pragma unroll
+        for (int i = 0; i < ROWS / 8; ++i) {
+            unpack_f32x2(mul_f32x2(pack_f32x2(v[i].x, v[i].y), mult_xy), v[i].x, v[i].y);
+            unpack_f32x2(mul_f32x2(pack_f32x2(v[i].z, v[i].w), mult_zw), v[i].z, v[i].w);
+        }
+    }
+    __device__ __forceinline__ void store(uint32_t tile, int t) const
     {
         // (rows t / 16 + 8 i: the same place in every group of 8 rows)
         const uint32_t at = tile + sw128_offset(t >> 4, (t & 15) >> 1) + 8 * (t & 1);
-        const uint64_t m2 = pack_f32x2(mult, mult);
 #pragma unroll
         for (int i = 0; i < ROWS / 8; ++i) {
             uint2 hi, lo;
-            split2(mul_f32x2(pack_f32x2(v[i].x, v[i].y), m2), hi.x, lo.x);
-            split2(mul_f32x2(pack_f32x2(v[i].z, v[i].w), m2), hi.y, lo.y);
+            split2(pack_f32x2(v[i].x, v[i].y), hi.x, lo.x);
+            split2(pack_f32x2(v[i].z, v[i].w), hi.y, lo.y);
             asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + 1024 * i), "r"(hi.x), "r"(hi.y) : "memory");
             asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + 1024 * i + ROWS * 128), "r"(lo.x), "r"(lo.y) : "memory");
         }
@@ -199,6 +219,13 @@ template <int N>
 __device__ __forceinline__ void shrink_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 __device__ __forceinline__ void staging_barrier() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+__device__ __forceinline__ bool staging_any(bool mine)  // whether it holds in any of the staging threads
+{
+    uint32_t any;
+    asm volatile("{\n\t.reg .pred m, a;\n\tsetp.ne.u32 m, %1, 0;\n\tbar.red.or.pred a, 2, 128, m;\n\tselp.u32 %0, 1, 0, a;\n\t}"
+                 : "=r"(any) : "r"(mine ? 1u : 0u) : "memory");
+    return any != 0;
+}
 
 __global__ void __launch_bounds__(kThreads, 2)
 attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__restrict__ ctx,
@@ -213,15 +240,21 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
     __shared__ __align__(8) uint64_t bars[11];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ __align__(16) uint32_t warp_max[2][2][kStagingWarps];  // [chunk parity][K, V][warp]
-    // K = K' 2^exponent, V = V' 2^exponent, by chunk number modulo 4 (K of chunk c + 2 may be staged while the softmax of
-    // chunk c still reads its exponent; K of chunk c + 4 is staged after P of chunk c + 1 was handed over)
-    __shared__ int k_exponent[4], v_exponent[4];
+    __shared__ __align__(16) uint32_t k_max[2][kStagingWarps];  // [chunk parity][warp]
+    __shared__ __align__(16) float v_max[kStagingWarps][kHeadDim];
+    // K = K' 2^exponent, V = V' unit (a power of two for each feature).  By chunk number modulo 4: K's exponent, whether V's units
+    // rose and what the output so far is multiplied by then.  (K of chunk c + 2 may be staged while the softmax of chunk c still
+    // reads its exponent; K of chunk c + 4 is staged after P of chunk c + 1 was handed over, V's units of chunk c + 4 after
+    // P of chunk c + 1 was.)
+    __shared__ int k_exponent[4], v_rose[4];
+    __shared__ __align__(16) float v_factor[4][kHeadDim];
+    __shared__ __align__(16) float v_unit[kHeadDim];  // after the last chunk
     // barrier of each kind for buffer `buf` = chunk parity
     const uint32_t bar0 = smem_u32(bars), q_ready = bar0 + 80;
     auto k_ready = [&](int buf) { return bar0 + 8 * buf; };        // staging -> MMA: K is in place
-    auto v_ready = [&](int buf) { return bar0 + 16 + 8 * buf; };   // staging -> MMA, softmax: V (and its exponent)
-    auto s_done = [&](int buf) { return bar0 + 32 + 8 * buf; };    // MMA -> softmax, staging: scores complete, K read
+    auto v_ready = [&](int buf) { return bar0 + 16 + 8 * buf; };   // staging -> MMA, softmax: V (and its units)
+    // MMA -> softmax, staging: scores complete, K read; and staging -> softmax: K's exponent
+    auto s_done = [&](int buf) { return bar0 + 32 + 8 * buf; };
     auto p_ready = [&](int buf) { return bar0 + 48 + 8 * buf; };   // softmax -> MMA: P is in tensor memory
     auto pv_done = [&](int buf) { return bar0 + 64 + 8 * buf; };   // MMA -> staging, softmax: P V complete, P and V read
 
@@ -239,7 +272,7 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
         for (int buf = 0; buf < 2; ++buf) {
             mbar_init(k_ready(buf), kStagingWarps);
             mbar_init(v_ready(buf), kStagingWarps);
-            mbar_init(s_done(buf), 1);
+            mbar_init(s_done(buf), 2);
             mbar_init(p_ready(buf), kSoftmaxWarps);
             mbar_init(pv_done(buf), 1);
         }
@@ -344,17 +377,60 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
         // ================= staging warps
         grow_registers<kStagingRegs>();
         const int t = tid - 32 * kSoftmaxWarps, w = warp - kSoftmaxWarps;
-        const float *kbase = base + H, *vbase = base + 2 * H;
+        const float *kv = base + H;  // K of the next chunk; V lies H further
         const uint32_t pitch_bytes = (uint32_t)row_pitch * 4u;
         Tile<kChunk> kt, vt;
-        auto chunk_exponent = [&](const Tile<kChunk> &tile, int which, int c) {
-            const uint32_t m = __reduce_max_sync(0xffffffffu, absmax_bits(tile.v));
-            if (lane == 0) warp_max[c & 1][which][w] = m;
+        auto k_chunk_exponent = [&](int c) {
+            const uint32_t m = __reduce_max_sync(0xffffffffu, absmax_bits(kt.v));
+            if (lane == 0) k_max[c & 1][w] = m;
             staging_barrier();
-            const uint4 x = *reinterpret_cast<const uint4 *>(warp_max[c & 1][which]);
+            const uint4 x = *reinterpret_cast<const uint4 *>(k_max[c & 1]);
             return scale_exponent(max(max(x.x, x.y), max(x.z, x.w)));
         };
-        int gv_largest = -126;
+        // V's units of this thread's four features, one byte each: exponent + 126.  Chunk 0 brings its largest values into
+        // [2^12, 2^13); a unit rises only when a later value would reach 2^15 in it, which is rare, so that a chunk costs one vote.
+        uint32_t units = 0;
+        auto unit = [&](int i) { return (int)((units >> (8 * i)) & 255u); };
+        auto in_units = [&]() { vt.scale(make_float4(pow2(126 - unit(0)), pow2(126 - unit(1)), pow2(126 - unit(2)), pow2(126 - unit(3)))); };
+        auto scale_v = [&](int c) {
+            if (c > 0) {
+                in_units();
+                float top = 0.0f;
+#pragma unroll
+                for (int i = 0; i < kChunk / 8; ++i) {
+                    top = fmaxf(fmaxf(top, fabsf(vt.v[i].x)), fabsf(vt.v[i].y));
+                    top = fmaxf(fmaxf(top, fabsf(vt.v[i].z)), fabsf(vt.v[i].w));
+                }
+                if (!staging_any(top >= 32768.0f)) {
+                    if (t == 0) v_rose[c & 3] = 0;
+                    return;
+                }
+                vt.fetch(kv + H - kChunk * row_pitch, pitch_bytes, t, S - c * kChunk);  // (in_units() may have overflowed)
+            }
+            float4 m = absmax_columns(vt.v);
+            m = make_float4(fmaxf(m.x, __shfl_xor_sync(0xffffffffu, m.x, 16)), fmaxf(m.y, __shfl_xor_sync(0xffffffffu, m.y, 16)),
+                            fmaxf(m.z, __shfl_xor_sync(0xffffffffu, m.z, 16)), fmaxf(m.w, __shfl_xor_sync(0xffffffffu, m.w, 16)));
+            if (lane < 16) *reinterpret_cast<float4 *>(&v_max[w][4 * lane]) = m;
+            staging_barrier();
+#pragma unroll
+            for (int i = 0; i < kStagingWarps; ++i) {
+                const float4 x = *reinterpret_cast<const float4 *>(&v_max[i][4 * (t & 15)]);
+                m = make_float4(fmaxf(m.x, x.x), fmaxf(m.y, x.y), fmaxf(m.z, x.z), fmaxf(m.w, x.w));
+            }
+            auto above = [&](float x, int i) { return __float_as_uint(x) >= (uint32_t)min(unit(i) + 16, 255) << 23; };  // 2^15 units
+            auto raised = [&](float x, int i) { return c == 0 || above(x, i) ? scale_exponent(__float_as_uint(x)) + 127 : unit(i); };
+            const int e[4] = {raised(m.x, 0), raised(m.y, 1), raised(m.z, 2), raised(m.w, 3)};
+            if (t < 16) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    v_factor[c & 3][4 * t + i] = pow2(max(unit(i) - e[i], -126));
+                    v_unit[4 * t + i] = pow2(e[i] - 126);
+                }
+            }
+            if (t == 0) v_rose[c & 3] = c > 0;
+            units = (uint32_t)(e[0] | e[1] << 8 | e[2] << 16 | e[3] << 24);
+            in_units();
+        };
         // (chunk -1: nothing to stage yet, its fetches bring in chunk 0; after a time-out the loop still runs, for the
         // barriers of its group alone)
 #pragma unroll 1
@@ -362,28 +438,27 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             const int buf = c & 1, left = S - (c + 1) * kChunk;  // keys behind this chunk
             const uint32_t freed = (uint32_t)(((c >> 1) & 1) ^ 1);
             if (c >= 0) {
-                const int gk = chunk_exponent(kt, 0, c);
+                const int gk = k_chunk_exponent(c);
                 if (c >= 2 && ok) wait(s_done(buf), freed);  // K of chunk c - 2 has been read
                 if (ok) {
-                    kt.store(k_tile(buf), t, pow2(-gk));
+                    kt.scale(make_float4(pow2(-gk), pow2(-gk), pow2(-gk), pow2(-gk)));
+                    kt.store(k_tile(buf), t);
                     if (t == 0) k_exponent[c & 3] = gk;
+                    if (t == 0) mbar_arrive(s_done(buf));
                     arrive(k_ready(buf), true);
                 }
             }
-            if (left > 0) kt.fetch(kbase + (int64_t)(c + 1) * kChunk * row_pitch, pitch_bytes, t, left);
+            if (left > 0) kt.fetch(kv, pitch_bytes, t, left);
             if (c >= 0) {
-                // (a chunk of far smaller values shares the scale of the largest so far to within 2^60: P carries the exponent
-                // too, and fp32 has to hold it for the row sum)
-                const int gv = max(chunk_exponent(vt, 1, c), gv_largest - 60);
-                gv_largest = max(gv_largest, gv);
+                scale_v(c);
                 if (c >= 2 && ok) wait(pv_done(buf), freed);  // V of chunk c - 2 has been read
                 if (ok) {
-                    vt.store(v_tile(buf), t, pow2(-gv));
-                    if (t == 0) v_exponent[c & 3] = gv;
+                    vt.store(v_tile(buf), t);
                     arrive(v_ready(buf), true);
                 }
             }
-            if (left > 0) vt.fetch(vbase + (int64_t)(c + 1) * kChunk * row_pitch, pitch_bytes, t, left);
+            if (left > 0) vt.fetch(kv + H, pitch_bytes, t, left);
+            kv += kChunk * row_pitch;
         }
     } else {
         // ================= softmax warps: thread = query row = TMEM lane
@@ -432,11 +507,11 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             tmem_st_wait();
             arrive(q_ready, false);
         }
-        // Reference maxima, whole numbers so that every power of two between them is exact: M of s + v_exponent
-        // (P is 2^(s + v_exponent - M)), ml of s (for the row sum l)
-        float M = 0.0f, ml = 0.0f;
+        // Reference maximum R of the scores, a whole number so that every power of two between two of them is exact: P is 2^(s - R),
+        // the row sum l is in units of 2^R, the running output O in units of 2^(R - kPShift) times V's units
+        float R = 0.0f;
         float l = 0.0f;
-        uint64_t O[kHeadDim / 2];  // running output of the row, in units of 2^M
+        uint64_t O[kHeadDim / 2];
 #pragma unroll
         for (int j = 0; j < kHeadDim / 2; ++j) O[j] = 0;  // (+0, +0)
         auto add_product = [&](int c) {  // O += P(c) V(c)
@@ -454,9 +529,9 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
         for (int c = 0; c < chunks && ok; ++c) {
             const int buf = c & 1, left = S - c * kChunk;
             const uint32_t par = (uint32_t)((c >> 1) & 1), t_s = t_row + (uint32_t)(buf * kChunk);
-            if (!wait(s_done(buf), par) || !wait(v_ready(buf), par)) break;
+            if (!wait(s_done(buf), par)) break;
             if (warp_live) {
-                const float f = pow2(max(-126, min(120, gq + k_exponent[c & 3]))) * kLog2eOver8, gv = (float)v_exponent[c & 3];
+                const float f = pow2(max(-126, min(120, gq + k_exponent[c & 3]))) * kLog2eOver8;
                 // half 1 of the scores is read twice (for the maximum, then for the exponentials), half 0 stays in registers
                 uint32_t sv[32];
                 float mc = -INFINITY;
@@ -483,23 +558,14 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
                 if (two) take_max(1);
                 take_max(0);
                 mc = ceilf(mc * f);
-                const float a = mc + gv;
                 float rescale = 1.0f;
                 if (c == 0) {
-                    M = a;
-                    ml = mc;
-                } else {
-                    if (a > M + kStaleSlack) {
-                        rescale = exp2_fast(M - a);
-                        M = a;
-                    }
-                    if (mc > ml + 20.0f) {
-                        l *= exp2_fast(ml - mc);
-                        ml = mc;
-                    }
+                    R = mc;
+                } else if (mc > R + kStaleSlack) {
+                    rescale = exp2_fast(R - mc);
+                    R = mc;
                 }
-                const float b = gv - M;
-                const uint64_t f2 = pack_f32x2(f, f), b2 = pack_f32x2(b, b);
+                const uint64_t f2 = pack_f32x2(f, f), b2 = pack_f32x2(-R, -R);
                 const uint64_t shift2 = pack_f32x2((float)(1 << kPShift), (float)(1 << kPShift));
                 uint64_t sum_a = 0, sum_b = 0;  // (+0, +0)
                 auto exponentials = [&](int h) {  // 16 keys: 8 columns of hi parts, then 8 of lo parts, over their scores
@@ -528,7 +594,7 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
                 float sum0, sum1, sum2, sum3;
                 unpack_f32x2(sum_a, sum0, sum1);
                 unpack_f32x2(sum_b, sum2, sum3);
-                l = fmaf((sum0 + sum1) + (sum2 + sum3), exp2_fast(-b - ml), l);
+                l = fmaf(l, rescale, (sum0 + sum1) + (sum2 + sum3));
                 if (c > 0) {
                     add_product(c - 1);
                     if (__any_sync(0xffffffffu, rescale != 1.0f)) {
@@ -539,14 +605,25 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
                 }
                 tmem_st_wait();
             }
+            // V's units of this chunk.  (Before P is handed over: V of chunk c + 2 would complete the barrier's next phase.)
+            if (!wait(v_ready(buf), par)) break;
             arrive(p_ready(buf), false);
+            if (v_rose[c & 3] != 0) {
+                const uint32_t factor = smem_u32(v_factor[c & 3]);
+#pragma unroll
+                for (int j = 0; j < kHeadDim / 2; ++j) {
+                    uint64_t f2;
+                    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(f2) : "r"(factor + 8 * j) : "memory");
+                    O[j] = mul_f32x2(O[j], f2);
+                }
+            }
         }
         // ---------------- ctx = O / row sum
         if (ok && warp_live) add_product(chunks - 1);
         if (ok && warp_live) {
             // Normalised rows to shared memory (where Q came in), then a half-warp takes a row at a time, so that whole lines
             // are stored.  In a short loop: written out for a thread's 64 values this was a third of the kernel's code.
-            const float inv = exp2_fast(M - (float)kPShift - ml) / l;
+            const float inv = pow2(-kPShift) / l;
             const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
@@ -556,10 +633,12 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             __syncwarp();
             const int live_rows = min(32, S - q0 - 32 * warp), pc = lane & 15;
             const int64_t out0 = (seq * (int64_t)S + q0 + 32 * warp) * H + head * kHeadDim + 4 * pc;
+            const float4 unit = *reinterpret_cast<const float4 *>(&v_unit[4 * pc]);
             float am = 0.0f;
 #pragma unroll 2
             for (int r = lane >> 4; r < live_rows; r += 2) {
-                const float4 y = ld_shared_f4(piece(r, pc));
+                float4 y = ld_shared_f4(piece(r, pc));
+                y = make_float4(y.x * unit.x, y.y * unit.y, y.z * unit.z, y.w * unit.w);
                 const int64_t at = out0 + (int64_t)r * H;
                 am = fmaxf(fmaxf(am, fmaxf(fabsf(y.x), fabsf(y.y))), fmaxf(fabsf(y.z), fabsf(y.w)));
                 if (ctx != nullptr) *reinterpret_cast<float4 *>(ctx + at) = y;

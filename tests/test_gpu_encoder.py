@@ -388,6 +388,27 @@ def test_attention_non_finite_rows_stay_in_their_rows():
     assert np.abs(got[np.ix_(rows, features)] - ref[np.ix_(rows, features)]).max() <= EDGE_TOL * np.abs(ref).max()
 
 
+def _many(seed, B, S, heads, sigma=1.0):
+    """Different sequences of several heads, more CTAs than SMs: (qkv, its parts as views [B, S, (q, k, v), heads, 64])."""
+    assert B * heads * ((S + 127) // 128) > torch.cuda.get_device_properties(0).multi_processor_count
+    qkv = synth.normal((B * S, 3 * heads * 64), sigma, seed)
+    return qkv, qkv.reshape(B, S, 3, heads, 64)
+
+
+@pytest.mark.parametrize("power", [10, 16, 24, 40])
+@pytest.mark.parametrize("keys", [slice(0, 64), slice(7, 8), slice(64, 200)])
+def test_attention_features_of_v_are_independent_of_each_other(power, keys):
+    """One feature that is larger in some keys leaves the others as accurate as they are by themselves, each measured against its own
+    largest output."""
+    B, S, heads = 40, 200, 2
+    qkv, parts = _many(3600 + power, B, S, heads)
+    parts[:, keys, 2, :, 5] *= np.float32(2.0 ** power)
+    got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy()
+    assert q8.q8_attention_status() == (q8.Q8_OK, 0)
+    ref = o.attention(qkv, B, S, heads)
+    assert (np.abs(got - ref).max(0) / np.abs(ref).max(0)).max() <= EDGE_TOL
+
+
 # ------------------------------------------------------------------ the input of an encoder in one pass
 @pytest.mark.parametrize("B,S,H", [(1, 1, 4), (3, 7, 100), (2, 33, 768), (5, 512, 1024), (700, 9, 132)])
 def test_embed_layernorm_equals_the_separate_calls(B, S, H):
