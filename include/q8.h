@@ -260,8 +260,10 @@ q8_status q8_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, const int
 
 /* q8_attention / q8_attention_quant run on the tensor cores when the pointers are 16-byte aligned: both products as
  * tcgen05.mma on operands split into two 16-bit (kind::f16, scaled by powers of two) or TF32 parts each, three
- * partial products accumulated in fp32, which keeps fp32-grade accuracy (an infinite input gives NaN where the
- * exact result would be infinite).  Otherwise a CUDA-core fp32 kernel computes the same thing.  The tensor-core
+ * partial products accumulated in fp32, which keeps fp32-grade accuracy; rows whose operands span more than the 16-bit
+ * parts carry are computed in plain fp32.  (Grids of at most one CTA of 128 queries per SM with S <= 384 use TF32 parts: an
+ * infinite input gives NaN there where the exact result would be infinite.)  Unaligned pointers: a CUDA-core fp32
+ * kernel computes the same thing.  The tensor-core
  * kernels bound their waits; a time-out sets the Q8_ERR_TIMEOUT bit in a per-device status word whose device
  * address q8_attention_status_word returns (poll it with q8_poll_status). */
 q8_status q8_attention_status_word(void **dev_status);

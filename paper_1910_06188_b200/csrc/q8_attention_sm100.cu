@@ -26,8 +26,16 @@
 //   warps 4..7  staging: K and V global -> registers -> scale, split -> shared memory, 128-byte-swizzled rows of 64 fp16.  K
 //               is a K-major operand; V keeps its [key][feature] order and is read as an MN-major operand.
 //   warp 8      issues the MMAs (converged, one elected lane); the rest of its warpgroup is there for setmaxnreg, which gives
-//               the softmax 128 registers a thread and the staging 88, the one split without spills (120 / 96: 3 % slower, 112 / 104:
+//               the softmax 128 registers a thread and the staging 88, the one split without spills in the loops (120 / 96: 3 % slower, 112 / 104:
 //               8 %; with 96 for all, O was spilled).
+// Where the split parts would not carry what fp32 carries, the row is computed over again in plain fp32 FMAs (plain_row()), by
+// its own thread and for itself alone:
+//   - largest |q| of the row times largest |k| of a chunk above 2^kScoreExponent.  Up to there a score is off by less than
+//     2^-20 in its exponent of 2 whatever the operands look like (64 products, each operand off by 2^-39 of its largest), and
+//     the reference maximum, a whole number below 2^18, is subtracted without a loss.
+//   - a row whose result is small beside V in every feature (kSmallResult): it hangs on keys whose V is tiny beside that of
+//     others, and what those are rounded by counts.
+//   - infinities.
 // Measured (64 x 384 x 16 heads / 16 x 512 x 12 / 32 x 128 x 12, Int8 output): 227 / 72 / 19.9 us; split TF32 with whole score
 // rows in TMEM, one CTA per SM, 512 threads staging: 304 / - / 23.8 us (it takes S <= 384; plain fp32 FMAs needed 413 us at
 // 512).  What bounds it now is latency: loads of K and V (without them 25 % less) and the chain softmax -> P V -> scores
@@ -64,6 +72,8 @@ constexpr uint32_t kColPV = 128, kColQ = 192;
 constexpr float kLog2eOver8 = 1.4426950408889634f / 8.0f;  // log2(e) / sqrt(64): the softmax uses 2^x
 constexpr int kPShift = 13;          // p is split as 2^13 p: at most 2^15 with the stale-maximum slack below, and small p keep
 constexpr float kStaleSlack = 2.0f;  // their precision (fp16 rounds absolutely below 2^-14)
+constexpr int kScoreExponent = 14;           // log2 of the largest |q| |k| that the split product takes (of values ~ N(0, 1): 2^4)
+constexpr float kSmallResult = 4.0f;           // in V's units, whose largest is 2^12 .. 2^15 (a mean of 4096 values ~ N(0, 1): 2^6)
 
 // tcgen05.mma kind::f16 instruction descriptor: D = F32, A = B = F16, M = 128; bit 16: B is MN-major.
 constexpr uint32_t kIdescBase = (1u << 4) | ((uint32_t)(kQTile >> 4) << 24);
@@ -145,15 +155,14 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at)
     return v;
 }
 
-// Largest finite magnitude among N float4 (NaN and infinities do not take part) of each component ...
-__device__ __forceinline__ float finite_abs(float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.0f; }
+// Largest magnitude among N float4 (a NaN does not take part; an infinity sends the rows to plain_row()) of each component ...
 template <int N>
 __device__ __forceinline__ float4 absmax_columns(const float4 (&v)[N])
 {
     float4 m = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int i = 0; i < N; ++i)
-        m = make_float4(fmaxf(m.x, finite_abs(v[i].x)), fmaxf(m.y, finite_abs(v[i].y)), fmaxf(m.z, finite_abs(v[i].z)), fmaxf(m.w, finite_abs(v[i].w)));
+        m = make_float4(fmaxf(m.x, fabsf(v[i].x)), fmaxf(m.y, fabsf(v[i].y)), fmaxf(m.z, fabsf(v[i].z)), fmaxf(m.w, fabsf(v[i].w)));
     return m;
 }
 // ... and of all of them, as fp32 bits.
@@ -165,10 +174,6 @@ __device__ __forceinline__ uint32_t absmax_bits(const float4 (&v)[N])
     for (int i = 0; i < N; ++i) {
         m = fmaxf(fmaxf(m, fabsf(v[i].x)), fabsf(v[i].y));
         m = fmaxf(fmaxf(m, fabsf(v[i].z)), fabsf(v[i].w));
-    }
-    if (m == INFINITY) {  // rare: leave the infinities out (fmaxf has left the NaN out)
-        const float4 c = absmax_columns(v);
-        m = fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w));
     }
     return __float_as_uint(m);
 }
@@ -213,6 +218,67 @@ struct Tile {
     }
 };
 
+// One query row in plain fp32 FMAs by one thread (see the top of the file): softmax(q K^T / 8) V over all S keys, four at a time, with
+// the running maximum and sum of q8_support.cu's kernel.  q_at(i): shared-memory address of the i-th 16 bytes of q.  Leaves the sum
+// of p v in O, returns the sum of p.
+template <typename QAt>
+__device__ __forceinline__ float plain_row(QAt q_at, const float *qkv, int S, int64_t H, uint64_t (&O)[kHeadDim / 2])
+{
+    uint32_t head, seq;  // read here, so that the caller's loop need not keep them
+    asm volatile("mov.u32 %0, %%ctaid.y;\n\tmov.u32 %1, %%ctaid.z;" : "=r"(head), "=r"(seq));
+    const int64_t row_pitch = 3 * H;
+    const float *k = qkv + seq * (int64_t)S * row_pitch + head * kHeadDim + H, *v = k + H;
+    float m = -INFINITY, l = 0.0f;
+#pragma unroll
+    for (int j = 0; j < kHeadDim / 2; ++j) O[j] = 0;  // (+0, +0)
+#pragma unroll 1
+    for (int j0 = 0; j0 < S; j0 += 4, k += 4 * row_pitch, v += 4 * row_pitch) {
+        float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
+        for (int i = 0; i < kHeadDim / 4; ++i) {
+            const float4 q = ld_shared_f4(q_at(i));
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if (j0 + a >= S) break;
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(k + a * row_pitch) + i);
+                s[a] = fmaf(q.x * kLog2eOver8, x.x, s[a]);
+                s[a] = fmaf(q.y * kLog2eOver8, x.y, s[a]);
+                s[a] = fmaf(q.z * kLog2eOver8, x.z, s[a]);
+                s[a] = fmaf(q.w * kLog2eOver8, x.w, s[a]);
+            }
+        }
+        float m_new = m;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (j0 + a < S) m_new = fmaxf(m_new, s[a]);
+        const float ref = m_new == -INFINITY ? 0.0f : m_new;  // (only scores of -inf so far: their p is 0)
+        const float corr = exp2f(m - ref);
+        l *= corr;
+        uint64_t p2[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float p = j0 + a < S ? exp2f(s[a] - ref) : 0.0f;
+            l += p;
+            p2[a] = pack_f32x2(p, p);
+        }
+        m = m_new;
+        const uint64_t corr2 = pack_f32x2(corr, corr);
+#pragma unroll
+        for (int i = 0; i < kHeadDim / 4; ++i) {
+            O[2 * i] = mul_f32x2(O[2 * i], corr2);
+            O[2 * i + 1] = mul_f32x2(O[2 * i + 1], corr2);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if (j0 + a >= S) break;
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(v + a * row_pitch) + i);
+                O[2 * i] = fma_f32x2(pack_f32x2(x.x, x.y), p2[a], O[2 * i]);
+                O[2 * i + 1] = fma_f32x2(pack_f32x2(x.z, x.w), p2[a], O[2 * i + 1]);
+            }
+        }
+    }
+    return l;
+}
+
 template <int N>
 __device__ __forceinline__ void grow_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N>
@@ -249,6 +315,7 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
     __shared__ int k_exponent[4], v_rose[4];
     __shared__ __align__(16) float v_factor[4][kHeadDim];
     __shared__ __align__(16) float v_unit[kHeadDim];  // after the last chunk
+    __shared__ int v_any, v_far;                      // any of V is not zero, is infinite
     // barrier of each kind for buffer `buf` = chunk parity
     const uint32_t bar0 = smem_u32(bars), q_ready = bar0 + 80;
     auto k_ready = [&](int buf) { return bar0 + 8 * buf; };        // staging -> MMA: K is in place
@@ -277,6 +344,8 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             mbar_init(pv_done(buf), 1);
         }
         abort_flag = 0;
+        v_any = 0;
+        v_far = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kSoftmaxWarps + kStagingWarps) tmem_alloc(smem_u32(&tmem_slot), kTmemCols);
@@ -421,6 +490,9 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             auto raised = [&](float x, int i) { return c == 0 || above(x, i) ? scale_exponent(__float_as_uint(x)) + 127 : unit(i); };
             const int e[4] = {raised(m.x, 0), raised(m.y, 1), raised(m.z, 2), raised(m.w, 3)};
             if (t < 16) {
+                const float top = fmaxf(fmaxf(m.x, m.y), fmaxf(m.z, m.w));
+                if (top > 0.0f) v_any = 1;
+                if (top == INFINITY) v_far = 1;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     v_factor[c & 3][4 * t + i] = pow2(max(unit(i) - e[i], -126));
@@ -531,7 +603,9 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             const uint32_t par = (uint32_t)((c >> 1) & 1), t_s = t_row + (uint32_t)(buf * kChunk);
             if (!wait(s_done(buf), par)) break;
             if (warp_live) {
-                const float f = pow2(max(-126, min(120, gq + k_exponent[c & 3]))) * kLog2eOver8;
+                const int g = gq + k_exponent[c & 3];
+                if (g + 28 > kScoreExponent) l = NAN;  // (largest |q| |k| may reach 2^(g + 28): the row goes to plain_row())
+                const float f = pow2(max(-126, min(120, g))) * kLog2eOver8;
                 // half 1 of the scores is read twice (for the maximum, then for the exponentials), half 0 stays in registers
                 uint32_t sv[32];
                 float mc = -INFINITY;
@@ -623,7 +697,18 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
         if (ok && warp_live) {
             // Normalised rows to shared memory (where Q came in), then a half-warp takes a row at a time, so that whole lines
             // are stored.  In a short loop: written out for a thread's 64 values this was a third of the kernel's code.
-            const float inv = pow2(-kPShift) / l;
+            float inv = pow2(-kPShift) / l;
+            float top = v_any != 0 ? 0.0f : INFINITY;
+#pragma unroll
+            for (int j = 0; j < kHeadDim / 2; ++j) {
+                float a, b;
+                unpack_f32x2(O[j], a, b);
+                top = fmaxf(fmaxf(top, fabsf(a)), fabsf(b));
+            }
+            const bool plain = (v_far != 0 || !(top * inv >= kSmallResult)) && q0 + 32 * warp + lane < S;
+            const uint32_t plain_rows = __ballot_sync(0xffffffffu, plain);
+            if (plain) inv = 1.0f / plain_row([&](int i) { return piece(lane, i); }, qkv, S, H, O);
+            __syncwarp();
             const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
@@ -638,7 +723,7 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
 #pragma unroll 2
             for (int r = lane >> 4; r < live_rows; r += 2) {
                 float4 y = ld_shared_f4(piece(r, pc));
-                y = make_float4(y.x * unit.x, y.y * unit.y, y.z * unit.z, y.w * unit.w);
+                if (((plain_rows >> r) & 1u) == 0u) y = make_float4(y.x * unit.x, y.y * unit.y, y.z * unit.z, y.w * unit.w);
                 const int64_t at = out0 + (int64_t)r * H;
                 am = fmaxf(fmaxf(am, fmaxf(fabsf(y.x), fabsf(y.y))), fmaxf(fabsf(y.z), fabsf(y.w)));
                 if (ctx != nullptr) *reinterpret_cast<float4 *>(ctx + at) = y;

@@ -409,6 +409,98 @@ def test_attention_features_of_v_are_independent_of_each_other(power, keys):
     assert (np.abs(got - ref).max(0) / np.abs(ref).max(0)).max() <= EDGE_TOL
 
 
+def _dot_error(q, k):
+    """Largest rounding error of a score in fp32: about four roundings' worth of sum |q_d k_d| / 8."""
+    return float(np.einsum("bshd,bthd->bhst", np.abs(q).astype(np.float64), np.abs(k)).max()) / 8 * 2.0 ** -22
+
+
+@pytest.mark.parametrize("sigma", [6.0, 30.0, 4000.0, 30000.0, 1e15])
+def test_attention_of_large_scores(sigma):
+    """Scores beyond what whole numbers in fp32 can tell apart, in a grid that fills the device: an average of V, the arg-max row
+    of V where one score is ahead of the others, and the same values in every output form."""
+    B, S, heads = 26, 130, 3
+    qkv, parts = _many(3700, B, S, heads)
+    parts[:, :, :2] *= np.float32(sigma)
+    got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy()
+    assert q8.q8_attention_status() == (q8.Q8_OK, 0)
+    q, k, v = (parts[:, :, i] for i in range(3))
+    assert np.isfinite(got).all()
+    assert (np.abs(got.reshape(B, S, heads, 64)) <= np.abs(v).max(1, keepdims=True) * (1 + EDGE_TOL)).all()
+    slack = _dot_error(q, k)
+    if slack < 0.01:  # the weights are off by as much
+        ref = o.attention(qkv, B, S, heads)
+        assert np.abs(got - ref).max() <= (EDGE_TOL + slack) * np.abs(ref).max()
+    s = np.einsum("bshd,bthd->bhst", q.astype(np.float64), k) / 8
+    top = np.sort(s, axis=-1)[..., -2:]
+    clear = top[..., 1] - top[..., 0] > 2 * slack + 120  # e^-120: the other weights are zero in fp32
+    assert sigma < 1000 or clear.mean() > 0.9
+    want = np.take_along_axis(v.transpose(0, 2, 1, 3), s.argmax(-1)[..., None], axis=2)
+    assert np.abs(got.reshape(B, S, heads, 64).transpose(0, 2, 1, 3) - want)[clear].max(initial=0.0) <= EDGE_TOL * np.abs(v).max()
+    scale, peak = dev(np.array([20.0], np.float32)), _word()
+    got_q = q8.q8_attention_quant(dev(qkv), B, S, heads, scale).cpu().numpy()
+    assert np.array_equal(got_q, o.quantize(got, 20.0))
+    assert np.array_equal(q8.q8_attention_absmax(dev(qkv), B, S, heads, peak).cpu().numpy(), got)
+    assert peak.view(torch.float32).item() == np.abs(got).max()
+
+
+@pytest.mark.parametrize("power", [10, 12, 16, 24])
+@pytest.mark.parametrize("S", [130, 200])
+def test_attention_of_operands_that_differ_widely_from_feature_to_feature(power, S):
+    """Q large in one feature and small in another, K the other way round: the scores are ordinary ones, and so is their accuracy."""
+    B, heads = 40, 2
+    qkv, parts = _many(3720 + power, B, S, heads)
+    big = np.float32(2.0 ** power)
+    parts[:, :, 0, :, 3] *= big
+    parts[:, :, 1, :, 3] /= big
+    parts[:, :, 0, :, 40] /= big
+    parts[:, :, 1, :, 40] *= big
+    got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy()
+    ref = o.attention(qkv, B, S, heads)
+    assert np.abs(got - ref).max() <= EDGE_TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("S", [129, 200])
+def test_attention_rows_that_hang_on_a_small_value(S):
+    """Every third query attends to key 7 alone, whose V is 2^-30 of the others': that row is v_7, to its own precision."""
+    B, heads = 40, 2
+    qkv, parts = _many(3740, B, S, heads)
+    parts[:, ::3, 0, :, 0] = 8.0
+    parts[:, :, 1, :, 0] = 0.0
+    parts[:, 7, 1, :, 0] = 64.0   # 64 score units ahead
+    parts[:, 7, 2] *= np.float32(2.0 ** -30)
+    got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy().reshape(B, S, heads, 64)[:, ::3]
+    ref = o.attention(qkv, B, S, heads).reshape(B, S, heads, 64)[:, ::3]
+    assert (np.abs(got - ref).max(-1) / np.abs(ref).max(-1)).max() <= EDGE_TOL
+
+
+@pytest.mark.parametrize("power", [-120, 0, 78, 90, 118])
+def test_attention_of_v_over_the_range_of_fp32(power):
+    B, S, heads = 40, 200, 2
+    qkv, parts = _many(3760, B, S, heads)
+    ref = o.attention(qkv, B, S, heads)
+    parts[:, :, 2] *= np.float32(2.0 ** power)
+    got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy().astype(np.float64) * 2.0 ** -power
+    assert np.abs(got - ref).max() <= EDGE_TOL * np.abs(ref).max()
+    parts[:, :, 2] = 0.0
+    assert not q8.q8_attention(dev(qkv), B, S, heads).any()
+
+
+def test_attention_of_an_infinite_key():
+    """A score of -inf takes its key out of the average, a score of +inf makes the row NaN."""
+    B, S, heads = 40, 200, 2
+    qkv, parts = _many(3780, B, S, heads)
+    parts[:, 70, 1, :, 9] = np.inf
+    got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy().reshape(B, S, heads, 64)
+    assert q8.q8_attention_status() == (q8.Q8_OK, 0)
+    out = parts[:, :, 0, :, 9] < 0
+    rest = np.ascontiguousarray(np.delete(parts, 70, axis=1)).reshape(-1, qkv.shape[1])
+    rest = o.attention(rest, B, S - 1, heads).reshape(B, S - 1, heads, 64)
+    ref = np.insert(rest, 70, np.nan, axis=1)
+    out[:, 70] = False  # (the query of that position is not in the reference)
+    assert np.abs(got - ref)[out].max() <= EDGE_TOL * np.nanmax(np.abs(ref))
+    assert np.isnan(got[parts[:, :, 0, :, 9] > 0]).all()
+
+
 # ------------------------------------------------------------------ the input of an encoder in one pass
 @pytest.mark.parametrize("B,S,H", [(1, 1, 4), (3, 7, 100), (2, 33, 768), (5, 512, 1024), (700, 9, 132)])
 def test_embed_layernorm_equals_the_separate_calls(B, S, H):
