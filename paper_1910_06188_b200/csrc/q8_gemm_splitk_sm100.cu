@@ -105,6 +105,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    cluster_arrive();  // this CTA has started.  Every role waits for the others' arrivals off the critical path (and when aborting)
     grid_dependency_release_next(true);  // small by construction: one tile per cluster
     grid_dependency_wait();
 
@@ -124,6 +125,8 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const uint64_t t0 = global_timer_ns();
             while (global_timer_ns() - t0 < 1000000ull) {}
         }
+        __syncwarp();
+        cluster_wait();
     } else if (warp == 1) {
         const uint32_t elected = elect_one();
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -142,7 +145,10 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const uint64_t t0 = global_timer_ns();
             while (global_timer_ns() - t0 < 1000000ull) {}
         }
+        __syncwarp();
+        cluster_wait();
     } else {
+        cluster_wait();  // (before any CTA stores into another's shared memory)
         // Partial sums of the blocks that another CTA finishes go to that CTA's exchange slot: with ROWS the block of lane quarter
         // q is CTA q's, else the block of columns 32 r .. of every quarter is CTA r's.
         const int quarter = warp & 3;
