@@ -137,6 +137,29 @@ def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str) -> Optional[i
     return t.data_ptr()
 
 
+def _layer_shape(X: torch.Tensor, Wq: torch.Tensor, name: str = "X") -> Tuple[int, int, int]:
+    """(M, N, K) of a layer with activation [M, K] and weight [N, K]."""
+    M, K = X.shape
+    N, K2 = Wq.shape
+    if K != K2:
+        raise ValueError(f"{name} is [M,{K}] but Wq is [N,{K2}]")
+    return M, N, K
+
+
+def _check_covers(t: Optional[torch.Tensor], values: int, name: str) -> None:
+    if t is not None and t.numel() < values:
+        raise ValueError(f"{name} has {t.numel()} values, {values} are read")
+
+
+def _layernorm_shape(x, r1, r2, gamma, beta) -> Tuple[int, int]:
+    rows, H = x.shape
+    for t, name in ((r1, "r1"), (r2, "r2")):
+        _check_covers(t, rows * H, name)
+    for t, name in ((gamma, "gamma"), (beta, "beta")):
+        _check_covers(t, H, name)
+    return rows, H
+
+
 def _any_ptr(t: Optional[torch.Tensor], name: str) -> Optional[int]:
     if t is None:
         return None
@@ -254,10 +277,7 @@ def new_workspace(M: int, N: int, K: int, device="cuda") -> torch.Tensor:
 
 
 def _linear(fn_name: str, X, Wq, S_w, S_x, bias, act, Y, workspace, dbg_Xq, dbg_acc, stream):
-    M, K = X.shape
-    N, K2 = Wq.shape
-    if K != K2:
-        raise ValueError(f"X is [M,{K}] but Wq is [N,{K2}]")
+    M, N, K = _layer_shape(X, Wq)
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float32, device=X.device)
     if workspace is None:
@@ -293,10 +313,7 @@ def q8_linear_q(Xq, S_x, Wq, S_w, bias=None, act: int = Q8_ACT_NONE, Y=None, dbg
         r = (_native_module or _native()).linear_q(Xq, S_x, Wq, S_w, bias, act, Y, dbg_acc, dev_status)
         if r is not NotImplemented:
             return r
-    M, K = Xq.shape
-    N, K2 = Wq.shape
-    if K != K2:
-        raise ValueError(f"Xq is [M,{K}] but Wq is [N,{K2}]")
+    M, N, K = _layer_shape(Xq, Wq, "Xq")
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float32, device=Xq.device)
     st = load().q8_linear_q(_ptr(Xq, torch.int8, "Xq"), _ptr(S_x, torch.float32, "S_x"), _ptr(Wq, torch.int8, "Wq"),
@@ -315,10 +332,7 @@ def q8_linear_noalloc(X, Wq, S_w, S_x=None, bias=None, act: int = Q8_ACT_NONE, Y
     """q8_linear without a caller workspace: for callers that may not allocate device memory (the scratch
     is a fixed array inside the library, M*K <= Q8_NOALLOC_MAX_MK).  Y must be supplied by such callers;
     when it is None this binding allocates it with torch for convenience.  Returns (Y, status_word_address)."""
-    M, K = X.shape
-    N, K2 = Wq.shape
-    if K != K2:
-        raise ValueError(f"X is [M,{K}] but Wq is [N,{K2}]")
+    M, N, K = _layer_shape(X, Wq)
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float32, device=X.device)
     word = C.c_void_p(0)
@@ -385,7 +399,7 @@ def q8_add_layernorm(x, r1=None, r2=None, gamma=None, beta=None, eps: float = 1e
         r = (_native_module or _native()).add_layernorm(x, r1, r2, gamma, beta, eps, out, None, None, None)
         if r is not NotImplemented:
             return r
-    rows, H = x.shape
+    rows, H = _layernorm_shape(x, r1, r2, gamma, beta)
     if out is None:
         out = torch.empty_like(x)
     st = load().q8_add_layernorm(_ptr(x, torch.float32, "x"), _ptr(r1, torch.float32, "r1"),
@@ -420,7 +434,7 @@ def q8_add_layernorm_absmax(x, absmax_bits, r1=None, r2=None, gamma=None, beta=N
         r = (_native_module or _native()).add_layernorm_absmax(x, r1, r2, gamma, beta, eps, out, None, None, absmax_bits)
         if r is not NotImplemented:
             return r
-    rows, H = x.shape
+    rows, H = _layernorm_shape(x, r1, r2, gamma, beta)
     if out is None:
         out = torch.empty_like(x)
     st = load().q8_add_layernorm_absmax(_ptr(x, torch.float32, "x"), _ptr(r1, torch.float32, "r1"),
@@ -457,10 +471,7 @@ def q8_linear_dyn(X, x_absmax, Wq, S_w, bias=None, act: int = Q8_ACT_NONE, Y=Non
         r = (_native_module or _native()).linear_dyn(X, x_absmax, Wq, S_w, bias, act, Y, y_absmax, workspace, dbg_Xq, dbg_acc)
         if r is not NotImplemented:
             return r
-    M, K = X.shape
-    N, K2 = Wq.shape
-    if K != K2:
-        raise ValueError(f"X is [M,{K}] but Wq is [N,{K2}]")
+    M, N, K = _layer_shape(X, Wq)
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float32, device=X.device)
     if workspace is None:
@@ -490,8 +501,7 @@ def q8_quantize_weight_segments(W, seg_rows: int, dev_status=None, stream=None):
 def q8_linear_wseg(X, Wq, S_w, seg_rows: int, S_x=None, bias=None, act: int = Q8_ACT_NONE, Y=None, workspace=None,
                    dbg_Xq=None, dbg_acc=None, stream=None):
     """q8_linear with one weight scale per block of `seg_rows` output features."""
-    M, K = X.shape
-    N = Wq.shape[0]
+    M, N, K = _layer_shape(X, Wq)
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float32, device=X.device)
     if workspace is None:
@@ -507,8 +517,7 @@ def q8_linear_wseg(X, Wq, S_w, seg_rows: int, S_x=None, bias=None, act: int = Q8
 
 def q8_linear_q_wseg(Xq, S_x, Wq, S_w, seg_rows: int, bias=None, act: int = Q8_ACT_NONE, Y=None, dbg_acc=None,
                      dev_status=None, stream=None):
-    M, K = Xq.shape
-    N = Wq.shape[0]
+    M, N, K = _layer_shape(Xq, Wq, "Xq")
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float32, device=Xq.device)
     st = load().q8_linear_q_wseg(_ptr(Xq, torch.int8, "Xq"), _ptr(S_x, torch.float32, "S_x"), _ptr(Wq, torch.int8, "Wq"),
@@ -526,8 +535,7 @@ def q8_linear_requant(X, Wq, S_w, S_x, bias, act, S_y, Yq=None, Y=None, workspac
         r = (_native_module or _native()).linear_requant(X, Wq, S_w, S_x, bias, act, S_y, Yq, Y, workspace, dbg_Xq, dbg_acc)
         if r is not NotImplemented:
             return r
-    M, K = X.shape
-    N = Wq.shape[0]
+    M, N, K = _layer_shape(X, Wq)
     if Yq is None:
         Yq = torch.empty((M, N), dtype=torch.int8, device=X.device)
     if workspace is None:
@@ -549,8 +557,7 @@ def q8_linear_q_requant(Xq, S_x, Wq, S_w, bias, act, S_y, Yq=None, Y=None, dbg_a
         r = (_native_module or _native()).linear_q_requant(Xq, S_x, Wq, S_w, bias, act, S_y, Yq, Y, dbg_acc, dev_status)
         if r is not NotImplemented:
             return r
-    M, K = Xq.shape
-    N = Wq.shape[0]
+    M, N, K = _layer_shape(Xq, Wq, "Xq")
     if Yq is None:
         Yq = torch.empty((M, N), dtype=torch.int8, device=Xq.device)
     st = load().q8_linear_q_requant(_ptr(Xq, torch.int8, "Xq"), _ptr(S_x, torch.float32, "S_x"),
@@ -569,7 +576,7 @@ def q8_add_layernorm_quant(x, r1, r2, S_q, out_q=None, out=None, gamma=None, bet
         r = (_native_module or _native()).add_layernorm_quant(x, r1, r2, gamma, beta, eps, out, S_q, out_q, None)
         if r is not NotImplemented:
             return r
-    rows, H = x.shape
+    rows, H = _layernorm_shape(x, r1, r2, gamma, beta)
     if out_q is None:
         out_q = torch.empty((rows, H), dtype=torch.int8, device=x.device)
     st = load().q8_add_layernorm_quant(_ptr(x, torch.float32, "x"), _ptr(r1, torch.float32, "r1"),
@@ -588,6 +595,9 @@ def q8_attention_quant(qkv, B: int, S: int, heads: int, S_q, ctx_q=None, ctx=Non
         if r is not NotImplemented:
             return r
     H = heads * 64
+    if qkv.dim() == 2 and qkv.shape[1] != 3 * H:
+        raise ValueError(f"qkv must be [{B * S}, {3 * H}], got {tuple(qkv.shape)}")
+    _check_covers(qkv, B * S * 3 * H, "qkv")
     if ctx_q is None:
         ctx_q = torch.empty((B * S, H), dtype=torch.int8, device=qkv.device)
     st = load().q8_attention_quant(_ptr(qkv, torch.float32, "qkv"), B, S, heads, _ptr(ctx, torch.float32, "ctx"),

@@ -57,6 +57,14 @@ struct Call {
         }
         return static_cast<T *>(t->data_ptr());
     }
+    // the same for a tensor of which `values` values are read
+    template <typename T>
+    T *covering(PyObject *o, at::ScalarType type, int64_t values)
+    {
+        T *p = ptr<T>(o, type);
+        if (plain && o != Py_None && THPVariable_Unpack(o).numel() < values) plain = false;
+        return p;
+    }
     void *any_ptr(PyObject *o, size_t *bytes = nullptr)
     {
         const at::Tensor *t = tensor(o);
@@ -309,8 +317,9 @@ PyObject *add_layernorm(Args a)
     Call c;
     int64_t rows, H;
     if (!c.matrix(a[0], &rows, &H)) return other_form();
-    auto x = c.ptr<const float>(a[0], kF32), r1 = c.ptr<const float>(a[1], kF32), r2 = c.ptr<const float>(a[2], kF32),
-         gamma = c.ptr<const float>(a[3], kF32), beta = c.ptr<const float>(a[4], kF32), S_q = c.ptr<const float>(a[7], kF32);
+    auto x = c.ptr<const float>(a[0], kF32), r1 = c.covering<const float>(a[1], kF32, rows * H),
+         r2 = c.covering<const float>(a[2], kF32, rows * H), gamma = c.covering<const float>(a[3], kF32, H),
+         beta = c.covering<const float>(a[4], kF32, H), S_q = c.ptr<const float>(a[7], kF32);
     const float eps = c.real(a[5]);
     auto word = c.ptr<uint32_t>(a[9], kI32);
     if (KIND == 1) {
@@ -342,7 +351,7 @@ PyObject *attention(Args a)
     if (!c.matrix(a[0], &T, &W)) return other_form();
     const int64_t B = c.integer(a[1]), S = c.integer(a[2]), heads = c.integer(a[3]);
     if (!c.plain || B < 0 || S < 0 || heads < 0 || heads > 65535 || B > 65535 || S > (int64_t(1) << 31) || B * S != T ||
-        (KIND != 1 && heads * 192 != W))
+        heads * 192 != W)
         return other_form();
     const int64_t H = heads * 64;
     auto qkv = c.ptr<const float>(a[0], kF32);

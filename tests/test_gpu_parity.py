@@ -482,6 +482,37 @@ def test_native_calls_refuse_what_the_python_form_refuses():
         q8.q8_linear(X, Wq[:, :32].contiguous(), S_w, workspace=torch.empty(256, dtype=torch.uint8, device="cuda"))
 
 
+def test_operands_that_do_not_fit_together_are_refused():
+    """In both forms of a call, before anything is launched: shapes under which a kernel would read past an operand, or read it as
+    something that it is not."""
+    f32 = lambda *shape: torch.ones(shape, device="cuda")
+    i8 = lambda *shape: torch.ones(shape, dtype=torch.int8, device="cuda")
+    s, word, b = f32(1), torch.zeros(1, dtype=torch.int32, device="cuda"), f32(8)
+    X, Xq, ids = f32(4, 32), i8(4, 32), torch.zeros(6, dtype=torch.int32, device="cuda")
+    cases = []
+    for W in (i8(8, 16), i8(8, 48)):
+        cases += [(q8.q8_linear, (X, W, s)), (q8.q8_linear_generic, (X, W, s)), (q8.q8_linear_q, (Xq, s, W, s)),
+                  (q8.q8_linear_requant, (X, W, s, s, b, 0, s)), (q8.q8_linear_q_requant, (Xq, s, W, s, b, 0, s)),
+                  (q8.q8_linear_dyn, (X, word, W, s)), (q8.q8_linear_wseg, (X, W, s, 32)), (q8.q8_linear_q_wseg, (Xq, s, W, s, 32))]
+    for qkv, B, S, heads in ((f32(20, 192), 3, 10, 1), (f32(20, 192), 2, 10, 2), (f32(20, 384), 2, 10, 1)):
+        cases += [(q8.q8_attention, (qkv, B, S, heads)), (q8.q8_attention_quant, (qkv, B, S, heads, s)),
+                  (q8.q8_attention_absmax, (qkv, B, S, heads, word))]
+    for extra in ((f32(3, 32),), (None, f32(4, 31)), (None, None, f32(31)), (None, None, None, f32(31))):
+        extra = tuple(extra) + (None,) * (4 - len(extra))
+        cases += [(q8.q8_add_layernorm, (X,) + extra), (q8.q8_add_layernorm_absmax, (X, word) + extra),
+                  (q8.q8_add_layernorm_quant, (X, extra[0], extra[1], s, None, None, extra[2], extra[3]))]
+    for pos, typ in ((i8(9, 16), i8(2, 32)), (i8(9, 32), i8(2, 16)), (i8(9, 32), i8(0, 32))):
+        cases.append((q8.q8_embed_layernorm, (ids, 3, i8(9, 32), s, pos, s, typ, s)))
+    for fn, args in cases:
+        for stream in (None, torch.cuda.current_stream()):
+            with pytest.raises(ValueError):
+                fn(*args, stream=stream)
+    # larger ones than needed stay as they were
+    x, r, qkv = torch.randn((4, 32), device="cuda"), torch.randn((5, 32), device="cuda"), torch.randn((21, 192), device="cuda")
+    assert torch.equal(q8.q8_add_layernorm(x, r), q8.q8_add_layernorm(x, r[:4].contiguous()))
+    assert torch.equal(q8.q8_attention_quant(qkv, 2, 10, 1, s), q8.q8_attention_quant(qkv[:20].contiguous(), 2, 10, 1, s))
+
+
 # ------------------------------------------------------------------ K split over a cluster
 @pytest.mark.parametrize("M,N,K", [(1, 32, 2048), (37, 90, 2064), (128, 768, 3072), (129, 500, 4096), (128, 1184, 2048),
                                    (300, 1000, 2176), (512, 1152, 2048), (16, 33, 16400)])
