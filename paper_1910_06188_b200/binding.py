@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import warnings
 from typing import Optional, Tuple
 
 import torch
@@ -105,16 +106,25 @@ def load() -> C.CDLL:
     return _lib
 
 
+class _PythonForms:
+    """In the place of the native marshalling module: every call takes its Python form."""
+
+    def __getattr__(self, name):
+        return lambda *args: NotImplemented
+
+
 def _native():
-    """The native marshalling module, bound to the loaded library."""
+    """The native marshalling module, bound to the loaded library, or what stands in for it where it cannot be loaded."""
     global _native_module
     if _native_module is None:
         lib = load()
         try:
             from . import _q8_native
         except ImportError as ex:
-            raise RuntimeError("_q8_native.so not found or not loadable: build it first "
-                               "(python -m paper_1910_06188_b200.build)") from ex
+            warnings.warn(f"calls are marshalled in Python, some 8 us slower each: {ex} "
+                          "(python -m paper_1910_06188_b200.build builds the native form)", RuntimeWarning, stacklevel=3)
+            _native_module = _PythonForms()
+            return _native_module
         _q8_native.bind({name: C.cast(getattr(lib, name), C.c_void_p).value for name in _NATIVE_CALLS}, _check)
         _native_module = _q8_native
     return _native_module

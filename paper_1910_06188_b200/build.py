@@ -9,6 +9,7 @@ import os
 import shutil
 import subprocess
 import sys
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -48,10 +49,15 @@ def _native_command() -> list:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile the library and the native marshalling when they are missing or older than any source; returns the
-    library's path."""
+    library's path.  Without a compiler or headers for the native marshalling, which only makes calls cheaper, the library is all."""
     _build_library(force, verbose)
     if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < _newest_source_mtime():
-        subprocess.check_call(_native_command())
+        try:
+            subprocess.check_call(_native_command())
+        except (OSError, subprocess.CalledProcessError) as ex:
+            if os.path.exists(NATIVE):
+                os.remove(NATIVE)  # made from other sources
+            warnings.warn(f"{os.path.basename(NATIVE)} was not built, calls will be marshalled in Python: {ex}", RuntimeWarning)
     return LIB
 
 
