@@ -120,6 +120,8 @@ def _native():
         lib = load()
         try:
             from . import _q8_native
+            if _q8_native.built_for != torch.__version__:  # torch promises nothing about the ABI of another version
+                raise ImportError(f"_q8_native was built for torch {_q8_native.built_for}, this is {torch.__version__}")
         except ImportError as ex:
             warnings.warn(f"calls are marshalled in Python, some 8 us slower each: {ex} "
                           "(python -m paper_1910_06188_b200.build builds the native form)", RuntimeWarning, stacklevel=3)

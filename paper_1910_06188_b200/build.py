@@ -42,16 +42,30 @@ def _native_command() -> list:
     include = [os.path.join(home, "include"), os.path.join(home, "include", "torch", "csrc", "api", "include"),
                os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *("-isystem" + i for i in include),
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DQ8_TORCH_VERSION="{torch.__version__}"', *("-isystem" + i for i in include),
             "-I", os.path.join(ROOT, "include"), os.path.join(CSRC, "q8_python.cpp"), "-o", NATIVE,
             "-L" + os.path.join(home, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
+def _built_for() -> str:
+    """What the native marshalling is compiled against, as q8_python.cpp writes it into the module."""
+    import torch
+
+    return f"q8 native for torch {torch.__version__}, python {sys.version_info.major}.{sys.version_info.minor}\0"
+
+
+def _native_is_current() -> bool:
+    if not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < _newest_source_mtime():
+        return False
+    with open(NATIVE, "rb") as f:
+        return _built_for().encode() in f.read()
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile the library and the native marshalling when they are missing or older than any source; returns the
-    library's path.  Without a compiler or headers for the native marshalling, which only makes calls cheaper, the library is all."""
+    """Compile the library and the native marshalling when they are missing or older than any source (or made for
+    another torch or Python); returns the library's path.  Without a compiler or headers for the native marshalling, which only makes calls cheaper, the library is all."""
     _build_library(force, verbose)
-    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < _newest_source_mtime():
+    if force or not _native_is_current():
         try:
             subprocess.check_call(_native_command())
         except (OSError, subprocess.CalledProcessError) as ex:

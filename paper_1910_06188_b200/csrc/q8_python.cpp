@@ -528,4 +528,18 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_q8_native", nullptr, -1, kMethod
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__q8_native() { return PyModule_Create(&kModule); }
+#define Q8_STRING(x) #x
+#define Q8_VALUE(x) Q8_STRING(x)
+// build.py looks for this in the file, binding.py asks the module: torch's ABI holds for one version
+extern "C" __attribute__((visibility("default"), used)) const char q8_native_built_for[] =
+    "q8 native for torch " Q8_TORCH_VERSION ", python " Q8_VALUE(PY_MAJOR_VERSION) "." Q8_VALUE(PY_MINOR_VERSION);
+
+PyMODINIT_FUNC PyInit__q8_native()
+{
+    PyObject *m = PyModule_Create(&kModule);
+    if (m != nullptr && PyModule_AddStringConstant(m, "built_for", Q8_TORCH_VERSION) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

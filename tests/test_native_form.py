@@ -35,3 +35,11 @@ def test_the_library_is_built_where_the_native_module_cannot_be(monkeypatch, tmp
         monkeypatch.setattr(build, "_native_command", lambda: command)
         with pytest.warns(RuntimeWarning, match="was not built"):
             assert build.build() == build.LIB
+
+
+def test_a_module_for_another_torch_is_rebuilt_and_not_used(no_module_loaded, monkeypatch):
+    assert build._native_is_current()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert not build._native_is_current()
+    with pytest.warns(RuntimeWarning, match="built for torch"):
+        _takes_the_python_form()
