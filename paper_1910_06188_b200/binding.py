@@ -65,6 +65,7 @@ SIGNATURES = {
     "q8_selftest_wait_timeout": (_int, [C.c_uint64, _vp, _vp, _vp]),
     "q8_attention_status_word": (_int, [C.POINTER(C.c_void_p)]),
     "q8_tune_gemm_epilogue_warps": (_int, [_int]),
+    "q8_tune_quantize_grid": (None, [_int]),
     "q8_last_launch_tail_split": (_int, []),
     "q8_last_launch_store_mode": (_int, []),
     "q8_measure_hbm_peak": (_int, [C.c_void_p, C.c_size_t, _int, _int, C.POINTER(C.c_double), C.POINTER(C.c_double),
@@ -688,6 +689,11 @@ def q8_attention_status() -> Tuple[int, int]:
     raw = C.c_uint32(0)
     st = load().q8_poll_status(C.c_void_p(q8_attention_status_word()), C.byref(raw), None)
     return int(st), int(raw.value)
+
+
+def q8_tune_quantize_grid(ctas: int = 0) -> None:
+    """Forces the grid of the cooperative dynamic quantisation for later calls (0 = automatic)."""
+    load().q8_tune_quantize_grid(int(ctas))
 
 
 def q8_tune_gemm_epilogue_warps(warps: int = 0) -> None:

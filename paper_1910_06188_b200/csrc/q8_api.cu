@@ -37,9 +37,13 @@ q8_status quantize_tensor(const float *X, int64_t numel, const float *S_given, i
         return Q8_OK;
     }
     if (S_given == nullptr && quantize_dynamic_grid_supported(X, numel, Xq, Xq_copy)) {
-        Q8_CUDA_TRY(launch_quantize_dynamic_grid(X, numel, S_dyn, status, Xq, Xq_copy, s));
-        li.launches += 1;
-        return Q8_OK;
+        const cudaError_t e = launch_quantize_dynamic_grid(X, numel, S_dyn, status, Xq, Xq_copy, s);
+        if (e != cudaErrorCooperativeLaunchTooLarge) {
+            Q8_CUDA_TRY(e);
+            li.launches += 1;
+            return Q8_OK;
+        }
+        cudaGetLastError();  // not every SM is this process's to use (a partition of the device): the separate passes run anywhere
     }
     if (S_given == nullptr) {
         // The scale word first holds the float bits of the running maximum, then the scale itself.
@@ -537,6 +541,7 @@ q8_status q8_attention_status_word(void **dev_status)
     return *dev_status != nullptr ? Q8_OK : Q8_ERR_CUDA;
 }
 
+void q8_tune_quantize_grid(int ctas) { set_quantize_grid(ctas); }
 void q8_tune_gemm_tail_split(int enable) { set_gemm_tail_split(enable != 0); }
 void q8_tune_gemm_direct_store(int mode) { set_gemm_direct_store(mode); }
 

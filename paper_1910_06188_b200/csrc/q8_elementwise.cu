@@ -585,6 +585,9 @@ bool quantize_dynamic_grid_supported(const float *x, int64_t n, const int8_t *xq
     return n > 0 && n <= kCoopMaxElems && aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy));
 }
 
+static int g_quantize_grid = 0;
+void set_quantize_grid(int ctas) { g_quantize_grid = ctas > 0 ? ctas : 0; }
+
 cudaError_t launch_quantize_dynamic_grid(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq, int8_t *xq_copy,
                                          cudaStream_t s)
 {
@@ -603,7 +606,7 @@ cudaError_t launch_quantize_dynamic_grid(const float *x, int64_t n, float *S_out
     }
     const int64_t want = ((n >> 2) + kCoopThreads * 4 - 1) / (kCoopThreads * 4);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(want < 1 ? 1 : want < resident[dev] ? want : resident[dev]));
+    cfg.gridDim = dim3((unsigned)(g_quantize_grid > 0 ? g_quantize_grid : want < 1 ? 1 : want < resident[dev] ? want : resident[dev]));
     cfg.blockDim = dim3(kCoopThreads);
     cfg.stream = s;
     cudaLaunchAttribute attr;

@@ -85,9 +85,11 @@ cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_ou
                                           int8_t *xq_copy, cudaStream_t s);
 // Larger ones, up to 4 Mi values (16-byte aligned): the same in one cooperative launch.  *S_out also serves as the reduction
 // word; *status (may be NULL) is OR-ed into.
+// cudaErrorCooperativeLaunchTooLarge where the process may not use every SM: nothing was launched then.
 bool quantize_dynamic_grid_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
 cudaError_t launch_quantize_dynamic_grid(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq, int8_t *xq_copy,
                                          cudaStream_t s);
+void set_quantize_grid(int ctas);  // CTAs of the cooperative launch, 0 automatic
 cudaError_t launch_fake_quantize(const float *x, int64_t n, const float *S, float *xhat, cudaStream_t s);
 cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, const float *S_e, int64_t V,
                              int64_t H, float *out, int8_t *rows_q, int32_t *status, cudaStream_t s);

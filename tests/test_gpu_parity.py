@@ -366,6 +366,25 @@ def test_dynamic_quantisation_in_one_or_several_launches(n, peak_at):
     assert zs.item() == 1.0 and not zq.any() and word.item() == (1 << 20) | (1 << q8.Q8_ERR_SCALE)
 
 
+@pytest.mark.parametrize("n", [196612, 1 << 20, (4 << 20) - 1])
+def test_dynamic_quantisation_where_the_cooperative_launch_is_refused(n):
+    """As in a process that may use a part of the SMs only: the separate passes give the same values, and no error stays behind."""
+    x = dev(synth.normal((n,), 1.0, 9050))
+    want, s_want = q8.q8_quantize_activation(x)
+    assert q8.q8_last_launch_info()["launches"] == 1
+    try:  # (an SM holds 2048 threads, eight of its CTAs: nine for each SM are refused before anything is launched)
+        q8.q8_tune_quantize_grid(9 * torch.cuda.get_device_properties(0).multi_processor_count)
+        got, s_got = q8.q8_quantize_activation(x)
+        assert q8.q8_last_launch_info()["launches"] == 3
+        assert torch.equal(got, want) and torch.equal(s_got, s_want)
+        Wq, S_w = q8.q8_quantize_weight(x.view(1, n))
+        assert torch.equal(Wq.view(-1), want) and torch.equal(S_w, s_want)
+    finally:
+        q8.q8_tune_quantize_grid(0)
+    torch.cuda.synchronize()
+    assert torch.equal(q8.q8_quantize_activation(x)[0], want)
+
+
 @pytest.mark.parametrize("M,K", [(1, 13), (3, 65537), (257, 768), (1000, 300), (4096, 1040)])
 def test_dynamic_linear_finds_the_peak_of_every_share(M, K):
     """The partial maxima of the abs-max pass: the scale is that of the largest value, in whichever CTA's share it lies."""
