@@ -16,7 +16,7 @@ extern "C" {
 
 /* Tuning / test hook: force the tile shape of the tcgen05 GEMM for later calls in this process.
  * (block_n, ctas) = (0, 0) restores the automatic choice; otherwise ctas = 1 with block_n in
- * {32, 64, 128, 256} (one SM per 128 x block_n tile) or ctas = 2 with block_n = 256 (a pair of
+ * {32, 64, 128, 192, 256} (one SM per 128 x block_n tile) or ctas = 2 with block_n = 256 (a pair of
  * SMs per 256 x 256 tile).  Results do not depend on the choice.  Not thread-safe. */
 q8_status q8_tune_gemm_tile(int block_n, int ctas);
 

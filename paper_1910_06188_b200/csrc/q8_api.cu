@@ -518,7 +518,7 @@ void q8_last_launch_info(int *gemm_kernel, int *launches, int *block_n, int *gri
 q8_status q8_tune_gemm_tile(int block_n, int ctas)
 {
     const bool automatic = block_n == 0 && ctas == 0;
-    const bool single = ctas == 1 && (block_n == 32 || block_n == 64 || block_n == 128 || block_n == 256);
+    const bool single = ctas == 1 && (block_n == 32 || block_n == 64 || block_n == 128 || block_n == 192 || block_n == 256);
     const bool pair = ctas == 2 && block_n == 256;
     if (!automatic && !single && !pair) return Q8_ERR_ARG;
     set_gemm_tile_override(block_n, ctas);

@@ -557,6 +557,16 @@ def test_split_k_layers_bit_exact(M, N, K, act):
     assert peak.view(torch.float32).item() == Y.abs().max().item()
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 1, 16), (129, 193, 144), (300, 500, 272)])
+def test_192_wide_tiles_can_be_asked_for(M, N, K):
+    try:
+        q8.q8_tune_gemm_tile(192, 1)
+        info = check_linear(synth.activation(M, K, 9450), synth.weight(N, K, 9451), synth.bias(N, 9452), 1)
+    finally:
+        q8.q8_tune_gemm_tile(0, 0)
+    assert (info["gemm_kernel"], info["block_n"], info["ctas"]) == (1, 192, 1)
+
+
 @pytest.mark.parametrize("M,N,K", [(4096, 768, 256), (4000, 700, 144), (2900, 1024, 272)])
 def test_192_wide_tiles_bit_exact(M, N, K):
     X, W, b = synth.activation(M, K, 9400 + N), synth.weight(N, K, 9401), synth.bias(N, 9402)
