@@ -28,8 +28,8 @@
 //   warp 8      issues the MMAs (converged, one elected lane); the rest of its warpgroup is there for setmaxnreg, which gives
 //               the softmax 128 registers a thread and the staging 88, the one split without spills in the loops (120 / 96: 3 % slower, 112 / 104:
 //               8 %; with 96 for all, O was spilled).
-// Where the split parts would not carry what fp32 carries, the row is computed over again in plain fp32 FMAs (plain_row()), by
-// its own thread and for itself alone:
+// Where the split parts would not carry what fp32 carries, the row is computed over again in plain fp32 FMAs, by its own thread
+// (plain_rows_of_warp()):
 //   - largest |q| of the row times largest |k| of a chunk above 2^kScoreExponent.  Up to there a score is off by less than
 //     2^-20 in its exponent of 2 whatever the operands look like (64 products, each operand off by 2^-39 of its largest), and
 //     the reference maximum, a whole number below 2^18, is subtracted without a loss.
@@ -155,7 +155,7 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t at)
     return v;
 }
 
-// Largest magnitude among N float4 (a NaN does not take part; an infinity sends the rows to plain_row()) of each component ...
+// Largest magnitude among N float4 (a NaN does not take part; an infinity sends the rows to plain_rows_of_warp()) of each component ...
 template <int N>
 __device__ __forceinline__ float4 absmax_columns(const float4 (&v)[N])
 {
@@ -218,64 +218,70 @@ struct Tile {
     }
 };
 
-// One query row in plain fp32 FMAs by one thread (see the top of the file): softmax(q K^T / 8) V over all S keys, four at a time, with
-// the running maximum and sum of q8_support.cu's kernel.  q_at(i): shared-memory address of the i-th 16 bytes of q.  Leaves the sum
-// of p v in O, returns the sum of p.
+// The 32 query rows of a warp in plain fp32 FMAs, a thread each (see the top of the file): softmax(q K^T / 8) V over all S keys, one at
+// a time, with the running maximum and sum of q8_support.cu's kernel.  q_at(i): shared-memory address of the i-th 16 bytes of
+// the thread's q.  stage: 16 KB of shared memory for keys on their way, 16 of K and of V at a time through two buffers.  Leaves the
+// sum of p v in O, returns the sum of p.  (With every row of 16 x 512 x 12 heads here: 1.05 ms; keys read from where they lie
+// 3.6 ms; the CUDA-core kernel 0.41 ms.  Four keys at a time took 0.72 ms, but their registers are spilled in the loops of the
+// ordinary path: 64 x 384 x 16 heads 227 -> 231 us.)
 template <typename QAt>
-__device__ __forceinline__ float plain_row(QAt q_at, const float *qkv, int S, int64_t H, uint64_t (&O)[kHeadDim / 2])
+__device__ __forceinline__ float plain_rows_of_warp(QAt q_at, const float *qkv, int S, int64_t H, uint32_t stage, int lane,
+                                                    uint64_t (&O)[kHeadDim / 2])
 {
     uint32_t head, seq;  // read here, so that the caller's loop need not keep them
     asm volatile("mov.u32 %0, %%ctaid.y;\n\tmov.u32 %1, %%ctaid.z;" : "=r"(head), "=r"(seq));
     const int64_t row_pitch = 3 * H;
-    const float *k = qkv + seq * (int64_t)S * row_pitch + head * kHeadDim + H, *v = k + H;
+    const float *k = qkv + seq * (int64_t)S * row_pitch + head * kHeadDim + H + 4 * (lane & 15);
+    constexpr int kKeys = 16;
+    auto fetch = [&](int j0, uint32_t to) {
+#pragma unroll 1
+        for (int i = 0; i < kKeys / 2; ++i) {
+            const int r = 2 * i + (lane >> 4);
+            const bool in = j0 + r < S;  // past the end: zeros
+            const float *src = k + (int64_t)(in ? j0 + r : 0) * row_pitch;
+            const uint32_t at = to + (uint32_t)(r * kRowBytes + 16 * (lane & 15));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at), "l"(src), "r"(in ? 16 : 0) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at + kKeys * kRowBytes), "l"(src + H), "r"(in ? 16 : 0) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     float m = -INFINITY, l = 0.0f;
 #pragma unroll
     for (int j = 0; j < kHeadDim / 2; ++j) O[j] = 0;  // (+0, +0)
+    fetch(0, stage);
 #pragma unroll 1
-    for (int j0 = 0; j0 < S; j0 += 4, k += 4 * row_pitch, v += 4 * row_pitch) {
-        float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 2
-        for (int i = 0; i < kHeadDim / 4; ++i) {
-            const float4 q = ld_shared_f4(q_at(i));
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                if (j0 + a >= S) break;
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(k + a * row_pitch) + i);
-                s[a] = fmaf(q.x * kLog2eOver8, x.x, s[a]);
-                s[a] = fmaf(q.y * kLog2eOver8, x.y, s[a]);
-                s[a] = fmaf(q.z * kLog2eOver8, x.z, s[a]);
-                s[a] = fmaf(q.w * kLog2eOver8, x.w, s[a]);
-            }
+    for (int j = 0; j < S; ++j) {
+        const int r = j & (kKeys - 1), buf = (j / kKeys) & 1;
+        const uint32_t row = stage + (uint32_t)(2 * buf * kKeys * kRowBytes + r * kRowBytes);
+        if (r == 0) {
+            __syncwarp();  // everybody has left the other buffer
+            fetch(j + kKeys, stage + (uint32_t)(2 * (buf ^ 1) * kKeys * kRowBytes));
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
         }
-        float m_new = m;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-            if (j0 + a < S) m_new = fmaxf(m_new, s[a]);
+        float4 dot = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 4
+        for (int i = 0; i < kHeadDim / 4; ++i) {
+            const float4 q = ld_shared_f4(q_at(i)), x = ld_shared_f4(row + 16u * i);  // (a key is at the same address in every lane)
+            dot.x = fmaf(q.x * kLog2eOver8, x.x, dot.x);
+            dot.y = fmaf(q.y * kLog2eOver8, x.y, dot.y);
+            dot.z = fmaf(q.z * kLog2eOver8, x.z, dot.z);
+            dot.w = fmaf(q.w * kLog2eOver8, x.w, dot.w);
+        }
+        const float s = (dot.x + dot.y) + (dot.z + dot.w), m_new = fmaxf(m, s);
         const float ref = m_new == -INFINITY ? 0.0f : m_new;  // (only scores of -inf so far: their p is 0)
-        const float corr = exp2f(m - ref);
-        l *= corr;
-        uint64_t p2[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const float p = j0 + a < S ? exp2f(s[a] - ref) : 0.0f;
-            l += p;
-            p2[a] = pack_f32x2(p, p);
-        }
+        const float corr = exp2f(m - ref), p = exp2f(s - ref);
+        l = fmaf(l, corr, p);
         m = m_new;
-        const uint64_t corr2 = pack_f32x2(corr, corr);
+        const uint64_t p2 = pack_f32x2(p, p), corr2 = pack_f32x2(corr, corr);
 #pragma unroll
         for (int i = 0; i < kHeadDim / 4; ++i) {
-            O[2 * i] = mul_f32x2(O[2 * i], corr2);
-            O[2 * i + 1] = mul_f32x2(O[2 * i + 1], corr2);
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                if (j0 + a >= S) break;
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(v + a * row_pitch) + i);
-                O[2 * i] = fma_f32x2(pack_f32x2(x.x, x.y), p2[a], O[2 * i]);
-                O[2 * i + 1] = fma_f32x2(pack_f32x2(x.z, x.w), p2[a], O[2 * i + 1]);
-            }
+            const float4 x = ld_shared_f4(row + (uint32_t)(kKeys * kRowBytes + 16 * i));
+            O[2 * i] = fma_f32x2(pack_f32x2(x.x, x.y), p2, mul_f32x2(O[2 * i], corr2));
+            O[2 * i + 1] = fma_f32x2(pack_f32x2(x.z, x.w), p2, mul_f32x2(O[2 * i + 1], corr2));
         }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     return l;
 }
 
@@ -604,7 +610,7 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             if (!wait(s_done(buf), par)) break;
             if (warp_live) {
                 const int g = gq + k_exponent[c & 3];
-                if (g + 28 > kScoreExponent) l = NAN;  // (largest |q| |k| may reach 2^(g + 28): the row goes to plain_row())
+                if (g + 28 > kScoreExponent) l = NAN;  // (largest |q| |k| may reach 2^(g + 28): the row goes to plain_rows_of_warp())
                 const float f = pow2(max(-126, min(120, g))) * kLog2eOver8;
                 // half 1 of the scores is read twice (for the maximum, then for the exponentials), half 0 stays in registers
                 uint32_t sv[32];
@@ -707,8 +713,24 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
             }
             const bool plain = (v_far != 0 || !(top * inv >= kSmallResult)) && q0 + 32 * warp + lane < S;
             const uint32_t plain_rows = __ballot_sync(0xffffffffu, plain);
-            if (plain) inv = 1.0f / plain_row([&](int i) { return piece(lane, i); }, qkv, S, H, O);
-            __syncwarp();
+            if (__builtin_expect(plain_rows != 0, 0)) {
+                // K and V have been read by every product; each warp has a quarter of their buffers.  The whole warp fetches the keys;
+                // a thread whose row is done puts it aside, where its q was, and computes something of no use.
+                auto row = [&](int i) { return piece(lane, i); };
+                if (!plain) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(row(i)), "l"(O[2 * i]), "l"(O[2 * i + 1]) : "memory");
+                }
+                const float sum = plain_rows_of_warp(row, qkv, S, H, smem + (uint32_t)(warp * kKvBytes), lane, O);
+                if (plain) {
+                    inv = 1.0f / sum;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(O[2 * i]), "=l"(O[2 * i + 1]) : "r"(row(i)) : "memory");
+                }
+            }
             const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
