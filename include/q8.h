@@ -244,7 +244,7 @@ const char *q8_status_string(q8_status s);
 
 /* What the most recent call on this host thread enqueued: which GEMM kernel it chose (0 none,
  * 1 tcgen05, 2 generic), how many kernels it launched, the tile width, the grid size and how many
- * CTAs share one tile (2 = cta_group::2 pairs).  Host-side bookkeeping for benchmarks and tests;
+ * CTAs share one tile (2 with 256-wide tiles = cta_group::2 pairs; 2 or 4 with narrower ones = K split over a cluster).  Host-side bookkeeping for benchmarks and tests;
  * any pointer may be NULL. */
 void q8_last_launch_info(int *gemm_kernel, int *launches, int *block_n, int *grid, int *ctas);
 

@@ -253,7 +253,7 @@ cudaError_t launch_out(const GemmArgs &a, cudaStream_t s)
     LaunchInfo &li = last_launch_info();
     li.gemm_kernel = 1;
     li.block_n = BN;
-    li.ctas = 1;
+    li.ctas = KS;
     li.epilogue_warps = 4;
     li.grid = (int)(tiles * KS);
     li.tail_split = 1;

@@ -51,7 +51,7 @@ struct LaunchInfo {
     int gemm_kernel = 0;  // 0 none, 1 tcgen05, 2 generic
     int launches = 0;
     int block_n = 0;
-    int ctas = 0;  // CTAs cooperating on one tile (1, or 2 for cta_group::2)
+    int ctas = 0;  // CTAs cooperating on one tile (1, 2 for cta_group::2, 2 or 4 with K split over a cluster)
     int epilogue_warps = 0;
     int grid = 0;
     int tail_split = 1;  // tiles of the last scheduling round cut into this many narrower ones

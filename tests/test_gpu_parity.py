@@ -557,6 +557,15 @@ def test_split_k_layers_bit_exact(M, N, K, act):
     assert peak.view(torch.float32).item() == Y.abs().max().item()
 
 
+@pytest.mark.parametrize("M,N,K,block_n,ctas", [(1, 32, 2048, 32, 4), (300, 1000, 2176, 64, 2)])
+def test_split_k_reports_the_ctas_of_a_tile(M, N, K, block_n, ctas):
+    Xq, Wq = (torch.ones((n, K), dtype=torch.int8, device="cuda") for n in (M, N))
+    one = torch.ones(1, device="cuda")
+    q8.q8_linear_q(Xq, one, Wq, one)
+    info = q8.q8_last_launch_info()
+    assert (info["block_n"], info["ctas"]) == (block_n, ctas)
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 1, 16), (129, 193, 144), (300, 500, 272)])
 def test_192_wide_tiles_can_be_asked_for(M, N, K):
     try:
