@@ -75,8 +75,8 @@ class Q8BertEncoder:
         if self._bufs is None or self._bufs["T"] != T:
             d, f32 = self.device, torch.float32
             e = lambda n: torch.empty((T, n), dtype=f32, device=d)
-            self._bufs = dict(T=T, ew=e(self.H), ep=e(self.H), et=e(self.H), h=e(self.H), qkv=e(3 * self.H),
-                              ctx=e(self.H), ao=e(self.H), h1=e(self.H), f=e(self.F), f2=e(self.H),
+            self._bufs = dict(T=T, h=e(self.H), qkv=e(3 * self.H), ctx=e(self.H), ao=e(self.H), h1=e(self.H),
+                              f=e(self.F), f2=e(self.H),
                               ws=q8.new_workspace(T, self.F, max(self.H, self.F), d),
                               status=torch.zeros(1, dtype=torch.int32, device=d))
         return self._bufs
@@ -94,6 +94,8 @@ class Q8BertEncoder:
     def _embed(self, ids: torch.Tensor, B: int, S: int) -> None:
         """The three table look-ups of B sequences of S tokens, each into its own fp32 buffer."""
         bf = self._bufs
+        if "ew" not in bf:
+            bf.update((name, torch.empty_like(bf["h"])) for name in ("ew", "ep", "et"))
         pos_ids = torch.arange(S, dtype=torch.int32, device=self.device).repeat(B)
         typ_ids = torch.zeros(B * S, dtype=torch.int32, device=self.device)
         q8.q8_embedding(ids, self.word, self.S_word, out=bf["ew"], dev_status=bf["status"])

@@ -247,6 +247,17 @@ def test_fused_forward_is_bit_identical_to_the_unfused_one():
         assert torch.equal(replayed, enc.forward(ids, B, S, scales="static"))
 
 
+def test_forwards_of_one_input_pass_hold_no_buffers_for_the_three_tables():
+    dims = dict(hidden=128, ffn=512, heads=2, layers=1, vocab=500, max_pos=96)
+    enc = enc_mod.Q8BertEncoder(dims, config=32)
+    ids = enc_mod.random_ids(2 * 40, dims["vocab"], 32)
+    want = enc.forward(ids, 2, 40, scales="dynamic").clone()
+    tables = {name for name, t in enc._bufs.items() if name in ("ew", "ep", "et") and t.shape == (80, 128)}
+    enc._bufs = None
+    assert torch.equal(enc.forward_dynamic_fused(ids, 2, 40), want)
+    assert tables == {"ew", "ep", "et"} and not tables & set(enc._bufs)
+
+
 # ------------------------------------------------------------------ dynamic quantisation with fused abs-max (Sec. 4.1)
 def _word():
     return torch.zeros(1, dtype=torch.int32, device="cuda")
