@@ -220,6 +220,7 @@ class Q8BertEncoder:
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph):
             out = run()
+        graph.buffers = self._bufs  # what it reads and writes, also after a forward of another size has replaced the buffers
         return graph, out
 
     def launches_per_forward(self, scales: str = "static", fused: bool = False) -> int:

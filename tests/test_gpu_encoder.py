@@ -258,6 +258,22 @@ def test_forwards_of_one_input_pass_hold_no_buffers_for_the_three_tables():
     assert tables == {"ew", "ep", "et"} and not tables & set(enc._bufs)
 
 
+def test_a_captured_forward_keeps_its_buffers():
+    """Forwards of other sizes replace the encoder's buffers; the graph's own stay allocated, so nothing else is written over."""
+    dims = dict(hidden=128, ffn=512, heads=2, layers=1, vocab=500, max_pos=96)
+    enc = enc_mod.Q8BertEncoder(dims, config=33)
+    ids, other = enc_mod.random_ids(80, dims["vocab"], 33), enc_mod.random_ids(60, dims["vocab"], 34)
+    enc.forward(ids, 2, 40, scales="calibrate")
+    graph, out = enc.capture(ids, 2, 40)
+    graph.replay()
+    want, held = out.clone(), {t.data_ptr() for t in enc._bufs.values() if isinstance(t, torch.Tensor)}
+    enc.forward_fused(other, 2, 30)
+    fresh = [torch.zeros(80, 512, device="cuda") for _ in range(64)]  # (what was given back would be handed out again here)
+    assert not held & {t.data_ptr() for t in fresh}
+    graph.replay()
+    assert torch.equal(out, want) and not any(t.any() for t in fresh)
+
+
 # ------------------------------------------------------------------ dynamic quantisation with fused abs-max (Sec. 4.1)
 def _word():
     return torch.zeros(1, dtype=torch.int32, device="cuda")
