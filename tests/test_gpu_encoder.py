@@ -45,8 +45,8 @@ def test_attention(B, S, heads):
 
 @pytest.mark.parametrize("B,S,heads", [(2, 100, 2), (1, 384, 2), (1, 448, 1), (1, 500, 1)])
 def test_attention_tensor_core_and_cuda_core_kernels_both_match_the_oracle(B, S, heads):
-    """S <= 448 runs on the tensor cores (split TF32 products), longer sequences and q8_tune_attention(0)
-    on the CUDA-core kernel; both must meet the fp32 tolerance."""
+    """Small grids: up to 384 keys on split TF32 products, more on split fp16; with q8_tune_attention(0) the CUDA-core kernel.
+    All must meet the fp32 tolerance."""
     qkv = synth.normal((B * S, 3 * heads * 64), 1.0, 3150 + S)
     ref = o.attention(qkv, B, S, heads)
     try:
@@ -59,9 +59,10 @@ def test_attention_tensor_core_and_cuda_core_kernels_both_match_the_oracle(B, S,
         q8.q8_tune_attention(True)
 
 
-def test_attention_large_logits_stay_finite():
-    B, S, heads = 1, 130, 1
-    qkv = synth.normal((B * S, 3 * 64), 6.0, 3150)             # logits of several hundred
+@pytest.mark.parametrize("B,heads", [(1, 1), (30, 3)])          # the kernel for small grids, and the one for grids that fill the device
+def test_attention_large_logits_stay_finite(B, heads):
+    S = 130
+    qkv = synth.normal((B * S, 3 * heads * 64), 6.0, 3150)     # logits of several hundred
     got = q8.q8_attention(dev(qkv), B, S, heads).cpu().numpy()
     assert np.isfinite(got).all()
     # fp32 logits of magnitude ~500 carry an absolute rounding error of ~500 * 2^-24 = 3e-5, which the
@@ -369,12 +370,22 @@ EDGE_TOL = 2e-6
 FULL = 150  # sequences of one head that make more CTAs than there are SMs: the kernel for grids that fill the device
 
 
+def _many(seed, B, S, heads, sigma=1.0):
+    """Different sequences of several heads, more CTAs than SMs: (qkv, its parts as views [B, S, (q, k, v), heads, 64])."""
+    assert B * heads * ((S + 127) // 128) > torch.cuda.get_device_properties(0).multi_processor_count
+    qkv = synth.normal((B * S, 3 * heads * 64), sigma, seed)
+    return qkv, qkv.reshape(B, S, 3, heads, 64)
+
+
 def _attention_errors(qkv, S):
-    """FULL copies of one sequence of one head: (error of the first, error of the last) against the oracle."""
-    got = q8.q8_attention(dev(np.tile(qkv, (FULL, 1))), FULL, S, 1).cpu().numpy()
+    """A sequence of one head as the first one, and as the last of the last head, among many others: errors of both."""
+    B, heads = 50, 3
+    many, parts = _many(3290 + S, B, S, heads)
+    parts[0, :, :, 0] = parts[-1, :, :, -1] = qkv.reshape(S, 3, 64)
+    got = q8.q8_attention(dev(many), B, S, heads).cpu().numpy()
     assert q8.q8_attention_status() == (q8.Q8_OK, 0)
     ref = o.attention(qkv, 1, S, 1)
-    return [np.abs(x - ref).max() / np.abs(ref).max() for x in (got[:S], got[-S:])]
+    return [np.abs(x - ref).max() / np.abs(ref).max() for x in (got[:S, :64], got[-S:, -64:])]
 
 
 @pytest.mark.parametrize("S", [1, 31, 33, 63, 65, 95, 97, 127, 129, 193, 385, 512, 513])
@@ -384,8 +395,8 @@ def test_attention_at_chunk_and_tile_edges(S):
 
 @pytest.mark.parametrize("S", [100, 200])
 def test_attention_scales_of_its_operands(S):
-    """Powers of two moved between Q and K, and between the chunks of V, leave the accuracy as it is: every operand tile is
-    brought into fp16's range by a scale of its own.  A maximum that rises from chunk to chunk rescales what is summed."""
+    """Powers of two moved between the whole of Q and of K, and between the chunks of V, leave the accuracy as it is.  A maximum that
+    rises from chunk to chunk rescales what is summed.  (Ranges within an operand: the tests below.)"""
     qkv = synth.normal((S, 3 * 64), 1.0, 3400 + S)
     moved = qkv.copy()
     moved[:, :64] *= 2.0 ** 40
@@ -413,13 +424,6 @@ def test_attention_non_finite_rows_stay_in_their_rows():
     rows, features = np.delete(np.arange(S), [70, 71]), np.delete(np.arange(64), 5)
     assert np.isnan(got[70]).all() and np.isnan(got[71]).all() and not np.isfinite(got[:, 5]).any()
     assert np.abs(got[np.ix_(rows, features)] - ref[np.ix_(rows, features)]).max() <= EDGE_TOL * np.abs(ref).max()
-
-
-def _many(seed, B, S, heads, sigma=1.0):
-    """Different sequences of several heads, more CTAs than SMs: (qkv, its parts as views [B, S, (q, k, v), heads, 64])."""
-    assert B * heads * ((S + 127) // 128) > torch.cuda.get_device_properties(0).multi_processor_count
-    qkv = synth.normal((B * S, 3 * heads * 64), sigma, seed)
-    return qkv, qkv.reshape(B, S, 3, heads, 64)
 
 
 @pytest.mark.parametrize("power", [10, 16, 24, 40])
