@@ -14,16 +14,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-int sm_count()
-{
-    static int n = [] {
-        int dev = 0, v = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        return v > 0 ? v : 148;
-    }();
-    return n;
-}
-
 int grid_for(int64_t work_items, int items_per_block, int blocks_per_sm)
 {
     int64_t want = (work_items + items_per_block - 1) / items_per_block;

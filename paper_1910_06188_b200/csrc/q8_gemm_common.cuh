@@ -398,15 +398,5 @@ inline bool make_tmap_out_q(CUtensorMap *map, int8_t *base, int64_t M, int64_t N
     });
 }
 
-inline int sm_count()
-{
-    static int n = [] {
-        int dev = 0, v = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        return v > 0 ? v : 148;
-    }();
-    return n;
-}
-
 }  // namespace gemm_detail
 }  // namespace q8

@@ -234,7 +234,7 @@ cudaError_t launch_gemm_generic(const GemmArgs &a, cudaStream_t s)
     // 1500 x 1004 -> 1500, 144 tiles: 32 / 31 us, both before a common gain; rows that start at any byte, whose loads go through registers, never gain:
     // 4000 x 1001 -> 2000 270 / 163 us), and where 64-wide tiles would be too many for a grid
     const int64_t big_tiles = ((a.M + 127) / 128) * ((a.N + 127) / 128);
-    if ((big_tiles >= 148 && any % 4 == 0) || a.N > 64 * 65535ll) {
+    if ((big_tiles >= sm_count() && any % 4 == 0) || a.N > 64 * 65535ll) {
         if (any % 8 == 0) return launch_shape<128, 8>(a, s);
         return any % 4 == 0 ? launch_shape<128, 4>(a, s) : launch_shape<128, 1>(a, s);
     }

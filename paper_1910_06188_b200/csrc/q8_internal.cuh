@@ -59,6 +59,16 @@ struct LaunchInfo {
 };
 LaunchInfo &last_launch_info();
 
+inline int sm_count()
+{
+    static int n = [] {
+        int dev = 0, v = 148;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 148;
+    }();
+    return n;
+}
+
 // ---- elementwise / reduction launchers (q8_elementwise.cu) ----
 // max|x| folded into *bits (must hold 0 or an earlier maximum) with atomicMax on the float bits.  With st the Eq. 4 update
 // of that state follows in the same launch and *bits is zero again afterwards.
