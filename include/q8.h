@@ -77,7 +77,9 @@ q8_status q8_quantize_activation(const float *X, int64_t numel, const float *S_x
 
 /* Eq. 4: one calibration batch.  `state` is a q8_calibrate_state_bytes()-byte, 16-byte aligned,
  * zero-initialised device block laid out as
- *   { float ema; float S_x; int32 n_batches; uint32 scratch; int32 status; int32 pad[3]; }
+ *   { float ema; float S_x; int32 n_batches; uint32 scratch; int32 status; uint32 counter; int32 pad[2]; }
+ * scratch and counter are the kernel's own: zero between calls, and to be zero in a block that a caller fills in itself
+ * (a saved state restored field by field).  Calls on one state must be ordered on the stream.
  * The first batch sets ema = max|X|; later ones do ema += (1 - decay) * (max|X| - ema) in fp32;
  * then S_x = 127 / ema.  decay must lie in [0, 1); decay 0 keeps no history: ema is exactly this batch's
  * max|X| and S_x exactly the dynamic scale of Sec. 4.1.  A batch with numel == 0 carries no observation and
@@ -122,7 +124,7 @@ q8_status q8_linear_q(const int8_t *Xq, const float *S_x, const int8_t *Wq, cons
                       const float *bias, int act, float *Y, int64_t M, int64_t N, int64_t K,
                       int32_t *dbg_acc, int32_t *dev_status, void *stream);
 
-/* q8_linear / q8_linear_q forced onto the generic (any shape, any alignment, CUDA-core) GEMM
+/* q8_linear / q8_linear_q forced onto the generic (any shape, any alignment, mma.sync) GEMM
  * kernel that q8_linear uses by itself when K % 16 != 0 or an operand is not 16-byte aligned.
  * Same arguments, same results; kept public as an on-device cross-check of the tensor-core kernel. */
 q8_status q8_linear_generic(const float *X, const int8_t *Wq, const float *S_w, const float *S_x,

@@ -114,15 +114,16 @@ __device__ __forceinline__ void umma_i8(uint32_t tmem_d, uint64_t desc_a, uint64
         ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]^T with TF32 operands (the upper 19 bits of each fp32 word) and fp32 accumulation.
-// For a converged warp: every lane executes the call with identical operands and one elected lane issues.  Keeping the issuing warp converged lets the compiler hold descriptors and addresses in uniform
-// registers instead of moving them there for every instruction.  `elected` comes from elect_one().
+// One lane of a converged warp.  The *_elected calls below are executed by every lane with identical operands and issued by that
+// one: keeping the issuing warp converged lets the compiler hold descriptors and addresses in uniform registers instead of
+// moving them there for every instruction.
 __device__ __forceinline__ uint32_t elect_one()
 {
     uint32_t e;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
     return e;
 }
+// D[tmem] (+)= A[smem] * B[smem]^T with TF32 operands (the upper 19 bits of each fp32 word) and fp32 accumulation.
 __device__ __forceinline__ void umma_tf32_elected(uint32_t elected, uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b,
                                                   uint32_t idesc, uint32_t accumulate)
 {
