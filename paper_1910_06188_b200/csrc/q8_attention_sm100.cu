@@ -36,7 +36,7 @@
 //   - a row whose result is small beside V in every feature (kSmallResult): it hangs on keys whose V is tiny beside that of
 //     others, and what those are rounded by counts.
 //   - infinities.
-// Measured (64 x 384 x 16 heads / 16 x 512 x 12 / 32 x 128 x 12, Int8 output): 227 / 72 / 19.9 us; split TF32 with whole score
+// Measured (64 x 384 x 16 heads / 16 x 512 x 12 / 32 x 128 x 12, Int8 output): 227 / 72 / 20 us; split TF32 with whole score
 // rows in TMEM, one CTA per SM, 512 threads staging: 304 / - / 23.8 us (it takes S <= 384; plain fp32 FMAs needed 413 us at
 // 512).  What bounds it now is latency: loads of K and V (without them 25 % less) and the chain softmax -> P V -> scores
 // between the roles, with the issue slots 40 % busy and the tensor pipe 20 %.  Tried and dropped: a persistent grid (the
