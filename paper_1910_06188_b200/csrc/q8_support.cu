@@ -15,12 +15,16 @@ namespace {
 // One CTA per row.  The summed row is kept in shared memory, so the inputs are read once; mean and
 // variance are the two-pass forms (sum, then sum of squared deviations), reduced through warp shuffles.
 constexpr int kLnThreads = 256;
-// CTAs per SM of the warp-per-row kernel.  Two, with registers for all loads of a row and of its residual at once (with four CTAs
+// The warp-per-row kernel has registers for a row and its residual, all loads of both in flight at once, of up to 256, 512, 768 or 1024
+// values, and four CTAs per SM where these leave room for them (H <= 512), else two.  (One form of 1024 values and two CTAs for every
+// H, four of 64 registers in sequence before it, us: 65536 x 64 27.8 / 38.0 / 17.2 now, 32768 x 128 15.0 / 20.3 / 9.7, 16384 x 256 10.6 /
+// 12.3 / 7.3, 8192 x 512 8.1 / 9.0 / 7.3, 4096 x 768 6.0 / 6.5 / 6.0, 24576 x 768 44.9 / 36.9 / 36.4; three CTAs up to 768: 1421 x 768 4.4
+// for 4.0; six up to 256: 65536 x 64 19.2.)
+// Of the two-CTA forms: two, with registers for all loads of a row and of its residual at once (with four CTAs
 // of 64 registers the loads of the two come one after the other: 128 x 768 3.85 -> 3.10 us, 1421 x 768 5.05 -> 4.10, 24576 x 1024
 // with Int8 copy 61.9 -> 54.0 us = 6.05 TB/s; three CTAs spill: 57.4).  Also where four would take all rows in one round and two
 // need a second one: 4096 x 768 10.2 -> 9.3.  (Whole static forwards of 32 x 128 and 16 x 512 tokens are 0.6 % slower with it all the
 // same, 516 -> 520 and 739 -> 743 us; 1 x 128 is 7 %, 7 x 203 6 %, BERT-Large 64 x 384 2.5 % faster.)
-constexpr int kLnCtasPerSm = 2;
 constexpr int kEmbedLnCtasPerSm = 4;  // the one-pass input kernel: Int8 rows, fewer registers
 
 __device__ __forceinline__ float block_sum(float v, float *scratch)
@@ -136,9 +140,10 @@ __global__ void __launch_bounds__(kLnThreads) add_layernorm_vec_kernel(const flo
     if (amax) warp_fold_absmax(am, amax);
 }
 
-// The row of one warp, H <= 1024: v[i] holds the values 4 (lane + 32 i) .. + 3 of the summed row and s this lane's share of
+// The row of one warp, H <= 128 NV: v[i] holds the values 4 (lane + 32 i) .. + 3 of the summed row and s this lane's share of
 // their sum.  Both moments are reduced with shuffles only, so there is no block-level barrier at all.
-__device__ __forceinline__ void normalise_row(const float4 (&v)[8], float s, int lane, int n4, int64_t H, float eps,
+template <int NV>
+__device__ __forceinline__ void normalise_row(const float4 (&v)[NV], float s, int lane, int n4, int64_t H, float eps,
                                               const float *__restrict__ gamma, const float *__restrict__ beta, float4 *out4,
                                               uint32_t *q4, float Sq, float &am)
 {
@@ -147,7 +152,7 @@ __device__ __forceinline__ void normalise_row(const float4 (&v)[8], float s, int
     const float mean = s / (float)H;
     float q = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < NV; ++i)
         if (lane + 32 * i < n4) {
             const float dx = v[i].x - mean, dy = v[i].y - mean, dz = v[i].z - mean, dw = v[i].w - mean;
             q += (dx * dx + dy * dy) + (dz * dz + dw * dw);
@@ -156,7 +161,7 @@ __device__ __forceinline__ void normalise_row(const float4 (&v)[8], float s, int
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     const float rstd = 1.0f / sqrtf(q / (float)H + eps);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < NV; ++i) {
         const int c = lane + 32 * i;
         if (c >= n4) continue;
         const float4 g = gamma ? __ldg(reinterpret_cast<const float4 *>(gamma) + c) : make_float4(1.f, 1.f, 1.f, 1.f);
@@ -172,8 +177,9 @@ __device__ __forceinline__ void normalise_row(const float4 (&v)[8], float s, int
     }
 }
 
-// One warp per row for H <= 1024 (BERT's hidden sizes): up to eight float4 per lane, eight rows per CTA.
-__global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_kernel(const float *__restrict__ x,
+// One warp per row for H <= 1024 (BERT's hidden sizes): NV float4 per lane (H <= 128 NV), eight rows per CTA.
+template <int NV, int CTAS_PER_SM>
+__global__ void __launch_bounds__(kLnThreads, CTAS_PER_SM) add_layernorm_warp_kernel(const float *__restrict__ x,
                                                                         const float *__restrict__ r1,
                                                                         const float *__restrict__ r2,
                                                                         const float *__restrict__ gamma,
@@ -195,16 +201,16 @@ __global__ void __launch_bounds__(kLnThreads, kLnCtasPerSm) add_layernorm_warp_k
         const float4 *x4 = reinterpret_cast<const float4 *>(x) + base4;
         const float4 *a4 = r1 ? reinterpret_cast<const float4 *>(r1) + base4 : nullptr;
         const float4 *b4 = r2 ? reinterpret_cast<const float4 *>(r2) + base4 : nullptr;
-        float4 v[8], r[8];
+        float4 v[NV], r[NV];
         float s = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = lane + 32 * i < n4 ? __ldg(x4 + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < NV; ++i) v[i] = lane + 32 * i < n4 ? __ldg(x4 + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
         if (a4) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = lane + 32 * i < n4 ? __ldg(a4 + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int i = 0; i < NV; ++i) r[i] = lane + 32 * i < n4 ? __ldg(a4 + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < NV; ++i) {
             const int c = lane + 32 * i;
             if (c < n4) {
                 if (a4) { v[i].x += r[i].x; v[i].y += r[i].y; v[i].z += r[i].z; v[i].w += r[i].w; }
@@ -440,10 +446,15 @@ cudaError_t launch_add_layernorm(const float *x, const float *r1, const float *r
         const int64_t want = (rows + kLnThreads / 32 - 1) / (kLnThreads / 32);
         int dev = 0, sms = 148;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int64_t cap = (int64_t)(sms > 0 ? sms : 148) * kLnCtasPerSm;
-        const unsigned blocks = (unsigned)(want < cap ? want : cap);
-        return launch_overlapping_tail(add_layernorm_warp_kernel, dim3(blocks), dim3(kLnThreads), 0, s, x, r1, r2, gamma, beta,
-                                       eps, rows, H, out, S_q, out_q, amax);
+        auto launch = [&](auto kernel, int ctas_per_sm) {
+            const int64_t cap = (int64_t)(sms > 0 ? sms : 148) * ctas_per_sm;
+            return launch_overlapping_tail(kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kLnThreads), 0, s, x, r1, r2, gamma,
+                                           beta, eps, rows, H, out, S_q, out_q, amax);
+        };
+        if (H <= 256) return launch(add_layernorm_warp_kernel<2, 4>, 4);
+        if (H <= 512) return launch(add_layernorm_warp_kernel<4, 4>, 4);
+        if (H <= 768) return launch(add_layernorm_warp_kernel<6, 2>, 2);
+        return launch(add_layernorm_warp_kernel<8, 2>, 2);
     } else if (vec) {
         add_layernorm_vec_kernel<<<(unsigned)rows, kLnThreads, 0, s>>>(x, r1, r2, gamma, beta, eps, H, out, S_q, out_q, amax);
     } else {
