@@ -233,8 +233,10 @@ cudaError_t launch_gemm_generic(const GemmArgs &a, cudaStream_t s)
     // the large tile once its grid fills the device (2000 x 1004 -> 2000, 256 tiles: 35 against 46 us with the small one,
     // 1500 x 1004 -> 1500, 144 tiles: 32 / 31 us, both before a common gain; rows that start at any byte, whose loads go through registers, never gain:
     // 4000 x 1001 -> 2000 270 / 163 us), and where 64-wide tiles would be too many for a grid
+    // Not for N <= 128, one column of large tiles, where its few wide CTAs leave the loads of X_q waiting: 40000 x 100 -> 4 34.0 us, 9.4 with
+    // the small tile, -> 128 35.1 / 15.1, 125829 x 1004 -> 100 140 / 123 (but -> 65 111 / 125).
     const int64_t big_tiles = ((a.M + 127) / 128) * ((a.N + 127) / 128);
-    if ((big_tiles >= sm_count() && any % 4 == 0) || a.N > 64 * 65535ll) {
+    if ((a.N > 128 && big_tiles >= sm_count() && any % 4 == 0) || a.N > 64 * 65535ll) {
         if (any % 8 == 0) return launch_shape<128, 8>(a, s);
         return any % 4 == 0 ? launch_shape<128, 4>(a, s) : launch_shape<128, 1>(a, s);
     }

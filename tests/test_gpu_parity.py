@@ -385,7 +385,7 @@ def test_dynamic_quantisation_where_the_cooperative_launch_is_refused(n):
     assert torch.equal(q8.q8_quantize_activation(x)[0], want)
 
 
-@pytest.mark.parametrize("M,K", [(1, 13), (3, 65537), (257, 768), (1000, 300), (4096, 1040)])
+@pytest.mark.parametrize("M,K", [(1, 13), (3, 65537), (257, 768), (1000, 300), (4096, 1040), (8192, 1024), (8192, 1040)])
 def test_dynamic_linear_finds_the_peak_of_every_share(M, K):
     """The partial maxima of the abs-max pass: the scale is that of the largest value, in whichever CTA's share it lies."""
     W = synth.weight(16, K, 9100)
@@ -423,6 +423,18 @@ def test_generic_gemm_pieces_and_tile_edges(M, N, K):
     acc = torch.empty((M, N), dtype=torch.int32, device="cuda")
     q8.q8_linear_q(dev(Xq), torch.ones(1, device="cuda"), dev(Wq), torch.ones(1, device="cuda"), None, 0, dbg_acc=acc)
     assert q8.q8_last_launch_info()["gemm_kernel"] == 2
+    assert np.array_equal(acc.cpu().numpy(), Xq.astype(np.int32) @ Wq.astype(np.int32).T)
+
+
+@pytest.mark.parametrize("N,tile", [(1, 64), (64, 64), (65, 64), (128, 64), (129, 128)])
+def test_generic_gemm_tall_and_narrow(N, tile):
+    M, K = 20003, 20
+    rng = np.random.default_rng(N)
+    Xq, Wq = (rng.integers(-127, 128, size=(n, K), dtype=np.int8) for n in (M, N))
+    acc = torch.empty((M, N), dtype=torch.int32, device="cuda")
+    q8.q8_linear_q(dev(Xq), torch.ones(1, device="cuda"), dev(Wq), torch.ones(1, device="cuda"), None, 0, dbg_acc=acc)
+    info = q8.q8_last_launch_info()
+    assert (info["gemm_kernel"], info["block_n"]) == (2, tile)
     assert np.array_equal(acc.cpu().numpy(), Xq.astype(np.int32) @ Wq.astype(np.int32).T)
 
 
