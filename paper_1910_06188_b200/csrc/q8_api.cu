@@ -120,9 +120,14 @@ q8_status linear_impl(const float *X, const int8_t *Wq, const float *S_w, const 
         Q8_CUDA_TRY(launch_quantize_dynamic_small(X, M * K, &hdr->S_x_dyn, &hdr->status, true, Xq, dbg_Xq, s));
         last_launch_info().launches += 1;
     } else {
-        int words = 0;
-        Q8_CUDA_TRY(launch_absmax_partial(X, M * K, hdr->absmax_partial,
-                                          (int)(sizeof(hdr->absmax_partial) / sizeof(hdr->absmax_partial[0])), &words, s));
+        int words = 1;
+        if (absmax_partial_preferred(M * K)) {
+            Q8_CUDA_TRY(launch_absmax_partial(X, M * K, hdr->absmax_partial,
+                                              (int)(sizeof(hdr->absmax_partial) / sizeof(hdr->absmax_partial[0])), &words, s));
+        } else {
+            Q8_CUDA_TRY(cudaMemsetAsync(hdr->absmax_partial, 0, sizeof(hdr->absmax_partial[0]), s));
+            Q8_CUDA_TRY(launch_absmax(X, M * K, hdr->absmax_partial, s));
+        }
         Q8_CUDA_TRY(launch_quantize_dynamic(X, M * K, hdr->absmax_partial, &hdr->S_x_dyn, &hdr->status, Xq, dbg_Xq, s, true, words));
         last_launch_info().launches += 2;
     }

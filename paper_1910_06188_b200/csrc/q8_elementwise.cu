@@ -548,6 +548,11 @@ cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_
                                    st, decay);
 }
 
+// Two CTAs per SM read less at a time than the eight of absmax_kernel: a dynamic layer of 1024 columns with changing inputs, partial
+// maxima / clear and atomics, us: 2.1 M values 11.2 / 13.0, 4.2 M 16.0 / 16.9, 6.3 M 18.8 / 19.1, 9.4 M 23.6 / 23.1, 12.6 M 29.3 / 25.3,
+// 52 M 113 / 97.  (CTAs of 1024 threads in the clusters do not help: 29.6 at 12.6 M.)
+bool absmax_partial_preferred(int64_t n) { return n <= (int64_t(8) << 20); }
+
 cudaError_t launch_absmax_partial(const float *x, int64_t n, uint32_t *partial, int max_words, int *words, cudaStream_t s)
 {
     const bool vec = aligned16(x);
