@@ -25,6 +25,15 @@ inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
         if (e__ != cudaSuccess) return Q8_ERR_CUDA; \
     } while (0)
 
+// A launch that is refused (see below) while its stream is captured would end the capture.
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // Eq. 1 with either a given scale or the dynamic one of Eq. 3 / Sec. 4.1 (scratch == output scale word).
 q8_status quantize_tensor(const float *X, int64_t numel, const float *S_given, int8_t *Xq, int8_t *Xq_copy,
                           float *S_dyn, bool S_dyn_is_zero, int32_t *status, cudaStream_t s)
@@ -36,7 +45,7 @@ q8_status quantize_tensor(const float *X, int64_t numel, const float *S_given, i
         li.launches += 1;
         return Q8_OK;
     }
-    if (S_given == nullptr && quantize_dynamic_grid_supported(X, numel, Xq, Xq_copy)) {
+    if (S_given == nullptr && quantize_dynamic_grid_supported(X, numel, Xq, Xq_copy) && !capturing(s)) {
         const cudaError_t e = launch_quantize_dynamic_grid(X, numel, S_dyn, status, Xq, Xq_copy, s);
         if (e != cudaErrorCooperativeLaunchTooLarge) {
             Q8_CUDA_TRY(e);

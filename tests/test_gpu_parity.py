@@ -379,6 +379,11 @@ def test_dynamic_quantisation_where_the_cooperative_launch_is_refused(n):
         assert torch.equal(got, want) and torch.equal(s_got, s_want)
         Wq, S_w = q8.q8_quantize_weight(x.view(1, n))
         assert torch.equal(Wq.view(-1), want) and torch.equal(S_w, s_want)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):  # (a launch that is refused would end the capture)
+            captured, s_captured = q8.q8_quantize_activation(x)
+        graph.replay()
+        assert torch.equal(captured, want) and torch.equal(s_captured, s_want)
     finally:
         q8.q8_tune_quantize_grid(0)
     torch.cuda.synchronize()
