@@ -53,7 +53,7 @@ int q8_last_launch_store_mode(void);
  * (non-zero, the default) or always the CUDA-core fp32 kernel (0), for later calls in this process. */
 void q8_tune_attention(int use_tensor_cores);
 
-/* Tuning / test hook: CTAs of the cooperative launch that finds a dynamic scale and quantises with it (up to 4 Mi values), for later
+/* Tuning / test hook: CTAs of the cooperative launch that finds a dynamic scale and quantises with it (up to 2 Mi values), for later
  * calls in this process; 0 (the default) = automatic.  More than fit on the device at a time make the CUDA runtime refuse the
  * launch, as it does where the process may use a part of the SMs only, and the separate passes run instead.  Results do not
  * depend on it. */

@@ -325,14 +325,13 @@ __global__ void __launch_bounds__(kDqThreads) quantize_dynamic_cluster_kernel(co
 }
 
 // The same in ONE launch for tensors that no longer fit one cluster's registers: a cooperative grid finds max|x|, meets,
-// derives S and quantises.  Up to kCoopMaxElems: the barriers cost about as much device time as the launches they replace
-// (a 2048 x 768 weight 8.55 against 8.59 us for memset, abs-max, scale, quantise), but one call to the driver takes the place
-// of four; a 125 MB matrix would take 54 us instead of 51, the second pass being bound by the conversions and latency
-// even where it hits L2.
+// derives S and quantises.  Up to kCoopMaxElems, where the barriers cost about as much device time as the launches they replace and
+// one call to the driver takes the place of four.  Calls in a row with changing inputs, one launch / memset, abs-max, scale, quantise,
+// us: 0.3 M values 8.2 / 11.6, 1 M 8.7 / 11.5, 2 Mi 11.3 / 11.6, 2.5 M 13.6 / 12.4, 3 Mi 14.4 / 12.4, 4 Mi 16.4 / 13.7.
 // *word holds the running maximum (float bits) during the first pass and S at the end, so a single device word is enough;
 // a bad maximum is OR-ed into *status (may be NULL).
 constexpr int kCoopThreads = 256, kCoopCtasPerSm = 4;
-constexpr int64_t kCoopMaxElems = int64_t(4) << 20;
+constexpr int64_t kCoopMaxElems = int64_t(2) << 20;
 
 __global__ void __launch_bounds__(kCoopThreads, kCoopCtasPerSm)
 quantize_dynamic_grid_kernel(const float *__restrict__ x, int64_t n, uint32_t *word, int32_t *status,

@@ -95,7 +95,7 @@ cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *a
 bool quantize_dynamic_small_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
 cudaError_t launch_quantize_dynamic_small(const float *x, int64_t n, float *S_out, int32_t *status, bool set_status, int8_t *xq,
                                           int8_t *xq_copy, cudaStream_t s);
-// Larger ones, up to 4 Mi values (16-byte aligned): the same in one cooperative launch.  *S_out also serves as the reduction
+// Larger ones, up to 2 Mi values (16-byte aligned): the same in one cooperative launch.  *S_out also serves as the reduction
 // word; *status (may be NULL) is OR-ed into.
 // cudaErrorCooperativeLaunchTooLarge where the process may not use every SM: nothing was launched then.
 bool quantize_dynamic_grid_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
