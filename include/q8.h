@@ -262,8 +262,9 @@ q8_status q8_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, const int
 
 /* q8_attention / q8_attention_quant run on the tensor cores when the pointers are 16-byte aligned: both products as
  * tcgen05.mma on operands split into two 16-bit (kind::f16, scaled by powers of two) or TF32 parts each, three
- * partial products accumulated in fp32, which keeps fp32-grade accuracy; rows whose operands span more than the 16-bit
- * parts carry are computed in plain fp32.  (Grids of at most one CTA of 128 queries per SM with S <= 384 use TF32 parts: an
+ * partial products accumulated in fp32, which keeps fp32-grade accuracy: a product is off by 2^-22 of itself, and by 2^-37 of the
+ * largest |q| |k| of its row and 64 keys, or of the largest |v| of its feature.  Rows for which that is more than plain fp32 sums are
+ * off by (largest |q| |k| above 2^14, a result small beside V in every feature, infinities) are computed in plain fp32.  (Grids of at most one CTA of 128 queries per SM with S <= 384 use TF32 parts: an
  * infinite input gives NaN there where the exact result would be infinite.)  Unaligned pointers: a CUDA-core fp32
  * kernel computes the same thing.  The tensor-core
  * kernels bound their waits; a time-out sets the Q8_ERR_TIMEOUT bit in a per-device status word whose device

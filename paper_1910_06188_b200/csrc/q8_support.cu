@@ -23,8 +23,9 @@ constexpr int kLnThreads = 256;
 // Of the two-CTA forms: two, with registers for all loads of a row and of its residual at once (with four CTAs
 // of 64 registers the loads of the two come one after the other: 128 x 768 3.85 -> 3.10 us, 1421 x 768 5.05 -> 4.10, 24576 x 1024
 // with Int8 copy 61.9 -> 54.0 us = 6.05 TB/s; three CTAs spill: 57.4).  Also where four would take all rows in one round and two
-// need a second one: 4096 x 768 10.2 -> 9.3.  (Whole static forwards of 32 x 128 and 16 x 512 tokens are 0.6 % slower with it all the
-// same, 516 -> 520 and 739 -> 743 us; 1 x 128 is 7 %, 7 x 203 6 %, BERT-Large 64 x 384 2.5 % faster.)
+// need a second one: 4096 x 768 10.2 -> 9.3.  (Whole static forwards of 32 x 128 and 16 x 512 tokens were 0.6 % slower with it all the
+// same, 516 -> 520 and 739 -> 743 us, which the form of 768 values takes back; 1 x 128 is 7 %, 7 x 203 6 %, BERT-Large 64 x 384 2.5 %
+// faster.)
 constexpr int kEmbedLnCtasPerSm = 4;  // the one-pass input kernel: Int8 rows, fewer registers
 
 __device__ __forceinline__ float block_sum(float v, float *scratch)
