@@ -223,8 +223,7 @@ q8_status q8_ste_backward(const float *grad_out, int64_t numel, float *grad_in, 
     if (numel < 0) return Q8_ERR_SHAPE;
     if (numel == 0 || grad_in == grad_out) return Q8_OK;  // the estimator is the identity: in place is a no-op
     if (!grad_out || !grad_in) return Q8_ERR_NULL;
-    Q8_CUDA_TRY(cudaMemcpyAsync(grad_in, grad_out, (size_t)numel * sizeof(float), cudaMemcpyDeviceToDevice,
-                                static_cast<cudaStream_t>(stream)));
+    Q8_CUDA_TRY(launch_copy(grad_out, numel, grad_in, static_cast<cudaStream_t>(stream)));
     return Q8_OK;
 }
 

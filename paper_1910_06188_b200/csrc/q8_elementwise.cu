@@ -1,8 +1,7 @@
 // HBM-bound kernels of the Q8BERT inference path: max|x| reduction (Eq. 3 / Eq. 4 / Sec. 4.1),
 // the quantiser of Eq. 1, the EMA update of Eq. 4 and the Int8 embedding gather of Sec. 3.
 //
-// All of them stream their input once with 16-byte loads and stores; the grid is a multiple of
-// the SM count with a grid-stride loop so every SM keeps several independent loads in flight.
+// All of them stream their input once with 16-byte loads and stores, several independent loads of a thread in flight.
 
 #include <cooperative_groups.h>
 
@@ -22,6 +21,20 @@ int grid_for(int64_t work_items, int items_per_block, int blocks_per_sm)
     return (int)(want < cap ? want : cap);
 }
 
+// The passes that read and write (quantise, copy) run as many short CTAs, one run of 4 x 128 float4 each: measured
+// faster than a grid of the device's size whose threads stride through the tensor, the more so the larger the tensor, and than
+// more or fewer loads a thread or larger CTAs.  Quantise, us, grid of 4 CTAs of 256 per SM before / 4 x 128 / 4 x 256 / 2 x 256 /
+// 8 x 128 / 4 x 512: 4096 x 768 3.34 / 3.36 / 3.63 / 3.70 / 3.73 / 3.51, 8192 x 768 6.45 / 5.63 / 5.3 / 6.65 / 7.93 / 6.56,
+// 4096 x 3072 11.9 / 11.0 / 11.1 / 11.9 / 14.9 / 12.8, 24576 x 1024 21.3 / 19.8 / 19.8 / 21.4 / 27.1 / 22.9, 24576 x 4096 75.4 / 71.2 /
+// 71.3 / 78.8 / 100 / 83 (= 7.07 TB/s).
+constexpr int kStreamThreads = 128, kStreamBatch = 4;
+
+int stream_grid(int64_t n)
+{
+    const int64_t runs = ((n >> 2) + kStreamThreads * kStreamBatch - 1) / (kStreamThreads * kStreamBatch);
+    return (int)(runs < 1 ? 1 : runs < INT32_MAX ? runs : INT32_MAX);
+}
+
 // ------------------------------------------------------------------ max|x|
 __device__ __forceinline__ float absmax4(float m, float4 v)
 {
@@ -34,10 +47,39 @@ __device__ __forceinline__ float absmax4(float m, float4 v)
 
 __device__ __forceinline__ void ema_update(CalibState *st, float m, float decay);
 
+// Streams n4 float4 through a thread, kBatch loads in flight at a time, then take(index, value) for each of them.  A CTA takes
+// runs of kBatch * blockDim.x neighbouring float4; how many runs is the grid's choice.
+template <int kBatch, typename Load, typename Take>
+__device__ __forceinline__ void for_each_batch(int64_t n4, Load load, Take take)
+{
+    const int64_t run = (int64_t)kBatch * blockDim.x;
+    for (int64_t base = (int64_t)blockIdx.x * run; base < n4; base += (int64_t)gridDim.x * run) {
+        const int64_t i = base + threadIdx.x;
+        float4 v[kBatch];
+        if (base + run <= n4) {
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) v[k] = load(i + k * blockDim.x);
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) take(i + k * blockDim.x, v[k]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k)
+                if (i + k * blockDim.x < n4) v[k] = load(i + k * blockDim.x);
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k)
+                if (i + k * blockDim.x < n4) take(i + k * blockDim.x, v[k]);
+        }
+    }
+}
+
+// Two CTAs of 512 per SM, eight loads a thread in flight also at the end (a thread's last loads one after the other, and an atomic
+// of each of 1184 CTAs: 12.6 M values 14 us, now 10.6).
 // With st the last CTA to finish (counted in the state's own counter, which it leaves at zero) also makes the Eq. 4 update.
+constexpr int kAbsmaxThreads = 512, kAbsmaxCtasPerSm = 2;
+
 template <bool VEC>
-__global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restrict__ x, int64_t n, uint32_t *bits,
-                                                          CalibState *st, float decay)
+__global__ void __launch_bounds__(kAbsmaxThreads, kAbsmaxCtasPerSm) absmax_kernel(const float *__restrict__ x, int64_t n, uint32_t *bits,
+                                                                                  CalibState *st, float decay)
 {
     grid_dependency_release_next(n <= kSmallProblemElems);
     grid_dependency_wait();
@@ -47,32 +89,19 @@ __global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restric
     if (VEC) {
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
         const int64_t n4 = n >> 2;
-        int64_t i = tid;
-        // eight independent 16-byte loads per iteration
-        for (; i + 7 * nthreads < n4; i += 8 * nthreads) {
-            float4 v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = __ldg(x4 + i + k * nthreads);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) m = absmax4(m, v[k]);
-        }
-        for (; i < n4; i += nthreads) m = absmax4(m, __ldg(x4 + i));
+        for_each_batch<8>(n4, [&](int64_t i) { return __ldg(x4 + i); }, [&](int64_t, float4 v) { m = absmax4(m, v); });
         for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
     } else {
         for (int64_t j = tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __shared__ float warp_max[kThreads / 32];
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+    const uint32_t warp_bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));  // non-negative floats order like their bits
+    __shared__ uint32_t warp_max[kAbsmaxThreads / 32];
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = warp_bits;
     __syncthreads();
     if (threadIdx.x < 32) {
-        m = threadIdx.x < kThreads / 32 ? warp_max[threadIdx.x] : 0.0f;
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        const uint32_t all = __reduce_max_sync(0xffffffffu, threadIdx.x < kAbsmaxThreads / 32 ? warp_max[threadIdx.x] : 0u);
         if (threadIdx.x == 0) {
-            // non-negative floats (and +Inf) order like their bit patterns
-            if (m > 0.0f) atomicMax(bits, __float_as_uint(m));
+            if (all != 0u) atomicMax(bits, all);
             if (st != nullptr) {
                 __threadfence();
                 if (atomicInc(&st->finished_ctas, gridDim.x - 1) == gridDim.x - 1)
@@ -154,8 +183,7 @@ __device__ __forceinline__ int32_t quantize_one(float x, float S) { return quant
 
 __device__ __forceinline__ uint32_t quantize_pack4(float4 v, float S) { return q8::quantize_pack4(v.x, v.y, v.z, v.w, S); }
 
-// VEC: a thread turns one 16-byte load (4 floats) into one 4-byte store, four of them in flight
-// per iteration; consecutive lanes touch consecutive addresses on both sides.
+// VEC: a thread turns one 16-byte load (4 floats) into one 4-byte store, four of them in flight; consecutive lanes touch consecutive addresses on both sides.
 // With absmax_bits (dynamic scale, Sec. 4.1) every thread derives S = 127 / max|x| from the finished abs-max word
 // itself (one correctly rounded division, the same value in every thread) and thread 0 of the grid publishes it
 // in *S_out for the GEMM that follows, so no separate scale kernel runs; otherwise S is read from S_ptr.
@@ -204,28 +232,12 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
         uint32_t *q4 = reinterpret_cast<uint32_t *>(xq);
         uint32_t *c4 = reinterpret_cast<uint32_t *>(xq_copy);
         const int64_t n4 = n >> 2;
-        int64_t i = tid;
-        for (; i + 3 * nthreads < n4; i += 4 * nthreads) {
-            float4 a = __ldg(x4 + i), b = __ldg(x4 + i + nthreads), c = __ldg(x4 + i + 2 * nthreads),
-                   d = __ldg(x4 + i + 3 * nthreads);
-            uint32_t qa = quantize_pack4(a, S), qb = quantize_pack4(b, S), qc = quantize_pack4(c, S),
-                     qd = quantize_pack4(d, S);
-            q4[i] = qa;
-            q4[i + nthreads] = qb;
-            q4[i + 2 * nthreads] = qc;
-            q4[i + 3 * nthreads] = qd;
-            if (xq_copy) {
-                c4[i] = qa;
-                c4[i + nthreads] = qb;
-                c4[i + 2 * nthreads] = qc;
-                c4[i + 3 * nthreads] = qd;
-            }
-        }
-        for (; i < n4; i += nthreads) {
-            uint32_t q = quantize_pack4(__ldg(x4 + i), S);
-            q4[i] = q;
-            if (xq_copy) c4[i] = q;
-        }
+        for_each_batch<kStreamBatch>(n4, [&](int64_t i) { return __ldg(x4 + i); },
+                                     [&](int64_t i, float4 v) {
+                                         const uint32_t q = quantize_pack4(v, S);
+                                         q4[i] = q;
+                                         if (xq_copy) c4[i] = q;
+                                     });
         for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) {
             int8_t q = (int8_t)quantize_one(x[j], S);
             xq[j] = q;
@@ -533,6 +545,20 @@ __global__ void __launch_bounds__(kThreads) fake_quantize_kernel(const float *x,
     }
 }
 
+// ------------------------------------------------------------------ Eq. 5: the gradient passes unchanged
+// (A kernel of its own so that it starts under the tail of the one before it; 4096 x 3072 17.3 us = 5.8 TB/s with its launch, the
+// runtime's copy 19.0.)
+__global__ void __launch_bounds__(kStreamThreads) copy_kernel(const float *__restrict__ from, int64_t n, float *__restrict__ to)
+{
+    grid_dependency_release_next(n <= kSmallProblemElems);
+    grid_dependency_wait();
+    const float4 *f4 = reinterpret_cast<const float4 *>(from);
+    float4 *t4 = reinterpret_cast<float4 *>(to);
+    const int64_t n4 = n >> 2;
+    for_each_batch<kStreamBatch>(n4, [&](int64_t i) { return __ldcs(f4 + i); }, [&](int64_t i, float4 v) { __stcs(t4 + i, v); });
+    if (blockIdx.x == 0 && threadIdx.x < (n & 3)) to[(n4 << 2) + threadIdx.x] = from[(n4 << 2) + threadIdx.x];
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -540,11 +566,10 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_t s, CalibState *st, float decay)
 {
     if (n <= 0) return cudaSuccess;
-    if (aligned16(x))
-        return launch_overlapping_tail(absmax_kernel<true>, dim3(grid_for(n >> 2, kThreads * 4, 8)), dim3(kThreads), 0, s, x, n,
-                                       bits, st, decay);
-    return launch_overlapping_tail(absmax_kernel<false>, dim3(grid_for(n, kThreads * 4, 8)), dim3(kThreads), 0, s, x, n, bits,
-                                   st, decay);
+    const bool vec = aligned16(x);
+    const int grid = grid_for(vec ? n >> 2 : n, kAbsmaxThreads * 2, kAbsmaxCtasPerSm);
+    return launch_overlapping_tail(vec ? absmax_kernel<true> : absmax_kernel<false>, dim3(grid), dim3(kAbsmaxThreads), 0, s, x, n, bits, st,
+                                   decay);
 }
 
 // Two CTAs per SM read less at a time than the eight of absmax_kernel: a dynamic layer of 1024 columns with changing inputs, partial
@@ -617,19 +642,12 @@ cudaError_t launch_scale_from_absmax(const uint32_t *bits, float *S, int32_t *st
     return launch_overlapping_tail(scale_from_absmax_kernel, dim3(1), dim3(1), 0, s, bits, S, status);
 }
 
-// Grid of the vectorised quantise pass: CTAs per SM, grid-stride.  Measured on 24576 x 1024 / 24576 x 4096 fp32 inputs
-// (graph replays of three passes over separate buffers): 2 CTAs per SM 26.6 / 92.2 us, 3: 23.0 / 78.6, 4: 21.4 / 75.4,
-// 5: 25.4 / 89.6, 8: 21.6 / 77.3, 16: 24.8 / 78.4: a power-of-two stride between a thread's successive loads suits
-// the memory system best, and four CTAs already keep enough loads in flight (64 KB per SM).
-constexpr int kQuantCtasPerSm = 4;
-
 cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *xq, int8_t *xq_copy, cudaStream_t s,
                             int32_t *clear_word, int32_t *status)
 {
     if (n <= 0) return cudaSuccess;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
-        return launch_overlapping_tail(quantize_kernel<true>, dim3(grid_for((n + 3) >> 2, kThreads * 4, kQuantCtasPerSm)),
-                                       dim3(kThreads), 0, s, x, n, S, xq, xq_copy, nullptr, 1, nullptr, status, clear_word);
+        return launch_overlapping_tail(quantize_kernel<true>, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, x, n, S, xq, xq_copy, nullptr, 1, nullptr, status, clear_word);
     } else {
         quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, S, xq, xq_copy, nullptr, 1, nullptr,
                                                                                  status, clear_word);
@@ -643,8 +661,7 @@ cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *a
     if (n <= 0) return cudaSuccess;
     int32_t *clear_word = clear_status ? status : nullptr;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
-        return launch_overlapping_tail(quantize_kernel<true>, dim3(grid_for((n + 3) >> 2, kThreads * 4, kQuantCtasPerSm)),
-                                       dim3(kThreads), 0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
+        return launch_overlapping_tail(quantize_kernel<true>, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
     } else {
         quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, nullptr, xq, xq_copy, absmax_bits,
                                                                                  absmax_count, S_out, status, clear_word);
@@ -685,6 +702,13 @@ cudaError_t launch_fake_quantize(const float *x, int64_t n, const float *S, floa
                                        0, s, x, n, S, xhat);
     return launch_overlapping_tail(fake_quantize_kernel<false>, dim3(grid_for(n, kThreads * 4, 8)), dim3(kThreads), 0, s, x, n,
                                    S, xhat);
+}
+
+cudaError_t launch_copy(const float *from, int64_t n, float *to, cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    if (!aligned16(from) || !aligned16(to)) return cudaMemcpyAsync(to, from, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    return launch_overlapping_tail(copy_kernel, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, from, n, to);
 }
 
 cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, const float *S_e, int64_t V,

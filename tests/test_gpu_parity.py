@@ -605,3 +605,22 @@ def test_192_wide_tiles_bit_exact(M, N, K):
     Y = q8.q8_linear_q(Xq, S_x, Wq, S_w, dev(b), 1)
     only = q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), 1, S_y)
     assert np.array_equal(only.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(25.0)))
+
+
+# ------------------------------------------------------------------ the streaming passes at the ends of their runs
+@pytest.mark.parametrize("n", [1, 5, 511, 2047, 2048, 2049, 4 * 2048 - 3, 16 * 148 * 512 + 7])
+def test_streaming_passes_at_the_ends_of_their_runs(n):
+    """Quantise, abs-max with the Eq. 4 update, fake quantise and the straight-through copy: a CTA's run is 4 x 128 float4 (8 x 512
+    of the abs-max), the last run is ragged and up to three values are left over."""
+    x = synth.normal((n,), 1.0, 9100 + n % 1000)
+    x[-1] = 7.5  # the largest value is the last one
+    xd, S = dev(x), dev(np.array([12.7], np.float32))
+    assert np.array_equal(q8.q8_quantize_activation(xd, S)[0].cpu().numpy(), o.quantize(x, np.float32(12.7)))
+    state = q8.new_calibrate_state()
+    q8.q8_calibrate(xd, 0.5, state)
+    assert state.view(torch.float32)[0].item() == 7.5
+    assert torch.equal(q8.q8_ste_backward(xd), xd)
+    want = o.quantize(x, np.float32(12.7)).astype(np.float32) / np.float32(12.7)
+    assert np.array_equal(q8.q8_fake_quantize(xd, S).cpu().numpy(), want)
+    inplace = xd.clone()
+    assert np.array_equal(q8.q8_fake_quantize(inplace, S, inplace).cpu().numpy(), want)
