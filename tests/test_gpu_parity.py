@@ -624,3 +624,15 @@ def test_streaming_passes_at_the_ends_of_their_runs(n):
     assert np.array_equal(q8.q8_fake_quantize(xd, S).cpu().numpy(), want)
     inplace = xd.clone()
     assert np.array_equal(q8.q8_fake_quantize(inplace, S, inplace).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("S", [2.0 ** -125, 1e-25, 2.0 ** -60, 1.0000001, 12.7, 1e9 / 3, 2.0 ** 60, 1e25, 3.4e38])
+def test_fake_quantise_quotient_is_rounded_to_nearest(S):
+    """Every integer of -127..127 over S, at the ends of the range where the quotient comes from a reciprocal and beyond."""
+    S = np.float32(S)
+    q = np.arange(-127, 128, dtype=np.float32)
+    with np.errstate(over="ignore"):
+        x = (q / S).astype(np.float32)
+        want = o.quantize(x, S).astype(np.float32) / S
+    got = q8.q8_fake_quantize(dev(x), dev(np.array([S], np.float32))).cpu().numpy()
+    assert np.array_equal(got, want)
