@@ -54,6 +54,11 @@ q8_status quantize_tensor(const float *X, int64_t numel, const float *S_given, i
         }
         cudaGetLastError();  // not every SM is this process's to use (a partition of the device): the separate passes run anywhere
     }
+    if (S_given == nullptr && quantize_two_pass_supported(X, numel, Xq, Xq_copy)) {
+        Q8_CUDA_TRY(launch_quantize_two_pass(X, numel, S_dyn, status, Xq, Xq_copy, s));
+        li.launches += 3;
+        return Q8_OK;
+    }
     if (S_given == nullptr) {
         // The scale word first holds the float bits of the running maximum, then the scale itself.
         if (!S_dyn_is_zero) Q8_CUDA_TRY(cudaMemsetAsync(S_dyn, 0, sizeof(float), s));
@@ -130,14 +135,16 @@ q8_status linear_impl(const float *X, const int8_t *Wq, const float *S_w, const 
         last_launch_info().launches += 1;
     } else {
         int words = 1;
-        if (absmax_partial_preferred(M * K)) {
+        const bool partial = absmax_partial_preferred(M * K);
+        if (partial) {
             Q8_CUDA_TRY(launch_absmax_partial(X, M * K, hdr->absmax_partial,
                                               (int)(sizeof(hdr->absmax_partial) / sizeof(hdr->absmax_partial[0])), &words, s));
         } else {
             Q8_CUDA_TRY(cudaMemsetAsync(hdr->absmax_partial, 0, sizeof(hdr->absmax_partial[0]), s));
             Q8_CUDA_TRY(launch_absmax(X, M * K, hdr->absmax_partial, s));
         }
-        Q8_CUDA_TRY(launch_quantize_dynamic(X, M * K, hdr->absmax_partial, &hdr->S_x_dyn, &hdr->status, Xq, dbg_Xq, s, true, words));
+        Q8_CUDA_TRY(launch_quantize_dynamic(X, M * K, hdr->absmax_partial, &hdr->S_x_dyn, &hdr->status, Xq, dbg_Xq, s, true, words,
+                                            !partial));
         last_launch_info().launches += 2;
     }
 

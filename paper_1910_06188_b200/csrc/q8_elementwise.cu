@@ -29,9 +29,9 @@ int grid_for(int64_t work_items, int items_per_block, int blocks_per_sm)
 // 71.3 / 78.8 / 100 / 83 (= 7.07 TB/s).
 constexpr int kStreamThreads = 128, kStreamBatch = 4;
 
-int stream_grid(int64_t n)
+int stream_grid(int64_t n, int threads = kStreamThreads)
 {
-    const int64_t runs = ((n >> 2) + kStreamThreads * kStreamBatch - 1) / (kStreamThreads * kStreamBatch);
+    const int64_t runs = ((n >> 2) + threads * kStreamBatch - 1) / (threads * kStreamBatch);
     return (int)(runs < 1 ? 1 : runs < INT32_MAX ? runs : INT32_MAX);
 }
 
@@ -72,43 +72,57 @@ __device__ __forceinline__ void for_each_batch(int64_t n4, Load load, Take take)
     }
 }
 
-// Two CTAs of 512 per SM, eight loads a thread in flight also at the end (a thread's last loads one after the other, and an atomic
-// of each of 1184 CTAs: 12.6 M values 14 us, now 10.6).
-// With st the last CTA to finish (counted in the state's own counter, which it leaves at zero) also makes the Eq. 4 update.
-constexpr int kAbsmaxThreads = 512, kAbsmaxCtasPerSm = 2;
+// The CTA's share of max|x| in every thread of warp 0, as float bits (non-negative floats order like them).
+// Eight CTAs of 256 per SM, four loads a thread in flight, the last ones as well (eight loads, with the last made one after the other,
+// 14 us for 12.6 M values where this takes 8.5; two CTAs of 512 with eight loads 9.4; a run per CTA 8.7).
+constexpr int kAbsmaxCtasPerSm = 8, kAbsmaxBatch = 4;
 
 template <bool VEC>
-__global__ void __launch_bounds__(kAbsmaxThreads, kAbsmaxCtasPerSm) absmax_kernel(const float *__restrict__ x, int64_t n, uint32_t *bits,
-                                                                                  CalibState *st, float decay)
+__device__ __forceinline__ uint32_t cta_absmax(const float *__restrict__ x, int64_t n)
 {
-    grid_dependency_release_next(n <= kSmallProblemElems);
-    grid_dependency_wait();
     float m = 0.0f;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     if (VEC) {
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
         const int64_t n4 = n >> 2;
-        for_each_batch<8>(n4, [&](int64_t i) { return __ldg(x4 + i); }, [&](int64_t, float4 v) { m = absmax4(m, v); });
+        for_each_batch<kAbsmaxBatch>(n4, [&](int64_t i) { return __ldg(x4 + i); }, [&](int64_t, float4 v) { m = absmax4(m, v); });
         for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
     } else {
         for (int64_t j = tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
     }
-    const uint32_t warp_bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));  // non-negative floats order like their bits
-    __shared__ uint32_t warp_max[kAbsmaxThreads / 32];
+    const uint32_t warp_bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    __shared__ uint32_t warp_max[kThreads / 32];
     if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = warp_bits;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const uint32_t all = __reduce_max_sync(0xffffffffu, threadIdx.x < kAbsmaxThreads / 32 ? warp_max[threadIdx.x] : 0u);
-        if (threadIdx.x == 0) {
-            if (all != 0u) atomicMax(bits, all);
-            if (st != nullptr) {
-                __threadfence();
-                if (atomicInc(&st->finished_ctas, gridDim.x - 1) == gridDim.x - 1)
-                    ema_update(st, __uint_as_float(atomicExch(bits, 0u)), decay);
-            }
+    if (threadIdx.x >= 32) return 0u;
+    return __reduce_max_sync(0xffffffffu, threadIdx.x < kThreads / 32 ? warp_max[threadIdx.x] : 0u);
+}
+
+// With st the last CTA to finish (counted in the state's own counter, which it leaves at zero) also makes the Eq. 4 update.
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads) absmax_kernel(const float *__restrict__ x, int64_t n, uint32_t *bits, CalibState *st, float decay)
+{
+    grid_dependency_release_next(n <= kSmallProblemElems);
+    grid_dependency_wait();
+    const uint32_t all = cta_absmax<VEC>(x, n);
+    if (threadIdx.x == 0) {
+        if (all != 0u) atomicMax(bits, all);
+        if (st != nullptr) {
+            __threadfence();
+            if (atomicInc(&st->finished_ctas, gridDim.x - 1) == gridDim.x - 1)
+                ema_update(st, __uint_as_float(atomicExch(bits, 0u)), decay);
         }
     }
+}
+
+// The same with a word for each CTA, all of which are written, so that nothing is cleared first.
+__global__ void __launch_bounds__(kThreads) absmax_words_kernel(const float *__restrict__ x, int64_t n, uint32_t *__restrict__ words)
+{
+    grid_dependency_release_next(true);  // to the one CTA of scale_from_words_kernel
+    grid_dependency_wait();
+    const uint32_t all = cta_absmax<true>(x, n);
+    if (threadIdx.x == 0) words[blockIdx.x] = all;
 }
 
 // max|x| as one partial maximum per cluster of CTAs (exchanged through distributed shared memory): every word of `partial`
@@ -127,15 +141,7 @@ __global__ void __launch_bounds__(kThreads) absmax_partial_kernel(const float *_
     if (VEC) {
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
         const int64_t n4 = n >> 2;
-        int64_t i = tid;
-        for (; i + 7 * nthreads < n4; i += 8 * nthreads) {
-            float4 v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = __ldg(x4 + i + k * nthreads);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) m = absmax4(m, v[k]);
-        }
-        for (; i < n4; i += nthreads) m = absmax4(m, __ldg(x4 + i));
+        for_each_batch<8>(n4, [&](int64_t i) { return __ldg(x4 + i); }, [&](int64_t, float4 v) { m = absmax4(m, v); });
         for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
     } else {
         for (int64_t j = tid; j < n; j += nthreads) m = fmaxf(m, fabsf(x[j]));
@@ -162,20 +168,35 @@ __global__ void __launch_bounds__(kThreads) absmax_partial_kernel(const float *_
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// S = 127 / max|.| (Eq. 3), in place over the scratch word when bits and S alias.
+// S = 127 / max|.| (Eq. 3); 1, and the flag, for a maximum that is zero or not finite.
+__device__ __forceinline__ void put_scale(float a, float *S, int32_t *status)
+{
+    const bool bad = !(a > 0.0f) || isinf(a);
+    if (bad && status) atomicOr(status, 1 << Q8_ERR_SCALE);
+    *S = bad ? 1.0f : __fdiv_rn(127.0f, a);
+}
+
+// (in place over the scratch word when bits and S alias)
 __global__ void scale_from_absmax_kernel(const uint32_t *bits, float *S, int32_t *status)
 {
     grid_dependency_release_next(true);
     grid_dependency_wait();
-    float a = __uint_as_float(*bits);
-    float s;
-    if (!(a > 0.0f) || isinf(a)) {
-        s = 1.0f;
-        if (status) atomicOr(status, 1 << Q8_ERR_SCALE);
-    } else {
-        s = __fdiv_rn(127.0f, a);
-    }
-    *S = s;
+    put_scale(__uint_as_float(*bits), S, status);
+}
+
+__global__ void __launch_bounds__(kThreads) scale_from_words_kernel(const uint32_t *words, int count, float *S, int32_t *status)
+{
+    grid_dependency_wait();
+    grid_dependency_release_next(true);  // (not before the pass over x is over, which the CTAs of the next kernel would hold up)
+    uint32_t m = 0u;
+    for (int i = threadIdx.x; i < count; i += kThreads) m = max(m, words[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    __shared__ uint32_t warp_max[kThreads / 32];
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    m = __reduce_max_sync(0xffffffffu, threadIdx.x < kThreads / 32 ? warp_max[threadIdx.x] : 0u);
+    if (threadIdx.x == 0) put_scale(__uint_as_float(m), S, status);
 }
 
 // ------------------------------------------------------------------ Eq. 1
@@ -187,7 +208,11 @@ __device__ __forceinline__ uint32_t quantize_pack4(float4 v, float S) { return q
 // With absmax_bits (dynamic scale, Sec. 4.1) every thread derives S = 127 / max|x| from the finished abs-max word
 // itself (one correctly rounded division, the same value in every thread) and thread 0 of the grid publishes it
 // in *S_out for the GEMM that follows, so no separate scale kernel runs; otherwise S is read from S_ptr.
-template <bool VEC>
+// AGAIN: the abs-max pass has just read x.  From its end, which L2 still holds some of, the lines marked as the first to go.
+// (30522 x 1024, both passes, us: in the order of the abs-max pass 43.8, from the end 40.2, with the mark 38.5, with CTAs of 256 instead of 128 another 1.2 less; marking the first lines
+// of the abs-max pass as well, or keeping its last, changes less than 1; all of it in one cooperative launch of a CTA per SM that keeps
+// 53 MB in registers and shared memory takes 54.)
+template <bool VEC, bool AGAIN = false>
 __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restrict__ x, int64_t n,
                                                             const float *__restrict__ S_ptr,
                                                             int8_t *__restrict__ xq, int8_t *__restrict__ xq_copy,
@@ -232,12 +257,23 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
         uint32_t *q4 = reinterpret_cast<uint32_t *>(xq);
         uint32_t *c4 = reinterpret_cast<uint32_t *>(xq_copy);
         const int64_t n4 = n >> 2;
-        for_each_batch<kStreamBatch>(n4, [&](int64_t i) { return __ldg(x4 + i); },
-                                     [&](int64_t i, float4 v) {
-                                         const uint32_t q = quantize_pack4(v, S);
-                                         q4[i] = q;
-                                         if (xq_copy) c4[i] = q;
-                                     });
+        uint64_t first_to_go;
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first_to_go));
+        auto place = [&](int64_t i) { return AGAIN ? n4 - 1 - i : i; };
+        for_each_batch<kStreamBatch>(
+            n4,
+            [&](int64_t i) {
+                if (!AGAIN) return __ldg(x4 + i);
+                float4 v;
+                asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                             : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(x4 + place(i)), "l"(first_to_go));
+                return v;
+            },
+            [&](int64_t i, float4 v) {
+                const uint32_t q = quantize_pack4(v, S);
+                q4[place(i)] = q;
+                if (xq_copy) c4[place(i)] = q;
+            });
         for (int64_t j = (n4 << 2) + tid; j < n; j += nthreads) {
             int8_t q = (int8_t)quantize_one(x[j], S);
             xq[j] = q;
@@ -560,20 +596,20 @@ cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_
 {
     if (n <= 0) return cudaSuccess;
     const bool vec = aligned16(x);
-    const int grid = grid_for(vec ? n >> 2 : n, kAbsmaxThreads * 2, kAbsmaxCtasPerSm);
-    return launch_overlapping_tail(vec ? absmax_kernel<true> : absmax_kernel<false>, dim3(grid), dim3(kAbsmaxThreads), 0, s, x, n, bits, st,
-                                   decay);
+    return launch_overlapping_tail(vec ? absmax_kernel<true> : absmax_kernel<false>,
+                                   dim3(grid_for(vec ? n >> 2 : n, kThreads * kAbsmaxBatch, kAbsmaxCtasPerSm)), dim3(kThreads), 0, s, x, n, bits,
+                                   st, decay);
 }
 
-// Two CTAs per SM read less at a time than the eight of absmax_kernel: a dynamic layer of 1024 columns with changing inputs, partial
-// maxima / clear and atomics, us: 2.1 M values 11.2 / 13.0, 4.2 M 16.0 / 16.9, 6.3 M 18.8 / 19.1, 9.4 M 23.6 / 23.1, 12.6 M 29.3 / 25.3,
-// 52 M 113 / 97.  (CTAs of 1024 threads in the clusters do not help: 29.6 at 12.6 M.)
-bool absmax_partial_preferred(int64_t n) { return n <= (int64_t(8) << 20); }
+// A dynamic layer of 1024 columns with changing inputs, partial maxima / clear and atomics of eight CTAs per SM, us: 0.6 M values 10.4 /
+// 12.5, 2.0 M 12.3 / 14.3, 4.1 M 14.7 / 16.4, 6.1 M 22.7 / 18.7, 8.2 M 27.3 / 22.5: what no longer stays in L2 wants all of the
+// loads that 8 CTAs have in flight.
+bool absmax_partial_preferred(int64_t n) { return n <= (int64_t(9) << 19); }  // 4.7 M
 
 cudaError_t launch_absmax_partial(const float *x, int64_t n, uint32_t *partial, int max_words, int *words, cudaStream_t s)
 {
     const bool vec = aligned16(x);
-    int clusters = (grid_for(vec ? n >> 2 : n, kThreads * 4, 2) + kAmCluster - 1) / kAmCluster;
+    int clusters = (grid_for(vec ? n >> 2 : n, kThreads * 4, 4) + kAmCluster - 1) / kAmCluster;
     if (clusters > max_words) clusters = max_words;
     *words = clusters;
     cudaLaunchConfig_t cfg = {};
@@ -635,6 +671,25 @@ cudaError_t launch_scale_from_absmax(const uint32_t *bits, float *S, int32_t *st
     return launch_overlapping_tail(scale_from_absmax_kernel, dim3(1), dim3(1), 0, s, bits, S, status);
 }
 
+// Every access of the three kernels is whole, and the first bytes of xq, which the last of them fills, have room for a word per CTA
+// (each of which has a run of 4096 values unless the tensor is smaller than that).
+bool quantize_two_pass_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy)
+{
+    return n >= 4 && aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy));
+}
+
+cudaError_t launch_quantize_two_pass(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq, int8_t *xq_copy, cudaStream_t s)
+{
+    const int ctas = grid_for(n >> 2, kThreads * kAbsmaxBatch, kAbsmaxCtasPerSm);
+    uint32_t *words = reinterpret_cast<uint32_t *>(xq);
+    cudaError_t e = launch_overlapping_tail(absmax_words_kernel, dim3(ctas), dim3(kThreads), 0, s, x, n, words);
+    if (e == cudaSuccess)
+        e = launch_overlapping_tail(scale_from_words_kernel, dim3(1), dim3(kThreads), 0, s, words, ctas, S_out, status);
+    if (e != cudaSuccess) return e;
+    return launch_overlapping_tail(quantize_kernel<true, true>, dim3(stream_grid(n, kThreads)), dim3(kThreads), 0, s, x, n, S_out, xq, xq_copy,
+                                   nullptr, 1, nullptr, nullptr, nullptr);
+}
+
 cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *xq, int8_t *xq_copy, cudaStream_t s,
                             int32_t *clear_word, int32_t *status)
 {
@@ -649,12 +704,14 @@ cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *x
 }
 
 cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *absmax_bits, float *S_out, int32_t *status,
-                                    int8_t *xq, int8_t *xq_copy, cudaStream_t s, bool clear_status, int absmax_count)
+                                    int8_t *xq, int8_t *xq_copy, cudaStream_t s, bool clear_status, int absmax_count, bool again)
 {
     if (n <= 0) return cudaSuccess;
     int32_t *clear_word = clear_status ? status : nullptr;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
-        return launch_overlapping_tail(quantize_kernel<true>, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
+        const int threads = again ? kThreads : kStreamThreads;
+        return launch_overlapping_tail(again ? quantize_kernel<true, true> : quantize_kernel<true>, dim3(stream_grid(n, threads)), dim3(threads),
+                                       0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
     } else {
         quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, nullptr, xq, xq_copy, absmax_bits,
                                                                                  absmax_count, S_out, status, clear_word);

@@ -86,10 +86,13 @@ cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *x
                             cudaStream_t s, int32_t *clear_word = nullptr, int32_t *status = nullptr);
 // Eq. 1 with S = 127 / float(*absmax_bits) derived inside the kernel (dynamic scale); *S_out receives S and
 // *status the Q8_ERR_SCALE bit when the maximum is 0 or not finite (S = 1 then).  absmax_bits and S_out differ.
-// absmax_count: that many partial maxima from absmax_bits on.  clear_status: start *status at zero first (the call's status word, when no memset precedes the kernel).
+// absmax_count: that many partial maxima from absmax_bits on.  again: an abs-max pass has just read all of a large x.  clear_status: start *status at zero first (the call's status word, when no memset precedes the kernel).
 cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *absmax_bits, float *S_out,
                                     int32_t *status, int8_t *xq, int8_t *xq_copy, cudaStream_t s,
-                                    bool clear_status = false, int absmax_count = 1);
+                                    bool clear_status = false, int absmax_count = 1, bool again = false);
+// max|x|, its scale (into *S_out; a bad maximum is OR-ed into *status, which may be NULL) and Eq. 1 in three launches and no scratch but xq.
+bool quantize_two_pass_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
+cudaError_t launch_quantize_two_pass(const float *x, int64_t n, float *S_out, int32_t *status, int8_t *xq, int8_t *xq_copy, cudaStream_t s);
 // Small tensors (n <= 196608, n % 4 == 0, 16-byte aligned): abs-max, scale and Eq. 1 in one launch of one cluster.
 // *status (may be NULL) is SET (0 or the Q8_ERR_SCALE bit) with set_status, else OR-ed into.
 bool quantize_dynamic_small_supported(const float *x, int64_t n, const int8_t *xq, const int8_t *xq_copy);
