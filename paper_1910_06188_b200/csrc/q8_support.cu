@@ -15,18 +15,15 @@ namespace {
 // One CTA per row.  The summed row is kept in shared memory, so the inputs are read once; mean and
 // variance are the two-pass forms (sum, then sum of squared deviations), reduced through warp shuffles.
 constexpr int kLnThreads = 256;
-// The warp-per-row kernel has registers for a row and its residual, all loads of both in flight at once, of up to 256, 512, 768 or 1024
-// values, and four CTAs per SM where these leave room for them (H <= 512), else two.  (One form of 1024 values and two CTAs for every
-// H, four of 64 registers in sequence before it, us: 65536 x 64 27.8 / 38.0 / 17.2 now, 32768 x 128 15.0 / 20.3 / 9.7, 16384 x 256 10.6 /
-// 12.3 / 7.3, 8192 x 512 8.1 / 9.0 / 7.3, 4096 x 768 6.0 / 6.5 / 6.0, 24576 x 768 44.9 / 36.9 / 36.4; three CTAs up to 768: 1421 x 768 4.4
-// for 4.0; six up to 256: 65536 x 64 19.2.)
-// Of the two-CTA forms: two, with registers for all loads of a row and of its residual at once (with four CTAs
-// of 64 registers the loads of the two come one after the other: 128 x 768 3.85 -> 3.10 us, 1421 x 768 5.05 -> 4.10, 24576 x 1024
-// with Int8 copy 61.9 -> 54.0 us = 6.05 TB/s; three CTAs spill: 57.4).  Also where four would take all rows in one round and two
-// need a second one: 4096 x 768 10.2 -> 9.3.  (Whole static forwards of 32 x 128 and 16 x 512 tokens were 0.6 % slower with it all the
-// same, 516 -> 520 and 739 -> 743 us, which the form of 768 values takes back; 1 x 128 is 7 %, 7 x 203 6 %, BERT-Large 64 x 384 2.5 %
-// faster.)
-constexpr int kEmbedLnCtasPerSm = 4;  // the one-pass input kernel: Int8 rows, fewer registers
+// The warp-per-row kernels: CTAs of four rows, as many as there are rows for.  (Until all rows are taken by a device-sized grid whose
+// warps stride through them, CTAs of eight rows, us: 128 x 768 2.91 -> 2.73, 1421 x 768 3.92 -> 3.75, 4096 x 768 9.13 -> 8.87, 8192 x 768 16.1 ->
+// 14.7, 24576 x 1024 with its Int8 copy 53.8 -> 49.6 = 6.4 TB/s, 16384 x 256 11.2 -> 10.4; CTAs of eight rows without the stride
+// 9.7, 15.8 and 49.7 on the middle ones.)
+// add_layernorm_warp_kernel has registers for a row and its residual, all loads of both in flight at once, of up to 256, 512, 768 or 1024
+// values.  (One form of 1024 values for every H: 65536 x 64 38.0 us where the form of 256 takes 17.2; the loads of the row and of the
+// residual one after the other: 24576 x 1024 61.9 for 54.0.)
+constexpr int kLnWarpThreads = 128;
+constexpr int kEmbedLnCtasPerSm = 8;  // the one-pass input kernel: Int8 rows, fewer registers (four CTAs: 24576 x 1024 45.4 us for 35.0)
 
 __device__ __forceinline__ float block_sum(float v, float *scratch)
 {
@@ -178,9 +175,24 @@ __device__ __forceinline__ void normalise_row(const float4 (&v)[NV], float s, in
     }
 }
 
-// One warp per row for H <= 1024 (BERT's hidden sizes): NV float4 per lane (H <= 128 NV), eight rows per CTA.
+// max|y| of a CTA of the warp-per-row kernels into the word of a dynamically quantised consumer (Sec. 4.1): one atomic per CTA, since
+// those of one word take turns.  (16384 x 256, us: one per warp with a look at the word first 12.3, one per CTA with a look 11.6, without 11.3.)
+__device__ __forceinline__ void cta_fold_absmax(float m, uint32_t *word)
+{
+    __shared__ uint32_t warp_max[kLnWarpThreads / 32];
+    const uint32_t bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));  // non-negative floats order like their bits
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = bits;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    uint32_t all = 0u;
+#pragma unroll
+    for (int w = 0; w < kLnWarpThreads / 32; ++w) all = max(all, warp_max[w]);
+    if (all != 0u) atomicMax(word, all);
+}
+
+// One warp per row for H <= 1024 (BERT's hidden sizes): NV float4 per lane (H <= 128 NV).
 template <int NV, int CTAS_PER_SM>
-__global__ void __launch_bounds__(kLnThreads, CTAS_PER_SM) add_layernorm_warp_kernel(const float *__restrict__ x,
+__global__ void __launch_bounds__(kLnWarpThreads, CTAS_PER_SM) add_layernorm_warp_kernel(const float *__restrict__ x,
                                                                         const float *__restrict__ r1,
                                                                         const float *__restrict__ r2,
                                                                         const float *__restrict__ gamma,
@@ -195,9 +207,8 @@ __global__ void __launch_bounds__(kLnThreads, CTAS_PER_SM) add_layernorm_warp_ke
     const int n4 = (int)(H >> 2);
     const float Sq = out_q ? __ldg(S_q) : 1.0f;
     float am = 0.0f;  // running max|y| of this lane over all rows of the warp
-    // the grid is sized to the device and every warp walks rows with a grid stride (no partial last wave)
-    for (int64_t row = (int64_t)blockIdx.x * (kLnThreads / 32) + (threadIdx.x >> 5); row < rows;
-         row += (int64_t)gridDim.x * (kLnThreads / 32)) {
+    for (int64_t row = (int64_t)blockIdx.x * (kLnWarpThreads / 32) + (threadIdx.x >> 5); row < rows;
+         row += (int64_t)gridDim.x * (kLnWarpThreads / 32)) {
         const int64_t base4 = row * n4;
         const float4 *x4 = reinterpret_cast<const float4 *>(x) + base4;
         const float4 *a4 = r1 ? reinterpret_cast<const float4 *>(r1) + base4 : nullptr;
@@ -222,14 +233,14 @@ __global__ void __launch_bounds__(kLnThreads, CTAS_PER_SM) add_layernorm_warp_ke
         normalise_row(v, s, lane, n4, H, eps, gamma, beta, out ? reinterpret_cast<float4 *>(out) + base4 : nullptr,
                       out_q ? reinterpret_cast<uint32_t *>(out_q) + base4 : nullptr, Sq, am);
     }
-    if (amax) warp_fold_absmax(am, amax);  // one atomic per warp: max|y| for a dynamically quantised consumer (Sec. 4.1)
+    if (amax) cta_fold_absmax(am, amax);
 }
 
 // LayerNorm(word[ids[t]] + position[t % S] + type[0]) in one pass, one warp per token: the three Int8 rows are dequantised in
 // registers instead of travelling through three fp32 tensors (which is what the separate kernels are bound by: for
 // 24576 x 1024 they move 12 + 4 + 4 bytes per value where this one moves 4 and the table rows).  The same roundings as
 // q8_embedding and q8_add_layernorm: every product and sum is rounded by itself.
-__global__ void __launch_bounds__(kLnThreads, kEmbedLnCtasPerSm)
+__global__ void __launch_bounds__(kLnWarpThreads, kEmbedLnCtasPerSm)
 embed_layernorm_kernel(const int32_t *__restrict__ ids, int64_t T, int64_t S, const int8_t *__restrict__ word,
                        const float *__restrict__ S_word, int64_t V, const int8_t *__restrict__ pos,
                        const float *__restrict__ S_pos, int64_t P, const int8_t *__restrict__ typ,
@@ -243,8 +254,8 @@ embed_layernorm_kernel(const int32_t *__restrict__ ids, int64_t T, int64_t S, co
     const float Sq = out_q ? __ldg(S_q) : 1.0f;
     const float inv_w = __fdiv_rn(1.0f, __ldg(S_word)), inv_p = __fdiv_rn(1.0f, __ldg(S_pos)), inv_t = __fdiv_rn(1.0f, __ldg(S_typ));
     float am = 0.0f;
-    for (int64_t t = (int64_t)blockIdx.x * (kLnThreads / 32) + (threadIdx.x >> 5); t < T;
-         t += (int64_t)gridDim.x * (kLnThreads / 32)) {
+    for (int64_t t = (int64_t)blockIdx.x * (kLnWarpThreads / 32) + (threadIdx.x >> 5); t < T;
+         t += (int64_t)gridDim.x * (kLnWarpThreads / 32)) {
         const int64_t id = __ldg(ids + t), place = t % S;
         const bool id_ok = id >= 0 && id < V, place_ok = place < P;
         if (!(id_ok && place_ok) && lane == 0 && status) atomicOr(status, 1 << Q8_ERR_INDEX);  // a zero row, as in q8_embedding
@@ -273,7 +284,7 @@ embed_layernorm_kernel(const int32_t *__restrict__ ids, int64_t T, int64_t S, co
         normalise_row(v, s, lane, n4, H, eps, nullptr, nullptr, out ? reinterpret_cast<float4 *>(out) + t * n4 : nullptr,
                       out_q ? reinterpret_cast<uint32_t *>(out_q) + t * n4 : nullptr, Sq, am);
     }
-    if (amax) warp_fold_absmax(am, amax);
+    if (amax) cta_fold_absmax(am, amax);
 }
 
 // ------------------------------------------------------------------ self-attention, head dimension 64, no mask
@@ -435,6 +446,11 @@ __global__ void __launch_bounds__(256) attention_kernel(const float *__restrict_
 
 }  // namespace
 
+static unsigned warp_row_grid(int64_t rows)  // (rows fit 31 bits)
+{
+    return (unsigned)((rows + kLnWarpThreads / 32 - 1) / (kLnWarpThreads / 32));
+}
+
 cudaError_t launch_add_layernorm(const float *x, const float *r1, const float *r2, const float *gamma,
                                  const float *beta, float eps, int64_t rows, int64_t H, float *out, const float *S_q,
                                  int8_t *out_q, uint32_t *amax, cudaStream_t s)
@@ -444,18 +460,14 @@ cudaError_t launch_add_layernorm(const float *x, const float *r1, const float *r
     const bool vec = (H % 4 == 0) && H <= 4 * 4 * kLnThreads && al16(x) && al16(r1) && al16(r2) && al16(gamma) &&
                      al16(beta) && al16(out) && (reinterpret_cast<uintptr_t>(out_q) & 3u) == 0;
     if (vec && H <= 1024) {
-        const int64_t want = (rows + kLnThreads / 32 - 1) / (kLnThreads / 32);
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        auto launch = [&](auto kernel, int ctas_per_sm) {
-            const int64_t cap = (int64_t)(sms > 0 ? sms : 148) * ctas_per_sm;
-            return launch_overlapping_tail(kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kLnThreads), 0, s, x, r1, r2, gamma,
-                                           beta, eps, rows, H, out, S_q, out_q, amax);
+        auto launch = [&](auto kernel) {
+            return launch_overlapping_tail(kernel, dim3(warp_row_grid(rows)), dim3(kLnWarpThreads), 0, s, x, r1, r2, gamma, beta, eps, rows, H,
+                                           out, S_q, out_q, amax);
         };
-        if (H <= 256) return launch(add_layernorm_warp_kernel<2, 4>, 4);
-        if (H <= 512) return launch(add_layernorm_warp_kernel<4, 4>, 4);
-        if (H <= 768) return launch(add_layernorm_warp_kernel<6, 2>, 2);
-        return launch(add_layernorm_warp_kernel<8, 2>, 2);
+        if (H <= 256) return launch(add_layernorm_warp_kernel<2, 8>);
+        if (H <= 512) return launch(add_layernorm_warp_kernel<4, 8>);
+        if (H <= 768) return launch(add_layernorm_warp_kernel<6, 4>);
+        return launch(add_layernorm_warp_kernel<8, 4>);
     } else if (vec) {
         add_layernorm_vec_kernel<<<(unsigned)rows, kLnThreads, 0, s>>>(x, r1, r2, gamma, beta, eps, H, out, S_q, out_q, amax);
     } else {
@@ -478,11 +490,8 @@ cudaError_t launch_embed_layernorm(const int32_t *ids, int64_t T, int64_t S, con
                                    int32_t *status, cudaStream_t s)
 {
     if (T <= 0 || H <= 0) return cudaSuccess;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (T + kLnThreads / 32 - 1) / (kLnThreads / 32), cap = (int64_t)(sms > 0 ? sms : 148) * kEmbedLnCtasPerSm;
-    return launch_overlapping_tail(embed_layernorm_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kLnThreads), 0, s, ids, T,
-                                   S, word, S_word, V, pos, S_pos, P, typ, S_typ, eps, H, out, S_q, out_q, amax, status);
+    return launch_overlapping_tail(embed_layernorm_kernel, dim3(warp_row_grid(T)), dim3(kLnWarpThreads), 0, s, ids, T, S, word, S_word, V, pos,
+                                   S_pos, P, typ, S_typ, eps, H, out, S_q, out_q, amax, status);
 }
 
 cudaError_t launch_attention(const float *qkv, int64_t B, int64_t S, int64_t heads, float *ctx, const float *S_q,
