@@ -33,7 +33,7 @@ using namespace gemm_detail;
 
 constexpr int kAccStages = 2;      // TMEM accumulator double buffering
 // Epilogue warps per CTA (template parameter EW): 8 = two per TMEM lane quarter, each taking half of the tile's
-// columns; 16 = four per quarter.  A warp walks its 32-column blocks one after the other and every block is a
+// columns; 12 = three, 16 = four per quarter.  A warp walks its 32-column blocks one after the other and every block is a
 // chain of dependent latencies (TMEM load, arithmetic, staging, proxy fence, TMA store), so when the main loop is
 // short (small K) more warps shorten the epilogue; the extra staging buffers cost one stage of the operand ring.
 
@@ -544,6 +544,17 @@ cudaError_t launch_by_shape(int bn, int ctas, const GemmArgs &a, cudaStream_t s)
         // a short main loop (small K) leaves the epilogue on the critical path: give it twice the warps
         const bool wide_epilogue = g_force_epilogue_warps ? g_force_epilogue_warps == 16 : a.K <= 2048;
         return wide_epilogue ? launch_cfg<256, 2, 16>(a, s) : launch_cfg<256, 2, 8>(a, s);
+    }
+    // A one-CTA tile is mostly the only one of its CTA, so its epilogue is exposed: with GELU in it as many warps as there are 64-column
+    // (128: 32-column) shares, 1421 x 768 -> 3072 10.0 -> 9.2 us, 1000 x 768 -> 3072 8.3 -> 7.6, 509 x 1024 -> 4096 to Int8 7.1 -> 6.5;
+    // without GELU it is short enough and the staging buffers are better spent on the ring (4096 x 4096 -> 1024 17.9 for 19.7).
+    if (a.act == Q8_ACT_GELU) {
+        switch (bn) {
+            case 256: return launch_cfg<256, 1, 16>(a, s);
+            case 192: return launch_cfg<192, 1, 12>(a, s);
+            case 128: return launch_cfg<128, 1, 16>(a, s);
+            default: break;
+        }
     }
     switch (bn) {
         case 256: return launch_cfg<256, 1>(a, s);

@@ -607,6 +607,33 @@ def test_192_wide_tiles_bit_exact(M, N, K):
     assert np.array_equal(only.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(25.0)))
 
 
+@pytest.mark.parametrize("block_n", [128, 192, 256])
+@pytest.mark.parametrize("M,N,K", [(1, 32, 16), (130, 260, 272), (511, 1000, 1040), (40000, 384, 48)])
+def test_one_cta_tiles_in_every_output_mode(block_n, M, N, K):
+    """Tiles of one CTA have 12 or 16 epilogue warps with GELU and 8 without: ragged rows and columns, several tiles to a CTA, fp32, Int8,
+    both, and with the running maximum."""
+    X, W, b = synth.activation(M, K, 9460), synth.weight(N, K, 9461), synth.bias(N, 9462)
+    S_y = torch.full((1,), 25.0, device="cuda")
+    try:
+        q8.q8_tune_gemm_tile(block_n, 1)
+        for act in (0, 1):
+            info = check_linear(X, W, b, act)
+            assert (info["gemm_kernel"], info["block_n"], info["ctas"]) == (1, block_n, 1)
+            Wq, S_w = q8.q8_quantize_weight(dev(W))
+            Xd = dev(X)
+            Xq, S_x = q8.q8_quantize_activation(Xd)
+            Y = q8.q8_linear_q(Xq, S_x, Wq, S_w, dev(b), act)
+            want = o.quantize(Y.cpu().numpy(), np.float32(25.0))
+            assert np.array_equal(q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), act, S_y).cpu().numpy(), want)
+            Y2 = torch.empty_like(Y)
+            assert np.array_equal(q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), act, S_y, Y=Y2).cpu().numpy(), want)
+            word = torch.zeros(1, dtype=torch.int32, device="cuda")
+            Y3 = q8.q8_linear_dyn(Xd, Xd.abs().max().view(torch.int32).reshape(1), Wq, S_w, dev(b), act, y_absmax=word)
+            assert torch.equal(Y2, Y) and torch.equal(Y3, Y) and word.view(torch.float32).item() == Y.abs().max().item()
+    finally:
+        q8.q8_tune_gemm_tile(0, 0)
+
+
 # ------------------------------------------------------------------ the streaming passes at the ends of their runs
 @pytest.mark.parametrize("n", [1, 5, 511, 2047, 2048, 2049, 4 * 2048 - 3, 16 * 148 * 512 + 7])
 def test_streaming_passes_at_the_ends_of_their_runs(n):
