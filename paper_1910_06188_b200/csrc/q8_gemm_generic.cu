@@ -8,9 +8,10 @@
 // Operand rows that start anywhere cannot be fetched by TMA, and tcgen05 reads nothing but shared memory in TMA's layout, so
 // the tiles are staged by all threads (cp.async in pieces of 8 or 4 bytes where K and the pointers allow it, otherwise
 // 4-byte words shifted into place) and multiplied by mma.sync m16n8k32.s8 from rows of 64 bytes, 80 apart (ldmatrix without
-// bank conflicts).  1000 x 300 -> 1200 with GELU: 39.4 -> 10.0 us against byte loads and dp4a, 128 x 1000 -> 768 103 -> 8.0,
-// 2000 x 1004 -> 2000 330 -> 31 (259 TOPS), 4000 x 1001 -> 2000 558 -> 140.  Bound by the loads: instructions per piece
-// (with per-piece index arithmetic 13 us on the first shape) and, for rows that start at any byte, two words per piece.
+// bank conflicts).  1000 x 300 -> 1200 with GELU 7.6 us (39.4 with byte loads and dp4a), 128 x 1000 -> 768 6.2 (103),
+// 2000 x 1004 -> 2000 21 (330; 382 TOPS), 4000 x 1001 -> 2000 140 (558).  Bound by the loads: instructions per piece
+// (with per-piece index arithmetic 3 us more on the first shape) and, for rows that start at any byte, two words per piece; and, in
+// grids of one wave, by fetching the instructions themselves (PLAIN below).
 
 #include "q8_internal.cuh"
 
@@ -43,8 +44,16 @@ __device__ __forceinline__ void mma_s8(int32_t (&d)[4], const uint32_t (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// A call, not a copy for each of a thread's outputs: the epilogue runs once, so its instructions are all fetched for the first time.
+// (Four at a time, so that their chains overlap.)
+__device__ __noinline__ float4 gelu_of(float4 y) { return make_float4(gelu_erf(y.x), gelu_erf(y.y), gelu_erf(y.z), gelu_erf(y.w)); }
+
 // PIECE: bytes per cp.async (8 or 4: K and both pointers are multiples of it), or 1: rows start at any byte.
-template <int TILE, int PIECE>
+// PLAIN: one weight scale and nothing but the fp32 output; the other outputs are compiled out, whose skipped instructions are fetched
+// like the rest.  (Warps spent 40 % of 1000 x 300 -> 1200 waiting for instructions.  Without / with GELU, us: 8.0 / 9.9 -> 6.4 / 7.6, 128 x
+// 300 -> 768 5.1 / 6.0 -> 3.3 / 3.9, 2000 x 1004 -> 2000 30.9 / 32.1 -> 20.7 / 24.2, 3000 x 700 -> 3000 51.8 / 52.5 -> 30.6 / 36.7, 40000 x 100 -> 4 8.2 /
+// 11.2 -> 4.6 / 5.3.)
+template <int TILE, int PIECE, bool PLAIN>
 __global__ void __launch_bounds__(kThreads, TILE == 128 ? 2 : PIECE == 1 ? 4 : 3) gemm_generic_kernel(GemmArgs a)
 {
     using C = Shape<TILE>;
@@ -116,7 +125,7 @@ __global__ void __launch_bounds__(kThreads, TILE == 128 ? 2 : PIECE == 1 ? 4 : 3
     int32_t acc[C::kMT][C::kNT][4] = {};
     // what the epilogue needs travels under the main loop
     auto col = [&](int j, int c) { return n0 + wn + 8 * j + 2 * (lane & 3) + c; };
-    const float S_x = __ldg(a.S_x), S_w = __ldg(a.S_w), S_y = a.Yq ? __ldg(a.S_y) : 1.0f;
+    const float S_x = __ldg(a.S_x), S_w = __ldg(a.S_w), S_y = !PLAIN && a.Yq ? __ldg(a.S_y) : 1.0f;
     float bias[C::kNT][2];
 #pragma unroll
     for (int j = 0; j < C::kNT; ++j)
@@ -167,6 +176,36 @@ __global__ void __launch_bounds__(kThreads, TILE == 128 ? 2 : PIECE == 1 ? 4 : 3
         }
     }
 
+    if (PLAIN) {
+        const float S_out = __fmul_rn(S_x, S_w), inv = __fdiv_rn(1.0f, S_out);
+#pragma unroll
+        for (int j = 0; j < C::kNT; ++j) {
+            const int32_t b0 = a.bias ? quantize_bias(bias[j][0], S_out) : 0, b1 = a.bias ? quantize_bias(bias[j][1], S_out) : 0;
+            const int64_t n = col(j, 0);
+            if (n >= a.N) continue;
+            float *y = a.Y + (m0 + wm + (lane >> 2)) * a.N + n;
+#pragma unroll
+            for (int i = 0; i < C::kMT; ++i) {
+                const int m = wm + 16 * i + (lane >> 2);
+                if (m >= x_rows) continue;
+                auto value = [&](int e, int32_t b_q) { return __fmul_rn(__int2float_rn(add_wrap(acc[i][j][e], b_q)), inv); };
+                float4 v = make_float4(value(0, b0), value(1, b1), value(2, b0), value(3, b1));  // rows m and m + 8
+                if (a.act == Q8_ACT_GELU) v = gelu_of(v);
+                float *to = y + 16 * i * a.N, *to8 = to + 8 * a.N;
+                const bool second = m + 8 < x_rows;
+                if (pairs) {
+                    *reinterpret_cast<float2 *>(to) = make_float2(v.x, v.y);
+                    if (second) *reinterpret_cast<float2 *>(to8) = make_float2(v.z, v.w);
+                } else {
+                    to[0] = v.x;
+                    if (n + 1 < a.N) to[1] = v.y;
+                    if (second) to8[0] = v.z;
+                    if (second && n + 1 < a.N) to8[1] = v.w;
+                }
+            }
+        }
+        return;
+    }
     float am = 0.0f;
 #pragma unroll
     for (int j = 0; j < C::kNT; ++j) {
@@ -200,8 +239,8 @@ __global__ void __launch_bounds__(kThreads, TILE == 128 ? 2 : PIECE == 1 ? 4 : 3
     if (a.y_absmax) warp_fold_absmax(am, a.y_absmax);
 }
 
-template <int TILE, int PIECE>
-cudaError_t launch_shape(const GemmArgs &a, cudaStream_t s)
+template <int TILE, int PIECE, bool PLAIN>
+cudaError_t launch_form(const GemmArgs &a, cudaStream_t s)
 {
     using C = Shape<TILE>;
     static bool attr_set[64] = {};  // opt-in shared-memory size: per device, per function
@@ -210,19 +249,26 @@ cudaError_t launch_shape(const GemmArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr_set[dev]) {
-        e = cudaFuncSetAttribute(gemm_generic_kernel<TILE, PIECE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+        e = cudaFuncSetAttribute(gemm_generic_kernel<TILE, PIECE, PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
     dim3 grid((unsigned)((a.M + TILE - 1) / TILE), (unsigned)((a.N + TILE - 1) / TILE));
     if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
-    e = launch_overlapping_tail(gemm_generic_kernel<TILE, PIECE>, grid, dim3(kThreads), C::kSmemBytes, s, a);
+    e = launch_overlapping_tail(gemm_generic_kernel<TILE, PIECE, PLAIN>, grid, dim3(kThreads), C::kSmemBytes, s, a);
     LaunchInfo &li = last_launch_info();
     li.gemm_kernel = 2;
     li.block_n = TILE;
     li.grid = (int)(grid.x * grid.y);
     li.launches += 1;
     return e;
+}
+
+template <int TILE, int PIECE>
+cudaError_t launch_shape(const GemmArgs &a, cudaStream_t s)
+{
+    const bool plain = a.Yq == nullptr && a.dbg_acc == nullptr && a.y_absmax == nullptr && a.w_seg <= 0;
+    return plain ? launch_form<TILE, PIECE, true>(a, s) : launch_form<TILE, PIECE, false>(a, s);
 }
 
 }  // namespace

@@ -663,3 +663,20 @@ def test_fake_quantise_quotient_is_rounded_to_nearest(S):
         want = o.quantize(x, S).astype(np.float32) / S
     got = q8.q8_fake_quantize(dev(x), dev(np.array([S], np.float32))).cpu().numpy()
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (65, 66, 300), (100, 130, 301), (64, 1201, 72), (1000, 1200, 300), (2050, 1930, 100),
+                                   (2049, 1931, 104), (3000, 700, 77), (40000, 4, 100)])
+def test_generic_gemm_with_and_without_the_other_outputs(M, N, K):
+    """A call that wants the fp32 output only has its own form of the generic kernel: same bits as the one that also copies the Int32
+    accumulator, for pieces of 8, 4 and 1 bytes, both tiles, ragged edges, odd widths and an output that takes no pairs."""
+    X, W, b = dev(synth.activation(M, K, 9700)), dev(synth.weight(N, K, 9701)), dev(synth.bias(N, 9702))
+    Wq, S_w = q8.q8_quantize_weight(W)
+    ws, acc = q8.new_workspace(M, N, K), torch.empty((M, N), dtype=torch.int32, device="cuda")
+    for act in (0, 1):
+        for bias in (b, None):
+            want = q8.q8_linear_generic(X, Wq, S_w, None, bias, act, workspace=ws, dbg_acc=acc)
+            assert torch.equal(q8.q8_linear_generic(X, Wq, S_w, None, bias, act, workspace=ws), want)
+            room = torch.full((M * N + 3,), 5.0, device="cuda")
+            q8.q8_linear_generic(X, Wq, S_w, None, bias, act, Y=room[1:1 + M * N].view(M, N), workspace=ws)
+            assert torch.equal(room[1:1 + M * N].view(M, N), want) and room[0] == 5.0 and (room[1 + M * N:] == 5.0).all()
