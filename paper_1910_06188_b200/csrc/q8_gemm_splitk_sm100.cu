@@ -106,6 +106,8 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     cluster_arrive();  // this CTA has started.  Every role waits for the others' arrivals off the critical path (and when aborting)
+    if (warp == 3 && lane == 0 && m0 == 0)  // the weights on their way into L2 while the kernel before this one still runs
+        for (int kb = kb0; kb < kb1; ++kb) tma_prefetch_2d(&tmap_w, kb * BLOCK_K, (int32_t)n0);
     grid_dependency_release_next(true);  // small by construction: one tile per cluster
     grid_dependency_wait();
 
