@@ -359,7 +359,7 @@ attention_tc_kernel(const float *__restrict__ qkv, int S, int64_t H, float *__re
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
-    grid_dependency_release_next(gridDim.x * gridDim.y * gridDim.z <= 600u);  // up to ~2 waves of CTAs count as small
+    grid_dependency_release_next(true);
     grid_dependency_wait();  // the set-up above may overlap the tail of the kernel that produced qkv
 
     bool ok = true;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kLnWarpThreads, CTAS_PER_SM) add_layernorm_war
                                                                         const float *__restrict__ S_q,
                                                                         int8_t *__restrict__ out_q, uint32_t *__restrict__ amax)
 {
-    grid_dependency_release_next(rows * H <= kSmallProblemElems);
+    grid_dependency_release_next(true);
     grid_dependency_wait();  // launched so that its start may overlap the tail of the kernel before it
     const int lane = threadIdx.x & 31;
     const int n4 = (int)(H >> 2);
@@ -247,7 +247,7 @@ embed_layernorm_kernel(const int32_t *__restrict__ ids, int64_t T, int64_t S, co
                        const float *__restrict__ S_typ, float eps, int64_t H, float *__restrict__ out,
                        const float *__restrict__ S_q, int8_t *__restrict__ out_q, uint32_t *__restrict__ amax, int32_t *status)
 {
-    grid_dependency_release_next(T * H <= kSmallProblemElems);
+    grid_dependency_release_next(true);
     grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int n4 = (int)(H >> 2);
