@@ -541,12 +541,15 @@ cudaError_t launch_cfg_impl(const GemmArgs &a, cudaStream_t s)
     return e;
 }
 
-// Relative time of one 32-deep K step of a 128 x bn tile on one SM: the tensor pipe needs bn/2 cycles,
-// reading the (128 + bn) x 32 operand bytes from shared memory needs (128 + bn)/4; plus a fixed per-step cost.
-double tile_step_cost(int bn)
+// Cycles of one-CTA tiles of bn columns, as many on an SM one after the other as `rounds`: a 32-deep K step (the tensor pipe needs
+// bn / 2, reading the (128 + bn) x 32 operand bytes from shared memory (128 + bn) / 4, the loads under both the rest), the way into
+// and out of a tile, and the last tile's epilogue, which nothing overlaps.  The numbers are fitted to times of 190 layers (64 to 8192
+// rows, K = 256 to 4096, all widths).  Without the last term one round of 256-wide tiles was preferred to two of 128: 1421 x 768 ->
+// 3072 with GELU 9.5 us for 8.9, 2048 x 768 -> 2304 8.6 for 8.1, 5000 x 768 -> 768 8.35 for 7.95, 6500 x 256 -> 512 7.05 for 6.25.
+double tile_cost(int bn, int64_t rounds, int64_t K)
 {
-    const double mma = bn / 2.0, smem = (128 + bn) / 4.0;
-    return (mma > smem ? mma : smem) + 8.0;
+    const double step = bn == 256 ? 160.0 : bn == 192 ? 125.0 : bn == 128 ? 90.0 : bn == 64 ? 64.0 : 50.0;
+    return (double)rounds * (step * (double)K / 32.0 + 500.0) + 10.0 * bn;
 }
 
 cudaError_t launch_by_shape(int bn, int ctas, const GemmArgs &a, cudaStream_t s)
@@ -601,10 +604,13 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
     if (g_force_ctas == 2 || (g_force_ctas == 1 && g_force_block_n != 0))
         return launch_by_shape(g_force_block_n, g_force_ctas, a, s);
     const int sms = sm_count();
-    // Large problems: CTA pairs on 256 x 256 tiles (least operand traffic per MAC) once every pair has work.
+    // Large problems: CTA pairs on 256 x 256 tiles (least operand traffic per MAC) once every pair has work.  Not for a round and up to a
+    // half of a short K, whose second round leaves most pairs idle: 8192 x 768 -> 768 11.05 us with pairs, 10.6 with one-CTA tiles,
+    // 2048 x 768 -> 3072 with GELU 11.85 / 11.3, 3200 x 512 -> 2048 11.4 / 10.4 (but 2048 x 1024 -> 3072 11.0 / 11.15).
     const int64_t pair_tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
-    if (a.N >= 192 && a.M > 128 && pair_tiles >= sms / 2) return launch_by_shape(256, 2, a, s);
-    // Otherwise single-CTA tiles: pick the width that minimises (waves over the SMs) x (time of one tile).
+    const bool second_round_thin = a.K <= 768 && 2 * pair_tiles > sms && 4 * pair_tiles <= 3 * sms;
+    if (a.N >= 192 && a.M > 128 && pair_tiles >= sms / 2 && !second_round_thin) return launch_by_shape(256, 2, a, s);
+    // Otherwise single-CTA tiles of the cheapest width.
     const int64_t tm = (a.M + BLOCK_M - 1) / BLOCK_M;
     int best = 32;
     double best_cost = 0.0;
@@ -614,7 +620,7 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
     for (int bn : {256, 192, 128, 64, 32}) {
         if (bn > 32 && bn / 2 >= a.N) continue;  // more than half of the tile would be padding
         const int64_t tiles = tm * ((a.N + bn - 1) / bn);
-        const double cost = (double)((tiles + sms - 1) / sms) * tile_step_cost(bn);
+        const double cost = tile_cost(bn, (tiles + sms - 1) / sms, a.K);
         if (best_cost == 0.0 || cost < best_cost) {
             best = bn;
             best_cost = cost;
@@ -627,6 +633,8 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
         if (4 * narrow_tiles <= sms) return launch_gemm_splitk(a, true, s);
         if (best == 32 && 2 * tm * ((a.N + 63) / 64) <= sms) return launch_gemm_splitk(a, false, s);
     }
+    // One round of the widest tiles with a long K: the pair does the same with fewer operand bytes (4096 x 4096 -> 1024 18.1 us / 17.2).
+    if (best == 256 && a.K >= 2048 && a.M > 128) return launch_by_shape(256, 2, a, s);
     return launch_by_shape(best, 1, a, s);
 }
 
