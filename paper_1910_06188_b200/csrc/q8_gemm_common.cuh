@@ -45,6 +45,18 @@ __device__ __forceinline__ void gelu_fast_x2(uint64_t y2, float &out_lo, float &
     unpack_f32x2(r, out_lo, out_hi);
 }
 
+// quantize_pack4() where no integer is below -127: two pairs, their products with S one packed instruction each.
+__device__ __forceinline__ uint32_t quantize_pack4_unclamped(float a, float b, float c, float d, float S)
+{
+    const uint64_t S2 = pack_f32x2(S, S);
+    unpack_f32x2(mul_f32x2(pack_f32x2(a, b), S2), a, b);
+    unpack_f32x2(mul_f32x2(pack_f32x2(c, d), S2), c, d);
+    uint32_t hi, r;
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(__float2int_rn(d)), "r"(__float2int_rn(c)), "r"(0));
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(__float2int_rn(b)), "r"(__float2int_rn(a)), "r"(hi));
+    return r;
+}
+
 // ------------------------------------------------------------------ epilogue of one warp
 // The warp owns 32 accumulator rows (its TMEM lane quarter) x COLS columns of the tile and walks
 // them in 32-column blocks: tcgen05.ld (one row per lane) -> + b_q -> int-to-float ->
@@ -59,12 +71,12 @@ __device__ __forceinline__ void gelu_fast_x2(uint64_t y2, float &out_lo, float &
 // warp walks four blocks per tile; with two blocks per warp it measured 1 % slower).
 // BIAS_IN_STAGE: bq_s points into `stage`, so a staged fp32 block must have been read by its TMA store before the
 // next block's bias values are exchanged there.
-// OUT: which outputs the instantiation can write.  kOutPlain: the fp32 Y only; kOutInt8: the Int8 copy only (the
-// fused FFN1 of a forward whose next layer is quantised); kOutFull: whatever the call asks for (fp32, Int8, the
+// OUT: which outputs the instantiation can write.  kOutPlain: the fp32 Y only; kOutInt8 and, with GELU, kOutInt8Gelu: the Int8 copy
+// only (the fused FFN1 of a forward whose next layer is quantised); kOutFull: whatever the call asks for (fp32, Int8, the
 // debug copy of the accumulator).  Compiling the other paths out keeps the 16-warp kernel (96 registers per thread)
 // free of spills; a spilled value is reloaded from local memory in every block, and under the main loop's traffic
 // that load is not a cache hit.
-constexpr int kOutPlain = 0, kOutFull = 1, kOutDirect = 2, kOutInt8 = 3;
+constexpr int kOutPlain = 0, kOutFull = 1, kOutDirect = 2, kOutInt8 = 3, kOutInt8Gelu = 4;
 template <int COLS, bool ABSMAX, bool PREFETCH, bool BIAS_IN_STAGE, int OUT, typename Release>
 __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorMap *tmap_y, bool tma_store,
                                               const CUtensorMap *tmap_yq, bool yq_tma, uint32_t taddr, int64_t row0,
@@ -75,7 +87,8 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
     constexpr int NCHUNK = COLS / 32;  // compile-time maximum; this tile has nch <= NCHUNK blocks (warp-uniform)
     const int64_t row = row0 + lane;
     const bool row_ok = row < a.M;
-    constexpr bool kHasY = OUT != kOutInt8, kHasYq = OUT == kOutFull || OUT == kOutInt8, kHasDbg = OUT == kOutFull;
+    constexpr bool kInt8Only = OUT == kOutInt8 || OUT == kOutInt8Gelu;
+    constexpr bool kHasY = !kInt8Only, kHasYq = OUT == kOutFull || kInt8Only, kHasDbg = OUT == kOutFull;
     const float S_y = (kHasYq && a.Yq != nullptr) ? __ldg(a.S_y) : 1.0f;
     const bool yq_vec = ((a.N & 15) == 0) && ((reinterpret_cast<uintptr_t>(a.Yq) & 15u) == 0);
     // Int8-only output of a full-width tile: the warp's 32 x COLS bytes are collected in its staging buffer (free,
@@ -85,6 +98,10 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
     const bool yq_staged = kHasYq && kYqStageable && yq_tma && nch == NCHUNK;
     const int yq_xor = COLS == 128 ? (lane & 7) : ((lane >> 1) & 3);  // 128-byte / 64-byte swizzle of row `lane`
     bool yq_pending = false;
+    // GELU is never below -0.17, so its integers need no lower clamp at scales below 127 / 0.17 = 747.  Such an epilogue is bound by
+    // its instructions: with neither the clamp nor scalar products (quantize_pack4_unclamped()) 24576 x 1024 -> 4096 97.7 -> 91.0 us, 8192 x 768
+    // -> 3072 28.7 -> 25.4, 4096 x 768 -> 3072 17.5 -> 15.7.
+    const bool above_low_clamp = OUT == kOutInt8Gelu && S_y < 700.0f;
 
     // Everything after the TMEM load, for the 32-column block ci held in v, up to and including the staging of the
     // fp32 block in shared memory.  Returns the first column of the block when a staged fp32 block now waits for its
@@ -112,7 +129,7 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
             for (int j = 0; j < 32; ++j)
                 if (nb + j < a.N) drow[j] = (int32_t)v[j];
         }
-        if (a.act == Q8_ACT_GELU) {
+        if (OUT == kOutInt8Gelu || (OUT != kOutInt8 && a.act == Q8_ACT_GELU)) {
             const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
@@ -165,16 +182,16 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
                 yq_pending = true;
             }
             uint8_t *srow = stage + lane * COLS;
-            *reinterpret_cast<uint4 *>(srow + (((2 * ci) ^ yq_xor) << 4)) = make_uint4(
-                quantize_pack4(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]), __uint_as_float(v[3]), S_y),
-                quantize_pack4(__uint_as_float(v[4]), __uint_as_float(v[5]), __uint_as_float(v[6]), __uint_as_float(v[7]), S_y),
-                quantize_pack4(__uint_as_float(v[8]), __uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]), S_y),
-                quantize_pack4(__uint_as_float(v[12]), __uint_as_float(v[13]), __uint_as_float(v[14]), __uint_as_float(v[15]), S_y));
-            *reinterpret_cast<uint4 *>(srow + (((2 * ci + 1) ^ yq_xor) << 4)) = make_uint4(
-                quantize_pack4(__uint_as_float(v[16]), __uint_as_float(v[17]), __uint_as_float(v[18]), __uint_as_float(v[19]), S_y),
-                quantize_pack4(__uint_as_float(v[20]), __uint_as_float(v[21]), __uint_as_float(v[22]), __uint_as_float(v[23]), S_y),
-                quantize_pack4(__uint_as_float(v[24]), __uint_as_float(v[25]), __uint_as_float(v[26]), __uint_as_float(v[27]), S_y),
-                quantize_pack4(__uint_as_float(v[28]), __uint_as_float(v[29]), __uint_as_float(v[30]), __uint_as_float(v[31]), S_y));
+            auto quantise = [&](auto pack4) {
+                uint32_t w[8];
+#pragma unroll
+                for (int g = 0; g < 8; ++g)
+                    w[g] = pack4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]), __uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3]));
+                *reinterpret_cast<uint4 *>(srow + (((2 * ci) ^ yq_xor) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4 *>(srow + (((2 * ci + 1) ^ yq_xor) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+            };
+            if (above_low_clamp) quantise([&](float x, float y, float z, float w) { return quantize_pack4_unclamped(x, y, z, w, S_y); });
+            else quantise([&](float x, float y, float z, float w) { return quantize_pack4(x, y, z, w, S_y); });
         }
         if (!kHasY || a.Y == nullptr) return -1;
         if (tma_store) {

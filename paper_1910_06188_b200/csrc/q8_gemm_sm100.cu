@@ -70,7 +70,7 @@ struct Cfg {
 
 // ------------------------------------------------------------------ the kernel
 // OUT: what the epilogue writes.  kOutPlain: fp32 Y, staged in shared memory and stored by TMA (or by the lanes
-// when Y is not aligned for that); kOutInt8: only the Int8 copy; kOutFull: fp32 and / or Int8 and / or the debug copy
+// when Y is not aligned for that); kOutInt8, kOutInt8Gelu: only the Int8 copy; kOutFull: fp32 and / or Int8 and / or the debug copy
 // of the accumulator, as asked for; kOutDirect: fp32 Y stored straight from the accumulator fragments.  Separate
 // instantiations, so that a layer does not carry the registers of the paths it does not take.
 
@@ -427,7 +427,8 @@ template <int BLOCK_N, int CTAS, int EW, bool ABSMAX>
 cudaError_t launch_cfg_out(const GemmArgs &a, cudaStream_t s)
 {
     if (a.Yq != nullptr && a.Y == nullptr && a.dbg_acc == nullptr)
-        return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8>(a, s);
+        return a.act == Q8_ACT_GELU ? launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8Gelu>(a, s)
+                                    : launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8>(a, s);
     if (a.Yq != nullptr || a.dbg_acc != nullptr) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutFull>(a, s);
     if constexpr (CTAS == 2) {
         if (wants_direct_store<CTAS, EW>(a)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutDirect>(a, s);

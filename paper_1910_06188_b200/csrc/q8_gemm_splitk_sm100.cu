@@ -269,6 +269,7 @@ cudaError_t launch_split(const GemmArgs &a, cudaStream_t s)
 {
     const bool int8_only = a.Yq != nullptr && a.Y == nullptr && a.dbg_acc == nullptr, plain = a.Yq == nullptr && a.dbg_acc == nullptr;
     if (a.y_absmax != nullptr) return plain ? launch_out<ROWS, true, kOutPlain>(a, s) : launch_out<ROWS, true, kOutFull>(a, s);
+    if (int8_only && a.act == Q8_ACT_GELU) return launch_out<ROWS, false, kOutInt8Gelu>(a, s);
     if (int8_only) return launch_out<ROWS, false, kOutInt8>(a, s);
     return plain ? launch_out<ROWS, false, kOutPlain>(a, s) : launch_out<ROWS, false, kOutFull>(a, s);
 }
