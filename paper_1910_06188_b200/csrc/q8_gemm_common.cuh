@@ -71,12 +71,20 @@ __device__ __forceinline__ uint32_t quantize_pack4_unclamped(float a, float b, f
 // warp walks four blocks per tile; with two blocks per warp it measured 1 % slower).
 // BIAS_IN_STAGE: bq_s points into `stage`, so a staged fp32 block must have been read by its TMA store before the
 // next block's bias values are exchanged there.
-// OUT: which outputs the instantiation can write.  kOutPlain: the fp32 Y only; kOutInt8 and, with GELU, kOutInt8Gelu: the Int8 copy
+// OUT: which outputs the instantiation can write.  kOutPlain: the fp32 Y only; kOutInt8: the Int8 copy
 // only (the fused FFN1 of a forward whose next layer is quantised); kOutFull: whatever the call asks for (fp32, Int8, the
 // debug copy of the accumulator).  Compiling the other paths out keeps the 16-warp kernel (96 registers per thread)
 // free of spills; a spilled value is reloaded from local memory in every block, and under the main loop's traffic
 // that load is not a cache hit.
-constexpr int kOutPlain = 0, kOutFull = 1, kOutDirect = 2, kOutInt8 = 3, kOutInt8Gelu = 4;
+// All but kOutFull are for one activation: plus kOutGelu with GELU, else without.
+constexpr int kOutPlain = 0, kOutFull = 1, kOutDirect = 2, kOutInt8 = 3, kOutGelu = 4;
+template <int OUT>
+constexpr int kOutKind = OUT & 3;
+template <int OUT>
+__device__ __forceinline__ bool has_gelu(const GemmArgs &a)
+{
+    return kOutKind<OUT> == kOutFull ? a.act == Q8_ACT_GELU : (OUT & kOutGelu) != 0;
+}
 template <int COLS, bool ABSMAX, bool PREFETCH, bool BIAS_IN_STAGE, int OUT, typename Release>
 __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorMap *tmap_y, bool tma_store,
                                               const CUtensorMap *tmap_yq, bool yq_tma, uint32_t taddr, int64_t row0,
@@ -87,8 +95,8 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
     constexpr int NCHUNK = COLS / 32;  // compile-time maximum; this tile has nch <= NCHUNK blocks (warp-uniform)
     const int64_t row = row0 + lane;
     const bool row_ok = row < a.M;
-    constexpr bool kInt8Only = OUT == kOutInt8 || OUT == kOutInt8Gelu;
-    constexpr bool kHasY = !kInt8Only, kHasYq = OUT == kOutFull || kInt8Only, kHasDbg = OUT == kOutFull;
+    constexpr int kKind = kOutKind<OUT>;
+    constexpr bool kHasY = kKind != kOutInt8, kHasYq = kKind == kOutFull || kKind == kOutInt8, kHasDbg = kKind == kOutFull;
     const float S_y = (kHasYq && a.Yq != nullptr) ? __ldg(a.S_y) : 1.0f;
     const bool yq_vec = ((a.N & 15) == 0) && ((reinterpret_cast<uintptr_t>(a.Yq) & 15u) == 0);
     // Int8-only output of a full-width tile: the warp's 32 x COLS bytes are collected in its staging buffer (free,
@@ -101,7 +109,7 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
     // GELU is never below -0.17, so its integers need no lower clamp at scales below 127 / 0.17 = 747.  Such an epilogue is bound by
     // its instructions: with neither the clamp nor scalar products (quantize_pack4_unclamped()) 24576 x 1024 -> 4096 97.7 -> 91.0 us, 8192 x 768
     // -> 3072 28.7 -> 25.4, 4096 x 768 -> 3072 17.5 -> 15.7.
-    const bool above_low_clamp = OUT == kOutInt8Gelu && S_y < 700.0f;
+    const bool above_low_clamp = OUT == (kOutInt8 | kOutGelu) && S_y < 700.0f;
 
     // Everything after the TMEM load, for the 32-column block ci held in v, up to and including the staging of the
     // fp32 block in shared memory.  Returns the first column of the block when a staged fp32 block now waits for its
@@ -129,7 +137,7 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
             for (int j = 0; j < 32; ++j)
                 if (nb + j < a.N) drow[j] = (int32_t)v[j];
         }
-        if (OUT == kOutInt8Gelu || (OUT != kOutInt8 && a.act == Q8_ACT_GELU)) {
+        if (has_gelu<OUT>(a)) {
             const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
@@ -245,7 +253,7 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
 // stores its pairs straight to Y (8-byte stores, every sector written whole by one instruction).  No proxy fence,
 // no TMA store, no staging buffer to wait for.  Needs an even N and an 8-byte aligned Y; like the plain form of the
 // staged epilogue it writes Y only (a call that wants the Int8 or the debug copy takes the staged path).
-template <int COLS, bool ABSMAX, typename Release>
+template <int COLS, bool ABSMAX, int OUT, typename Release>
 __device__ __forceinline__ void epilogue_warp_direct(const GemmArgs &a, uint32_t taddr, int64_t row0, int64_t col0,
                                                      const int32_t (&bqv)[COLS / 32], const float (&invv)[COLS / 32],
                                                      int32_t *bq_s, int lane, int nch, Release release, float &absmax_run)
@@ -276,7 +284,7 @@ __device__ __forceinline__ void epilogue_warp_direct(const GemmArgs &a, uint32_t
                 v[k + 1] = (uint32_t)add_wrap((int32_t)v[k + 1], b.y);
             }
         }
-        if (a.act == Q8_ACT_GELU) {
+        if (has_gelu<OUT>(a)) {
             const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {

@@ -70,7 +70,7 @@ struct Cfg {
 
 // ------------------------------------------------------------------ the kernel
 // OUT: what the epilogue writes.  kOutPlain: fp32 Y, staged in shared memory and stored by TMA (or by the lanes
-// when Y is not aligned for that); kOutInt8, kOutInt8Gelu: only the Int8 copy; kOutFull: fp32 and / or Int8 and / or the debug copy
+// when Y is not aligned for that); kOutInt8: only the Int8 copy; kOutFull: fp32 and / or Int8 and / or the debug copy
 // of the accumulator, as asked for; kOutDirect: fp32 Y stored straight from the accumulator fragments.  Separate
 // instantiations, so that a layer does not carry the registers of the paths it does not take.
 
@@ -368,8 +368,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     else mbar_arrive(smem_u32(tmem_empty_bar + as));
                 }
             };
-            if (active && OUT == kOutDirect)
-                epilogue_warp_direct<C::kColsPerWarp, ABSMAX>(
+            if (active && kOutKind<OUT> == kOutDirect)
+                epilogue_warp_direct<C::kColsPerWarp, ABSMAX, OUT>(
                     a, tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(as * BLOCK_N + col_off),
                     m0 + quarter * 32, n0 + col_off, bqv, invv, bq_s, lane, cpw / 32, release, absmax_run);
             else if (active)
@@ -423,17 +423,27 @@ bool wants_direct_store(const GemmArgs &a)
 
 // The layer that also reports max|y| (Sec. 4.1 chained dynamically) and each output mode run their own
 // instantiation of the kernel.
+template <int BLOCK_N, int CTAS, int EW, bool ABSMAX, int GELU>
+cudaError_t launch_cfg_act(const GemmArgs &a, cudaStream_t s)
+{
+    if (a.Yq != nullptr && a.Y == nullptr) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8 | GELU>(a, s);
+    if constexpr (CTAS == 2) {
+        if (wants_direct_store<CTAS, EW>(a)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutDirect | GELU>(a, s);
+    }
+    return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutPlain | GELU>(a, s);
+}
 template <int BLOCK_N, int CTAS, int EW, bool ABSMAX>
 cudaError_t launch_cfg_out(const GemmArgs &a, cudaStream_t s)
 {
-    if (a.Yq != nullptr && a.Y == nullptr && a.dbg_acc == nullptr)
-        return a.act == Q8_ACT_GELU ? launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8Gelu>(a, s)
-                                    : launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8>(a, s);
-    if (a.Yq != nullptr || a.dbg_acc != nullptr) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutFull>(a, s);
-    if constexpr (CTAS == 2) {
-        if (wants_direct_store<CTAS, EW>(a)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutDirect>(a, s);
+    if (a.dbg_acc != nullptr || (a.Yq != nullptr && a.Y != nullptr)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutFull>(a, s);
+    // (launch_by_shape() has one-CTA tiles of 128 columns and more for each activation)
+    if constexpr (CTAS == 2 || BLOCK_N < 128 || EW > 8) {
+        if (a.act == Q8_ACT_GELU) return launch_cfg_act<BLOCK_N, CTAS, EW, ABSMAX, kOutGelu>(a, s);
     }
-    return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutPlain>(a, s);
+    if constexpr (CTAS == 2 || BLOCK_N < 128 || EW == 8) {
+        if (a.act != Q8_ACT_GELU) return launch_cfg_act<BLOCK_N, CTAS, EW, ABSMAX, 0>(a, s);
+    }
+    return cudaErrorInvalidValue;
 }
 template <int BLOCK_N, int CTAS, int EW = 8>
 cudaError_t launch_cfg(const GemmArgs &a, cudaStream_t s)
@@ -501,7 +511,7 @@ cudaError_t launch_cfg_impl(const GemmArgs &a, cudaStream_t s)
         tw4 = tw;
     }
     // the TMA store needs a 16-byte aligned base and row pitch; otherwise lanes store their rows directly
-    int tma_store = OUT != kOutDirect && a.Y != nullptr && ((a.N & 3) == 0) &&
+    int tma_store = kOutKind<OUT> != kOutDirect && a.Y != nullptr && ((a.N & 3) == 0) &&
                     ((reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0);
     if (tma_store) {
         if (!make_tmap_out(&ty, a.Y, a.M, a.N)) return cudaErrorInvalidValue;
@@ -537,7 +547,7 @@ cudaError_t launch_cfg_impl(const GemmArgs &a, cudaStream_t s)
     li.epilogue_warps = EW;
     li.grid = units * CTAS;
     li.tail_split = split;
-    li.store_mode = OUT == kOutDirect ? 2 : tma_store;
+    li.store_mode = kOutKind<OUT> == kOutDirect ? 2 : tma_store;
     li.launches += 1;
     return e;
 }

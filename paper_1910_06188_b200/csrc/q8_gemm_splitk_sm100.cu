@@ -268,10 +268,12 @@ template <bool ROWS>
 cudaError_t launch_split(const GemmArgs &a, cudaStream_t s)
 {
     const bool int8_only = a.Yq != nullptr && a.Y == nullptr && a.dbg_acc == nullptr, plain = a.Yq == nullptr && a.dbg_acc == nullptr;
-    if (a.y_absmax != nullptr) return plain ? launch_out<ROWS, true, kOutPlain>(a, s) : launch_out<ROWS, true, kOutFull>(a, s);
-    if (int8_only && a.act == Q8_ACT_GELU) return launch_out<ROWS, false, kOutInt8Gelu>(a, s);
-    if (int8_only) return launch_out<ROWS, false, kOutInt8>(a, s);
-    return plain ? launch_out<ROWS, false, kOutPlain>(a, s) : launch_out<ROWS, false, kOutFull>(a, s);
+    const bool gelu = a.act == Q8_ACT_GELU;
+    if (a.y_absmax != nullptr && plain) return gelu ? launch_out<ROWS, true, kOutPlain | kOutGelu>(a, s) : launch_out<ROWS, true, kOutPlain>(a, s);
+    if (a.y_absmax != nullptr) return launch_out<ROWS, true, kOutFull>(a, s);
+    if (int8_only) return gelu ? launch_out<ROWS, false, kOutInt8 | kOutGelu>(a, s) : launch_out<ROWS, false, kOutInt8>(a, s);
+    if (plain) return gelu ? launch_out<ROWS, false, kOutPlain | kOutGelu>(a, s) : launch_out<ROWS, false, kOutPlain>(a, s);
+    return launch_out<ROWS, false, kOutFull>(a, s);
 }
 
 }  // namespace
