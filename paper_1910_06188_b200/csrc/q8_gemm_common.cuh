@@ -77,6 +77,9 @@ __device__ __forceinline__ uint32_t quantize_pack4_unclamped(float a, float b, f
 // free of spills; a spilled value is reloaded from local memory in every block, and under the main loop's traffic
 // that load is not a cache hit.
 // All but kOutFull are for one activation: plus kOutGelu with GELU, else without.
+// ROLLED: an fp32 block that TMA does not take leaves through the staging buffer in a loop over its rows, else column by column in line.
+// Tiles of one CTA and 64 columns or more: with it the encoder's 32-wide tiles took 0.4 % longer (1 x 128: 204.6 -> 205.4 us) and the
+// pairs' plain fp32 epilogue 2-4 % (8192 x 1024 -> 1024 12.7 -> 13.2), although neither runs it: the compiler orders the rest differently.
 constexpr int kOutPlain = 0, kOutFull = 1, kOutDirect = 2, kOutInt8 = 3, kOutGelu = 4;
 template <int OUT>
 constexpr int kOutKind = OUT & 3;
@@ -85,7 +88,7 @@ __device__ __forceinline__ bool has_gelu(const GemmArgs &a)
 {
     return kOutKind<OUT> == kOutFull ? a.act == Q8_ACT_GELU : (OUT & kOutGelu) != 0;
 }
-template <int COLS, bool ABSMAX, bool PREFETCH, bool BIAS_IN_STAGE, int OUT, typename Release>
+template <int COLS, bool ABSMAX, bool PREFETCH, bool BIAS_IN_STAGE, bool ROLLED, int OUT, typename Release>
 __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorMap *tmap_y, bool tma_store,
                                               const CUtensorMap *tmap_yq, bool yq_tma, uint32_t taddr, int64_t row0,
                                               int64_t col0, const int32_t (&bqv)[COLS / 32], const float (&invv)[COLS / 32],
@@ -211,12 +214,32 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
                 *reinterpret_cast<uint4 *>(srow + ((g ^ (lane & 7)) << 4)) =
                     make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
             return nb;
-        } else if (row_ok) {
-            float *yrow = a.Y + row * a.N + nb;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (nb + j < a.N) yrow[j] = __uint_as_float(v[j]);
         }
+        if (!ROLLED) {
+            if (row_ok) {
+                float *yrow = a.Y + row * a.N + nb;
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (nb + j < a.N) yrow[j] = __uint_as_float(v[j]);
+            }
+            return -1;
+        }
+        uint8_t *srow = stage + lane * 128;
+        // a width or an address that TMA does not take: row by row, a column a lane, so that a warp's store is one run of 128 bytes.  A lane's
+        // own row, a word at a time, is 32 lines a store: 3000 x 512 -> 2047 with GELU 43-45 -> 17.8 us.
+        __syncwarp();
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4 *>(srow + ((g ^ (lane & 7)) << 4)) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        __syncwarp();
+        const int rows = (int)min((int64_t)32, a.M - row0);
+        if (nb + lane < a.N) {
+#pragma unroll 1
+            for (int r = 0; r < rows; ++r)
+                a.Y[(row0 + r) * a.N + nb + lane] =
+                    *reinterpret_cast<const float *>(stage + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2)));
+        }
+        __syncwarp();
         return -1;
     };
     auto issue_store = [&](int64_t nb) {

@@ -200,7 +200,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         tmem_st_32x32(t_own, part);
         tmem_st_wait();
         float am = 0.0f;
-        epilogue_warp<32, ABSMAX, false, false, OUT>(a, &tmap_y, tma_store == 1, &tmap_y, false, t_own, m0 + quarter * 32, n, bqv, invv,
+        epilogue_warp<32, ABSMAX, false, false, false, OUT>(a, &tmap_y, tma_store == 1, &tmap_y, false, t_own, m0 + quarter * 32, n, bqv, invv,
                                                      smem_stage + mine * kStagingBytesPerWarp, smem_bq + mine * 32, lane, 1, [] {}, am);
         if (ABSMAX) warp_fold_absmax(am, a.y_absmax);
         if (lane == 0) tma_store_wait_all();

@@ -634,6 +634,32 @@ def test_one_cta_tiles_in_every_output_mode(block_n, M, N, K):
         q8.q8_tune_gemm_tile(0, 0)
 
 
+@pytest.mark.parametrize("block_n", [64, 128, 192, 256])
+@pytest.mark.parametrize("M,N,K", [(1, 33, 16), (127, 63, 64), (161, 1001, 272), (20000, 257, 48)])
+def test_one_cta_tiles_of_widths_that_tma_does_not_store(block_n, M, N, K):
+    """Rows that are no multiple of 16 bytes leave in a loop over the block's rows: fp32 alone, with the integers, with the maximum."""
+    X, W, b = synth.activation(M, K, 9470), synth.weight(N, K, 9471), synth.bias(N, 9472)
+    S_y = torch.full((1,), 25.0, device="cuda")
+    try:
+        q8.q8_tune_gemm_tile(block_n, 1)
+        for act in (0, 1):
+            info = check_linear(X, W, b, act)
+            assert (info["gemm_kernel"], info["block_n"], info["ctas"]) == (1, block_n, 1)
+            Wq, S_w = q8.q8_quantize_weight(dev(W))
+            Xd = dev(X)
+            Xq, S_x = q8.q8_quantize_activation(Xd)
+            Y = q8.q8_linear_q(Xq, S_x, Wq, S_w, dev(b), act)
+            Y2 = torch.full((M * N + 64,), 7.0, device="cuda")
+            Yq = q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, dev(b), act, S_y, Y=Y2[: M * N].view(M, N))
+            assert np.array_equal(Yq.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(25.0)))
+            assert torch.equal(Y2[: M * N].view(M, N), Y) and bool((Y2[M * N :] == 7.0).all())
+            word = torch.zeros(1, dtype=torch.int32, device="cuda")
+            Y3 = q8.q8_linear_dyn(Xd, Xd.abs().max().view(torch.int32).reshape(1), Wq, S_w, dev(b), act, y_absmax=word)
+            assert torch.equal(Y3, Y) and word.view(torch.float32).item() == Y.abs().max().item()
+    finally:
+        q8.q8_tune_gemm_tile(0, 0)
+
+
 # ------------------------------------------------------------------ the streaming passes at the ends of their runs
 @pytest.mark.parametrize("n", [1, 5, 511, 2047, 2048, 2049, 4 * 2048 - 3, 16 * 148 * 512 + 7])
 def test_streaming_passes_at_the_ends_of_their_runs(n):
