@@ -753,10 +753,22 @@ cudaError_t launch_fake_quantize(const float *x, int64_t n, const float *S, floa
                                    S, xhat);
 }
 
+// Memory of the current device, which a kernel reaches without more; between devices, from pinned or managed memory the runtime copies.
+static bool on_current_device(const void *p)
+{
+    int device = -1;
+    cudaPointerAttributes at{};
+    if (cudaGetDevice(&device) == cudaSuccess && cudaPointerGetAttributes(&at, p) == cudaSuccess)
+        return at.type == cudaMemoryTypeDevice && at.device == device;
+    cudaGetLastError();
+    return false;
+}
+
 cudaError_t launch_copy(const float *from, int64_t n, float *to, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    if (!aligned16(from) || !aligned16(to)) return cudaMemcpyAsync(to, from, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    if (!aligned16(from) || !aligned16(to) || !on_current_device(from) || !on_current_device(to))
+        return cudaMemcpyAsync(to, from, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
     return launch_overlapping_tail(copy_kernel, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, from, n, to);
 }
 
