@@ -109,10 +109,10 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
     const bool yq_staged = kHasYq && kYqStageable && yq_tma && nch == NCHUNK;
     const int yq_xor = COLS == 128 ? (lane & 7) : ((lane >> 1) & 3);  // 128-byte / 64-byte swizzle of row `lane`
     bool yq_pending = false;
-    // GELU is never below -0.17, so its integers need no lower clamp at scales below 127 / 0.17 = 747.  Such an epilogue is bound by
+    // GELU is never below -0.17, so its integers need no lower clamp at positive scales below 127 / 0.17 = 747.  Such an epilogue is bound by
     // its instructions: with neither the clamp nor scalar products (quantize_pack4_unclamped()) 24576 x 1024 -> 4096 97.7 -> 91.0 us, 8192 x 768
     // -> 3072 28.7 -> 25.4, 4096 x 768 -> 3072 17.5 -> 15.7.
-    const bool above_low_clamp = OUT == (kOutInt8 | kOutGelu) && S_y < 700.0f;
+    const bool above_low_clamp = OUT == (kOutInt8 | kOutGelu) && S_y > 0.0f && S_y < 700.0f;
 
     // Everything after the TMEM load, for the 32-column block ci held in v, up to and including the staging of the
     // fp32 block in shared memory.  Returns the first column of the block when a staged fp32 block now waits for its

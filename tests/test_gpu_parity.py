@@ -634,6 +634,29 @@ def test_one_cta_tiles_in_every_output_mode(block_n, M, N, K):
         q8.q8_tune_gemm_tile(0, 0)
 
 
+@pytest.mark.parametrize("block_n,ctas,warps", [(64, 1, 0), (128, 1, 0), (192, 1, 0), (256, 1, 0), (256, 2, 8), (256, 2, 16)])
+def test_gelu_to_int8_at_any_scale(block_n, ctas, warps):
+    """Eq. 1 on GELU's output at scales on both sides of the line from which its lowest value (-0.17) needs the lower clamp, and at scales
+    that are not positive (-128 never appears), infinite or NaN: the integers of the fp32 output, whatever the tile."""
+    M, N, K = 515, 1040, 272
+    Wq, S_w = q8.q8_quantize_weight(dev(synth.weight(N, K, 9480)))
+    b = dev(synth.bias(N, 9481))
+    Xq, S_x = q8.q8_quantize_activation(dev(synth.activation(M, K, 9482)))
+    try:
+        q8.q8_tune_gemm_tile(block_n, ctas)
+        q8.q8_tune_gemm_epilogue_warps(warps)
+        for scale_x in (S_x, torch.zeros_like(S_x)):  # (a zero product scale: every value is NaN or infinite)
+            Y = q8.q8_linear_q(Xq, scale_x, Wq, S_w, b, 1)
+            if scale_x is S_x:
+                assert Y.min().item() < -0.1699 and Y.max().item() > 0.3  # (-0.17 x 760 is beyond -127.5, 0.3 x 1000 beyond 127)
+            for S in (25.0, 699.0, 700.0, 701.0, 760.0, 5000.0, 0.0, -1.0, -1000.0, np.inf, -np.inf, np.nan):
+                got = q8.q8_linear_q_requant(Xq, scale_x, Wq, S_w, b, 1, dev(np.array([S], np.float32)))
+                assert np.array_equal(got.cpu().numpy(), o.quantize(Y.cpu().numpy(), np.float32(S))), S
+    finally:
+        q8.q8_tune_gemm_epilogue_warps(0)
+        q8.q8_tune_gemm_tile(0, 0)
+
+
 @pytest.mark.parametrize("block_n", [64, 128, 192, 256])
 @pytest.mark.parametrize("M,N,K", [(1, 33, 16), (127, 63, 64), (161, 1001, 272), (20000, 257, 48)])
 def test_one_cta_tiles_of_widths_that_tma_does_not_store(block_n, M, N, K):
