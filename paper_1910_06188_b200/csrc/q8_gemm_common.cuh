@@ -63,7 +63,7 @@ __device__ __forceinline__ uint32_t quantize_pack4_unclamped(float a, float b, f
 // * 1/(S_x S_w) -> GELU -> store.  With tma_store (N % 4 == 0, Y 16-byte aligned) the 32 x 32 fp32
 // block is staged in shared memory in the 128-byte-swizzled layout of the output tensor map
 // (row = lane, 16-byte piece g at position g ^ (lane & 7): bank-conflict free) and written by one
-// TMA store, clipped at the matrix edge by the hardware; otherwise every lane stores its own row.
+// TMA store, clipped at the matrix edge by the hardware; otherwise row by row or every lane its own row (ROLLED).
 // Once the last TMEM load of the tile has landed the accumulator buffer is handed back (release()).
 // ABSMAX: also keep the running max|y| of what is stored (a compile-time switch, so that the ordinary layer carries
 // neither the extra register nor the branch).
@@ -74,12 +74,15 @@ __device__ __forceinline__ uint32_t quantize_pack4_unclamped(float a, float b, f
 // OUT: which outputs the instantiation can write.  kOutPlain: the fp32 Y only; kOutInt8: the Int8 copy
 // only (the fused FFN1 of a forward whose next layer is quantised); kOutFull: whatever the call asks for (fp32, Int8, the
 // debug copy of the accumulator).  Compiling the other paths out keeps the 16-warp kernel (96 registers per thread)
-// free of spills; a spilled value is reloaded from local memory in every block, and under the main loop's traffic
-// that load is not a cache hit.
+// free of spills in its blocks: a value reloaded from local memory in every block is no cache hit under the main loop's traffic.
+// (What is left: one word in the fp32 pairs without GELU, which a form without it does not beat, 8192 x 1024 -> 1024 12.6 / 12.7 us, one
+// in the 256-wide one-CTA GELU to Int8, one or five in the 256-wide one-CTA kOutFull.)
 // All but kOutFull are for one activation: plus kOutGelu with GELU, else without.
 // ROLLED: an fp32 block that TMA does not take leaves through the staging buffer in a loop over its rows, else column by column in line.
 // Tiles of one CTA and 64 columns or more: with it the encoder's 32-wide tiles took 0.4 % longer (1 x 128: 204.6 -> 205.4 us) and the
 // pairs' plain fp32 epilogue 2-4 % (8192 x 1024 -> 1024 12.7 -> 13.2), although neither runs it: the compiler orders the rest differently.
+// The row loop shares the staging of the TMA store and steps a pointer: with a staging and an index of its own the 256-wide tiles with
+// GELU, which the loop is compiled into, spilled 60 bytes (2048 x 1280 -> 2304 11.5 -> 11.0 us, and the loop itself 3000 x 512 -> 2047 15.2 -> 14.2).
 constexpr int kOutPlain = 0, kOutFull = 1, kOutDirect = 2, kOutInt8 = 3, kOutGelu = 4;
 template <int OUT>
 constexpr int kOutKind = OUT & 3;
@@ -109,6 +112,7 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
     const bool yq_staged = kHasYq && kYqStageable && yq_tma && nch == NCHUNK;
     const int yq_xor = COLS == 128 ? (lane & 7) : ((lane >> 1) & 3);  // 128-byte / 64-byte swizzle of row `lane`
     bool yq_pending = false;
+    constexpr bool kStageOnce = kKind != kOutFull;  // one staging of the fp32 block for both ways it leaves (with it the 128-wide kOutFull spills)
     // GELU is never below -0.17, so its integers need no lower clamp at positive scales below 127 / 0.17 = 747.  Such an epilogue is bound by
     // its instructions: with neither the clamp nor scalar products (quantize_pack4_unclamped()) 24576 x 1024 -> 4096 97.7 -> 91.0 us, 8192 x 768
     // -> 3072 28.7 -> 25.4, 4096 x 768 -> 3072 17.5 -> 15.7.
@@ -156,11 +160,12 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
             for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__fmul_rn(__int2float_rn((int32_t)v[j]), inv));
         }
         if (ABSMAX && row_ok) {
-            // running max|y| of this lane over the outputs that exist (Sec. 4.1: the consumer's dynamic scale)
-            const bool whole = nb + 32 <= a.N;
+            // running max|y| of this lane over the outputs that exist (Sec. 4.1: the consumer's dynamic scale).  (Their number and not 64-bit
+            // columns against N: 4096 x 768 -> 3072 with its quantise pass 24.2 -> 22.5 us.)
+            const int cols = (int)min((int64_t)32, a.N - nb);
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-                if (whole || nb + j < a.N) absmax_run = fmaxf(absmax_run, fabsf(__uint_as_float(v[j])));
+                if (j < cols) absmax_run = fmaxf(absmax_run, fabsf(__uint_as_float(v[j])));
         }
         if (kHasYq && a.Yq != nullptr && row_ok) {
             // re-quantised output for the next quantised layer: Eq. 1 at that layer's activation scale
@@ -205,15 +210,18 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
             else quantise([&](float x, float y, float z, float w) { return quantize_pack4(x, y, z, w, S_y); });
         }
         if (!kHasY || a.Y == nullptr) return -1;
-        if (tma_store) {
-            if (!BIAS_IN_STAGE && lane == 0) tma_store_wait_read();  // the previous block has left the staging buffer
+        auto stage_block = [&] {
             __syncwarp();  // (also: every lane has read the bias values before the block overwrites them)
             uint8_t *srow = stage + lane * 128;
 #pragma unroll
             for (int g = 0; g < 8; ++g)
                 *reinterpret_cast<uint4 *>(srow + ((g ^ (lane & 7)) << 4)) =
                     make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-            return nb;
+        };
+        if (tma_store || (ROLLED && kStageOnce)) {
+            if (!BIAS_IN_STAGE && lane == 0) tma_store_wait_read();  // the previous block has left the staging buffer
+            stage_block();
+            if (tma_store) return nb;
         }
         if (!ROLLED) {
             if (row_ok) {
@@ -224,20 +232,16 @@ __device__ __forceinline__ void epilogue_warp(const GemmArgs &a, const CUtensorM
             }
             return -1;
         }
-        uint8_t *srow = stage + lane * 128;
         // a width or an address that TMA does not take: row by row, a column a lane, so that a warp's store is one run of 128 bytes.  A lane's
         // own row, a word at a time, is 32 lines a store: 3000 x 512 -> 2047 with GELU 43-45 -> 17.8 us.
-        __syncwarp();
-#pragma unroll
-        for (int g = 0; g < 8; ++g)
-            *reinterpret_cast<uint4 *>(srow + ((g ^ (lane & 7)) << 4)) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        if (!kStageOnce) stage_block();
         __syncwarp();
         const int rows = (int)min((int64_t)32, a.M - row0);
         if (nb + lane < a.N) {
+            float *y = a.Y + row0 * a.N + nb + lane;
 #pragma unroll 1
-            for (int r = 0; r < rows; ++r)
-                a.Y[(row0 + r) * a.N + nb + lane] =
-                    *reinterpret_cast<const float *>(stage + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2)));
+            for (int r = 0; r < rows; ++r, y += a.N)
+                *y = *reinterpret_cast<const float *>(stage + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2)));
         }
         __syncwarp();
         return -1;
