@@ -135,7 +135,7 @@ q8_status linear_impl(const float *X, const int8_t *Wq, const float *S_w, const 
         last_launch_info().launches += 1;
     } else {
         int words = 1;
-        const bool partial = absmax_partial_preferred(M * K);
+        const bool partial = absmax_partial_preferred(X, M * K);
         if (partial) {
             Q8_CUDA_TRY(launch_absmax_partial(X, M * K, hdr->absmax_partial,
                                               (int)(sizeof(hdr->absmax_partial) / sizeof(hdr->absmax_partial[0])), &words, s));

@@ -601,11 +601,17 @@ cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_
                                    st, decay);
 }
 
-// A dynamic layer of 1024 columns with changing inputs, partial maxima / clear and atomics of eight CTAs per SM, us: 0.6 M values 10.4 /
-// 12.5, 2.0 M 12.3 / 14.3, 4.1 M 14.7 / 16.4, 6.1 M 22.7 / 18.7, 8.2 M 27.3 / 22.5: what no longer stays in L2 wants all of the
-// loads that 8 CTAs have in flight.
-bool absmax_partial_preferred(int64_t n) { return n <= (int64_t(9) << 19); }  // 4.7 M
+// A dynamic layer of 1024 columns, partial maxima / clear and atomics of eight CTAs per SM, us, with changing inputs: 2.1 M values 12.0 /
+// 14.6, 4.6 M 13.9 / 17.8, 6.1 M 16.6 / 19.0, 8.4 M 19.6 / 21.8, 9.2 M 20.3 / 22.7, 9.7 M 25.4 / 23.0, 12.6 M 29.3 / 26.8; with the same one 6.1 M
+// 14.2 / 17.0, 9.2 M 16.8 / 19.1, 12.6 M 22.2 / 22.6: from where the second pass no longer finds the tensor in L2 all of the loads that 8 CTAs
+// have in flight are wanted, and the order of that pass from the end.  Off 16 bytes, where a thread loads a value at a time, 480 CTAs have
+// too few in flight sooner: 4.6 M 20.4 / 20.4, 4.9 M 20.1 / 20.7, 6.1 M 23.0 / 22.3, 8.4 M 27.1 / 25.7.
+bool absmax_partial_preferred(const float *x, int64_t n) { return n <= (int64_t(aligned16(x) ? 17 : 9) << 19); }  // 8.9 M, 4.7 M
 
+// Clusters for a run of 1024 float4 a CTA, four CTAs per SM; the 60 words of the header bound them at 480 CTAs, from 3.9 M values on.  (The
+// kernel takes runs of 2048, so below that half of the CTAs find none.  With as many CTAs as runs, us: 1421 x 768 -> 768 10.3 -> 9.8,
+// 1000 x 300 -> 1200 12.5 -> 12.1, but 1000 x 512 -> 2048 11.1 -> 12.0, 300 x 1000 -> 1000 16.7 -> 18.0, 1000 x 300 -> 256 10.3 -> 11.2: what the idle ones
+// change is where the CTAs of the two kernels behind them start.  Runs of 1024 are slower from 1.4 M values on, 4.2 M 13.6 -> 14.4.)
 cudaError_t launch_absmax_partial(const float *x, int64_t n, uint32_t *partial, int max_words, int *words, cudaStream_t s)
 {
     const bool vec = aligned16(x);

@@ -76,7 +76,7 @@ cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_
                           float decay = 0.0f);
 // max|x| as up to max_words partial maxima; *words receives how many were written (n > 0).  Preferred to a cleared word and
 // launch_absmax() while the tensor is small enough.
-bool absmax_partial_preferred(int64_t n);
+bool absmax_partial_preferred(const float *x, int64_t n);
 cudaError_t launch_absmax_partial(const float *x, int64_t n, uint32_t *partial, int max_words, int *words, cudaStream_t s);
 // *S = 127 / float(*bits) in place (bits and S may alias); flags Q8_ERR_SCALE on 0 / non-finite.
 cudaError_t launch_scale_from_absmax(const uint32_t *bits, float *S, int32_t *status, cudaStream_t s);

@@ -391,7 +391,8 @@ def test_dynamic_quantisation_where_the_cooperative_launch_is_refused(n):
     assert torch.equal(q8.q8_quantize_activation(x)[0], want)
 
 
-@pytest.mark.parametrize("M,K", [(1, 13), (3, 65537), (257, 768), (1000, 300), (4096, 1040), (8192, 1024), (8192, 1040)])
+@pytest.mark.parametrize("M,K", [(1, 13), (3, 65537), (257, 768), (1000, 300), (4096, 1040), (8192, 1024), (8192, 1040),
+                                 (8704, 1024), (8705, 1024), (9000, 1040), (14300, 1024)])
 def test_dynamic_linear_finds_the_peak_of_every_share(M, K):
     """The partial maxima of the abs-max pass: the scale is that of the largest value, in whichever CTA's share it lies."""
     W = synth.weight(16, K, 9100)
@@ -399,10 +400,14 @@ def test_dynamic_linear_finds_the_peak_of_every_share(M, K):
         x = synth.normal((M, K), 1.0, 9101)
         x.flat[at] = 11.0
         Wq, S_w = q8.q8_quantize_weight(dev(W))
-        ws = q8.new_workspace(M, 16, K)
-        q8.q8_linear(dev(x), Wq, S_w, None, None, 0, workspace=ws)
-        assert ws[4:8].view(torch.float32).item() == np.float32(127.0) / np.float32(11.0)
-        assert q8.q8_poll_status(ws) == (q8.Q8_OK, 0)
+        buf = torch.empty(M * K + 1, device="cuda")
+        for off in (0, 1):  # (off 16 bytes a thread loads a value at a time)
+            X = buf[off:M * K + off].view(M, K)
+            X.copy_(torch.from_numpy(x))
+            ws = q8.new_workspace(M, 16, K)
+            q8.q8_linear(X, Wq, S_w, None, None, 0, workspace=ws)
+            assert ws[4:8].view(torch.float32).item() == np.float32(127.0) / np.float32(11.0)
+            assert q8.q8_poll_status(ws) == (q8.Q8_OK, 0)
 
 
 @pytest.mark.parametrize("n", [1, 5, 1023, 4096, 1 << 20, (1 << 20) + 3])
