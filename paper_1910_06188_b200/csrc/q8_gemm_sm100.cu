@@ -409,15 +409,17 @@ bool g_tail_split_enabled = true;          // cut the tiles of a partial last ro
 template <int BLOCK_N, int CTAS, int EW, bool ABSMAX, int OUT>
 cudaError_t launch_cfg_impl(const GemmArgs &a, cudaStream_t s);
 
+// A TMA store needs a 16-byte aligned base and row pitch.
+bool tma_stores(const GemmArgs &a) { return (a.N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0; }
+
 // Unstaged stores of a plain fp32 output: chosen automatically where they measured faster, i.e. with a long main loop
 // (the 8-warp epilogue of the CTA pair, K > 2048: FFN2 75.1 -> 73.7 us, no staging traffic in shared memory, which the
 // operand ring and the tensor cores already load fully); with a short one the staged TMA stores win (QKV 79.5
 // against 85.7 us).  The pair kernels alone have the instantiation.
-template <int CTAS, int EW>
-bool wants_direct_store(const GemmArgs &a)
+bool wants_direct_store(const GemmArgs &a, int epilogue_warps)
 {
-    const bool direct = g_direct_store < 0 ? (CTAS == 2 && EW == 8) : g_direct_store != 0;
-    return CTAS == 2 && direct && a.Y != nullptr && a.Yq == nullptr && a.dbg_acc == nullptr && ((a.N & 1) == 0) &&
+    const bool direct = g_direct_store < 0 ? epilogue_warps == 8 : g_direct_store != 0;
+    return direct && a.Y != nullptr && a.Yq == nullptr && a.dbg_acc == nullptr && ((a.N & 1) == 0) &&
            ((reinterpret_cast<uintptr_t>(a.Y) & 7u) == 0);
 }
 
@@ -428,7 +430,7 @@ cudaError_t launch_cfg_act(const GemmArgs &a, cudaStream_t s)
 {
     if (a.Yq != nullptr && a.Y == nullptr) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8 | GELU>(a, s);
     if constexpr (CTAS == 2) {
-        if (wants_direct_store<CTAS, EW>(a)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutDirect | GELU>(a, s);
+        if (wants_direct_store(a, EW)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutDirect | GELU>(a, s);
     }
     return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutPlain | GELU>(a, s);
 }
@@ -510,9 +512,7 @@ cudaError_t launch_cfg_impl(const GemmArgs &a, cudaStream_t s)
         tw2 = tw;  // never used
         tw4 = tw;
     }
-    // the TMA store needs a 16-byte aligned base and row pitch; otherwise lanes store their rows directly
-    int tma_store = kOutKind<OUT> != kOutDirect && a.Y != nullptr && ((a.N & 3) == 0) &&
-                    ((reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0);
+    int tma_store = kOutKind<OUT> != kOutDirect && a.Y != nullptr && tma_stores(a);
     if (tma_store) {
         if (!make_tmap_out(&ty, a.Y, a.M, a.N)) return cudaErrorInvalidValue;
     } else {
@@ -563,13 +563,12 @@ double tile_cost(int bn, int64_t rounds, int64_t K)
     return (double)rounds * (step * (double)K / 32.0 + 500.0) + 10.0 * bn;
 }
 
+// a short main loop (small K) leaves the epilogue on the critical path: give it twice the warps
+int pair_epilogue_warps(const GemmArgs &a) { return g_force_epilogue_warps ? g_force_epilogue_warps : a.K <= 2048 ? 16 : 8; }
+
 cudaError_t launch_by_shape(int bn, int ctas, const GemmArgs &a, cudaStream_t s)
 {
-    if (ctas == 2) {
-        // a short main loop (small K) leaves the epilogue on the critical path: give it twice the warps
-        const bool wide_epilogue = g_force_epilogue_warps ? g_force_epilogue_warps == 16 : a.K <= 2048;
-        return wide_epilogue ? launch_cfg<256, 2, 16>(a, s) : launch_cfg<256, 2, 8>(a, s);
-    }
+    if (ctas == 2) return pair_epilogue_warps(a) == 16 ? launch_cfg<256, 2, 16>(a, s) : launch_cfg<256, 2, 8>(a, s);
     // A one-CTA tile is mostly the only one of its CTA, so its epilogue is exposed: with GELU in it as many warps as there are 64-column
     // (128: 32-column) shares, 1421 x 768 -> 3072 10.0 -> 9.2 us, 1000 x 768 -> 3072 8.3 -> 7.6, 509 x 1024 -> 4096 to Int8 7.1 -> 6.5;
     // without GELU it is short enough and the staging buffers are better spent on the ring (4096 x 4096 -> 1024 17.9 for 19.7).
@@ -620,7 +619,11 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
     // 2048 x 768 -> 3072 with GELU 11.85 / 11.3, 3200 x 512 -> 2048 11.4 / 10.4 (but 2048 x 1024 -> 3072 11.0 / 11.15).
     const int64_t pair_tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
     const bool second_round_thin = a.K <= 768 && 2 * pair_tiles > sms && 4 * pair_tiles <= 3 * sms;
-    if (a.N >= 192 && a.M > 128 && pair_tiles >= sms / 2 && !second_round_thin) return launch_by_shape(256, 2, a, s);
+    // Nor for an fp32 output that neither TMA nor the unstaged store takes: pairs store it a lane a row, 32 lines a store, one-CTA tiles row by
+    // row (4096 x 1024 -> 2047 63.5 us with pairs, 20.2 with one-CTA tiles, 24576 x 1024 -> 1023 189 / 52.5, 8192 x 4096 -> 1023 66.9 / 35.0,
+    // 256 x 768 -> 30522 69.1 / 19.5; of 2 x 20 layers with odd widths none is faster with pairs).
+    const bool pairs_store = a.Y == nullptr || tma_stores(a) || wants_direct_store(a, pair_epilogue_warps(a));
+    if (pairs_store && a.N >= 192 && a.M > 128 && pair_tiles >= sms / 2 && !second_round_thin) return launch_by_shape(256, 2, a, s);
     // Otherwise single-CTA tiles of the cheapest width.
     const int64_t tm = (a.M + BLOCK_M - 1) / BLOCK_M;
     int best = 32;
@@ -645,7 +648,7 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
         if (best == 32 && 2 * tm * ((a.N + 63) / 64) <= sms) return launch_gemm_splitk(a, false, s);
     }
     // One round of the widest tiles with a long K: the pair does the same with fewer operand bytes (4096 x 4096 -> 1024 18.1 us / 17.2).
-    if (best == 256 && a.K >= 2048 && a.M > 128) return launch_by_shape(256, 2, a, s);
+    if (pairs_store && best == 256 && a.K >= 2048 && a.M > 128) return launch_by_shape(256, 2, a, s);
     return launch_by_shape(best, 1, a, s);
 }
 

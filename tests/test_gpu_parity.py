@@ -688,6 +688,27 @@ def test_one_cta_tiles_of_widths_that_tma_does_not_store(block_n, M, N, K):
         q8.q8_tune_gemm_tile(0, 0)
 
 
+@pytest.mark.parametrize("N,off,K,ctas", [(1024, 0, 64, 2), (1023, 0, 64, 1), (1022, 0, 64, 1), (1024, 1, 64, 1), (1024, 2, 64, 1),
+                                          (1022, 0, 2064, 2), (1022, 1, 2064, 1), (1023, 0, 2064, 1)])
+def test_layers_whose_output_pairs_cannot_store_take_one_cta_tiles(N, off, K, ctas):
+    """A grid full of pairs: fp32 rows that neither TMA nor the paired 8-byte stores take (K > 2048 for these) leave through one-CTA tiles;
+    the Int8 output does not ask."""
+    M = 9500
+    Xq, S_x = q8.q8_quantize_activation(dev(synth.activation(M, K, 9490)))
+    Wq, S_w = q8.q8_quantize_weight(dev(synth.weight(N, K, 9491)))
+    b = dev(synth.bias(N, 9492))
+    room = torch.full((M * N + 64,), 7.0, device="cuda")
+    Y = room[off:M * N + off].view(M, N)
+    q8.q8_linear_q(Xq, S_x, Wq, S_w, b, 0, Y=Y)
+    assert q8.q8_last_launch_info()["ctas"] == ctas
+    assert bool((room[:off] == 7.0).all()) and bool((room[M * N + off:] == 7.0).all())
+    q8.q8_linear_q_requant(Xq, S_x, Wq, S_w, b, 0, torch.full_like(S_x, 25.0))
+    assert q8.q8_last_launch_info()["ctas"] == 2
+    acc = Xq.double() @ Wq.double().T + torch.round(b * (S_x * S_w)).double()  # exact: below 2^53
+    inv = torch.ones_like(S_x) / (S_x * S_w)
+    assert torch.equal(Y, acc.float() * inv)
+
+
 # ------------------------------------------------------------------ the streaming passes at the ends of their runs
 @pytest.mark.parametrize("n", [1, 5, 511, 2047, 2048, 2049, 4 * 2048 - 3, 16 * 148 * 512 + 7])
 def test_streaming_passes_at_the_ends_of_their_runs(n):
