@@ -428,7 +428,9 @@ bool wants_direct_store(const GemmArgs &a, int epilogue_warps)
 template <int BLOCK_N, int CTAS, int EW, bool ABSMAX, int GELU>
 cudaError_t launch_cfg_act(const GemmArgs &a, cudaStream_t s)
 {
-    if (a.Yq != nullptr && a.Y == nullptr) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutInt8 | GELU>(a, s);
+    if constexpr (!ABSMAX) {
+        if (a.Yq != nullptr) return launch_cfg_impl<BLOCK_N, CTAS, EW, false, kOutInt8 | GELU>(a, s);
+    }
     if constexpr (CTAS == 2) {
         if (wants_direct_store(a, EW)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutDirect | GELU>(a, s);
     }
@@ -437,7 +439,8 @@ cudaError_t launch_cfg_act(const GemmArgs &a, cudaStream_t s)
 template <int BLOCK_N, int CTAS, int EW, bool ABSMAX>
 cudaError_t launch_cfg_out(const GemmArgs &a, cudaStream_t s)
 {
-    if (a.dbg_acc != nullptr || (a.Yq != nullptr && a.Y != nullptr)) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutFull>(a, s);
+    // (no call asks for the maximum and the Int8 copy at once, so that has no form of its own)
+    if (a.dbg_acc != nullptr || (a.Yq != nullptr && (ABSMAX || a.Y != nullptr))) return launch_cfg_impl<BLOCK_N, CTAS, EW, ABSMAX, kOutFull>(a, s);
     // (launch_by_shape() has one-CTA tiles of 128 columns and more for each activation)
     if constexpr (CTAS == 2 || BLOCK_N < 128 || EW > 8) {
         if (a.act == Q8_ACT_GELU) return launch_cfg_act<BLOCK_N, CTAS, EW, ABSMAX, kOutGelu>(a, s);
