@@ -775,7 +775,9 @@ cudaError_t launch_copy(const float *from, int64_t n, float *to, cudaStream_t s)
     if (n <= 0) return cudaSuccess;
     if (!aligned16(from) || !aligned16(to) || !on_current_device(from) || !on_current_device(to))
         return cudaMemcpyAsync(to, from, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
-    return launch_overlapping_tail(copy_kernel, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, from, n, to);
+    const cudaError_t e = launch_overlapping_tail(copy_kernel, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, from, n, to);
+    last_launch_info().launches += e == cudaSuccess;
+    return e;
 }
 
 cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, const float *S_e, int64_t V,

@@ -325,6 +325,33 @@ def test_fake_quantize_and_ste(n):
     assert q8.q8_ste_backward(gd, gd).data_ptr() == gd.data_ptr()
 
 
+@pytest.mark.parametrize("n", [3, 2049, 100_003])
+def test_straight_through_copy_by_kernel_and_by_the_runtime(n):
+    """One launch for aligned memory of the device, also where a stream is captured; addresses off 16 bytes on either side and pinned host
+    memory go to the runtime's copy, which counts as no launch."""
+    g = dev(synth.normal((n,), 1.0, 1450))
+    assert torch.equal(q8.q8_ste_backward(g), g) and q8.q8_last_launch_info()["launches"] == 1
+    for off_in, off_out in ((1, 0), (0, 1), (2, 2), (3, 1)):
+        src, room = torch.zeros(n + 4, device="cuda"), torch.full((n + 8,), 9.0, device="cuda")
+        src[off_in:off_in + n] = g
+        q8.q8_ste_backward(src[off_in:off_in + n], room[off_out:off_out + n])
+        assert q8.q8_last_launch_info()["launches"] == 0
+        assert torch.equal(room[off_out:off_out + n], g)
+        assert bool((room[:off_out] == 9.0).all()) and bool((room[off_out + n:] == 9.0).all())
+    pinned, out = torch.empty(n, pin_memory=True), torch.zeros(n, device="cuda")
+    pinned.copy_(g)
+    torch.cuda.synchronize()
+    assert q8.load().q8_ste_backward(pinned.data_ptr(), n, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == q8.Q8_OK
+    assert torch.equal(out, g)
+    graph, moved, off = torch.cuda.CUDAGraph(), torch.zeros(n, device="cuda"), torch.zeros(n + 1, device="cuda")
+    with torch.cuda.graph(graph):
+        q8.q8_ste_backward(g, moved)
+        q8.q8_ste_backward(g, off[1:])
+    g.mul_(-3.0)
+    graph.replay()
+    assert torch.equal(moved, g) and torch.equal(off[1:], g)
+
+
 # ------------------------------------------------------------------ one weight scale per fused layer (Eq. 3 per layer)
 @pytest.mark.parametrize("M,H,seg,act", [(300, 128, 128, 0), (515, 256, 256, 1), (64, 40, 40, 0)])
 def test_fused_projection_with_per_layer_scales_equals_separate_layers(M, H, seg, act):
