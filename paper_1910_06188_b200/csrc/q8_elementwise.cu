@@ -776,6 +776,10 @@ cudaError_t launch_copy(const float *from, int64_t n, float *to, cudaStream_t s)
     if (!aligned16(from) || !aligned16(to) || !on_current_device(from) || !on_current_device(to))
         return cudaMemcpyAsync(to, from, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
     const cudaError_t e = launch_overlapping_tail(copy_kernel, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, from, n, to);
+    if (e == cudaErrorInvalidResourceHandle) {  // another device's stream, in which the runtime copies and launches nothing
+        cudaGetLastError();
+        return cudaMemcpyAsync(to, from, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    }
     last_launch_info().launches += e == cudaSuccess;
     return e;
 }

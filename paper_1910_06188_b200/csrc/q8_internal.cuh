@@ -106,7 +106,7 @@ cudaError_t launch_quantize_dynamic_grid(const float *x, int64_t n, float *S_out
                                          cudaStream_t s);
 void set_quantize_grid(int ctas);  // CTAs of the cooperative launch, 0 automatic
 cudaError_t launch_fake_quantize(const float *x, int64_t n, const float *S, float *xhat, cudaStream_t s);
-// By a kernel (counted as a launch) where both are 16-byte aligned memory of the current device, else by the runtime.
+// By a kernel (counted as a launch) where both are 16-byte aligned memory of the current device and of the stream's, else by the runtime.
 cudaError_t launch_copy(const float *from, int64_t n, float *to, cudaStream_t s);
 cudaError_t launch_embedding(const int32_t *ids, int64_t T, const int8_t *Eq, const float *S_e, int64_t V,
                              int64_t H, float *out, int8_t *rows_q, int32_t *status, cudaStream_t s);
