@@ -601,12 +601,12 @@ cudaError_t launch_absmax(const float *x, int64_t n, uint32_t *bits, cudaStream_
                                    st, decay);
 }
 
-// A dynamic layer of 1024 columns, partial maxima / clear and atomics of eight CTAs per SM, us, with changing inputs: 2.1 M values 12.0 /
-// 14.6, 4.6 M 13.9 / 17.8, 6.1 M 16.6 / 19.0, 8.4 M 19.6 / 21.8, 9.2 M 20.3 / 22.7, 9.7 M 25.4 / 23.0, 12.6 M 29.3 / 26.8; with the same one 6.1 M
-// 14.2 / 17.0, 9.2 M 16.8 / 19.1, 12.6 M 22.2 / 22.6: from where the second pass no longer finds the tensor in L2 all of the loads that 8 CTAs
-// have in flight are wanted, and the order of that pass from the end.  Off 16 bytes, where a thread loads a value at a time, 480 CTAs have
-// too few in flight sooner: 4.6 M 20.4 / 20.4, 4.9 M 20.1 / 20.7, 6.1 M 23.0 / 22.3, 8.4 M 27.1 / 25.7.
-bool absmax_partial_preferred(const float *x, int64_t n) { return n <= (int64_t(aligned16(x) ? 17 : 9) << 19); }  // 8.9 M, 4.7 M
+// A dynamic layer on 16-byte aligned inputs, partial maxima / clear and atomics of eight CTAs per SM, us, inputs that change / the same one:
+// 5000 x 1024 -> 1024 24.3 / 24.9 and 18.4 / 21.9, 6000 x 1024 -> 3072 33.6 / 37.1 and 33.2 / 37.0, 2407 x 3072 -> 2496 34.3 / 35.4 and 29.7 / 31.1,
+// 2000 x 4096 -> 1024 30.9 / 29.2 and 23.8 / 25.7, 8192 x 1024 -> 1024 32.2 / 31.5 and 26.2 / 26.9, 2407 x 3648 -> 2496 41.5 / 41.1: the line lies where
+// the second pass starts to miss what the first has left in L2, and the order of that pass from the end begins to count.  Off 16 bytes,
+// where a thread loads a value at a time, the 480 CTAs have too few in flight sooner: 4.6 M values 20.4 / 20.4, 6.1 M 23.0 / 22.3, 8.4 M 27.1 / 25.7.
+bool absmax_partial_preferred(const float *x, int64_t n) { return n <= (int64_t(aligned16(x) ? 14 : 9) << 19); }  // 7.3 M, 4.7 M
 
 // Clusters for a run of 1024 float4 a CTA, four CTAs per SM; the 60 words of the header bound them at 480 CTAs, from 3.9 M values on.  (The
 // kernel takes runs of 2048, so below that half of the CTAs find none.  With as many CTAs as runs, us: 1421 x 768 -> 768 10.3 -> 9.8,
