@@ -154,15 +154,19 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // The weights of the first tiles are on their way into L2 while the kernel before this one still runs, each column of tiles fetched
     // by one unit.  (Into L2 only: should that kernel write them, what is fetched there is what it leaves.  Forward of 32 x 128 tokens
     // 537 -> 524 us, 1 x 128 from a graph 215.6 -> 211; with every unit fetching its own tile's 16 x 512 is 1.2 % slower.)
+    // All of K for small weights, else its first 8 k-blocks: more is in the way of the kernel before and of this one's own loads (with all of K /
+    // with 8, behind their quantise pass, us: 2000 x 4496 -> 2496 43.8 / 39.5, 2407 x 3648 -> 1920 31.5 / 30.3, 1000 x 4096 -> 4096 23.2 / 22.5, 500 x
+    // 4096 -> 4096 18.0 / 17.1, 4096 x 4096 -> 1024 32.2 / 32.2, but 4096 x 3072 -> 768 22.2 / 23.1, 2500 x 2048 -> 1024 15.6 / 15.9).
     if (warp == 3 && lane == 0 && num_tiles <= 3 * num_units) {
         int64_t m_idx, n_start;
         int width;
         decode(unit, m_idx, n_start, width);
         const int b_rows = width / CTAS;
         const CUtensorMap *map_w = width == BLOCK_N ? &tmap_w : (width * 2 == BLOCK_N ? &tmap_w2 : &tmap_w4);
-        for (int kb = 0; m_idx == 0 && kb < num_kb; ++kb) tma_prefetch_2d(map_w, kb * BLOCK_K, (int32_t)(n_start + cta_rank * b_rows));
+        const int ahead = a.N * a.K <= (int64_t(3) << 20) ? num_kb : min(num_kb, 8);
+        for (int kb = 0; m_idx == 0 && kb < ahead; ++kb) tma_prefetch_2d(map_w, kb * BLOCK_K, (int32_t)(n_start + cta_rank * b_rows));
     }
-    // everything above touched only this CTA's own resources; the kernel before this one in the stream (which
+    // everything above touched only this CTA's own resources and L2; the kernel before this one in the stream (which
     // produced X_q) must be complete before anything below reads global memory
     grid_dependency_release_next(num_tiles <= 3 * num_units);  // up to three rounds of tiles count as small
     grid_dependency_wait();
