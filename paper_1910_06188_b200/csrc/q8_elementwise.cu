@@ -701,7 +701,8 @@ cudaError_t launch_quantize(const float *x, int64_t n, const float *S, int8_t *x
 {
     if (n <= 0) return cudaSuccess;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
-        return launch_overlapping_tail(quantize_kernel<true>, dim3(stream_grid(n)), dim3(kStreamThreads), 0, s, x, n, S, xq, xq_copy, nullptr, 1, nullptr, status, clear_word);
+        return launch_overlapping_tail_evenly<quantize_kernel<true>>(dim3(stream_grid(n)), dim3(kStreamThreads), s, x, n, S, xq, xq_copy, nullptr, 1,
+                                                                     nullptr, status, clear_word);
     } else {
         quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, S, xq, xq_copy, nullptr, 1, nullptr,
                                                                                  status, clear_word);
@@ -715,9 +716,13 @@ cudaError_t launch_quantize_dynamic(const float *x, int64_t n, const uint32_t *a
     if (n <= 0) return cudaSuccess;
     int32_t *clear_word = clear_status ? status : nullptr;
     if (aligned16(x) && aligned16(xq) && (xq_copy == nullptr || aligned16(xq_copy))) {
-        const int threads = again ? kThreads : kStreamThreads;
-        return launch_overlapping_tail(again ? quantize_kernel<true, true> : quantize_kernel<true>, dim3(stream_grid(n, threads)), dim3(threads),
-                                       0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
+        if (again || absmax_count > 1) {  // behind an abs-max pass, beside which they park as they would on a free SM
+            const int threads = again ? kThreads : kStreamThreads;
+            return launch_overlapping_tail(again ? quantize_kernel<true, true> : quantize_kernel<true>, dim3(stream_grid(n, threads)), dim3(threads),
+                                           0, s, x, n, nullptr, xq, xq_copy, absmax_bits, absmax_count, S_out, status, clear_word);
+        }
+        return launch_overlapping_tail_evenly<quantize_kernel<true>>(dim3(stream_grid(n)), dim3(kStreamThreads), s, x, n, nullptr, xq, xq_copy,
+                                                                     absmax_bits, absmax_count, S_out, status, clear_word);
     } else {
         quantize_kernel<false><<<grid_for(n, kThreads * 4, 8), kThreads, 0, s>>>(x, n, nullptr, xq, xq_copy, absmax_bits,
                                                                                  absmax_count, S_out, status, clear_word);
