@@ -574,7 +574,8 @@ def test_embed_layernorm_flags_what_is_out_of_range():
 @pytest.mark.parametrize("rows,H", [(2367, 96), (2369, 96), (4096, 96), (4736, 96), (4737, 96), (4737, 32), (9473, 256), (4737, 260),
                                     (4737, 512), (2369, 516), (2369, 768), (4737, 772), (2369, 1024), (301, 1028)])
 def test_add_layernorm_at_the_bounds_of_its_grids(rows, H):
-    """One, two and more rounds of rows (148 SMs x 16 or 32 rows), each of its forms: row by row the same results."""
+    """CTAs of four rows, the last one whole or not, fewer and more than the device takes at once, each of its forms: row by row the same
+    results."""
     g = torch.Generator(device="cuda").manual_seed(rows)
     x, r = (torch.randn((rows, H), generator=g, device="cuda") for _ in range(2))
     whole = q8.q8_add_layernorm(x, r)

@@ -378,7 +378,7 @@ def test_fused_projection_with_per_layer_scales_equals_separate_layers(M, H, seg
 
 # ------------------------------------------------------------------ routes of the dynamic scale
 @pytest.mark.parametrize("n", [1, 3, 4, 4095, 196607, 196608, 196612, 300001, 1 << 20, (2 << 20) - 1, 2 << 20, (2 << 20) + 5,
-                               (4 << 20) - 1, 4 << 20, (4 << 20) + 5])
+                               (4 << 20) - 1, 4 << 20, (4 << 20) + 5, 148 * 8 * 4096 + 5, 2 * 148 * 8 * 4096 + 12343])
 @pytest.mark.parametrize("peak_at", ["first", "last"])
 def test_dynamic_quantisation_in_one_or_several_launches(n, peak_at):
     """One cluster, one cooperative grid or separate passes (by size): the same integers, the same scale, and the largest
@@ -737,12 +737,15 @@ def test_layers_whose_output_pairs_cannot_store_take_one_cta_tiles(N, off, K, ct
 
 
 # ------------------------------------------------------------------ the streaming passes at the ends of their runs
-@pytest.mark.parametrize("n", [1, 5, 511, 2047, 2048, 2049, 4 * 2048 - 3, 16 * 148 * 512 + 7])
-def test_streaming_passes_at_the_ends_of_their_runs(n):
-    """Quantise, abs-max with the Eq. 4 update, fake quantise and the straight-through copy: a CTA's run is 4 x 128 float4 (8 x 512
-    of the abs-max), the last run is ragged and up to three values are left over."""
+@pytest.mark.parametrize("n", [1, 5, 511, 2047, 2048, 2049, 4 * 2048 - 3, 16 * 148 * 512 + 7, 148 * 8 * 2048, 148 * 8 * 2048 + 1,
+                               148 * 8 * 4096 + 5, 2 * 148 * 8 * 4096 + 12343])
+@pytest.mark.parametrize("peak_at", [0, -1])
+def test_streaming_passes_at_the_ends_of_their_runs(n, peak_at):
+    """Quantise, abs-max with the Eq. 4 update, fake quantise and the straight-through copy: a CTA's run is 4 x 128 float4 (4 x 256
+    of the abs-max, whose 8 CTAs per SM take a second and a third run on the two largest), the last run is ragged and up to three values
+    are left over."""
     x = synth.normal((n,), 1.0, 9100 + n % 1000)
-    x[-1] = 7.5  # the largest value is the last one
+    x[peak_at] = 7.5  # the largest value is the first or the last one
     xd, S = dev(x), dev(np.array([12.7], np.float32))
     assert np.array_equal(q8.q8_quantize_activation(xd, S)[0].cpu().numpy(), o.quantize(x, np.float32(12.7)))
     state = q8.new_calibrate_state()
