@@ -44,8 +44,8 @@ void q8_tune_gemm_direct_store(int mode);
  * of this host thread: 1 (not cut), 2 or 4. */
 int q8_last_launch_tail_split(void);
 
-/* How the most recent tcgen05 GEMM launch of this host thread wrote its fp32 output: 0 every lane stored its own
- * row (Y not aligned for a TMA store, or no fp32 output), 1 staged in shared memory and stored by TMA, 2 stored
+/* How the most recent tcgen05 GEMM launch of this host thread wrote its fp32 output: 0 by the lanes, row after row or each
+ * its own row (Y not aligned for a TMA store, or no fp32 output), 1 staged in shared memory and stored by TMA, 2 stored
  * straight from the accumulator fragments (see q8_tune_gemm_direct_store). */
 int q8_last_launch_store_mode(void);
 

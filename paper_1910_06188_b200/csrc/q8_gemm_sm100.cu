@@ -636,8 +636,8 @@ cudaError_t launch_gemm_tcgen05(const GemmArgs &a, cudaStream_t s)
     int best = 32;
     double best_cost = 0.0;
     // (192 is what fits BERT-Base's N = 768 on 32 rows of tiles: 4096 x 768 -> 768 8.2 -> 6.95 us, 4096 x 3072 -> 768 13.9 -> 11.3
-    // with 128 CTAs instead of 96.  An Int8-only output gains as much, although its 96 columns per warp leave in 16-byte pieces and
-    // not by TMA: 768 x 1024 -> 4096 with GELU 8.6 us, 9.9 with 128, 10.9 with 256; fp32 9.0 / 9.8 / 10.7)
+    // with 128 CTAs instead of 96.  An Int8-only output gains as much, also without GELU, where its 96 columns per warp leave in 16-byte
+    // pieces; with GELU a warp has 64, which leave by TMA.)
     for (int bn : {256, 192, 128, 64, 32}) {
         if (bn > 32 && bn / 2 >= a.N) continue;  // more than half of the tile would be padding
         const int64_t tiles = tm * ((a.N + bn - 1) / bn);

@@ -161,15 +161,18 @@ q8_status linear_impl(const float *X, const int8_t *Wq, const float *S_w, const 
 // A kernel launched with launch_overlapping_tail() may be scheduled while the kernel before it in the stream is
 // still draining (its last CTAs finishing), so that its own start-up overlaps that tail.  Such a kernel must call
 // grid_dependency_wait() before its first global-memory access: the call returns once the preceding kernel has
-// completed and its writes are visible (and at once when the kernel was launched the ordinary way).
+// completed and its writes are visible (and at once when the kernel was launched the ordinary way).  (The GEMMs ask for weights before
+// it, into L2 only, where what an earlier kernel writes lands as well.)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the NEXT kernel in the stream (if it was launched with launch_overlapping_tail) be scheduled as soon as every
 // CTA of this grid has started, instead of when the last one exits: its CTAs then sit resident, parked in their own
 // grid_dependency_wait(), and start the moment this grid has completed.  It does not weaken any ordering: the next
-// kernel still touches global memory only after its wait, i.e. after this whole grid has finished.  Kernels call it
-// only for SMALL problems (`small`, a grid-uniform condition), where launch latency is a visible share of the run
+// kernel still touches global memory only after its wait, i.e. after this whole grid has finished.  The GEMMs and the quantise
+// passes call it only for SMALL problems (`small`, a grid-uniform condition), where launch latency is a visible share of the run
 // time: a BERT-Base forward (32 x 128 tokens) replayed from a graph goes from 1.39 to 1.34 ms; on large problems
-// the parked CTAs only get in the way (the M = 24576 FC step went from 505 to 528 us), so those keep the default.
+// the parked CTAs only get in the way (the M = 24576 FC step went from 505 to 528 us), so those keep the default.  Attention, the
+// warp-per-row LayerNorms and the abs-max pass in front of one CTA call it at any size: their CTAs are short and many, so that the last of
+// them start when the grid is nearly done and nothing is parked for long.
 __device__ __forceinline__ void grid_dependency_release_next(bool small)
 {
     if (small) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
